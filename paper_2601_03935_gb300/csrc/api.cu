@@ -8,6 +8,7 @@
 #include <new>
 #include <random>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/gsis.h"
@@ -88,16 +89,15 @@ struct gsis_ctx {
                                  // last MACRO_TAIL inner iterations (2)
     int tcm = 0;                 // FP32 path: gas moments on tensor cores (1: standalone passes, 2: also the sweep)
     int tc_wait = 1 << 22;       // polls of the first tensor-core completion wait (gsis_set_wait_limit)
-    int *m_fi_i = nullptr, *m_fi_j = nullptr, *m_cface = nullptr, *m_pkind = nullptr;
-    double *m_fi_n = nullptr, *m_fi_S = nullptr, *m_fi_dn = nullptr, *m_fi_dist = nullptr, *m_fi_t = nullptr,
-           *m_fi_dx = nullptr, *m_lsq = nullptr, *m_eps2 = nullptr, *m_bf_n = nullptr,
-           *m_bf_S = nullptr, *m_bf_dn = nullptr, *m_pstate = nullptr;
+    int *m_cface = nullptr, *m_pkind = nullptr;
+    double *m_bf_n = nullptr, *m_pstate = nullptr, *m_binc = nullptr;
     double *vqd_x = nullptr, *vqd_w = nullptr, *oqd_x = nullptr, *oqd_w = nullptr;
-    double *W[2] = {nullptr, nullptr}, *mq = nullptr, *mgrad = nullptr, *mphi = nullptr, *Rg = nullptr,
-           *Dinv = nullptr, *gam = nullptr, *dG[2] = {nullptr, nullptr}, *rpart = nullptr, *hot = nullptr,
-           *hot_b = nullptr, *kbf = nullptr, *mbf = nullptr, *fields_h = nullptr, *fields_n = nullptr,
-           *mhist = nullptr;
-    MacroState *mstate = nullptr;
+    MacroWork mw{};              // state and work arrays of the synthetic equations (1-D and 2-D)
+    m3::Geom3 g3{};              // 3-D: geometry, state and work arrays of macro3d.cu
+    struct {
+        double *W[2], *q, *grad, *phi, *Rg, *Dinv, *gam, *dG[2], *rpart, *hot, *mbf;
+    } w3{};
+    double *hot_b = nullptr, *kbf = nullptr, *fields_h = nullptr, *fields_n = nullptr, *mhist = nullptr;
     MacroState *h_mstate = nullptr;   // pinned: initial state and the polled stop flag
     int last_inner = 0;
     cudaGraphExec_t macro_exec = nullptr;   // POLL inner iterations, captured once
@@ -400,39 +400,90 @@ int cis_iteration(gsis_ctx *c) {
 QuadD vquad_d(const gsis_ctx *c) { return QuadD{c->Vd, c->Vdp, c->vqd_x, c->vqd_w}; }
 QuadD oquad_d(const gsis_ctx *c) { return QuadD{c->NOd, c->Odp, c->oqd_x, c->oqd_w}; }
 
-// Pseudo-time iterations of the synthetic equations from W[0] until ||R|| <= tol_inner
-// ||R_0|| or max_inner; returns the index of the buffer that holds the result.  The
-// device stop flag is polled every POLL iterations (one stream synchronisation each).
-// enqueue one inner iteration reading W[w] and writing W[1 - w]; returns a CUDA status
-// fp32: the residual side of this iteration in FP32.
-cudaError_t enqueue_inner(gsis_ctx *c, int w, int fp32, int *kernels) {
-    const MacroGeom &g = c->mg;
-    const gsis_solver_params &sp = c->solver;
-    const int nparts = macro_rpart_count((int)c->nc);
-    const int sweeps = std::max(sp.macro_sweeps, 1);
-    cudaError_t e;
-    if ((e = launch_macro_grad(c->stream, g, c->order, fp32, c->model, c->mstate, c->W[w], c->mq, c->mgrad, c->mphi)))
-        return e;
-    if ((e = launch_macro_bflux(c->stream, g, fp32, c->model, vquad_d(c), oquad_d(c), c->mstate, c->mq, c->mbf))) return e;
-    if ((e = launch_macro_residual(c->stream, g, c->order, fp32, c->model, sp.cfl_macro, c->mstate, c->W[w], c->mq,
-                                   c->mgrad, c->mphi, c->hot, c->mbf, c->hot_b, c->Rg, c->Dinv, c->gam, c->rpart)))
-        return e;
-    if ((e = launch_macro_norm(c->stream, nparts, c->rpart, c->mstate, c->mhist))) return e;
-    for (int sw = 0; sw < sweeps; ++sw)
-        if ((e = launch_macro_jacobi(c->stream, g, fp32, c->model, c->mstate, sw == 0, sw == sweeps - 1, c->W[w],
-                                     c->mq, c->Rg, c->Dinv, c->gam, c->dG[sw & 1], c->dG[(sw + 1) & 1],
-                                     c->W[1 - w])))
-            return e;
-    *kernels += 4 + sweeps - (g.n_bf == 0 ? 1 : 0);
-    return cudaSuccess;
+// The velocity and direction sets of the synthetic equations' boundary fluxes (vqd_*, oqd_*)
+// as the kernels read them: the velocities in each compute type, and the sums that do not
+// change.  A solve captured before belongs to the previous sets.
+int macro_velocity_set(gsis_ctx *c) {
+    if (c->dim == 3) return GSIS_OK;
+    MacroGeom &g = c->mg;
+    g.d.vx = c->vqd_x;
+    g.d.vw = c->vqd_w;
+    if (c->mfp32) {
+        const size_t n = 4 * (size_t)c->Vdp;
+        std::vector<double> h(n);
+        CUDA_TRY(c, cudaMemcpy(h.data(), c->vqd_x, 3 * (size_t)c->Vdp * sizeof(double), cudaMemcpyDeviceToHost));
+        CUDA_TRY(c, cudaMemcpy(h.data() + 3 * (size_t)c->Vdp, c->vqd_w, (size_t)c->Vdp * sizeof(double),
+                               cudaMemcpyDeviceToHost));
+        const std::vector<float> hf(h.begin(), h.end());
+        float *p = nullptr;
+        TRY(dalloc(c, &p, n));
+        TRY(upload(c, p, hf));
+        g.f.vx = p;
+        g.f.vw = p + 3 * (size_t)c->Vdp;
+    }
+    for (cudaGraphExec_t *x : {&c->macro_exec, &c->macro_exec64})
+        if (*x) {
+            CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+            CUDA_TRY(c, cudaGraphExecDestroy(*x));
+            *x = nullptr;
+        }
+    return launch(c, K_MBFLUX, [&] {
+        return launch_macro_binc(c->stream, g, c->model, vquad_d(c), oquad_d(c), c->m_binc);
+    });
 }
 
-// Pseudo-time iterations of the synthetic equations from W[0] until ||R|| <= tol_inner
-// ||R_0|| or max_inner; returns the index of the buffer that holds the result.  Every
-// kernel returns at once after the device stop flag is set, so the host polls the flag
-// only every POLL iterations (one stream synchronisation each).  Without kernel
-// profiling, and on a non-default stream, the POLL iterations are a CUDA graph captured
-// once per context.
+// Inner iteration number k of the synthetic equations; fp32: its residual side in FP32.
+// 1-D and 2-D update W in place, 3-D reads W[k & 1] and writes the other (W[0] before the
+// first and after an even number of iterations).  `go(id, launcher)` runs each launch.
+template <typename F>
+int inner_iteration(gsis_ctx *c, int k, int fp32, F &&go) {
+    const int sweeps = std::max(c->solver.macro_sweeps, 1);
+    if (c->dim == 3) {
+        const m3::Geom3 &g = c->g3;
+        auto &w = c->w3;
+        MacroState *const st = c->mw.state;
+        const double *W = w.W[k & 1];
+        TRY(go(K_MGRAD, [&] {
+            return m3::launch_macro_grad(c->stream, g, c->order, fp32, c->model, st, W, w.q, w.grad, w.phi);
+        }));
+        TRY(go(K_MBFLUX, [&] {
+            return m3::launch_macro_bflux(c->stream, g, fp32, c->model, vquad_d(c), oquad_d(c), st, w.q, w.mbf);
+        }));
+        TRY(go(K_MRES, [&] {
+            return m3::launch_macro_residual(c->stream, g, c->order, fp32, c->model, c->solver.cfl_macro, st, W, w.q,
+                                             w.grad, w.phi, w.hot, w.mbf, c->hot_b, w.Rg, w.Dinv, w.gam, w.rpart);
+        }));
+        TRY(go(K_MNORM, [&] {
+            return m3::launch_macro_norm(c->stream, m3::macro_rpart_count((int)c->nc), w.rpart, st, c->mhist);
+        }));
+        for (int sw = 0; sw < sweeps; ++sw)
+            TRY(go(K_MJACOBI, [&] {
+                return m3::launch_macro_jacobi(c->stream, g, fp32, c->model, st, sw == 0, sw == sweeps - 1, W, w.q,
+                                               w.Rg, w.Dinv, w.gam, w.dG[sw & 1], w.dG[(sw + 1) & 1],
+                                               w.W[1 - (k & 1)]);
+            }));
+        return GSIS_OK;
+    }
+    const MacroGeom &g = c->mg;
+    const MacroWork &w = c->mw;
+    TRY(go(K_MGRAD, [&] { return launch_macro_grad(c->stream, g, c->order, fp32, w.state, w); }));
+    TRY(go(K_MBFLUX, [&] {
+        return launch_macro_flux(c->stream, g, c->order, fp32, c->model, vquad_d(c), w.state, w, false);
+    }));
+    TRY(go(K_MRES, [&] { return launch_macro_residual(c->stream, g, fp32, w.state, w, c->hot_b, c->mhist); }));
+    // the residual kernel makes the first of the sweeps (its only one is applied by itself)
+    for (int sw = sweeps > 1 ? 1 : 0; sw < sweeps; ++sw)
+        TRY(go(K_MJACOBI, [&] {
+            return launch_macro_jacobi(c->stream, g, fp32, c->model, w.state, sw, sw == sweeps - 1, w);
+        }));
+    return GSIS_OK;
+}
+
+// Pseudo-time iterations of the synthetic equations from W until ||R|| <= tol_inner
+// ||R_0|| or max_inner.  Every kernel returns at once after the device stop flag is set, so
+// the host polls the flag only every POLL iterations (one stream synchronisation each).
+// Without kernel profiling, and on a non-default stream, the POLL iterations are a CUDA
+// graph captured once per context.
 // Captures POLL inner iterations (residual side in FP32 when fp32) as one graph.
 int capture_inner(gsis_ctx *c, int fp32, cudaGraphExec_t *exec, int *nodes_out) {
     constexpr int POLL = 8;
@@ -440,7 +491,12 @@ int capture_inner(gsis_ctx *c, int fp32, cudaGraphExec_t *exec, int *nodes_out) 
     int nodes = 0;
     CUDA_TRY(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
-    for (int k = 0; k < POLL && e == cudaSuccess; ++k) e = enqueue_inner(c, k & 1, fp32, &nodes);
+    auto go = [&](int, auto &&fn) -> int {
+        e = fn();
+        ++nodes;
+        return e == cudaSuccess ? GSIS_OK : GSIS_ERR_CUDA;
+    };
+    for (int k = 0; k < POLL && e == cudaSuccess; ++k) inner_iteration(c, k, fp32, go);   // POLL is even
     cudaError_t e2 = cudaStreamEndCapture(c->stream, &gr);
     if (e != cudaSuccess || e2 != cudaSuccess) {
         if (gr) cudaGraphDestroy(gr);
@@ -457,62 +513,38 @@ int capture_inner(gsis_ctx *c, int fp32, cudaGraphExec_t *exec, int *nodes_out) 
     return GSIS_OK;
 }
 
-int macro_solve(gsis_ctx *c, int *w_out) {
+int macro_solve(gsis_ctx *c) {
     constexpr int POLL = 8;
     constexpr int MACRO_TAIL = 16;   // FP64 inner iterations that end a mixed-precision solve
     const gsis_solver_params &sp = c->solver;
+    MacroState *const mstate = c->mw.state;
     const bool mixed = c->mfp32 == 2;
     const int fp_main = c->mfp32 != 0 ? 1 : 0;
     const int tail = mixed ? std::min(MACRO_TAIL, sp.max_inner) : 0;
     c->h_mstate->it = 0;
     c->h_mstate->done = 0;
     c->h_mstate->max_inner = sp.max_inner - tail;
+    c->h_mstate->ticket = 0;
     c->h_mstate->r0 = 0.0;
     c->h_mstate->rn = 0.0;
     c->h_mstate->tol = sp.tol_inner;
-    CUDA_TRY(c, cudaMemcpyAsync(c->mstate, c->h_mstate, sizeof(MacroState), cudaMemcpyHostToDevice, c->stream));
+    CUDA_TRY(c, cudaMemcpyAsync(mstate, c->h_mstate, sizeof(MacroState), cudaMemcpyHostToDevice, c->stream));
     const bool graph = !c->prof && c->stream != nullptr;
     if (graph && !c->macro_exec) TRY(capture_inner(c, fp_main, &c->macro_exec, &c->macro_nodes));
     if (graph && mixed && !c->macro_exec64) TRY(capture_inner(c, 0, &c->macro_exec64, &c->macro_nodes64));
     // one chunk of POLL inner iterations (the main phase's precision, or the FP64 tail),
     // then (unless it is the last) a look at the stop flag
     auto chunk = [&](bool tail_phase, bool poll) -> int {
-        const int fp32 = tail_phase ? 0 : fp_main;
         if (graph) {
             CUDA_TRY(c, cudaGraphLaunch(tail_phase ? c->macro_exec64 : c->macro_exec, c->stream));
             c->launches += tail_phase ? c->macro_nodes64 : c->macro_nodes;
         } else {
-            for (int k = 0; k < POLL; ++k) {
-                const int wk = k & 1;
-                TRY(launch(c, K_MGRAD, [&] {
-                    return launch_macro_grad(c->stream, c->mg, c->order, fp32, c->model, c->mstate, c->W[wk], c->mq,
-                                             c->mgrad, c->mphi);
-                }));
-                TRY(launch(c, K_MBFLUX, [&] {
-                    return launch_macro_bflux(c->stream, c->mg, fp32, c->model, vquad_d(c), oquad_d(c), c->mstate,
-                                              c->mq, c->mbf);
-                }));
-                TRY(launch(c, K_MRES, [&] {
-                    return launch_macro_residual(c->stream, c->mg, c->order, fp32, c->model, sp.cfl_macro, c->mstate,
-                                                 c->W[wk], c->mq, c->mgrad, c->mphi, c->hot, c->mbf, c->hot_b, c->Rg,
-                                                 c->Dinv, c->gam, c->rpart);
-                }));
-                TRY(launch(c, K_MNORM, [&] {
-                    return launch_macro_norm(c->stream, macro_rpart_count((int)c->nc), c->rpart, c->mstate,
-                                             c->mhist);
-                }));
-                const int sweeps = std::max(sp.macro_sweeps, 1);
-                for (int sw = 0; sw < sweeps; ++sw)
-                    TRY(launch(c, K_MJACOBI, [&] {
-                        return launch_macro_jacobi(c->stream, c->mg, fp32, c->model, c->mstate, sw == 0,
-                                                   sw == sweeps - 1, c->W[wk], c->mq, c->Rg, c->Dinv, c->gam,
-                                                   c->dG[sw & 1], c->dG[(sw + 1) & 1], c->W[1 - wk]);
-                    }));
-            }
+            for (int k = 0; k < POLL; ++k)
+                TRY(inner_iteration(c, k, tail_phase ? 0 : fp_main,
+                                    [&](int id, auto &&fn) { return launch(c, id, fn); }));
         }
         if (poll) {
-            CUDA_TRY(c, cudaMemcpyAsync(c->h_mstate, c->mstate, sizeof(MacroState), cudaMemcpyDeviceToHost,
-                                        c->stream));
+            CUDA_TRY(c, cudaMemcpyAsync(c->h_mstate, mstate, sizeof(MacroState), cudaMemcpyDeviceToHost, c->stream));
             CUDA_TRY(c, cudaStreamSynchronize(c->stream));
         }
         return GSIS_OK;
@@ -526,14 +558,12 @@ int macro_solve(gsis_ctx *c, int *w_out) {
         // the FP64 residual side for up to `tail` more iterations, from where the FP32 ones stopped
         c->h_mstate->done = 0;
         c->h_mstate->max_inner = c->h_mstate->it + tail;
-        CUDA_TRY(c, cudaMemcpyAsync(c->mstate, c->h_mstate, sizeof(MacroState), cudaMemcpyHostToDevice, c->stream));
+        CUDA_TRY(c, cudaMemcpyAsync(mstate, c->h_mstate, sizeof(MacroState), cudaMemcpyHostToDevice, c->stream));
         for (int it = 0; it < tail; it += POLL) {
             TRY(chunk(true, it + POLL < tail));
             if (it + POLL < tail && c->h_mstate->done) break;
         }
     }
-    int w = 0;
-    *w_out = w;   // POLL is even: every chunk ends where it started
     return GSIS_OK;
 }
 
@@ -579,23 +609,85 @@ int defect_offset(gsis_ctx *c, int nxt) {
         return launch_resid_rows<Real>(c->stream, c->dim, (int)c->nc, c->nch, c->och, (const Real *)c->coef_h,
                                        (const Real *)c->partial, (const Real *)c->opartial, c->rrow);
     }));
+    if (c->dim == 3) {
+        m3::Geom3 g0 = c->g3;
+        g0.moff = nullptr;
+        auto &w = c->w3;
+        TRY(launch(c, K_MGRAD, [&] {
+            return m3::launch_macro_grad(c->stream, g0, c->order, 0, c->model, nullptr, w.W[0], w.q, w.grad, w.phi);
+        }));
+        TRY(launch(c, K_MBFLUX, [&] {
+            return m3::launch_macro_bflux(c->stream, g0, 0, c->model, vquad_d(c), oquad_d(c), nullptr, w.q, w.mbf);
+        }));
+        TRY(launch(c, K_MRES, [&] {
+            return m3::launch_macro_residual(c->stream, g0, c->order, 0, c->model, c->solver.cfl_macro, nullptr, w.W[0],
+                                             w.q, w.grad, w.phi, w.hot, w.mbf, c->hot_b, w.Rg, w.Dinv, w.gam, w.rpart);
+        }));
+        return launch(c, K_MCONV, [&] {
+            return launch_macro_offset(c->stream, c->dim, (int)c->nc, w.Rg, c->rrow, c->moff);
+        });
+    }
     MacroGeom g0 = c->mg;
     g0.moff = nullptr;
-    TRY(launch(c, K_MGRAD, [&] {
-        return launch_macro_grad(c->stream, g0, c->order, 0, c->model, nullptr, c->W[0], c->mq, c->mgrad, c->mphi);
-    }));
+    const MacroWork &w = c->mw;
+    TRY(launch(c, K_MGRAD, [&] { return launch_macro_grad(c->stream, g0, c->order, 0, nullptr, w); }));
     TRY(launch(c, K_MBFLUX, [&] {
-        return launch_macro_bflux(c->stream, g0, 0, c->model, vquad_d(c), oquad_d(c), nullptr, c->mq, c->mbf);
+        return launch_macro_flux(c->stream, g0, c->order, 0, c->model, vquad_d(c), nullptr, w, false);
     }));
-    TRY(launch(c, K_MRES, [&] {
-        return launch_macro_residual(c->stream, g0, c->order, 0, c->model, c->solver.cfl_macro, nullptr, c->W[0],
-                                     c->mq, c->mgrad, c->mphi, c->hot, c->mbf, c->hot_b, c->Rg, c->Dinv, c->gam,
-                                     c->rpart);
-    }));
+    TRY(launch(c, K_MRES, [&] { return launch_macro_residual(c->stream, g0, 0, nullptr, w, c->hot_b, nullptr); }));
     TRY(launch(c, K_MCONV, [&] {
-        return launch_macro_offset(c->stream, c->dim, (int)c->nc, c->Rg, c->rrow, c->moff);
+        return launch_macro_offset(c->stream, c->dim, (int)c->nc, w.Rg, c->rrow, c->moff);
     }));
     return GSIS_OK;
+}
+
+// fields_n of the synthetic solution; closed domains: scaled to the total mass of M^k
+int macro_result(gsis_ctx *c) {
+    const double *ref = c->closed ? c->fields : nullptr;
+    if (c->dim < 3)
+        return launch(c, K_MCONV, [&] {
+            return launch_macro_fields_from_W(c->stream, c->mg, c->model, c->mw, ref, c->fields_n);
+        });
+    if (ref)
+        TRY(launch(c, K_MCONV, [&] {
+            return m3::launch_macro_mass_rescale(c->stream, c->dim, (int)c->nc, c->vol, ref, c->w3.W[0]);
+        }));
+    return launch(c, K_MCONV, [&] {
+        return m3::launch_macro_fields_from_W(c->stream, c->dim, (int)c->nc, c->model, c->w3.W[0], c->fields_n);
+    });
+}
+
+// W and q of M^{k+1/2}, and the high-order terms against its NSF values (in FP32 only where
+// the whole synthetic side runs in FP32)
+int high_order_terms(gsis_ctx *c) {
+    const int fp32 = c->mfp32 == 1;
+    if (c->dim == 3) {
+        auto &w = c->w3;
+        TRY(launch(c, K_MCONV, [&] {
+            return m3::launch_macro_from_fields(c->stream, c->dim, (int)c->nc, c->model, c->fields_h, w.W[0]);
+        }));
+        TRY(launch(c, K_MGRAD, [&] {
+            return m3::launch_macro_grad(c->stream, c->g3, 1, fp32, c->model, nullptr, w.W[0], w.q, w.grad, w.phi);
+        }));
+        TRY(launch(c, K_MBFLUX, [&] {
+            return m3::launch_macro_bflux(c->stream, c->g3, fp32, c->model, vquad_d(c), oquad_d(c), nullptr, w.q, w.mbf);
+        }));
+        return launch(c, K_HOT, [&] {
+            return m3::launch_macro_hot(c->stream, c->g3, fp32, c->model, c->fields_h, w.q, w.grad, c->kbf, w.mbf,
+                                        w.hot, c->hot_b);
+        });
+    }
+    const MacroWork &w = c->mw;
+    TRY(launch(c, K_MCONV, [&] {
+        return launch_macro_from_fields(c->stream, c->dim, (int)c->nc, c->model, c->fields_h, w);
+    }));
+    TRY(launch(c, K_MGRAD, [&] { return launch_macro_grad(c->stream, c->mg, 1, fp32, nullptr, w); }));
+    TRY(launch(c, K_MBFLUX, [&] {
+        return launch_macro_flux(c->stream, c->mg, 1, fp32, c->model, vquad_d(c), nullptr, w, true);
+    }));
+    return launch(c, K_HOT, [&] {
+        return launch_macro_hot(c->stream, c->mg, fp32, c->model, c->fields_h, w, c->kbf, c->hot_b);
+    });
 }
 
 // One GSIS iteration (Section 3): kinetic step, high-order terms from f^{k+1/2}, the
@@ -615,30 +707,10 @@ int gsis_iteration(gsis_ctx *c) {
         return launch_kinetic_bflux<Real>(c->stream, g, c->model, vquad<Real>(c), oquad<Real>(c),
                                           (const Real *)c->f[nxt], (const Real *)c->I[nxt], c->kbf);
     }));
-    TRY(launch(c, K_MCONV, [&] {
-        return launch_macro_from_fields(c->stream, c->dim, (int)c->nc, c->model, c->fields_h, c->W[0]);
-    }));
-    TRY(launch(c, K_MGRAD, [&] {
-        return launch_macro_grad(c->stream, g, 1, c->mfp32 == 1, c->model, nullptr, c->W[0], c->mq, c->mgrad, c->mphi);
-    }));
-    TRY(launch(c, K_MBFLUX, [&] {
-        return launch_macro_bflux(c->stream, g, c->mfp32 == 1, c->model, vquad_d(c), oquad_d(c), nullptr, c->mq, c->mbf);
-    }));
-    TRY(launch(c, K_HOT, [&] {
-        return launch_macro_hot(c->stream, g, c->mfp32 == 1, c->model, c->fields_h, c->mq, c->mgrad, c->kbf, c->mbf, c->hot,
-                                c->hot_b);
-    }));
+    TRY(high_order_terms(c));
     if (c->moff) TRY(defect_offset<Real>(c, nxt));
-    int w = 0;
-    TRY(macro_solve(c, &w));
-    if (c->closed) {
-        TRY(launch(c, K_MCONV, [&] {
-            return launch_macro_mass_rescale(c->stream, c->dim, (int)c->nc, c->vol, c->fields, c->W[w]);
-        }));
-    }
-    TRY(launch(c, K_MCONV, [&] {
-        return launch_macro_fields_from_W(c->stream, c->dim, (int)c->nc, c->model, c->W[w], c->fields_n);
-    }));
+    TRY(macro_solve(c));
+    TRY(macro_result(c));
     TRY(launch(c, K_SYNC, [&] {
         return launch_sync<Real>(c->stream, c->dim, (int)c->nc, c->tcm >= 1, vquad<Real>(c), oquad<Real>(c), c->model,
                                  c->solver.sync_relax, c->fields_n, c->fields_h, (const Real *)c->coef,
@@ -1072,62 +1144,79 @@ int gsis_create(const gsis_mesh *m, const gsis_velocity_quad *vq, const gsis_pho
 
     // ---- synthetic-equation geometry: interior faces (owner -> neighbour), the cell -> face
     // map in the cell's face order, boundary faces, FP64 quadratures and patch states
-    std::vector<int> fi_i, fi_j, cface(nc * MAXF, 0), mpk(std::max(m->n_patches, 1), 0);
-    std::vector<double> fi_n, fi_S, fi_dn, fi_dist, fi_t, fi_dx, mbn, mbS, mbdn,
-        mps(8 * std::max(m->n_patches, 1), 0.0);
+    std::vector<int> fi4, cface(nc * MAXF, 0), mnb(nc * MAXF, -1), mpk(std::max(m->n_patches, 1), 0);
+    std::vector<unsigned char> mown(nc * MAXF, 0);
+    std::vector<double> mfgeo, mbn, mbgeo, mcdx(nc * MAXF * MGS, 0.0), mcnS(nc * MAXF * MGS, 0.0), mivol(nc), mhivol(nc),
+        micdx(nc), mps(8 * std::max(m->n_patches, 1), 0.0);
     {
         std::vector<int> id_of(nfc, -1);
         for (int64_t f = 0; f < nfc; ++f) {
             const int o = m->face_owner[f], nb = m->face_nbr[f];
             if (nb < 0) continue;
-            id_of[f] = (int)fi_i.size();
-            fi_i.push_back(o);
-            fi_j.push_back(nb);
-            double d[3] = {0, 0, 0}, dn = 0.0, dd = 0.0;
+            id_of[f] = (int)(fi4.size() / 4);
+            for (int x : {o, nb, 0, 0}) fi4.push_back(x);
+            double d[3] = {0, 0, 0}, n[3] = {0, 0, 0}, t[3] = {0, 0, 0}, dn = 0.0, dd = 0.0, tn = 0.0;
             for (int a = 0; a < dim; ++a) {
                 d[a] = wrap(m->cell_centroid[nb * dim + a] - m->cell_centroid[o * dim + a], a);
-                dn += m->face_normal[f * dim + a] * d[a];
+                n[a] = m->face_normal[f * dim + a];
+                dn += n[a] * d[a];
                 dd += d[a] * d[a];
             }
             dd = std::sqrt(dd);
-            for (int a = 0; a < MGS; ++a) {
-                fi_n.push_back(a < dim ? m->face_normal[f * dim + a] : 0.0);
-                fi_t.push_back(d[a] / dd);
+            for (int a = 0; a < 3; ++a) {
+                t[a] = d[a] / dd;
+                tn += t[a] * n[a];
             }
-            for (int s = 0; s < 2; ++s)
-                for (int a = 0; a < MGS; ++a)
-                    fi_dx.push_back(a < dim ? wrap(m->face_centroid[f * dim + a] -
-                                                   m->cell_centroid[(s == 0 ? o : nb) * dim + a], a)
-                                            : 0.0);
-            fi_S.push_back(m->face_area[f]);
-            fi_dn.push_back(std::fabs(dn));
-            fi_dist.push_back(dd);
-        }
-        for (int64_t i = 0; i < nc; ++i) {
-            for (int k = 0; k < MAXF; ++k) {
-                if (k >= nf[i]) { cface[i * MAXF + k] = -1 - std::max(c->n_bf, 1); continue; }
-                const int j = nbr[i * MAXF + k];
-                cface[i * MAXF + k] = j >= 0 ? id_of[face_of[i * MAXF + k]] : j;
+            double G[FGEO] = {0};
+            for (int a = 0; a < 3; ++a) {
+                G[a] = n[a];
+                G[3 + a] = t[a];
+                G[6 + a] = 0.5 * (n[a] - tn * t[a]);
             }
+            G[9] = 1.0 / dd;
+            G[10] = tn / dd;
+            G[11] = m->face_area[f];
+            G[12] = 1.0 / std::fabs(dn);
+            mfgeo.insert(mfgeo.end(), G, G + FGEO);
         }
-        // boundary faces in the order the kinetic connectivity numbered them
         mbn.assign(MGS * std::max(c->n_bf, 1), 0.0);
-        mbS.assign(std::max(c->n_bf, 1), 0.0);
-        mbdn.assign(std::max(c->n_bf, 1), 0.0);
-        for (int64_t i = 0; i < nc; ++i)
-            for (int k = 0; k < nf[i]; ++k) {
-                const int j = nbr[i * MAXF + k];
-                if (j >= 0) continue;
+        mbgeo.assign(8 * std::max(c->n_bf, 1), 0.0);
+        for (int64_t i = 0; i < nc; ++i) {
+            const double V = m->cell_volume[i];
+            mivol[i] = 1.0 / V;
+            mhivol[i] = 1.0 / (2.0 * V);
+            micdx[i] = 1.0 / (sp->cfl_macro * cdx[i]);
+            for (int k = 0; k < MAXF; ++k) {
+                const int64_t ik = i * MAXF + k;
+                if (k >= nf[i]) { cface[ik] = -1 - std::max(c->n_bf, 1); continue; }
+                const int j = nbr[ik];
+                const int64_t f = face_of[ik];
+                if (j >= 0) {
+                    const int id = id_of[f];
+                    cface[ik] = id;
+                    mnb[ik] = j;
+                    // owner i: this face is seen from the owner's side first (a face between the
+                    // same two cells across two periodic seams is two faces)
+                    mown[ik] = m->face_owner[f] == i;
+                    fi4[(size_t)id * 4 + (mown[ik] ? 2 : 3)] = k;
+                    for (int a = 0; a < dim; ++a) {
+                        mcdx[ik * MGS + a] = dxf[ik * 3 + a];
+                        mcnS[ik * MGS + a] = nrm[ik * 3 + a] * m->face_area[f] / (2.0 * V);
+                    }
+                    continue;
+                }
+                // boundary faces in the order the kinetic connectivity numbered them
                 const int b = -1 - j;
-                const int64_t f = face_of[i * MAXF + k];
+                cface[ik] = j;
                 double dn = 0.0;
                 for (int a = 0; a < dim; ++a) {
-                    mbn[b * MGS + a] = m->face_normal[f * dim + a];
+                    mbn[b * MGS + a] = mbgeo[b * 8 + a] = m->face_normal[f * dim + a];
                     dn += m->face_normal[f * dim + a] * wrap(m->face_centroid[f * dim + a] - m->cell_centroid[i * dim + a], a);
                 }
-                mbS[b] = m->face_area[f];
-                mbdn[b] = std::fabs(dn);
+                mbgeo[b * 8 + 3] = m->face_area[f];
+                mbgeo[b * 8 + 4] = 1.0 / std::fabs(dn);
             }
+        }
         for (int p = 0; p < m->n_patches; ++p) {
             const gsis_patch &P = m->patches[p];
             mpk[p] = P.kind;
@@ -1135,12 +1224,11 @@ int gsis_create(const gsis_mesh *m, const gsis_velocity_quad *vq, const gsis_pho
             const double st[8] = {P.rho, P.u[0], P.u[1], P.u[2], P.T_t, P.T_r, P.T_v, P.T_R};
             for (int k = 0; k < 8; ++k) mps[p * 8 + k] = st[k];
         }
-        if (fi_i.empty()) {   // keep every device array non-empty
-            fi_i.push_back(0); fi_j.push_back(0); fi_S.push_back(0.0); fi_dn.push_back(1.0); fi_dist.push_back(1.0);
-            for (int a = 0; a < MGS; ++a) { fi_n.push_back(0.0); fi_t.push_back(0.0); fi_dx.push_back(0.0); fi_dx.push_back(0.0); }
-        }
     }
-    const int n_fi = (int)std::count_if(fi_S.begin(), fi_S.end(), [](double x) { return x > 0.0; });
+    const int n_fi = (int)(fi4.size() / 4);
+    const size_t nfi1 = std::max(n_fi, 1);      // keep every device array non-empty
+    fi4.resize(nfi1 * 4, 0);
+    mfgeo.resize(nfi1 * FGEO, 0.0);
 
     // ---- device allocations
     const size_t fsz = (size_t)nc * c->Vp * 4, isz = (size_t)nc * c->Op;
@@ -1156,8 +1244,8 @@ int gsis_create(const gsis_mesh *m, const gsis_velocity_quad *vq, const gsis_pho
     A_(dalloc_real(c, &c->opartial, (size_t)nc * c->och * NMO));
     if (c->precision == GSIS_FP32) A_(dalloc_real(c, &c->sync_kc, (size_t)nc * SYNC_KC));
     if (c->order == 2) {
-        A_(dalloc_real(c, &c->fface, fi_i.size() * c->Vp * 4));
-        A_(dalloc_real(c, &c->oface, fi_i.size() * c->Op));
+        A_(dalloc_real(c, &c->fface, nfi1 * c->Vp * 4));
+        A_(dalloc_real(c, &c->oface, nfi1 * c->Op));
     }
     A_(dalloc(c, &c->fields, (size_t)nc * NF));
     A_(dalloc(c, &c->fields_old, (size_t)nc * NF));
@@ -1188,98 +1276,217 @@ int gsis_create(const gsis_mesh *m, const gsis_velocity_quad *vq, const gsis_pho
     if (cudaMallocHost(&c->h_pinned, (NEPS + 1) * sizeof(double)) != cudaSuccess) return bail(GSIS_ERR_OUT_OF_MEMORY);
     if (cudaMallocHost(&c->h_mstate, sizeof(MacroState)) != cudaSuccess) return bail(GSIS_ERR_OUT_OF_MEMORY);
     {
-        const size_t nbf1 = std::max(c->n_bf, 1), nfi1 = fi_i.size();
-        A_(dalloc(c, &c->m_fi_i, nfi1));
-        A_(dalloc(c, &c->m_fi_j, nfi1));
-        A_(dalloc(c, &c->m_cface, (size_t)nc * MAXF));
-        A_(dalloc(c, &c->m_pkind, mpk.size()));
-        A_(dalloc(c, &c->m_fi_n, nfi1 * MGS));
-        A_(dalloc(c, &c->m_fi_S, nfi1));
-        A_(dalloc(c, &c->m_fi_dn, nfi1));
-        A_(dalloc(c, &c->m_fi_dist, nfi1));
-        A_(dalloc(c, &c->m_fi_t, nfi1 * MGS));
-        A_(dalloc(c, &c->m_fi_dx, nfi1 * 2 * MGS));
-        A_(dalloc(c, &c->m_lsq, lsq.size()));
-        A_(dalloc(c, &c->m_eps2, (size_t)nc));
-        A_(dalloc(c, &c->m_bf_n, nbf1 * MGS));
-        A_(dalloc(c, &c->m_bf_S, nbf1));
-        A_(dalloc(c, &c->m_bf_dn, nbf1));
-        A_(dalloc(c, &c->m_pstate, mps.size()));
-        A_(dalloc(c, &c->vqd_x, vx.size()));
-        A_(dalloc(c, &c->vqd_w, vw.size()));
-        A_(dalloc(c, &c->oqd_x, ox.size()));
-        A_(dalloc(c, &c->oqd_w, ow.size()));
-        for (int k = 0; k < 2; ++k) {
-            A_(dalloc(c, &c->W[k], (size_t)nc * NVM));
-            A_(dalloc(c, &c->dG[k], (size_t)nc * NVM));
+        const size_t nbf1 = std::max(c->n_bf, 1);
+        MacroGeom &G = c->mg;
+        MacroWork &w = c->mw;
+        const size_t R8 = sizeof(double);            // the work arrays are sized for FP64
+        auto work = [&](void **p, size_t n) { return dalloc(c, reinterpret_cast<double **>(p), n); };
+        if (dim < 3) {
+            A_(dalloc(c, &w.W, (size_t)nc * NVM));
+            A_(dalloc(c, &w.qd, (size_t)nc * NVM));
+            A_(work(&w.grad, (size_t)nc * MGS * NVM));
+            A_(work(&w.rec, c->order == 2 ? (size_t)nc * MAXF * NVM : 1));
+            A_(work(&w.Fx, nfi1 * NVM));
+            A_(work(&w.fgam, nfi1 * 2));
+            A_(work(&w.src, (size_t)nc * SRC));
+            A_(work(&w.gam, (size_t)nc * MAXF * 2));
+            for (int k = 0; k < 2; ++k) {
+                A_(work(&w.rows[k], (size_t)nc * NVM * 4));
+                if (cudaMemset(w.rows[k], 0, (size_t)nc * NVM * 4 * R8) != cudaSuccess) return bail(GSIS_ERR_CUDA);
+            }
+            A_(dalloc(c, &w.Rg, (size_t)nc * NVM));
+            A_(dalloc(c, &w.Dinv, (size_t)nc * 24));
+            A_(dalloc(c, &w.rpart, (size_t)macro_rpart_count((int)nc)));
+            A_(dalloc(c, &w.fac, 1));
+            A_(dalloc(c, &w.hot, nfi1 * NVM));
+            A_(dalloc(c, &w.mbf, nbf1 * NVM));
         }
-        A_(dalloc(c, &c->mq, (size_t)nc * NVM));
-        A_(dalloc(c, &c->mgrad, (size_t)nc * MGS * NVM));
-        A_(dalloc(c, &c->mphi, (size_t)nc * NVM));
-        A_(dalloc(c, &c->Rg, (size_t)nc * NVM));
+        A_(dalloc(c, &w.state, 1));
+        if (cudaMemset(w.state, 0, sizeof(MacroState)) != cudaSuccess) return bail(GSIS_ERR_CUDA);
         if (sp->defect_correction) {
             A_(dalloc_real(c, &c->coef_h, (size_t)nc * cf::NC));
             A_(dalloc(c, &c->rrow, (size_t)nc * NVM));
             A_(dalloc(c, &c->moff, (size_t)nc * NVM));
             if (cudaMemset(c->moff, 0, (size_t)nc * NVM * sizeof(double)) != cudaSuccess) return bail(GSIS_ERR_CUDA);
         }
-        A_(dalloc(c, &c->Dinv, (size_t)nc * 24));
-        A_(dalloc(c, &c->gam, (size_t)nc * MAXF * 2));
-        A_(dalloc(c, &c->rpart, (size_t)macro_rpart_count((int)nc)));
-        A_(dalloc(c, &c->hot, nfi1 * NHOT));
         A_(dalloc(c, &c->hot_b, nbf1 * NVM));
         A_(dalloc(c, &c->kbf, nbf1 * NVM));
-        A_(dalloc(c, &c->mbf, nbf1 * NVM));
         A_(dalloc(c, &c->fields_h, (size_t)nc * NF));
         A_(dalloc(c, &c->fields_n, (size_t)nc * NF));
         A_(dalloc(c, &c->mhist, (size_t)std::max(sp->max_inner, 1)));
-        A_(dalloc(c, &c->mstate, 1));
-        A_(upload(c, c->m_fi_i, fi_i));
-        A_(upload(c, c->m_fi_j, fi_j));
+        A_(dalloc(c, &c->m_cface, (size_t)nc * MAXF));
+        A_(dalloc(c, &c->m_pkind, mpk.size()));
+        A_(dalloc(c, &c->m_bf_n, nbf1 * MGS));
+        A_(dalloc(c, &c->m_pstate, mps.size()));
+        A_(dalloc(c, &c->m_binc, nbf1 * BINC));
+        A_(dalloc(c, &c->vqd_x, vx.size()));
+        A_(dalloc(c, &c->vqd_w, vw.size()));
+        A_(dalloc(c, &c->oqd_x, ox.size()));
+        A_(dalloc(c, &c->oqd_w, ow.size()));
         A_(upload(c, c->m_cface, cface));
         A_(upload(c, c->m_pkind, mpk));
-        A_(upload(c, c->m_fi_n, fi_n));
-        A_(upload(c, c->m_fi_S, fi_S));
-        A_(upload(c, c->m_fi_dn, fi_dn));
-        A_(upload(c, c->m_fi_dist, fi_dist));
-        A_(upload(c, c->m_fi_t, fi_t));
-        A_(upload(c, c->m_fi_dx, fi_dx));
-        A_(upload(c, c->m_lsq, lsq));
-        A_(upload(c, c->m_eps2, eps2));
         A_(upload(c, c->m_bf_n, mbn));
-        A_(upload(c, c->m_bf_S, mbS));
-        A_(upload(c, c->m_bf_dn, mbdn));
         A_(upload(c, c->m_pstate, mps));
         A_(upload(c, c->vqd_x, vx));
         A_(upload(c, c->vqd_w, vw));
         A_(upload(c, c->oqd_x, ox));
         A_(upload(c, c->oqd_w, ow));
-        MacroGeom &G = c->mg;
+        auto table = [&](auto **dst, const auto &src) -> int {     // a constant device array of src
+            using T = std::remove_const_t<std::remove_pointer_t<std::remove_reference_t<decltype(*dst)>>>;
+            T *p = nullptr;
+            const std::vector<T> v(src.begin(), src.end());
+            int r = dalloc(c, &p, v.size());
+            if (r == GSIS_OK) r = upload(c, p, v);
+            *dst = p;
+            return r;
+        };
+        auto constants = [&](auto &r) -> int {                     // geometry and model constants in r's type
+            using R = std::remove_const_t<std::remove_pointer_t<std::remove_reference_t<decltype(r.q)>>>;
+            TRY(table(&r.lsq, lsq));
+            TRY(table(&r.eps2, eps2));
+            TRY(table(&r.ivol, mivol));
+            TRY(table(&r.hivol, mhivol));
+            TRY(table(&r.icdx, micdx));
+            TRY(table(&r.cdx, mcdx));
+            TRY(table(&r.cnS, mcnS));
+            TRY(table(&r.fgeo, mfgeo));
+            TRY(table(&r.bgeo, mbgeo));
+            double base[9];
+            kappa_base(md.A, md.d_r, md.d_v, base);
+            for (int k = 0; k < 9; ++k) r.base[k] = (R)base[k];
+            const double mu0 = std::sqrt(2.0 / M_PI) * md.Kn;
+            r.mu0 = (R)mu0;
+            r.i_mu0 = (R)(1.0 / mu0);
+            r.omega = (R)md.omega;
+            r.half_dr = (R)(0.5 * md.d_r);
+            r.half_dv = (R)(0.5 * md.d_v);
+            r.i_half_dr = (R)(2.0 / md.d_r);
+            r.i_half_dv = (R)(2.0 / md.d_v);
+            r.i_Zr = (R)(1.0 / md.Z_r);
+            r.i_Zv = (R)(1.0 / md.Z_v);
+            r.w_r = (R)(3.0 / (3.0 + md.d_r));
+            r.w_v = (R)(3.0 / (3.0 + md.d_v));
+            r.c_r = (R)(md.d_r / (3.0 + md.d_r));
+            r.e_v = (R)(md.d_v / (3.0 + md.d_v));
+            r.ik = (R)(1.0 / md.Kn_p);
+            r.kR0 = (R)(md.Kn_p / 3.0);
+            r.sigma = (R)md.sigma_R;
+            r.dens = md.k_eff_density_scaled;
+            return GSIS_OK;
+        };
+        if (dim < 3) {
+            A_(constants(G.d));
+            G.d.q = w.qd;
+            G.d.hot = w.hot;
+            if (c->mfp32) {
+                A_(dalloc(c, &w.qf, (size_t)nc * NVM));
+                A_(dalloc(c, &w.hotf, nfi1 * NVM));
+                A_(constants(G.f));
+                G.f.q = w.qf;
+                G.f.hot = w.hotf;
+            }
+            std::vector<int4> f4(nfi1);
+            std::memcpy(f4.data(), fi4.data(), nfi1 * sizeof(int4));
+            A_(table(&G.fi4, f4));
+        } else {
+            // macro3d.cu: the same geometry as separate arrays
+            m3::Geom3 &g3 = c->g3;
+            auto &w3 = c->w3;
+            std::vector<int> fi_i(nfi1), fi_j(nfi1);
+            std::vector<double> fi_n(nfi1 * MGS), fi_t(nfi1 * MGS), fi_S(nfi1), fi_dn(nfi1), fi_dist(nfi1, 1.0),
+                fi_dx(nfi1 * 2 * MGS), bS(nbf1), bdn(nbf1);
+            for (int64_t f = 0, id = 0; f < nfc; ++f) {
+                const int o = m->face_owner[f], nbc = m->face_nbr[f];
+                if (nbc < 0) continue;
+                double d[3], dn = 0.0, dd = 0.0;
+                for (int q = 0; q < 3; ++q) {
+                    d[q] = wrap(m->cell_centroid[nbc * dim + q] - m->cell_centroid[o * dim + q], q);
+                    dn += m->face_normal[f * dim + q] * d[q];
+                    dd += d[q] * d[q];
+                }
+                dd = std::sqrt(dd);
+                fi_i[id] = o;
+                fi_j[id] = nbc;
+                for (int q = 0; q < 3; ++q) {
+                    fi_n[id * MGS + q] = m->face_normal[f * dim + q];
+                    fi_t[id * MGS + q] = d[q] / dd;
+                    for (int sd = 0; sd < 2; ++sd)
+                        fi_dx[(id * 2 + sd) * MGS + q] =
+                            wrap(m->face_centroid[f * dim + q] - m->cell_centroid[(sd == 0 ? o : nbc) * dim + q], q);
+                }
+                fi_S[id] = m->face_area[f];
+                fi_dn[id] = std::fabs(dn);
+                fi_dist[id] = dd;
+                ++id;
+            }
+            for (int64_t i = 0; i < nc; ++i)
+                for (int k = 0; k < nf[i]; ++k) {
+                    const int j = nbr[i * MAXF + k];
+                    if (j >= 0) continue;
+                    const int64_t f = face_of[i * MAXF + k];
+                    double dn = 0.0;
+                    for (int q = 0; q < 3; ++q)
+                        dn += m->face_normal[f * dim + q] *
+                              wrap(m->face_centroid[f * dim + q] - m->cell_centroid[i * dim + q], q);
+                    bS[-1 - j] = m->face_area[f];
+                    bdn[-1 - j] = std::fabs(dn);
+                }
+            A_(table(&g3.fi_i, fi_i));
+            A_(table(&g3.fi_j, fi_j));
+            A_(table(&g3.fi_n, fi_n));
+            A_(table(&g3.fi_S, fi_S));
+            A_(table(&g3.fi_dn, fi_dn));
+            A_(table(&g3.fi_dist, fi_dist));
+            A_(table(&g3.fi_t, fi_t));
+            A_(table(&g3.fi_dx, fi_dx));
+            A_(table(&g3.lsq, lsq));
+            A_(table(&g3.eps2, eps2));
+            A_(table(&g3.bf_S, bS));
+            A_(table(&g3.bf_dn, bdn));
+            g3.n_cells = (int)nc;
+            g3.dim = dim;
+            g3.n_fi = n_fi;
+            g3.n_bf = c->n_bf;
+            g3.cface = c->m_cface;
+            g3.info = c->g_info;
+            g3.stn = c->g_stn;
+            g3.vol = c->vol;
+            g3.dx = c->cell_dx;
+            g3.bf_cell = c->bf_cell;
+            g3.bf_patch = c->bf_patch;
+            g3.bf_n = c->m_bf_n;
+            g3.patch_kind = c->m_pkind;
+            g3.patch_state = c->m_pstate;
+            g3.moff = c->moff;
+            for (int k = 0; k < 2; ++k) {
+                A_(dalloc(c, &w3.W[k], (size_t)nc * NVM));
+                A_(dalloc(c, &w3.dG[k], (size_t)nc * NVM));
+            }
+            A_(dalloc(c, &w3.q, (size_t)nc * NVM));
+            A_(dalloc(c, &w3.grad, (size_t)nc * MGS * NVM));
+            A_(dalloc(c, &w3.phi, (size_t)nc * NVM));
+            A_(dalloc(c, &w3.Rg, (size_t)nc * NVM));
+            A_(dalloc(c, &w3.Dinv, (size_t)nc * 24));
+            A_(dalloc(c, &w3.gam, (size_t)nc * MAXF * 2));
+            A_(dalloc(c, &w3.rpart, (size_t)m3::macro_rpart_count((int)nc)));
+            A_(dalloc(c, &w3.hot, nfi1 * m3::NHOT));
+            A_(dalloc(c, &w3.mbf, nbf1 * NVM));
+        }
+        A_(table(&G.nb, mnb));
+        A_(table(&G.own, mown));
         G.n_cells = (int)nc;
         G.dim = dim;
         G.n_fi = n_fi;
         G.n_bf = c->n_bf;
-        G.fi_i = c->m_fi_i;
-        G.fi_j = c->m_fi_j;
-        G.fi_n = c->m_fi_n;
-        G.fi_S = c->m_fi_S;
-        G.fi_dn = c->m_fi_dn;
-        G.fi_dist = c->m_fi_dist;
-        G.fi_t = c->m_fi_t;
-        G.fi_dx = c->m_fi_dx;
         G.cface = c->m_cface;
         G.info = c->g_info;
         G.stn = c->g_stn;
-        G.lsq = c->m_lsq;
-        G.eps2 = c->m_eps2;
         G.vol = c->vol;
-        G.dx = c->cell_dx;
         G.moff = c->moff;              // null unless the defect correction is on
         G.bf_cell = c->bf_cell;
         G.bf_patch = c->bf_patch;
         G.bf_n = c->m_bf_n;
-        G.bf_S = c->m_bf_S;
-        G.bf_dn = c->m_bf_dn;
+        G.binc = c->m_binc;
         G.patch_kind = c->m_pkind;
         G.patch_state = c->m_pstate;
     }
@@ -1356,9 +1563,9 @@ int gsis_create(const gsis_mesh *m, const gsis_velocity_quad *vq, const gsis_pho
         A_(upload(c, c->refl_v, rv));
         A_(upload(c, c->refl_o, ro));
         c->mirrors = !normals.empty();
-        c->mg.bf_tab = c->bf_tab;       // the synthetic equations' geometry was filled above
-        c->mg.refl_v = c->refl_v;
-        c->mg.refl_o = c->refl_o;
+        c->mg.bf_tab = c->g3.bf_tab = c->bf_tab;       // the synthetic equations' geometry was filled above
+        c->mg.refl_v = c->g3.refl_v = c->refl_v;
+        c->mg.refl_o = c->g3.refl_o = c->refl_o;
     }
     c->h_wall.assign((size_t)std::max(c->n_bf, 1) * 8, 0.0);
     for (int b = 0; b < c->n_bf; ++b) {     // per boundary face: wall flag, normal, wall T and u
@@ -1391,6 +1598,7 @@ int gsis_create(const gsis_mesh *m, const gsis_velocity_quad *vq, const gsis_pho
         }
         A_(upload(c, c->bf_inc, inc));
     }
+    A_(macro_velocity_set(c));
     if (cudaMemset(c->eps_ticket, 0, sizeof(unsigned int)) != cudaSuccess) return bail(GSIS_ERR_CUDA);
     A_(upload(c, c->patch_kind, pk));
     if (cudaMemset(c->err, 0, sizeof(int)) != cudaSuccess) return bail(GSIS_ERR_CUDA);
@@ -1653,29 +1861,9 @@ int shard_mid(gsis_ctx *c) {
                                    c->fields_h, c->eps_terms, c->err, 0, nullptr, nullptr, nullptr, c->xbuf);
     }));
     TRY(launch(c, K_KBFLUX, [&] { return launch_kbflux_combine(c->stream, g, xbuf_kbf(c), c->kbf); }));
-    TRY(launch(c, K_MCONV, [&] {
-        return launch_macro_from_fields(c->stream, c->dim, (int)c->nc, c->model, c->fields_h, c->W[0]);
-    }));
-    TRY(launch(c, K_MGRAD, [&] {
-        return launch_macro_grad(c->stream, g, 1, c->mfp32 == 1, c->model, nullptr, c->W[0], c->mq, c->mgrad, c->mphi);
-    }));
-    TRY(launch(c, K_MBFLUX, [&] {
-        return launch_macro_bflux(c->stream, g, c->mfp32 == 1, c->model, vquad_d(c), oquad_d(c), nullptr, c->mq, c->mbf);
-    }));
-    TRY(launch(c, K_HOT, [&] {
-        return launch_macro_hot(c->stream, g, c->mfp32 == 1, c->model, c->fields_h, c->mq, c->mgrad, c->kbf, c->mbf,
-                                c->hot, c->hot_b);
-    }));
-    int w = 0;
-    TRY(macro_solve(c, &w));
-    if (c->closed) {
-        TRY(launch(c, K_MCONV, [&] {
-            return launch_macro_mass_rescale(c->stream, c->dim, (int)c->nc, c->vol, c->fields, c->W[w]);
-        }));
-    }
-    TRY(launch(c, K_MCONV, [&] {
-        return launch_macro_fields_from_W(c->stream, c->dim, (int)c->nc, c->model, c->W[w], c->fields_n);
-    }));
+    TRY(high_order_terms(c));
+    TRY(macro_solve(c));
+    TRY(macro_result(c));
     TRY(launch(c, K_SYNC, [&] {
         return launch_sync<Real>(c->stream, c->dim, (int)c->nc, c->tcm >= 1, vquad<Real>(c), oquad<Real>(c), c->model,
                                  c->solver.sync_relax, c->fields_n, c->fields_h, (const Real *)c->coef,
@@ -1808,6 +1996,7 @@ int gsis_shard_setup(gsis_ctx *c, int32_t n_xi_all, const double *xi_all, const 
     c->Vdp = vdp;
     c->NOd = n_omega_all;
     c->Odp = odp;
+    TRY(macro_velocity_set(c));
     const size_t nbf1 = std::max(c->n_bf, 1);
     c->xcount = (int64_t)((size_t)c->nc * NXC + nbf1 * (1 + KBR));
     TRY(dalloc(c, &c->xbuf, (size_t)c->xcount));
@@ -2171,14 +2360,12 @@ int gsis_mlp_samples(gsis_ctx *c, float *X, float *Y, int64_t n_cells) {
     if (c->dim == 3) return fail(c, GSIS_ERR_UNSUPPORTED, "the learned closure's features are built for 1-D and 2-D");
     TRY(mlp_ensure(c, 1));
     TRY(launch(c, K_MCONV, [&] {
-        return launch_macro_from_fields(c->stream, c->dim, (int)c->nc, c->model, c->fields, c->W[0]);
+        return launch_macro_from_fields(c->stream, c->dim, (int)c->nc, c->model, c->fields, c->mw);
     }));
-    TRY(launch(c, K_MGRAD, [&] {
-        return launch_macro_grad(c->stream, c->mg, 1, 0, c->model, nullptr, c->W[0], c->mq, c->mgrad, c->mphi);
-    }));
+    TRY(launch(c, K_MGRAD, [&] { return launch_macro_grad(c->stream, c->mg, 1, 0, nullptr, c->mw); }));
     TRY(launch(c, K_MLP, [&] {
-        return launch_cell_features(c->stream, c->mg, c->model, c->fields, c->mq, c->mgrad, c->mlp_X,
-                                    Y ? c->mlp_Y : nullptr);
+        return launch_cell_features(c->stream, c->mg, c->model, c->fields, c->mw.qd, (const double *)c->mw.grad,
+                                    c->mlp_X, Y ? c->mlp_Y : nullptr);
     }));
     CUDA_TRY(c, cudaMemcpyAsync(X, c->mlp_X, c->nc * MLP_IN * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
     if (Y)
@@ -2195,15 +2382,15 @@ int warm_start(gsis_ctx *c, int n_presolve, bool use_mlp) {
     if (use_mlp) TRY(mlp_ensure(c, c->nc));
     for (int k = 0; k < n_presolve; ++k) {
         TRY(launch(c, K_MCONV, [&] {
-            return launch_macro_from_fields(c->stream, c->dim, (int)c->nc, c->model, c->fields, c->W[0]);
+            return c->dim == 3 ? m3::launch_macro_from_fields(c->stream, c->dim, (int)c->nc, c->model, c->fields, c->w3.W[0])
+                               : launch_macro_from_fields(c->stream, c->dim, (int)c->nc, c->model, c->fields, c->mw);
         }));
-        TRY(launch(c, K_MGRAD, [&] {
-            return launch_macro_grad(c->stream, g, 1, 0, c->model, nullptr, c->W[0], c->mq, c->mgrad, c->mphi);
-        }));
+        if (use_mlp) TRY(launch(c, K_MGRAD, [&] { return launch_macro_grad(c->stream, g, 1, 0, nullptr, c->mw); }));
         if (use_mlp) {
             MlpDev &d = c->mlp;
             TRY(launch(c, K_MLP, [&] {
-                return launch_cell_features(c->stream, g, c->model, c->fields, c->mq, c->mgrad, d.act[0], nullptr);
+                return launch_cell_features(c->stream, g, c->model, c->fields, c->mw.qd, (const double *)c->mw.grad,
+                                            d.act[0], nullptr);
             }));
             CUDA_TRY(c, launch_mlp_standardise(c->stream, (int)c->nc, MLP_IN, d.act[0], x_mean(c), x_std(c), 0));
             CUDA_TRY(c, launch_mlp_forward(c->stream, d, (int)c->nc));
@@ -2211,24 +2398,19 @@ int warm_start(gsis_ctx *c, int n_presolve, bool use_mlp) {
                                                1));
             c->launches += 6;
             TRY(launch(c, K_MLP, [&] {
-                return launch_hot_from_cells(c->stream, g, c->mq, d.act[MLP_LAYERS], c->hot, c->hot_b);
+                return launch_hot_from_cells(c->stream, g, d.act[MLP_LAYERS], c->mw, c->hot_b);
             }));
         } else {
-            CUDA_TRY(c, cudaMemsetAsync(c->hot, 0, (size_t)std::max(g.n_fi, 1) * NHOT * sizeof(double), c->stream));
+            const size_t nf1 = (size_t)std::max(g.n_fi, 1), nh = nf1 * NVM;
+            if (c->dim == 3) CUDA_TRY(c, cudaMemsetAsync(c->w3.hot, 0, nf1 * m3::NHOT * sizeof(double), c->stream));
+            else CUDA_TRY(c, cudaMemsetAsync(c->mw.hot, 0, nh * sizeof(double), c->stream));
+            if (c->mw.hotf) CUDA_TRY(c, cudaMemsetAsync(c->mw.hotf, 0, nh * sizeof(float), c->stream));
             CUDA_TRY(c, cudaMemsetAsync(c->hot_b, 0, (size_t)std::max(g.n_bf, 1) * NVM * sizeof(double), c->stream));
         }
         if (c->moff)   // the pre-solve has no kinetic residual: no offset
             CUDA_TRY(c, cudaMemsetAsync(c->moff, 0, (size_t)c->nc * NVM * sizeof(double), c->stream));
-        int w = 0;
-        TRY(macro_solve(c, &w));
-        if (c->closed) {
-            TRY(launch(c, K_MCONV, [&] {
-                return launch_macro_mass_rescale(c->stream, c->dim, (int)c->nc, c->vol, c->fields, c->W[w]);
-            }));
-        }
-        TRY(launch(c, K_MCONV, [&] {
-            return launch_macro_fields_from_W(c->stream, c->dim, (int)c->nc, c->model, c->W[w], c->fields_n);
-        }));
+        TRY(macro_solve(c));
+        TRY(macro_result(c));
         std::swap(c->fields, c->fields_n);
     }
     TRY(launch(c, K_EQUIL, [&] {
@@ -2255,7 +2437,7 @@ int gsis_warm_start(gsis_ctx *c, int32_t n_presolve, int32_t use_mlp) {
 
 int gsis_macro_stats(gsis_ctx *c, int32_t *inner_iters, double *r0, double *rn) {
     if (!c) return GSIS_ERR_INVALID_ARG;
-    CUDA_TRY(c, cudaMemcpyAsync(c->h_mstate, c->mstate, sizeof(MacroState), cudaMemcpyDeviceToHost, c->stream));
+    CUDA_TRY(c, cudaMemcpyAsync(c->h_mstate, c->mw.state, sizeof(MacroState), cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     if (inner_iters) *inner_iters = c->h_mstate->it;
     if (r0) *r0 = c->h_mstate->r0;

@@ -193,14 +193,131 @@ __host__ __device__ inline void mix_from_A(const ModelDev &m, const double *A, d
     Mx[8] = 1.0 - A[8] * Zi;
 }
 
-// ---- synthetic (macroscopic) equations, FP64 throughout (macro.cu)
+// base = A^-1 diag(5, d_r, d_v): kappa_gas = mu/2 base (Eq. NSF_thermal_conductivities)
+__host__ __device__ inline void kappa_base(const double *A, double dr, double dv, double *B) {
+    const double det = A[0] * (A[4] * A[8] - A[5] * A[7]) - A[1] * (A[3] * A[8] - A[5] * A[6]) +
+                       A[2] * (A[3] * A[7] - A[4] * A[6]);
+    const double Ai[9] = {A[4] * A[8] - A[5] * A[7], A[2] * A[7] - A[1] * A[8], A[1] * A[5] - A[2] * A[4],
+                          A[5] * A[6] - A[3] * A[8], A[0] * A[8] - A[2] * A[6], A[2] * A[3] - A[0] * A[5],
+                          A[3] * A[7] - A[4] * A[6], A[1] * A[6] - A[0] * A[7], A[0] * A[4] - A[1] * A[3]};
+    const double dg[3] = {5.0, dr, dv};
+    for (int k = 0; k < 9; ++k) B[k] = Ai[k] / det * dg[k % 3];
+}
+
+// ---- synthetic (macroscopic) equations (macro.cu)
 // Conservative variables W = [rho, rho u (dim), e, e_r, e_v, e_R] (nv = dim + 5) and
 // primitive variables q = [rho, u (dim), T_t, T_r, T_v, e_R] (the same count).
-constexpr int NVM = 8;         // largest nv (dim = 3)
-constexpr int NHOT = 21;       // per-face high-order terms: sigma (dim x dim), q_t, q_r, q_v, q_R (dim each)
+constexpr int NVM = 8;         // largest nv (dim = 3), stride of the per-cell and per-face rows
 constexpr int MGS = 3;         // stride of the synthetic equations' geometry vectors and gradients
+constexpr int FGEO = 16;       // per-face record of MacroReal::fgeo
+constexpr int SRC = 16;        // per-cell source record
+constexpr int BINC = 12;       // per-wall-face constant sums (dim + 7 used)
+
+// Geometry, model constants and state that the synthetic equations read, in the type they
+// are evaluated in (FP64, and FP32 where the solver's residual side runs in FP32)
+template <typename R>
+struct MacroReal {
+    const R *lsq;              // [nc][Lay::MAXS][Lay::LW]
+    const R *eps2;             // [nc] (K dx)^3
+    const R *ivol, *hivol;     // [nc] 1 / V, 1 / (2 V)
+    const R *icdx;             // [nc] 1 / (cfl_macro dx)
+    const R *cdx;              // [nc][MAXF][MGS] face centroid - cell centroid (interior faces; minimal image)
+    const R *cnS;              // [nc][MAXF][MGS] outward normal times S / (2 V) (interior faces)
+    const R *fgeo;             // [n_fi][FGEO]: normal n (owner -> neighbour), t = (x_j - x_i) / |x_j - x_i|,
+                               // (n - (t.n) t) / 2, 1 / |x_j - x_i|, t.n / |x_j - x_i|, S, 1 / |n.(x_j - x_i)|
+    const R *bgeo;             // [n_bf][8]: outward normal, S, 1 / |n.(x_f - x_c)|
+    const R *vx, *vw;          // the FP64 velocity quadrature in R
+    const R *q;                // [nc][NVM] primitive variables
+    const R *hot;              // [n_fi][NVM] high-order terms on the face normal: stress (dim), heat fluxes (4)
+    R mu0, i_mu0, omega;       // mu = mu0 T^omega
+    R half_dr, half_dv, i_half_dr, i_half_dv, i_Zr, i_Zv;
+    R w_r, w_v, c_r, e_v;      // 3/(3+d_r), 3/(3+d_v), d_r/(3+d_r), d_v/(3+d_v)
+    R ik, kR0, sigma;          // 1/Kn_p, Kn_p/3, sigma_R
+    R base[9];                 // A^-1 diag(5, d_r, d_v)
+    int dens;                  // k_eff scaled by the density
+};
 
 struct MacroGeom {
+    int n_cells, dim, n_fi, n_bf;
+    MacroReal<double> d;
+    MacroReal<float> f;        // set when the solver's residual side runs in FP32
+    const int4 *fi4;           // [n_fi] owner, neighbour, and the face's place among each one's faces
+    const int *cface;          // [nc][MAXF] interior face id, or -1 - boundary face id; -1 - n_bf.. unused
+    const int *nb;             // [nc][MAXF] neighbour across an interior face, else -1
+    const unsigned char *own;  // [nc][MAXF] 1 where the cell is the face's owner
+    const int4 *info;          // [nc] faces, stencil size, face neighbours leading the stencil
+    const int *stn;            // [nc][Lay::MAXS]
+    const double *vol;         // [nc]
+    const int *bf_cell, *bf_patch; // [n_bf]
+    const double *bf_n;        // [n_bf][MGS] outward normal
+    const double *binc;        // [n_bf][BINC] constant sums of the wall faces
+    const int *patch_kind;     // [n_patches]: 0 wall, 1 far field, 2 mirror plane
+    const double *patch_state; // [n_patches][8]: rho, u[3], T_t, T_r, T_v, T_R
+    const int *bf_tab;         // [n_bf] mirror-reflection table of the face or -1 (as Geom)
+    const int *refl_v, *refl_o;
+    const double *moff;        // [nc][NVM] added to the synthetic residual (defect correction), or null
+};
+
+// Double-precision quadratures for the macroscopic boundary fluxes.
+struct QuadD {
+    int n, n_pad;
+    const double *x;           // [3][n_pad]
+    const double *w;           // [n_pad]
+};
+
+// Device-side state of one synthetic solve: inner iteration counter, first and
+// current residual norms, the stop flag every macro kernel reads first, and the ticket
+// counter of the kernels whose last CTA sums the partials (zero between launches).
+struct MacroState {
+    int it, done, max_inner;
+    unsigned int ticket;
+    double r0, rn, tol;
+};
+
+// State and work arrays of the synthetic equations; void* ones hold the compute type
+struct MacroWork {
+    double *W, *qd;            // [nc][NVM] conservative and primitive variables
+    float *qf;                 // [nc][NVM] FP32 copy of qd (null: no FP32 residual side)
+    void *grad, *rec;          // [nc][MGS][NVM], [nc][MAXF][NVM]
+    void *Fx, *fgam;           // [n_fi][NVM], [n_fi][2]
+    void *src, *gam;           // [nc][SRC], [nc][MAXF][2]
+    void *rows[2];             // [nc][NVM][4] relaxation records, alternating between sweeps
+    double *Rg, *Dinv;         // [nc][NVM], [nc][24]
+    double *mbf;               // [n_bf][NVM] macroscopic boundary fluxes
+    double *hot;               // [n_fi][NVM]
+    float *hotf;               // FP32 copy of hot (or null)
+    double *rpart, *fac;       // CTA partials, mass factor
+    MacroState *state;
+};
+
+cudaError_t launch_macro_from_fields(cudaStream_t s, int dim, int n_cells, const ModelDev &m, const double *F,
+                                     const MacroWork &w);
+// F_ref: null, or the fields whose total mass W is scaled to
+cudaError_t launch_macro_fields_from_W(cudaStream_t s, const MacroGeom &g, const ModelDev &m, const MacroWork &w,
+                                       const double *F_ref, double *F);
+// fp32 != 0: the residual side (gradients, limiters, fluxes, sources, D) is evaluated in
+// FP32 from FP32 copies of the state; the diagonal solves, updates and norms stay FP64.
+// st: null, or the solve's state (every kernel returns at once after its stop flag is set)
+cudaError_t launch_macro_grad(cudaStream_t s, const MacroGeom &g, int order, int fp32, const MacroState *st,
+                              const MacroWork &w);
+// interior and boundary face fluxes and cell sources; boundary_only: the boundary faces alone
+cudaError_t launch_macro_flux(cudaStream_t s, const MacroGeom &g, int order, int fp32, const ModelDev &m,
+                              const QuadD &vq, const MacroState *st, const MacroWork &w, bool boundary_only);
+cudaError_t launch_macro_binc(cudaStream_t s, const MacroGeom &g, const ModelDev &m, const QuadD &vq, const QuadD &oq,
+                              double *binc);
+cudaError_t launch_macro_hot(cudaStream_t s, const MacroGeom &g, int fp32, const ModelDev &m, const double *F_kin,
+                             const MacroWork &w, const double *kin_bflux, double *hot_b);
+// residual, D and the first relaxation sweep; with st also the norm and the stop flag
+cudaError_t launch_macro_residual(cudaStream_t s, const MacroGeom &g, int fp32, MacroState *st, const MacroWork &w,
+                                  const double *hot_b, double *history);
+// relaxation sweep number `sweep` >= 1; the last one updates W and q.  sweep = 0 with last:
+// the only sweep of a solver with macro_sweeps = 1.
+cudaError_t launch_macro_jacobi(cudaStream_t s, const MacroGeom &g, int fp32, const ModelDev &m, const MacroState *st,
+                                int sweep, bool last, const MacroWork &w);
+// ---- the 3-D solver (macro3d.cu)
+namespace m3 {
+constexpr int NHOT = 21;       // per-face high-order terms: sigma (3 x 3), q_t, q_r, q_v, q_R (3 each)
+struct Geom3 {
     int n_cells, dim, n_fi, n_bf;
     const int *fi_i, *fi_j;    // [n_fi] owner and neighbour of each interior face
     const double *fi_n;        // [n_fi][MGS] unit normal, owner -> neighbour
@@ -226,51 +343,35 @@ struct MacroGeom {
     const int *refl_v, *refl_o;
     const double *moff;        // [nc][NVM] added to the synthetic residual (defect correction), or null
 };
-
-// Double-precision quadratures for the macroscopic boundary fluxes.
-struct QuadD {
-    int n, n_pad;
-    const double *x;           // [3][n_pad]
-    const double *w;           // [n_pad]
-};
-
-// Device-side state of one synthetic solve: inner iteration counter, first and
-// current residual norms, and the stop flag every macro kernel reads first.
-struct MacroState {
-    int it, done, max_inner, pad;
-    double r0, rn, tol;
-};
-
-template <int DIM> struct MacroDims {
-    static constexpr int NV = DIM + 5, E = 1 + DIM, ER = 4 + DIM, NQ = DIM + 5;
-};
-
 cudaError_t launch_macro_from_fields(cudaStream_t s, int dim, int n_cells, const ModelDev &m, const double *F,
                                      double *W);
 cudaError_t launch_macro_fields_from_W(cudaStream_t s, int dim, int n_cells, const ModelDev &m, const double *W,
                                        double *F);
 // fp32 != 0: the residual side (gradients, limiters, fluxes, high-order terms, D) is
 // evaluated in FP32 with FP64 storage; the relaxation sweeps and norms stay FP64
-cudaError_t launch_macro_grad(cudaStream_t s, const MacroGeom &g, int order, int fp32, const ModelDev &m,
+cudaError_t launch_macro_grad(cudaStream_t s, const Geom3 &g, int order, int fp32, const ModelDev &m,
                               const MacroState *st, const double *W, double *q, double *grad, double *phi);
-cudaError_t launch_macro_bflux(cudaStream_t s, const MacroGeom &g, int fp32, const ModelDev &m, const QuadD &vq,
+cudaError_t launch_macro_bflux(cudaStream_t s, const Geom3 &g, int fp32, const ModelDev &m, const QuadD &vq,
                                const QuadD &oq, const MacroState *st, const double *q, double *bflux);
-cudaError_t launch_macro_hot(cudaStream_t s, const MacroGeom &g, int fp32, const ModelDev &m, const double *F_kin,
+cudaError_t launch_macro_hot(cudaStream_t s, const Geom3 &g, int fp32, const ModelDev &m, const double *F_kin,
                              const double *q, const double *grad, const double *kin_bflux, const double *mac_bflux,
                              double *hot, double *hot_b);
-cudaError_t launch_macro_residual(cudaStream_t s, const MacroGeom &g, int order, int fp32, const ModelDev &m,
+cudaError_t launch_macro_residual(cudaStream_t s, const Geom3 &g, int order, int fp32, const ModelDev &m,
                                   double cfl_macro, const MacroState *st, const double *W, const double *q,
                                   const double *grad, const double *phi, const double *hot, const double *bflux,
                                   const double *hot_b, double *Rg, double *Dinv, double *gam, double *rpart);
 cudaError_t launch_macro_norm(cudaStream_t s, int n_parts, const double *rpart, MacroState *st, double *history);
 // one relaxation sweep; fp32: the neighbours' flux increments in FP32 from the primitive
 // state q of W (the diagonal solve and the update stay FP64)
-cudaError_t launch_macro_jacobi(cudaStream_t s, const MacroGeom &g, int fp32, const ModelDev &m,
+cudaError_t launch_macro_jacobi(cudaStream_t s, const Geom3 &g, int fp32, const ModelDev &m,
                                 const MacroState *st, int first, int last, const double *W, const double *q,
                                 const double *Rg, const double *Dinv, const double *gam, const double *dG_in,
                                 double *dG_out, double *W_next);
 cudaError_t launch_macro_mass_rescale(cudaStream_t s, int dim, int n_cells, const double *vol, const double *F_ref,
                                       double *W);
+int macro_rpart_count(int n_cells);
+}  // namespace m3
+
 template <typename Real>
 cudaError_t launch_kinetic_bflux(cudaStream_t s, const MacroGeom &g, const ModelDev &m, const Quad<Real> &vq,
                                  const Quad<Real> &oq, const Real *f, const Real *I, double *kin_bflux,
@@ -314,8 +415,8 @@ int mlp_loss_parts(int n);
 cudaError_t launch_mlp_gather(cudaStream_t s, int n, int width, const int *idx, const float *src, float *dst);
 cudaError_t launch_cell_features(cudaStream_t s, const MacroGeom &g, const ModelDev &m, const double *F,
                                  const double *q, const double *grad, float *X, float *Y);
-cudaError_t launch_hot_from_cells(cudaStream_t s, const MacroGeom &g, const double *q, const float *Yc,
-                                  double *hot, double *hot_b);
+cudaError_t launch_hot_from_cells(cudaStream_t s, const MacroGeom &g, const float *Yc, const MacroWork &w,
+                                  double *hot_b);
 
 // ---- kernel launchers (kernels.cu); every launcher returns the launch status
 template <typename Real>

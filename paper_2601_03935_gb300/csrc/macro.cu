@@ -1,31 +1,47 @@
-// Synthetic (macroscopic) equations of GSIS in FP64 (Sections 2.2, 3 and 5).
+// Synthetic (macroscopic) equations of GSIS on 1-D and 2-D meshes (Sections 2.2, 3 and 5).
 //
-//  macro_from_fields   W = conservative variables of a field record
-//  macro_grad          primitive variables, least-squares gradients and Venkatakrishnan
-//                      limiters of every cell (the stencil of the kinetic sweep)
-//  macro_bflux         macroscopic flux through every boundary face: at walls the flux of
-//                      an equilibrium leaving at the cell state against the diffuse wall
-//                      (discrete velocity and direction sums), at the far field Rusanov
-//                      plus NSF against the free stream
-//  macro_hot           face high-order terms of Eq. (getHoTs): kinetic stress and heat
-//                      fluxes averaged to the face minus the NSF values of the kinetic
-//                      state; boundary terms = kinetic minus macroscopic boundary flux
+//  macro_from_fields   W = conservative variables of a field record, and the primitive ones
+//  macro_grad          least-squares gradients, Venkatakrishnan limiters and (order 2) the
+//                      reconstructed face values of every cell (the stencil of the sweep)
+//  macro_flux          three kinds of thread blocks in one launch: the flux and the Gamma of
+//                      every interior face; the flux through every boundary face (walls: an
+//                      equilibrium leaving at the cell state against the diffuse wall, as
+//                      discrete velocity and direction sums; far field: Rusanov plus NSF
+//                      against the free stream); the sources of every cell and their
+//                      Jacobian's coefficients
+//  macro_hot           face high-order terms of Eq. (getHoTs), projected on the face normal:
+//                      kinetic stress and heat fluxes averaged to the face minus the NSF
+//                      values of the kinetic state; boundary terms = kinetic minus
+//                      macroscopic boundary flux
 //  macro_residual      R = -(1/V) sum (F_c + F_v) S + Q (Eq. delta_macro, right-hand side),
 //                      the implicit diagonal D (with the exact local Jacobian of the energy
-//                      sources) and its inverse, and the per-block partial sums of |R|^2
-//  macro_norm          ||R||_2, the first-iteration reference and the stop flag
-//  macro_jacobi        one point-relaxation sweep of
+//                      sources) and its inverse, the first relaxation sweep D dW = R, and
+//                      ||R||_2 with the stop flag (its last block)
+//  macro_jacobi        one further point-relaxation sweep of
 //                      D dW_i + (1/(2V)) sum_j (dF_j - Gamma dW_j) S = R_i
-//                      in the gas-energy form, W_next = W + dW after the last sweep
+//                      in the gas-energy form; the last one adds dW to W
 //  kinetic_bflux       moments of the kinetic boundary fluxes of the current distribution
 //  sync                f <- f + w [f_eq(M^{k+1}) - f_eq(M^{k+1/2})] (Section 3) fused with
 //                      the velocity moments of the result
 //
 // Every kernel of the inner loop returns at once when the solve's stop flag is set,
 // so a fixed launch sequence can run past convergence without changing W.
+//
+// What bounds these kernels is the number of FP64 instructions on the longest chain (64 to
+// 76 cycles each, see fp64.cuh), then the launches (about 1 us each) and the chains of
+// dependent loads; the data (a few MB) stay in L2.  Hence: no divisions by geometry or
+// model constants (stored as reciprocals, in the compute type, so that the FP32 path
+// converts nothing), one lane per variable or row of a cell where few warps are in flight,
+// face fluxes once per face, and the relaxation reads its neighbours' flux increments as
+// vectors F_a that the neighbour formed once, not once per adjacent face.
+// Per inner iteration (six sweeps, a GSIS iteration less its kinetic part over 100): 20 000
+// cells, mixed schedule 307 -> 74 us; 2 048 cells, FP64 209 -> 61 us, mixed 112 -> 43 us;
+// 800 cells in 1-D, FP64, order 2, 174 -> 45 us.
+#include <algorithm>
 #include <cmath>
 
 #include "gsis_impl.cuh"
+#include "fp64.cuh"
 
 namespace gsis {
 
@@ -33,208 +49,162 @@ namespace {
 
 constexpr double PI = 3.14159265358979323846;
 
-// Helpers are templates on the compute type R (double for the plain FP64 path, float for
-// the FP32 path's residual evaluation); literals are written R(x) so that a float
-// instantiation issues no FP64 instruction.
+// Device functions are templates on the compute type R (double for the plain FP64 path,
+// float for the FP32 path's residual evaluation).
 template <typename R>
-__device__ __forceinline__ R viscosity(R T_t, const ModelDev &m) {
-    return R(sqrt(2.0 / PI)) * R(m.Kn) * pow(T_t, R(m.omega));          // mu = p_t tau
-}
-template <typename R>
-__device__ __forceinline__ R sound_speed(R T_t) { return sqrt(R(5) * T_t / R(3)); }
-template <typename R>
-__device__ __forceinline__ R absorption(R rho, const ModelDev &m) {
-    const R k = R(1) / R(m.Kn_p);
-    return m.k_eff_density_scaled ? k * rho : k;
+__device__ __forceinline__ const MacroReal<R> &real(const MacroGeom &g) {
+    if constexpr (sizeof(R) == 8) return g.d;
+    else return g.f;
 }
 
-// base = A^-1 diag(5, d_r, d_v); kappa_gas = mu/2 base (Eq. NSF_thermal_conductivities).
-// dv < 0: the model's constant d_v and A; else A and the last diagonal entry at this d_v.
+// mu = p_t tau
 template <typename R>
-__device__ void kappa_base(const ModelDev &m, R (&B)[3][3], double dv = -1.0) {
-    double Aloc[9];
-    if (dv >= 0.0) relaxation_matrix_at(m, dv, Aloc);
-    const double *A = dv >= 0.0 ? Aloc : m.A;
-    const double det = A[0] * (A[4] * A[8] - A[5] * A[7]) - A[1] * (A[3] * A[8] - A[5] * A[6]) +
-                       A[2] * (A[3] * A[7] - A[4] * A[6]);
-    double Ai[3][3];
-    Ai[0][0] = (A[4] * A[8] - A[5] * A[7]) / det;
-    Ai[0][1] = (A[2] * A[7] - A[1] * A[8]) / det;
-    Ai[0][2] = (A[1] * A[5] - A[2] * A[4]) / det;
-    Ai[1][0] = (A[5] * A[6] - A[3] * A[8]) / det;
-    Ai[1][1] = (A[0] * A[8] - A[2] * A[6]) / det;
-    Ai[1][2] = (A[2] * A[3] - A[0] * A[5]) / det;
-    Ai[2][0] = (A[3] * A[7] - A[4] * A[6]) / det;
-    Ai[2][1] = (A[1] * A[6] - A[0] * A[7]) / det;
-    Ai[2][2] = (A[0] * A[4] - A[1] * A[3]) / det;
-    const double dg[3] = {5.0, m.d_r, dv >= 0.0 ? dv : m.d_v};
-    for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) B[a][b] = R(Ai[a][b] * dg[b]);
+__device__ __forceinline__ R viscosity(R T_t, const MacroReal<R> &c) { return c.mu0 * pow_r(T_t, c.omega); }
+template <typename R>
+__device__ __forceinline__ R sound_speed(R T_t) { return sqrt_r(R(5.0 / 3.0) * T_t); }
+template <typename R>
+__device__ __forceinline__ R absorption(R rho, const MacroReal<R> &c) { return c.dens ? c.ik * rho : c.ik; }
+template <typename R>
+__device__ __forceinline__ R vib_e(R T, const ModelDev &m, const MacroReal<R> &c) {
+    return m.dv_T ? vib_energy<R>(m, T) : c.half_dv * T;
 }
 
-template <typename R, int DIM, typename S>
-__device__ __forceinline__ void primitive(const S *W, const ModelDev &m, R *q) {
-    constexpr int E = 1 + DIM;
-    const R rho = R(W[0]);
-    R ke = R(0);
-    q[0] = rho;
-    for (int a = 0; a < DIM; ++a) {
-        q[1 + a] = R(W[1 + a]) / rho;
-        ke += q[1 + a] * q[1 + a];
+// base = A^-1 diag(5, d_r, d_v) at d_v(T_v) of the face (Eq. NSF_thermal_conductivities,
+// kappa_gas = mu/2 base), or the model's constant one
+template <typename R>
+__device__ void kappa_at(const ModelDev &m, const MacroReal<R> &c, double Tv, R (&B)[3][3]) {
+    if (!m.dv_T) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) B[a][b] = c.base[a * 3 + b];
+        return;
     }
-    const R e = R(W[E]), er = R(W[E + 1]), ev = R(W[E + 2]), eR = R(W[E + 3]);
-    q[E] = (e - eR - er - ev - R(0.5) * rho * ke) / (R(1.5) * rho);
-    q[E + 1] = R(2) * er / (R(m.d_r) * rho);
-    q[E + 2] = vib_temperature<R>(m, ev / rho);
-    q[E + 3] = eR;
+    double A[9], D[9];
+    const double dv = dv_at(m, Tv);
+    relaxation_matrix_at(m, dv, A);
+    kappa_base(A, m.d_r, dv, D);
+    for (int k = 0; k < 9; ++k) B[k / 3][k % 3] = R(D[k]);
 }
 
-template <typename R, int DIM>
-__device__ __forceinline__ void prim_to_W(const R *q, const ModelDev &m, R *W) {
+template <int DIM>
+__device__ __forceinline__ void primitive(const double *W, const ModelDev &m, const MacroReal<double> &c, double *q) {
     constexpr int E = 1 + DIM;
-    const R rho = q[0];
-    R uu = R(0);
+    const double rho = W[0], ir = rcp_r(rho);
+    double ke = 0.0;
+    q[0] = rho;
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) {
+        q[1 + a] = W[1 + a] * ir;
+        ke = fma(q[1 + a], W[1 + a], ke);
+    }
+    q[E] = (W[E] - W[E + 3] - W[E + 1] - W[E + 2] - 0.5 * ke) * ((2.0 / 3.0) * ir);
+    q[E + 1] = W[E + 1] * (c.i_half_dr * ir);
+    q[E + 2] = m.dv_T ? vib_temperature<double>(m, W[E + 2] * ir) : W[E + 2] * (c.i_half_dv * ir);
+    q[E + 3] = W[E + 3];
+}
+
+template <int DIM>
+__device__ __forceinline__ void prim_to_W(const double *q, const ModelDev &m, double *W) {
+    constexpr int E = 1 + DIM;
+    const double rho = q[0];
+    double uu = 0.0;
     for (int a = 0; a < DIM; ++a) uu += q[1 + a] * q[1 + a];
-    const R er = R(0.5) * R(m.d_r) * rho * q[E + 1], ev = rho * vib_energy<R>(m, q[E + 2]);
+    const double er = 0.5 * m.d_r * rho * q[E + 1], ev = rho * vib_energy<double>(m, q[E + 2]);
     W[0] = rho;
     for (int a = 0; a < DIM; ++a) W[1 + a] = rho * q[1 + a];
-    W[E] = R(1.5) * rho * q[E] + R(0.5) * rho * uu + er + ev + q[E + 3];
+    W[E] = 1.5 * rho * q[E] + 0.5 * rho * uu + er + ev + q[E + 3];
     W[E + 1] = er;
     W[E + 2] = ev;
     W[E + 3] = q[E + 3];
 }
 
-// F_c . n of Eq. (macroscopic_equation); e_R has no convective flux
+// One side of a face: the convected variables U (rho, m, gas energy, e_r, e_v), their flux
+// F_c . n of Eq. (macroscopic_equation) and |u_n| + c_s.  e_R has no convective flux.
 template <typename R, int DIM>
-__device__ __forceinline__ void convective_flux(const R *q, const R *n, const ModelDev &m, R *F) {
+__device__ __forceinline__ R face_side(const R *q, const R *n, const ModelDev &m, const MacroReal<R> &c, R *U, R *F) {
     constexpr int E = 1 + DIM;
-    const R rho = q[0], T_t = q[E];
-    R un = R(0), uu = R(0);
+    const R rho = q[0];
+    R un = R(0), ke = R(0);
+    U[0] = rho;
+#pragma unroll
     for (int a = 0; a < DIM; ++a) {
-        un += q[1 + a] * n[a];
-        uu += q[1 + a] * q[1 + a];
+        U[1 + a] = rho * q[1 + a];
+        un = fma(q[1 + a], n[a], un);
+        ke = fma(U[1 + a], q[1 + a], ke);
     }
-    const R p = rho * T_t;
-    const R er = R(0.5) * R(m.d_r) * rho * q[E + 1], ev = rho * vib_energy<R>(m, q[E + 2]);
-    const R eg = R(1.5) * rho * T_t + R(0.5) * rho * uu + er + ev;
+    const R p = rho * q[E];
+    U[E + 1] = c.half_dr * rho * q[E + 1];
+    U[E + 2] = rho * vib_e(q[E + 2], m, c);
+    U[E] = fma(R(1.5), p, fma(R(0.5), ke, U[E + 1] + U[E + 2]));
     F[0] = rho * un;
-    for (int a = 0; a < DIM; ++a) F[1 + a] = rho * q[1 + a] * un + p * n[a];
-    F[E] = un * (eg + p);
-    F[E + 1] = un * er;
-    F[E + 2] = un * ev;
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) F[1 + a] = fma(U[1 + a], un, p * n[a]);
+    F[E] = un * (U[E] + p);
+    F[E + 1] = un * U[E + 1];
+    F[E + 2] = un * U[E + 2];
+    return fabs(un) + sound_speed(q[E]);
+}
+
+// Rusanov flux times `scale`: average of the two fluxes minus half the largest |u_n| + c_s
+// times the jump of the convected variables (gas energy, not e_R)
+template <typename R, int DIM>
+__device__ __forceinline__ void rusanov(const R *qL, const R *qR, const R *n, R scale, const ModelDev &m,
+                                        const MacroReal<R> &c, R *F) {
+    constexpr int E = 1 + DIM;
+    R UL[E + 3], UR[E + 3], FL[E + 3], FR[E + 3];
+    const R lL = face_side<R, DIM>(qL, n, m, c, UL, FL), lR = face_side<R, DIM>(qR, n, m, c, UR, FR);
+    const R lam = max_pos(lL, lR), h = R(0.5) * scale;
+#pragma unroll
+    for (int k = 0; k < E + 3; ++k) F[k] = h * fma(lam, UL[k] - UR[k], FL[k] + FR[k]);
     F[E + 3] = R(0);
 }
 
-// Rusanov flux: average of the two fluxes minus half the largest |u_n| + c_s times the
-// jump of the convected variables (gas energy, not e_R)
-template <typename R, int DIM>
-__device__ void rusanov(const R *qL, const R *qR, const R *n, const ModelDev &m, R *F) {
-    constexpr int NV = DIM + 5, E = 1 + DIM;
-    R FL[NV], FR[NV], WL[NV], WR[NV];
-    convective_flux<R, DIM>(qL, n, m, FL);
-    convective_flux<R, DIM>(qR, n, m, FR);
-    R unL = R(0), unR = R(0);
-    for (int a = 0; a < DIM; ++a) {
-        unL += qL[1 + a] * n[a];
-        unR += qR[1 + a] * n[a];
-    }
-    const R lam = fmax(fabs(unL) + sound_speed(qL[E]), fabs(unR) + sound_speed(qR[E]));
-    prim_to_W<R, DIM>(qL, m, WL);
-    prim_to_W<R, DIM>(qR, m, WR);
-    for (int k = 0; k < NV; ++k) {
-        R dW = WR[k] - WL[k];
-        if (k == E) dW -= WR[E + 3] - WL[E + 3];
-        if (k == E + 3) dW = R(0);
-        F[k] = R(0.5) * (FL[k] + FR[k]) - R(0.5) * lam * dW;
-    }
-}
-
-// Venkatakrishnan's limiter function
+// Venkatakrishnan's limiter function phi_V = num / den
 template <typename R>
-__device__ __forceinline__ R venkat(R d1, R d2, R eps2) {
-    return (d1 * d1 + eps2 + R(2) * d1 * d2) / (d1 * d1 + R(2) * d2 * d2 + d1 * d2 + eps2);
-}
-
-// Q of Section 5: rotational and vibrational relaxation, gas-photon exchange
-template <typename R, int DIM>
-__device__ void source(const R *q, const ModelDev &m, R *Q) {
-    constexpr int NV = DIM + 5, E = 1 + DIM;
-    const R rho = q[0], Tt = q[E], Tr = q[E + 1], Tv = q[E + 2], eR = q[E + 3];
-    const R dr = R(m.d_r);
-    const R Ttr = (R(3) * Tt + dr * Tr) / (R(3) + dr);
-    const R ev = vib_energy<R>(m, Tv);
-    const R Ttv = equal_temperature<R>(m, R(3), R(3) * Tt + R(2) * ev);
-    const R tau = R(sqrt(2.0 / PI)) * pow(Tt, R(m.omega - 1.0)) * R(m.Kn) / rho;
-    const R k = absorption(rho, m);
-    const R evR = R(4) * R(m.sigma_R) * Tv * Tv * Tv * Tv;
-    for (int a = 0; a < NV; ++a) Q[a] = R(0);
-    Q[E + 1] = R(0.5) * dr * rho * (Ttr - Tr) / (R(m.Z_r) * tau);
-    // (e_tv - e_v) / (Z_v tau) - k_eff (e_vR - e_R), e_tv = d_v(T_tv) rho T_tv / 2
-    Q[E + 2] = rho * (vib_energy<R>(m, Ttv) - ev) / (R(m.Z_v) * tau) - k * (evR - eR);
-    Q[E + 3] = k * (evR - eR);
-}
-
-// exact d(Q_egas, Q_r, Q_v, Q_R)/d(e_gas, e_r, e_v, e_R) with rho, rho u, tau, k_eff frozen
-template <typename R, int DIM>
-__device__ void source_jacobian(const R *q, const ModelDev &m, R (&J)[4][4]) {
-    constexpr int E = 1 + DIM;
-    // Q_v = rho (eps(T_tv) - eps_v) / (Z_v tau) - k (e_vR - e_R), eps(T) = d_v(T) T / 2,
-    // 3 T_tv + 2 eps(T_tv) = 3 T_t + 2 eps_v: d(rho eps(T_tv)) = 3 a b (de_gas - de_r) with
-    // b = rho eps'(T_tv) / (3 + 2 eps'(T_tv)), a = dT_t/de_gas (the de_v terms cancel);
-    // d e_vR / d e_v = 16 sigma_R T_v^3 / (rho eps'(T_v))
-    const R rho = q[0], Tt = q[E], Tv = q[E + 2];
-    const R dr = R(m.d_r);
-    const R tau = R(sqrt(2.0 / PI)) * pow(Tt, R(m.omega - 1.0)) * R(m.Kn) / rho;
-    const R k = absorption(rho, m);
-    const R cr = rho * R(1.5) * dr / (R(3) + dr) / (R(m.Z_r) * tau);
-    const R Ttv = equal_temperature<R>(m, R(3), R(3) * Tt + R(2) * vib_energy<R>(m, Tv));
-    const R ctv = vib_cv<R>(m, Ttv);
-    const R b = rho * ctv / (R(3) + R(2) * ctv);
-    const R zv = R(1) / (R(m.Z_v) * tau);
-    const R beta = R(16) * R(m.sigma_R) * Tv * Tv * Tv / (rho * vib_cv<R>(m, Tv));
-    const R a = R(1) / (R(1.5) * rho);
-    for (int r = 0; r < 4; ++r)
-        for (int c = 0; c < 4; ++c) J[r][c] = R(0);
-    J[0][2] = -k * beta;
-    J[0][3] = k;
-    J[1][0] = cr * a;
-    J[1][1] = -cr * (a + R(2) / (dr * rho));
-    J[1][2] = -cr * a;
-    J[2][0] = R(3) * a * b * zv;
-    J[2][1] = -R(3) * a * b * zv;
-    J[2][2] = -zv - k * beta;
-    J[2][3] = k;
-    J[3][2] = k * beta;
-    J[3][3] = -k;
+__device__ __forceinline__ void venkat(R d1, R d2, R eps2, R &num, R &den) {
+    const R t = d1 + d2;
+    num = fma(d1, t + d2, eps2);
+    den = fma(d1, t, fma(d2 + d2, d2, eps2));
 }
 
 }  // namespace
 
 // ------------------------------------------------------------------ conversions (FP64)
+// q [nc][NVM] in FP64, and its rounding qf where the FP32 path reads it (else null)
 template <int DIM>
-__global__ void k_macro_from_fields(int n_cells, ModelDev m, const double *__restrict__ F, double *__restrict__ W) {
+__global__ void k_macro_from_fields(int n_cells, ModelDev m, const double *__restrict__ F, double *__restrict__ W,
+                                    double *__restrict__ q, float *__restrict__ qf) {
     constexpr int NV = DIM + 5, E = 1 + DIM;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_cells) return;
     const double *r = F + (size_t)i * NF;
-    double q[NV];
-    q[0] = r[0];
-    for (int a = 0; a < DIM; ++a) q[1 + a] = r[1 + a];
-    q[E] = r[4];
-    q[E + 1] = r[5];
-    q[E + 2] = r[6];
+    double x[NV];
+    x[0] = r[0];
+    for (int a = 0; a < DIM; ++a) x[1 + a] = r[1 + a];
+    x[E] = r[4];
+    x[E + 1] = r[5];
+    x[E + 2] = r[6];
     const double TR = r[7];
-    q[E + 3] = 4.0 * m.sigma_R * TR * TR * TR * TR;
-    prim_to_W<double, DIM>(q, m, W + (size_t)i * NVM);
+    x[E + 3] = 4.0 * m.sigma_R * TR * TR * TR * TR;
+    prim_to_W<DIM>(x, m, W + (size_t)i * NVM);
+    for (int v = 0; v < NV; ++v) {
+        q[(size_t)i * NVM + v] = x[v];
+        if (qf) qf[(size_t)i * NVM + v] = fp64::narrow(x[v]);
+    }
 }
 
+// fac: null, or the factor of k_macro_mass that W is scaled by
 template <int DIM>
-__global__ void k_macro_fields_from_W(int n_cells, ModelDev m, const double *__restrict__ W, double *__restrict__ F) {
+__global__ void k_macro_fields_from_W(int n_cells, ModelDev m, MacroReal<double> c, const double *__restrict__ W,
+                                      const double *__restrict__ fac, double *__restrict__ F) {
     constexpr int NV = DIM + 5, E = 1 + DIM;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_cells) return;
-    double q[NV];
-    primitive<double, DIM>(W + (size_t)i * NVM, m, q);
+    double w[NV], q[NV];
+    const double s = fac ? *fac : 1.0;
+    for (int v = 0; v < NV; ++v) w[v] = s * W[(size_t)i * NVM + v];
+    primitive<DIM>(w, m, c, q);
     double *r = F + (size_t)i * NF;
     for (int k = 0; k < NF; ++k) r[k] = 0.0;
     r[0] = q[0];
@@ -242,191 +212,160 @@ __global__ void k_macro_fields_from_W(int n_cells, ModelDev m, const double *__r
     r[4] = q[E];
     r[5] = q[E + 1];
     r[6] = q[E + 2];
-    r[7] = sqrt(sqrt(fmax(q[E + 3], 0.0) / (4.0 * m.sigma_R)));
+    r[7] = sqrt_r(sqrt_r(fmax(q[E + 3], 0.0) / (4.0 * m.sigma_R)));
 }
 
 // ------------------------------------------------------------------ gradients and limiters
-// q [nc][NVM], grad [nc][2][NVM], phi [nc][NVM] (stored in FP64, computed in R)
+// Eight lanes per cell, lane v = primitive variable v: q [nc][NVM] -> grad [nc][MGS][NVM]
+// and, at order 2, the limited reconstruction at every interior face of the cell,
+// rec [nc][MAXF][NVM].  The limiter's minimum over the faces is taken at the largest and the
+// most negative Delta_2 (phi_V falls beyond Delta_1 / 4 and exceeds 1 below Delta_1 / 2), and
+// in FP64 the smaller of the two quotients is found without dividing (their terms are positive).
 template <typename R, int DIM, int ORDER>
-__global__ void k_macro_grad(MacroGeom g, ModelDev m, const MacroState *__restrict__ st, const double *__restrict__ W,
-                             double *__restrict__ qo, double *__restrict__ grad, double *__restrict__ phi) {
-    constexpr int NQ = DIM + 5;
+__global__ void __launch_bounds__(128) k_macro_grad(MacroGeom g, const MacroState *__restrict__ st,
+                                                    R *__restrict__ grad, R *__restrict__ rec) {
+    constexpr int NV = DIM + 5, MS = Lay<DIM>::MAXS, LW = Lay<DIM>::LW;
     if (st && st->done) return;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= g.n_cells) return;
-    R qi[NQ], gr[DIM][NQ], dmax[NQ], dmin[NQ];
-    primitive<R, DIM>(W + (size_t)i * NVM, m, qi);
-    for (int k = 0; k < NQ; ++k) {
-        dmax[k] = R(0);
-        dmin[k] = R(0);
-        for (int a = 0; a < DIM; ++a) gr[a][k] = R(0);
-    }
+    const MacroReal<R> &c = real<R>(g);
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, i = t / NVM, v = t % NVM;
+    if (i >= g.n_cells || v >= NV) return;
+    const R qi = c.q[(size_t)i * NVM + v];
+    R gr[DIM], hi = R(0), lo = -R(0);
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) gr[a] = R(0);
     const int4 info = g.info[i];
-    for (int k = 0; k < info.y; ++k) {
-        const int s = g.stn[i * Lay<DIM>::MAXS + k];
-        R qs[NQ];
-        primitive<R, DIM>(W + (size_t)s * NVM, m, qs);
-        const double *C = g.lsq + ((size_t)i * Lay<DIM>::MAXS + k) * Lay<DIM>::LW;
-        for (int v = 0; v < NQ; ++v) {
-            const R dq = qs[v] - qi[v];
-            for (int a = 0; a < DIM; ++a) gr[a][v] += R(C[a]) * dq;
-            if (k < info.z) {
-                dmax[v] = fmax(dmax[v], dq);
-                dmin[v] = fmin(dmin[v], dq);
+    const int *stn = g.stn + (size_t)i * MS;
+    const R *lw = c.lsq + (size_t)i * MS * LW;
+    // two entries at a time: entries past the end hold cell 0 and zero weights
+    for (int k = 0; k < info.y; k += 2) {
+        const R q0 = c.q[(size_t)stn[k] * NVM + v], q1 = c.q[(size_t)stn[k + 1] * NVM + v];
+        const R d0 = q0 - qi, d1 = q1 - qi;
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) gr[a] = fma(lw[k * LW + a], d0, gr[a]);
+        if (k + 1 < info.y) {
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) gr[a] = fma(lw[(k + 1) * LW + a], d1, gr[a]);
+        }
+        if (ORDER == 2 && k < info.z) {
+            hi = max_pos(hi, d0);
+            lo = min_neg(lo, d0);
+            if (k + 1 < info.z) {
+                hi = max_pos(hi, d1);
+                lo = min_neg(lo, d1);
             }
         }
     }
-    for (int v = 0; v < NQ; ++v) {
-        qo[(size_t)i * NVM + v] = qi[v];
-        for (int a = 0; a < DIM; ++a) grad[((size_t)i * MGS + a) * NVM + v] = gr[a][v];
-    }
-    if constexpr (ORDER != 2) return;
-    R ph[NQ];
-    for (int v = 0; v < NQ; ++v) ph[v] = R(1);
-    const R eps2 = R(g.eps2[i]);
-    for (int k = 0; k < info.x; ++k) {
-        const int fid = g.cface[i * MAXF + k];
-        if (fid < 0) continue;
-        R d[DIM];
-        const double *dxf = g.fi_dx + ((size_t)fid * 2 + (g.fi_i[fid] == i ? 0 : 1)) * MGS;
-        for (int a = 0; a < DIM; ++a) d[a] = R(dxf[a]);
-        for (int v = 0; v < NQ; ++v) {
-            R d2 = R(0);
-            for (int a = 0; a < DIM; ++a) d2 += gr[a][v] * d[a];
-            const R d1 = d2 > R(0) ? dmax[v] : dmin[v];
-            const R pf = d2 != R(0) ? venkat(d1, d2, eps2) : R(1);
-            ph[v] = fmin(ph[v], pf);
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) grad[((size_t)i * MGS + a) * NVM + v] = gr[a];
+    if constexpr (ORDER == 2) {
+        R d2[MAXF], h2 = R(0), l2 = -R(0);
+#pragma unroll
+        for (int k = 0; k < MAXF; ++k) {
+            d2[k] = R(0);
+            if (g.nb[i * MAXF + k] < 0) continue;
+            const R *dx = c.cdx + ((size_t)i * MAXF + k) * MGS;
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) d2[k] = fma(gr[a], dx[a], d2[k]);
+            h2 = max_pos(h2, d2[k]);
+            l2 = min_neg(l2, d2[k]);
         }
+        const R eps2 = c.eps2[i];
+        R nh, dh, nl, dl;
+        venkat(hi, h2, eps2, nh, dh);       // h2 = 0: num = den, phi = 1
+        venkat(lo, l2, eps2, nl, dl);
+        R phi;
+        if constexpr (sizeof(R) == 8) {
+            const bool low = nl * dh < nh * dl;
+            const R num = low ? nl : nh, den = low ? dl : dh;
+            phi = num < den ? num * rcp_r(den) : R(1);
+        } else {
+            phi = fmin(fmin(R(1), nh < dh ? nh / dh : R(1)), nl < dl ? nl / dl : R(1));
+        }
+#pragma unroll
+        for (int k = 0; k < MAXF; ++k)
+            if (g.nb[i * MAXF + k] >= 0) rec[((size_t)i * MAXF + k) * NVM + v] = fma(phi, d2[k], qi);
     }
-    for (int v = 0; v < NQ; ++v) phi[(size_t)i * NVM + v] = ph[v];
 }
 
 // ------------------------------------------------------------------ face fluxes
 namespace {
 
-// NSF stress and heat fluxes of Eqs. (NSF_constitutive) and (NSF_thermal_conductivities)
-// at an interior face from the face-average state pf and the face gradient fg[a][v]
-// (gradient component a of primitive variable v); out layout as the high-order terms:
-// sigma (DIM x DIM), q_t, q_r, q_v, q_R (DIM each).
+// NSF terms of an interior face on its normal: sn = sigma . n (DIM), qn = q . n of the
+// translational, rotational and vibrational modes and of the photons (4); pf the
+// face-average state.  Eqs. (NSF_constitutive) and (NSF_thermal_conductivities) with the
+// face gradient = average of the cells' least-squares gradients with the component along
+// x_j - x_i replaced by the difference quotient; the scalars need its normal component only.
 template <typename R, int DIM>
-__device__ void nsf_face(const R *pf, const R (&fg)[DIM][DIM + 5], const ModelDev &m, const R (&base0)[3][3], R *out) {
-    constexpr int E = 1 + DIM;
-    R base[3][3];
-    if (m.dv_T) kappa_base<R>(m, base, dv_at(m, double(pf[E + 2])));   // at the face's T_v
-    else
-        for (int a = 0; a < 3; ++a)
-            for (int c = 0; c < 3; ++c) base[a][c] = base0[a][c];
-    const R mu = viscosity(pf[E], m);
-    R div = R(0);
-    for (int d = 0; d < DIM; ++d) div += fg[d][1 + d];
-    for (int a = 0; a < DIM; ++a)
-        for (int b = 0; b < DIM; ++b) {
-            const R S = fg[a][1 + b] + fg[b][1 + a];
-            out[a * DIM + b] = -mu * (S - (a == b ? R(2) / R(3) * div : R(0)));
-        }
-    for (int md = 0; md < 3; ++md)
-        for (int d = 0; d < DIM; ++d) {
-            R s = R(0);
-            for (int nn = 0; nn < 3; ++nn) s += R(0.5) * mu * base[md][nn] * fg[d][E + nn];
-            out[DIM * DIM + md * DIM + d] = -s;
-        }
-    const R kR = R(1) / (R(3) * absorption(pf[0], m));
-    for (int d = 0; d < DIM; ++d) out[DIM * DIM + 3 * DIM + d] = -kR * fg[d][E + 3];
-}
-
-// face-average state and face gradient (average of the cells' least-squares gradients
-// with the component along x_j - x_i replaced by the difference quotient)
-template <typename R, int DIM>
-__device__ void face_state(const MacroGeom &g, int fid, const double *q, const double *grad, R *pf,
-                           R (&fg)[DIM][DIM + 5]) {
-    constexpr int NQ = DIM + 5;
-    const int i = g.fi_i[fid], j = g.fi_j[fid];
-    const double *qi = q + (size_t)i * NVM, *qj = q + (size_t)j * NVM;
-    const double *t = g.fi_t + (size_t)fid * MGS;
-    const R dist = R(g.fi_dist[fid]);
-    for (int v = 0; v < NQ; ++v) {
-        const R qiv = R(qi[v]), qjv = R(qj[v]);
-        pf[v] = R(0.5) * (qiv + qjv);
-        R along = R(0);
-        R avg[DIM];
-        for (int a = 0; a < DIM; ++a) {
-            avg[a] = R(0.5) * (R(grad[((size_t)i * MGS + a) * NVM + v]) + R(grad[((size_t)j * MGS + a) * NVM + v]));
-            along += R(t[a]) * avg[a];
-        }
-        const R jump = (qjv - qiv) / dist;
-        for (int a = 0; a < DIM; ++a) fg[a][v] = avg[a] + R(t[a]) * (jump - along);
-    }
-}
-
-// (F_c + F_v) . n of interior face fid (owner -> neighbour orientation)
-template <typename R, int DIM, int ORDER>
-__device__ void interior_flux(const MacroGeom &g, const ModelDev &m, const R (&base)[3][3], int fid, const double *q,
-                              const double *grad, const double *phi, const double *hot, R *F) {
-    constexpr int NV = DIM + 5, E = 1 + DIM;
-    const int i = g.fi_i[fid], j = g.fi_j[fid];
-    R n[DIM];
-    for (int a = 0; a < DIM; ++a) n[a] = R(g.fi_n[(size_t)fid * MGS + a]);
-    R qL[NV], qR[NV];
+__device__ __forceinline__ void nsf_normal(const MacroGeom &g, const ModelDev &m, const R *fg16, int i, int j,
+                                           const R *__restrict__ grad, R *pf, R &mu, R &irho, R &kR, R *sn, R *qn) {
+    constexpr int E = 1 + DIM, NV = DIM + 5;
+    const MacroReal<R> &c = real<R>(g);
+    const R *n = fg16, *t = fg16 + 3, *mh = fg16 + 6;
+    const R invd = fg16[9], tnd = fg16[10];
+    const R *qi = c.q + (size_t)i * NVM, *qj = c.q + (size_t)j * NVM;
+    const R *gi = grad + (size_t)i * MGS * NVM, *gj = grad + (size_t)j * MGS * NVM;
+    R jump[NV];
+#pragma unroll
     for (int v = 0; v < NV; ++v) {
-        qL[v] = R(q[(size_t)i * NVM + v]);
-        qR[v] = R(q[(size_t)j * NVM + v]);
+        const R a = qi[v], b = qj[v];
+        pf[v] = R(0.5) * (a + b);
+        jump[v] = b - a;
     }
-    if (ORDER == 2) {
-        const double *dxf = g.fi_dx + (size_t)fid * 2 * MGS;
-        R di[DIM], dj[DIM];
+    R gu[DIM][DIM];       // gu[a][b] = d u_b / d x_a
+#pragma unroll
+    for (int b = 0; b < DIM; ++b) {
+        R s[DIM], along = R(0);
+#pragma unroll
         for (int a = 0; a < DIM; ++a) {
-            di[a] = R(dxf[a]);
-            dj[a] = R(dxf[MGS + a]);
+            s[a] = R(0.5) * (gi[a * NVM + 1 + b] + gj[a * NVM + 1 + b]);
+            along = fma(t[a], s[a], along);
         }
-        for (int v = 0; v < NV; ++v) {
-            R dL = R(0), dR = R(0);
-            for (int a = 0; a < DIM; ++a) {
-                dL += R(grad[((size_t)i * MGS + a) * NVM + v]) * di[a];
-                dR += R(grad[((size_t)j * MGS + a) * NVM + v]) * dj[a];
-            }
-            qL[v] += R(phi[(size_t)i * NVM + v]) * dL;
-            qR[v] += R(phi[(size_t)j * NVM + v]) * dR;
-        }
+        const R d = fma(jump[1 + b], invd, -along);
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) gu[a][b] = fma(t[a], d, s[a]);
     }
-    rusanov<R, DIM>(qL, qR, n, m, F);
-    R pf[NV], fg[DIM][DIM + 5], s[NHOT];
-    face_state<R, DIM>(g, fid, q, grad, pf, fg);
-    nsf_face<R, DIM>(pf, fg, m, base, s);
-    const double *h = hot + (size_t)fid * NHOT;
-    for (int k = 0; k < DIM * DIM + 4 * DIM; ++k) s[k] += R(h[k]);
-    R sn[DIM], un = R(0), qn[4] = {R(0), R(0), R(0), R(0)};
+    R gn[4];              // normal derivatives of T_t, T_r, T_v, e_R
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        gn[k] = tnd * jump[E + k];
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) gn[k] = fma(mh[a], gi[a * NVM + E + k] + gj[a * NVM + E + k], gn[k]);
+    }
+    R base[3][3];
+    kappa_at<R>(m, c, m.dv_T ? to_double(pf[E + 2]) : 0.0, base);
+    mu = viscosity(pf[E], c);
+    R div = R(0);
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) div += gu[a][a];
+    div *= R(2.0 / 3.0);
+#pragma unroll
     for (int a = 0; a < DIM; ++a) {
-        sn[a] = R(0);
-        for (int b = 0; b < DIM; ++b) sn[a] += s[a * DIM + b] * n[b];
-        un += sn[a] * pf[1 + a];
+        R s = -div * n[a];
+#pragma unroll
+        for (int b = 0; b < DIM; ++b) s = fma(gu[a][b] + gu[b][a], n[b], s);
+        sn[a] = -mu * s;
     }
-    R qtot = R(0);
-    for (int d = 0; d < DIM; ++d) {
-        const R *qq = s + DIM * DIM;
-        qtot += (qq[d] + qq[DIM + d] + qq[2 * DIM + d] + qq[3 * DIM + d]) * n[d];
-        for (int md = 0; md < 4; ++md) qn[md] += qq[md * DIM + d] * n[d];
-    }
-    for (int a = 0; a < DIM; ++a) F[1 + a] += sn[a];
-    F[E] += un + qtot;
-    F[E + 1] += qn[1];
-    F[E + 2] += qn[2];
-    F[E + 3] += qn[3];
+    const R hm = R(-0.5) * mu;
+#pragma unroll
+    for (int md = 0; md < 3; ++md) qn[md] = hm * fma(base[md][0], gn[0], fma(base[md][1], gn[1], base[md][2] * gn[2]));
+    irho = rcp_r(pf[0]);
+    kR = c.dens ? c.kR0 * irho : c.kR0;
+    qn[3] = -kR * gn[3];
 }
 
 // Far-field boundary flux: Rusanov against the free stream plus NSF terms over the
 // distance from the cell centre to the face
 template <typename R, int DIM>
-__device__ void farfield_flux(const MacroGeom &g, const ModelDev &m, const R (&base0)[3][3], int b, const R *qc, R *F) {
+__device__ void farfield_flux(const MacroGeom &g, const ModelDev &m, int b, const R *qc, R *F) {
     constexpr int E = 1 + DIM;
+    const MacroReal<R> &c = real<R>(g);
     const double *P = g.patch_state + (size_t)g.bf_patch[b] * 8;
     R base[3][3];
-    if (m.dv_T) kappa_base<R>(m, base, dv_at(m, 0.5 * (double(qc[E + 2]) + P[6])));   // at the face's T_v
-    else
-        for (int a = 0; a < 3; ++a)
-            for (int c = 0; c < 3; ++c) base[a][c] = base0[a][c];
+    kappa_at<R>(m, c, m.dv_T ? 0.5 * (to_double(qc[E + 2]) + P[6]) : 0.0, base);   // at the face's T_v
+    const R *bg = c.bgeo + (size_t)b * 8;
     R n[DIM];
-    for (int a = 0; a < DIM; ++a) n[a] = R(g.bf_n[(size_t)b * MGS + a]);
-    const R dn = R(g.bf_dn[b]);
+    for (int a = 0; a < DIM; ++a) n[a] = bg[a];
+    const R idn = bg[4];
     R qf[DIM + 5];
     qf[0] = R(P[0]);
     for (int a = 0; a < DIM; ++a) qf[1 + a] = R(P[1 + a]);
@@ -434,8 +373,8 @@ __device__ void farfield_flux(const MacroGeom &g, const ModelDev &m, const R (&b
     qf[E + 1] = R(P[5]);
     qf[E + 2] = R(P[6]);
     qf[E + 3] = R(4.0 * m.sigma_R * P[7] * P[7] * P[7] * P[7]);
-    rusanov<R, DIM>(qc, qf, n, m, F);
-    const R mu = viscosity(R(0.5) * (qc[E] + qf[E]), m);
+    rusanov<R, DIM>(qc, qf, n, R(1), m, c, F);
+    const R mu = viscosity(R(0.5) * (qc[E] + qf[E]), c);
     R du[DIM], dun = R(0);
     for (int a = 0; a < DIM; ++a) {
         du[a] = qf[1 + a] - qc[1 + a];
@@ -443,7 +382,7 @@ __device__ void farfield_flux(const MacroGeom &g, const ModelDev &m, const R (&b
     }
     R sn[DIM], snu = R(0);
     for (int a = 0; a < DIM; ++a) {
-        sn[a] = -mu / dn * (du[a] + (dun / R(3)) * n[a]);
+        sn[a] = -mu * idn * (du[a] + (dun * R(1.0 / 3.0)) * n[a]);
         snu += sn[a] * R(0.5) * (qf[1 + a] + qc[1 + a]);
     }
     const R dT[3] = {qf[E] - qc[E], qf[E + 1] - qc[E + 1], qf[E + 2] - qc[E + 2]};
@@ -451,10 +390,10 @@ __device__ void farfield_flux(const MacroGeom &g, const ModelDev &m, const R (&b
     for (int md = 0; md < 3; ++md) {
         R s = R(0);
         for (int nn = 0; nn < 3; ++nn) s += R(0.5) * mu * base[md][nn] * dT[nn];
-        qm[md] = -s / dn;
+        qm[md] = -s * idn;
     }
-    const R keff = absorption(qc[0], m);
-    const R qR = -(qf[E + 3] - qc[E + 3]) / (R(3) * keff * dn);
+    const R kR = c.dens ? c.kR0 * rcp_r(qc[0]) : c.kR0;
+    const R qR = -(qf[E + 3] - qc[E + 3]) * kR * idn;
     for (int a = 0; a < DIM; ++a) F[1 + a] += sn[a];
     F[E] += snu + (qm[0] + qm[1] + qm[2]) + qR;
     F[E + 1] += qm[1];
@@ -462,162 +401,307 @@ __device__ void farfield_flux(const MacroGeom &g, const ModelDev &m, const R (&b
     F[E + 3] += qR;
 }
 
-// block-wide sum of n values per thread; red[k] holds the sums for every thread after return
-template <int NT, typename R>
-__device__ void block_sum(R *vals, int n, R *red) {
-    __shared__ R buf[NT / 32][16];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int k = 0; k < n; ++k) {
-        R x = vals[k];
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if (lane == 0) buf[w][k] = x;
-    }
+constexpr int MF_NT = 128;            // threads of a flux CTA
+constexpr int MF_FACES = MF_NT / 2;   // interior faces of one: half the threads take each part
+
+// sum over the CTA of each of N values per thread, valid in thread 0
+template <int N, typename R>
+__device__ __forceinline__ void cta_sum(R (&x)[N], R (&buf)[MF_NT / 32][N]) {
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x[k] += __shfl_xor_sync(0xffffffffu, x[k], o);
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+        for (int k = 0; k < N; ++k) buf[threadIdx.x >> 5][k] = x[k];
     __syncthreads();
-    if (threadIdx.x < n) {
-        R x = R(0);
-        for (int ww = 0; ww < NT / 32; ++ww) x += buf[ww][threadIdx.x];
-        red[threadIdx.x] = x;
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int k = 0; k < N; ++k) x[k] = (buf[0][k] + buf[1][k]) + (buf[2][k] + buf[3][k]);
+}
+
+__device__ __forceinline__ double gauss(double mB, double c2) { return fp64::exp2n(mB * fp64::EXP_SCALE, c2); }
+__device__ __forceinline__ float gauss(float mB, float c2) { return expf(mB * c2); }
+
+// Flux through boundary face b (one CTA).  Walls: outgoing molecules in equilibrium at the
+// cell state, incoming ones the diffuse wall Maxwellian with the density that zeroes the
+// mass flux; photons leave isotropically (e_R / 4 pi) and enter black-body
+// (sigma_R T_w^4 / pi).  All four planes of the cell's equilibrium are multiples of F0, so
+// three kinds of sums give every row; the wall's own sums (unit density) and the direction
+// sums do not change and are kept in g.binc (k_macro_binc).
+template <typename R, int DIM>
+__device__ void boundary_face(const MacroGeom &g, const ModelDev &m, const QuadD &vq, int b, double *__restrict__ bflux) {
+    constexpr int NV = DIM + 5, E = 1 + DIM, MH = 3 - DIM, NS = DIM + 4, N = DIM + 2;
+    const MacroReal<R> &c = real<R>(g);
+    __shared__ R buf[MF_NT / 32][N];
+    const int cell = g.bf_cell[b], patch = g.bf_patch[b], pk = g.patch_kind[patch];
+    R qc[NV];
+    for (int k = 0; k < NV; ++k) qc[k] = c.q[(size_t)cell * NVM + k];
+    double *out = bflux + (size_t)b * NVM;
+    const R *bg = c.bgeo + (size_t)b * 8;
+    R n[DIM];
+    for (int a = 0; a < DIM; ++a) n[a] = bg[a];
+    if (pk != 0) {
+        if (threadIdx.x != 0) return;
+        R F[NV];
+        if (pk == 2) {   // mirror plane: Rusanov against the cell state with its normal velocity reversed
+            R qm[NV], un = R(0);
+            for (int a = 0; a < DIM; ++a) un += qc[1 + a] * n[a];
+            for (int k = 0; k < NV; ++k) qm[k] = qc[k];
+            for (int a = 0; a < DIM; ++a) qm[1 + a] = qc[1 + a] - R(2) * un * n[a];
+            rusanov<R, DIM>(qc, qm, n, R(1), m, c, F);
+        } else {
+            farfield_flux<R, DIM>(g, m, b, qc, F);
+        }
+        for (int k = 0; k < NV; ++k) out[k] = to_double(F[k]);
+        return;
     }
-    __syncthreads();
+    const R Tt = qc[E], mB = R(-0.5) * rcp_r(Tt);
+    R acc[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) acc[k] = R(0);
+    for (int v = threadIdx.x; v < vq.n; v += MF_NT) {
+        R xi[DIM], xn = R(0);
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+            xi[a] = c.vx[a * vq.n_pad + v];
+            xn = fma(xi[a], n[a], xn);
+        }
+        if (is_neg(xn)) continue;
+        R c2 = R(0), x2 = R(0);
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+            const R d = xi[a] - qc[1 + a];
+            c2 = fma(d, d, c2);
+            x2 = fma(xi[a], xi[a], x2);
+        }
+        const R wf = c.vw[v] * xn * gauss(mB, c2);
+        acc[0] += wf;
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) acc[1 + a] = fma(wf, xi[a], acc[1 + a]);
+        acc[1 + DIM] = fma(wf, x2, acc[1 + DIM]);
+    }
+    cta_sum<N>(acc, buf);
+    if (threadIdx.x != 0) return;
+    const double *in = g.binc + (size_t)b * BINC;
+    // F0 = rho (2 pi T)^(-DIM/2) exp(-c^2 / 2T)
+    const R i2piT = rcp_r(R(2.0 * PI) * Tt);
+    const R Ac = qc[0] * (DIM == 2 ? i2piT : DIM == 1 ? sqrt_r(i2piT) : i2piT * sqrt_r(i2piT));
+    const R hr = c.half_dr * qc[E + 1], hv = vib_e(qc[E + 2], m, c);
+    R r[NS];
+    r[0] = Ac * acc[0];
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) r[1 + a] = Ac * acc[1 + a];
+    r[E] = fma(R(0.5) * Ac, acc[1 + DIM], fma(R(0.5 * MH), Tt, hr + hv) * r[0]);
+    r[E + 1] = hr * r[0];
+    r[E + 2] = hv * r[0];
+    const double rw = -to_double(r[0]) * in[NS + 2];   // in[NS + 2] = 1 / in[0]
+    const double FR = fma(to_double(qc[E + 3]), in[NS], in[NS + 1]);
+    for (int k = 0; k < NS; ++k) {
+        const double x = fma(rw, in[k], to_double(r[k]));
+        out[k] = k == E ? x + FR : x;
+    }
+    out[E + 3] = FR;
 }
 
 }  // namespace
 
-// ------------------------------------------------------------------ boundary fluxes
-// One CTA per boundary face.  Walls: outgoing molecules in equilibrium at the cell state,
-// incoming ones the diffuse wall Maxwellian with the density that zeroes the mass flux;
-// photons leave isotropically (e_R / 4 pi) and enter black-body (sigma_R T_w^4 / pi).
-// The incoming sums are linear in the wall density and are taken for unit density.
-template <typename R, int DIM>
-__global__ void __launch_bounds__(128) k_macro_bflux(MacroGeom g, ModelDev m, QuadD vq, QuadD oq,
-                                                     const MacroState *__restrict__ st, const double *__restrict__ q,
-                                                     double *__restrict__ bflux) {
-    constexpr int NV = DIM + 5, E = 1 + DIM, MH = 3 - DIM;
-    constexpr int NS = DIM + 4;   // mass, momentum, gas energy, e_r, e_v
-    if (st && st->done) return;
-    const int b = blockIdx.x;
-    const int c = g.bf_cell[b];
-    R qc[NV];
-    for (int k = 0; k < NV; ++k) qc[k] = R(q[(size_t)c * NVM + k]);
-    double *out = bflux + (size_t)b * NVM;
-    const int pk = g.patch_kind[g.bf_patch[b]];
-    __shared__ R red[2 * NS + 2];
-    if (pk == 2) {   // mirror plane: Rusanov against the cell state with its normal velocity reversed
-        if (threadIdx.x == 0) {
-            R n[DIM], qm[NV], F[NV], un = R(0);
-            for (int a = 0; a < DIM; ++a) {
-                n[a] = R(g.bf_n[(size_t)b * MGS + a]);
-                un += qc[1 + a] * n[a];
-            }
-            for (int k = 0; k < NV; ++k) qm[k] = qc[k];
-            for (int a = 0; a < DIM; ++a) qm[1 + a] = qc[1 + a] - R(2) * un * n[a];
-            rusanov<R, DIM>(qc, qm, n, m, F);
-            F[E + 3] = R(0);
-            for (int k = 0; k < NV; ++k) out[k] = F[k];
-        }
-        return;
-    }
-    if (pk != 0) {   // far field
-        if (threadIdx.x == 0) {
-            R base[3][3], F[NV];
-            kappa_base<R>(m, base);
-            farfield_flux<R, DIM>(g, m, base, b, qc, F);
-            for (int k = 0; k < NV; ++k) out[k] = F[k];
-        }
-        return;
-    }
-    const double *P = g.patch_state + (size_t)g.bf_patch[b] * 8;
-    R n[DIM], uw[DIM];
-    for (int a = 0; a < DIM; ++a) {
-        n[a] = R(g.bf_n[(size_t)b * MGS + a]);
-        uw[a] = R(P[1 + a]);
-    }
-    const R rho = qc[0], Tt = qc[E], Tr = qc[E + 1], Tv = qc[E + 2], eR = qc[E + 3];
-    const R Tw = R(P[4]);
-    const R Ac = rho * pow(R(2.0 * PI) * Tt, R(-0.5 * DIM)), Bc = R(0.5) / Tt;
-    const R Aw = pow(R(2.0 * PI) * Tw, R(-0.5 * DIM)), Bw = R(0.5) / Tw;
-    const R hr = R(0.5 * m.d_r);
-    const R evc = vib_energy<R>(m, Tv), evw = vib_energy<R>(m, Tw);   // d_v(T) T / 2 of cell and wall
-    R acc[2 * NS + 2];
-    for (int k = 0; k < 2 * NS + 2; ++k) acc[k] = R(0);
-    for (int v = threadIdx.x; v < vq.n; v += blockDim.x) {
-        R xi[DIM], xn = R(0), x2 = R(0);
+// The constant sums of every wall face: rows of the unit-density wall Maxwellian over the
+// entering velocities (NS), sum of the leaving directions over 4 pi, black-body flux of the
+// entering ones, reciprocal of the first.  Runs when the velocity sets are set.
+template <int DIM>
+__global__ void __launch_bounds__(MF_NT) k_macro_binc(MacroGeom g, ModelDev m, QuadD vq, QuadD oq,
+                                                      double *__restrict__ binc) {
+    constexpr int E = 1 + DIM, NS = DIM + 4, MH = 3 - DIM;
+    __shared__ double buf[MF_NT / 32][NS + 2];
+    const int b = blockIdx.x, patch = g.bf_patch[b];
+    if (g.patch_kind[patch] != 0) return;
+    const double *P = g.patch_state + (size_t)patch * 8, *n = g.d.bgeo + (size_t)b * 8;
+    const double Tw = P[4], evw = vib_energy<double>(m, Tw);
+    double acc[NS + 2];
+    for (int k = 0; k < NS + 2; ++k) acc[k] = 0.0;
+    for (int v = threadIdx.x; v < vq.n; v += MF_NT) {
+        double xi[DIM], xn = 0.0, x2 = 0.0, c2 = 0.0;
         for (int a = 0; a < DIM; ++a) {
-            xi[a] = R(vq.x[a * vq.n_pad + v]);
+            xi[a] = vq.x[a * vq.n_pad + v];
             xn += xi[a] * n[a];
             x2 += xi[a] * xi[a];
+            c2 += (xi[a] - P[1 + a]) * (xi[a] - P[1 + a]);
         }
-        const R wf = R(vq.w[v]) * xn;
-        R f0, fh, f1, f2;
-        R *s;
-        if (xn > R(0)) {
-            R c2 = R(0);
-            for (int a = 0; a < DIM; ++a) c2 += (xi[a] - qc[1 + a]) * (xi[a] - qc[1 + a]);
-            f0 = Ac * exp(-Bc * c2);
-            fh = R(MH) * Tt * f0;
-            f1 = hr * Tr * f0;
-            f2 = evc * f0;
-            s = acc;
-        } else {
-            R c2 = R(0);
-            for (int a = 0; a < DIM; ++a) c2 += (xi[a] - uw[a]) * (xi[a] - uw[a]);
-            f0 = Aw * exp(-Bw * c2);
-            fh = R(MH) * Tw * f0;
-            f1 = hr * Tw * f0;
-            f2 = evw * f0;
-            s = acc + NS;
+        if (xn > 0.0) continue;
+        const double f0 = pow(2.0 * PI * Tw, -0.5 * DIM) * exp(-0.5 * c2 / Tw), wf = vq.w[v] * xn;
+        acc[0] += wf * f0;
+        for (int a = 0; a < DIM; ++a) acc[1 + a] += wf * f0 * xi[a];
+        acc[E] += wf * (0.5 * x2 + 0.5 * MH * Tw + 0.5 * m.d_r * Tw + evw) * f0;
+        acc[E + 1] += wf * 0.5 * m.d_r * Tw * f0;
+        acc[E + 2] += wf * evw * f0;
+    }
+    const double Iw = m.sigma_R * Tw * Tw * Tw * Tw / PI;
+    for (int o = threadIdx.x; o < oq.n; o += MF_NT) {
+        double on = 0.0;
+        for (int a = 0; a < DIM; ++a) on += oq.x[a * oq.n_pad + o] * n[a];
+        if (on > 0.0) acc[NS] += oq.w[o] * on / (4.0 * PI);
+        else acc[NS + 1] += oq.w[o] * on * Iw;
+    }
+    cta_sum<NS + 2>(acc, buf);
+    if (threadIdx.x != 0) return;
+    for (int k = 0; k < NS + 2; ++k) binc[(size_t)b * BINC + k] = acc[k];
+    binc[(size_t)b * BINC + NS + 2] = 1.0 / acc[0];
+}
+
+// Blocks [0, n_face_cta): MF_FACES interior faces each; the first half of the threads
+// evaluates the Rusanov flux of a face, the second half its NSF and high-order terms and its
+// Gamma (two chains of similar length instead of one of twice it).  Fx [n_fi][NVM] is the
+// flux times the area, owner -> neighbour; fgam [n_fi][2] the Gammas times the area.
+// Blocks [n_face_cta, n_face_cta + n_bf): one boundary face each.  The rest: the sources of
+// MF_NT cells each, src [nc][SRC].
+template <typename R, int DIM, int ORDER>
+__global__ void __launch_bounds__(MF_NT) k_macro_flux(MacroGeom g, ModelDev m, QuadD vq, int n_face_cta, int n_bf_cta,
+                                                      const MacroState *__restrict__ st,
+                                                      const R *__restrict__ grad, const R *__restrict__ rec,
+                                                      R *__restrict__ Fx, R *__restrict__ fgam, R *__restrict__ src,
+                                                      double *__restrict__ bflux) {
+    constexpr int NV = DIM + 5, E = 1 + DIM;
+    if (st && st->done) return;
+    const MacroReal<R> &c = real<R>(g);
+    if ((int)blockIdx.x < n_face_cta) {
+        __shared__ R conv[E + 3][MF_FACES];
+        const int l = threadIdx.x % MF_FACES, f = blockIdx.x * MF_FACES + l;
+        const bool first = threadIdx.x < MF_FACES, valid = f < g.n_fi;
+        const int4 fi = valid ? g.fi4[f] : make_int4(0, 0, 0, 0);
+        const R *G = c.fgeo + (size_t)(valid ? f : 0) * FGEO;
+        const R S = G[11];
+        if (first && valid) {
+            const R *qL = ORDER == 2 ? rec + ((size_t)fi.x * MAXF + fi.z) * NVM : c.q + (size_t)fi.x * NVM;
+            const R *qR = ORDER == 2 ? rec + ((size_t)fi.y * MAXF + fi.w) * NVM : c.q + (size_t)fi.y * NVM;
+            R n[DIM], F[NV];
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) n[a] = G[a];
+            rusanov<R, DIM>(qL, qR, n, S, m, c, F);
+#pragma unroll
+            for (int k = 0; k < E + 3; ++k) conv[k][l] = F[k];
         }
-        s[0] += wf * f0;
-        for (int a = 0; a < DIM; ++a) s[1 + a] += wf * f0 * xi[a];
-        s[E] += wf * (R(0.5) * x2 * f0 + R(0.5) * fh + f1 + f2);
-        s[E + 1] += wf * f1;
-        s[E + 2] += wf * f2;
-    }
-    const R Iw = R(m.sigma_R) * Tw * Tw * Tw * Tw / R(PI), Io = eR / R(4.0 * PI);
-    for (int o = threadIdx.x; o < oq.n; o += blockDim.x) {
-        R on = R(0);
-        for (int a = 0; a < DIM; ++a) on += R(oq.x[a * oq.n_pad + o]) * n[a];
-        acc[2 * NS] += R(oq.w[o]) * on * (on > R(0) ? Io : Iw);
-    }
-    block_sum<128, R>(acc, 2 * NS + 1, red);
-    if (threadIdx.x == 0) {
-        const R rw = -red[0] / red[NS];
         R F[NV];
-        for (int k = 0; k < NS; ++k) F[k] = red[k] + rw * red[NS + k];
-        F[E + 3] = red[2 * NS];
-        F[E] += F[E + 3];
-        for (int k = 0; k < NV; ++k) out[k] = F[k];
+        if (!first && valid) {
+            R pf[NV], mu, irho, kR, sn[DIM], qn[4];
+            nsf_normal<R, DIM>(g, m, G, fi.x, fi.y, grad, pf, mu, irho, kR, sn, qn);
+            const R idn = G[12];
+            const R *h = c.hot + (size_t)f * NVM;
+            R un = R(0), unf = R(0);
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) {
+                sn[a] += h[a];
+                un = fma(sn[a], pf[1 + a], un);
+                unf = fma(pf[1 + a], G[a], unf);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) qn[k] += h[DIM + k];
+            F[0] = R(0);
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) F[1 + a] = S * sn[a];
+            F[E] = S * (un + ((qn[0] + qn[1]) + (qn[2] + qn[3])));
+#pragma unroll
+            for (int k = 1; k < 4; ++k) F[E + k] = S * qn[k];
+            fgam[(size_t)f * 2] = S * (fabs(unf) + sound_speed(pf[E]) + R(2) * mu * irho * idn);
+            fgam[(size_t)f * 2 + 1] = S * (R(2) * kR * idn);
+        }
+        __syncthreads();
+        if (!first && valid) {
+#pragma unroll
+            for (int k = 0; k < NV; ++k) Fx[(size_t)f * NVM + k] = k < E + 3 ? F[k] + conv[k][l] : F[k];
+        }
+        return;
     }
+    const int b = (int)blockIdx.x - n_face_cta;
+    if (b < n_bf_cta) {
+        boundary_face<R, DIM>(g, m, vq, b, bflux);
+        return;
+    }
+    // sources Q of Section 5 (rotational and vibrational relaxation, gas-photon exchange) and
+    // the nonzero entries of their Jacobian d(Q_egas, Q_r, Q_v, Q_R)/d(e_gas, e_r, e_v, e_R)
+    // with rho, rho u, tau, k_eff frozen:
+    //   [ 0, 0, -kb, k ], [ c, -cr, -c, 0 ], [ e, -e, -zv - kb, k ], [ 0, 0, kb, -k ]
+    // c = d_r / (3 + d_r) zr, cr = zr, zr = 1 / (Z_r tau); e = 2 eps'(T_tv) / (3 + 2 eps'(T_tv)) zv,
+    // zv = 1 / (Z_v tau); kb = k_eff 16 sigma_R T_v^3 / (rho eps'(T_v)), eps(T) = d_v(T) T / 2.
+    const int i = (b - n_bf_cta) * MF_NT + threadIdx.x;
+    if (i >= g.n_cells) return;
+    const R *q = c.q + (size_t)i * NVM;
+    const R rho = q[0], Tt = q[E], Tr = q[E + 1], Tv = q[E + 2], eR = q[E + 3];
+    const R itau = rho * pow_r(Tt, R(1) - c.omega) * c.i_mu0;      // 1 / tau
+    const R zr = itau * c.i_Zr, zv = itau * c.i_Zv, k = absorption(rho, c);
+    const R s3 = R(4) * c.sigma * Tv * Tv * Tv, ex = k * fma(s3, Tv, -eR);
+    R *o = src + (size_t)i * SRC;
+    o[0] = c.half_dr * rho * c.w_r * (Tt - Tr) * zr;               // T_tr - T_r = 3 (T_t - T_r) / (3 + d_r)
+    R cvv, ctv, dev;                                               // eps'(T_v), eps'(T_tv), eps(T_tv) - eps(T_v)
+    if (m.dv_T) {
+        const R ev = vib_energy<R>(m, Tv), Ttv = equal_temperature<R>(m, R(3), R(3) * Tt + R(2) * ev);
+        cvv = vib_cv<R>(m, Tv);
+        ctv = vib_cv<R>(m, Ttv);
+        dev = vib_energy<R>(m, Ttv) - ev;
+        o[8] = R(2) * ctv * rcp_r(fma(R(2), ctv, R(3))) * zv;
+        o[4] = R(4) * k * s3 * rcp_r(rho * cvv);
+    } else {
+        dev = c.half_dv * c.w_v * (Tt - Tv);
+        o[8] = c.e_v * zv;
+        o[4] = R(4) * k * s3 * (c.i_half_dv * rcp_r(rho));
+    }
+    o[1] = fma(rho * dev, zv, -ex);
+    o[2] = ex;
+    R uu = R(0), ke = R(0);
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) uu = fma(q[1 + a], q[1 + a], uu);
+    o[3] = (sqrt_r(uu) + sound_speed(Tt)) * c.icdx[i];             // 1 / dt
+    o[5] = k;
+    o[6] = c.c_r * zr;
+    o[7] = zr;
+    o[9] = zv;
+    // the state that the relaxation's flux increments need: H = E_gas + p, e_r, e_v
+    const R p = rho * Tt, er = c.half_dr * rho * Tr, ev = rho * vib_e(Tv, m, c);
+    ke = rho * uu;
+    o[10] = fma(R(2.5), p, fma(R(0.5), ke, er + ev));
+    o[11] = er;
+    o[12] = ev;
 }
 
 // ------------------------------------------------------------------ high-order terms
-// one thread per interior face, then one per boundary face
+// one thread per interior face, then one per boundary face; hot [n_fi][NVM]: stress . n
+// (DIM), then the four heat fluxes . n
 template <typename R, int DIM>
-__global__ void k_macro_hot(MacroGeom g, ModelDev m, const double *__restrict__ Fk, const double *__restrict__ q,
-                            const double *__restrict__ grad, const double *__restrict__ kin_bflux,
-                            const double *__restrict__ mac_bflux, double *__restrict__ hot,
-                            double *__restrict__ hot_b) {
+__global__ void k_macro_hot(MacroGeom g, ModelDev m, const double *__restrict__ Fk, const R *__restrict__ grad,
+                            const double *__restrict__ kin_bflux, const double *__restrict__ mac_bflux,
+                            double *__restrict__ hot, float *__restrict__ hotf, double *__restrict__ hot_b) {
     constexpr int NV = DIM + 5;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < g.n_fi) {
-        R base[3][3];
-        kappa_base<R>(m, base);
-        R pf[NV], fg[DIM][DIM + 5], s[NHOT];
-        face_state<R, DIM>(g, t, q, grad, pf, fg);
-        nsf_face<R, DIM>(pf, fg, m, base, s);
-        const double *ri = Fk + (size_t)g.fi_i[t] * NF, *rj = Fk + (size_t)g.fi_j[t] * NF;
-        auto sig = [&](const double *r, int a, int b) {
-            const int idx[3][3] = {{20, 23, 24}, {23, 21, 25}, {24, 25, 22}};
-            return r[idx[a][b]];
-        };
-        double *h = hot + (size_t)t * NHOT;
-        for (int a = 0; a < DIM; ++a)
-            for (int b = 0; b < DIM; ++b) h[a * DIM + b] = 0.5 * (sig(ri, a, b) + sig(rj, a, b)) - (double)s[a * DIM + b];
-        for (int md = 0; md < 4; ++md)
-            for (int d = 0; d < DIM; ++d) {
-                const int k = 8 + 3 * md + d;
-                h[DIM * DIM + md * DIM + d] = 0.5 * (ri[k] + rj[k]) - (double)s[DIM * DIM + md * DIM + d];
+        const MacroReal<R> &c = real<R>(g);
+        const int4 fi = g.fi4[t];
+        R pf[NV], mu, irho, kR, sn[DIM], qn[4];
+        nsf_normal<R, DIM>(g, m, c.fgeo + (size_t)t * FGEO, fi.x, fi.y, grad, pf, mu, irho, kR, sn, qn);
+        const double *n = g.d.fgeo + (size_t)t * FGEO;
+        const double *ri = Fk + (size_t)fi.x * NF, *rj = Fk + (size_t)fi.y * NF;
+        double *h = hot + (size_t)t * NVM;
+        double x[DIM + 4];
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+            x[a] = -to_double(sn[a]);
+#pragma unroll
+            for (int b = 0; b < DIM; ++b) {
+                // record words of the stress: xx, yy, zz, xy, xz, yz at 20
+                const int k = a == b ? 20 + a : 22 + a + b;
+                x[a] = fma(0.5 * (ri[k] + rj[k]), n[b], x[a]);
             }
+        }
+#pragma unroll
+        for (int md = 0; md < 4; ++md) {
+            x[DIM + md] = -to_double(qn[md]);
+#pragma unroll
+            for (int d = 0; d < DIM; ++d) x[DIM + md] = fma(0.5 * (ri[8 + 3 * md + d] + rj[8 + 3 * md + d]), n[d], x[DIM + md]);
+        }
+#pragma unroll
+        for (int k = 0; k < DIM + 4; ++k) {
+            h[k] = x[k];
+            if (hotf) hotf[(size_t)t * NVM + k] = fp64::narrow(x[k]);
+        }
         return;
     }
     const int b = t - g.n_fi;
@@ -626,350 +710,433 @@ __global__ void k_macro_hot(MacroGeom g, ModelDev m, const double *__restrict__ 
             hot_b[(size_t)b * NVM + k] = kin_bflux[(size_t)b * NVM + k] - mac_bflux[(size_t)b * NVM + k];
 }
 
-// ------------------------------------------------------------------ residual and diagonal
-constexpr int MR_NT = 32;      // threads per CTA of the per-cell kernels (small CTAs spread FP64 work over SMs)
+// ------------------------------------------------------------------ residual and relaxation
 constexpr int DSTR = 24;       // Dinv record: NVM diagonal inverses (first E used), 4x4 block
 
 namespace {
 
-// Gauss-Jordan inverse of a 4x4 matrix with partial pivoting
-template <typename R>
-__device__ void inverse4(const R (&A)[4][4], R (&X)[4][4]) {
-    R M[4][8];
-    for (int r = 0; r < 4; ++r)
-        for (int c = 0; c < 4; ++c) {
-            M[r][c] = A[r][c];
-            M[r][4 + c] = r == c ? R(1) : R(0);
-        }
-    for (int c = 0; c < 4; ++c) {
-        int p = c;
-        for (int r = c + 1; r < 4; ++r)
-            if (fabs(M[r][c]) > fabs(M[p][c])) p = r;
-        if (p != c)
-            for (int k = 0; k < 8; ++k) {
-                const R t = M[c][k];
-                M[c][k] = M[p][k];
-                M[p][k] = t;
-            }
-        const R inv = R(1) / M[c][c];
-        for (int k = 0; k < 8; ++k) M[c][k] *= inv;
-        for (int r = 0; r < 4; ++r) {
-            if (r == c) continue;
-            const R f = M[r][c];
-            for (int k = 0; k < 8; ++k) M[r][k] -= f * M[c][k];
-        }
+// D of the energy rows, diag(d0, d0, d0, dR) minus the source Jacobian above, eliminated
+// photons first, then gas energy and e_r in terms of e_v.  Every pivot is a sum of positive
+// terms: dR + k, d0, d0 + zr, and the last one, d0 + zv + kb dR/(dR + k) + e (g - h), with
+// e < zv and h - g < c / (d0 + zr) < 1.
+template <typename T>
+struct EnergyD {
+    T ir3, k, id0, i1, c, e, g, h, is, kbi;
+    __device__ __forceinline__ EnergyD(T d0, T dR, T kb, T k_, T c_, T zr, T e_, T zv) {
+        k = k_;
+        c = c_;
+        e = e_;
+        ir3 = rcp_r(dR + k);
+        id0 = rcp_r(d0);
+        i1 = rcp_r(d0 + zr);
+        kbi = kb * ir3;
+        const T w = kbi * dR;
+        g = w * id0;
+        h = fma(c, g, c) * i1;
+        is = rcp_r(fma(e, g - h, d0 + zv + w));
     }
-    for (int r = 0; r < 4; ++r)
-        for (int c = 0; c < 4; ++c) X[r][c] = M[r][4 + c];
-}
+    // the same elimination with its coefficients widened
+    template <typename S>
+    __device__ __forceinline__ explicit EnergyD(const EnergyD<S> &o)
+        : ir3(to_double(o.ir3)), k(to_double(o.k)), id0(to_double(o.id0)), i1(to_double(o.i1)), c(to_double(o.c)),
+          e(to_double(o.e)), g(to_double(o.g)), h(to_double(o.h)), is(to_double(o.is)), kbi(to_double(o.kbi)) {}
+    __device__ __forceinline__ void solve(T b0, T b1, T b2, T b3, T (&x)[4]) const {
+        const T t3 = b3 * ir3;
+        const T y0 = fma(k, t3, b0) * id0, y1 = fma(c, y0, b1) * i1;
+        x[2] = fma(e, y0 - y1, fma(k, t3, b2)) * is;
+        x[0] = fma(-g, x[2], y0);
+        x[1] = fma(-h, x[2], y1);
+        x[3] = fma(kbi, x[2], t3);
+    }
+};
+
+// Increment of the convective flux vectors, F_a(W + dW) - F_a(W) in every direction a,
+// without forming either flux: every term is a product of an increment with a state value,
+// so that its rounding is relative to the increment.
+//   rho1 = rho + drho, du = (dm - u drho) / rho1, d(rho |u|^2) = drho |u1|^2 + rho du.(u1 + u),
+//   dp = 2/3 (dEg - der - dev - d(rho |u|^2) / 2),
+//   d(m_b u_a) = dm_b u_a1 + m_b du_a, d(u_a X) = du_a X1 + u_a dX (X = Eg + p, e_r, e_v).
+template <typename R, int DIM>
+struct FluxIncrement {
+    R du[DIM], u1[DIM], dp, dH;
+    __device__ __forceinline__ FluxIncrement(R rho, const R *u, R drho, const R *dm, R dEg, R der, R dev) {
+        const R inv1 = rcp_r(rho + drho);
+        R uu1 = R(0), dq = R(0);
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+            du[a] = fma(-u[a], drho, dm[a]) * inv1;
+            u1[a] = u[a] + du[a];
+            uu1 = fma(u1[a], u1[a], uu1);
+            dq = fma(du[a], u1[a] + u[a], dq);
+        }
+        dp = R(2.0 / 3.0) * fma(R(-0.5), fma(drho, uu1, rho * dq), dEg - der - dev);
+        dH = dEg + dp;
+    }
+};
+
+// One relaxation record per (cell, row): the flux increment vector of the row (DIM values)
+// and the row's dW at [3] (FP64: 32 bytes, FP32: 16)
+template <typename R>
+struct __align__(4 * sizeof(R)) Row {
+    R x[4];
+};
 
 }  // namespace
 
-// four lanes per cell (lane k = face k): each lane evaluates one face flux and its Gamma;
-// lane 0 adds the sources and builds D^-1
-template <typename R, int DIM, int ORDER>
-__global__ void __launch_bounds__(128) k_macro_residual(MacroGeom g, ModelDev m, double cfl_macro,
-                                                        const MacroState *__restrict__ st,
-                                                        const double *__restrict__ q, const double *__restrict__ grad,
-                                                        const double *__restrict__ phi, const double *__restrict__ hot,
-                                                        const double *__restrict__ bflux,
+// Eight lanes per cell, lane v = row v.  The first relaxation sweep has no neighbour terms
+// (dW = D^-1 R) and is made here.  With `st`, the last CTA to finish (an atomic ticket after
+// a fence, no waiting) adds the CTA partials of |R|^2 in a fixed order and sets the norm,
+// the iteration count and the stop flag.
+template <typename R, int DIM>
+__global__ void __launch_bounds__(128) k_macro_residual(MacroGeom g, MacroState *__restrict__ st,
+                                                        const R *__restrict__ Fx, const R *__restrict__ fgam,
+                                                        const R *__restrict__ src, const double *__restrict__ bflux,
                                                         const double *__restrict__ hot_b, double *__restrict__ Rg,
-                                                        double *__restrict__ Dinv, double *__restrict__ gam,
-                                                        double *__restrict__ rpart) {
-    constexpr int NV = DIM + 5, E = 1 + DIM, ER = 4 + DIM, L = 4;
+                                                        double *__restrict__ Dinv, R *__restrict__ gam,
+                                                        Row<R> *__restrict__ rows, double *__restrict__ rpart,
+                                                        double *__restrict__ history) {
+    constexpr int NV = DIM + 5, E = 1 + DIM, ER = 4 + DIM;
     if (st && st->done) return;
-    const int gt = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i = gt / L, k = gt % L;
-    const bool valid = i < g.n_cells;
-    const unsigned gmask = 0xFu << ((threadIdx.x & 31) & ~(L - 1));
-    R Rr[NV], gsum = R(0), gsumR = R(0);
-    for (int v = 0; v < NV; ++v) Rr[v] = R(0);
-    R qi[NV];
-    for (int v = 0; v < NV; ++v) qi[v] = valid ? R(q[(size_t)i * NVM + v]) : R(1);
-    if (valid && k < g.info[i].x) {
+    const MacroReal<R> &c = real<R>(g);
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, v = t % NVM;
+    const bool valid = t / NVM < g.n_cells;
+    const int i = valid ? t / NVM : g.n_cells - 1;
+    const unsigned lane = threadIdx.x & 31;
+    const int l0 = (int)(lane & ~(unsigned)(NVM - 1));       // the cell's first lane
+    const int nf = g.info[i].x;
+    const R *q = c.q + (size_t)i * NVM;
+    const R hiv = c.hivol[i];
+    R acc = R(0), gs = R(0), gsR = R(0);
+#pragma unroll
+    for (int k = 0; k < MAXF; ++k) {
+        if (k >= nf) break;
         const int fid = g.cface[i * MAXF + k];
         if (fid >= 0) {
-            R base[3][3];
-            kappa_base<R>(m, base);
-            R F[NV];
-            interior_flux<R, DIM, ORDER>(g, m, base, fid, q, grad, phi, hot, F);
-            const R S = R(g.fi_S[fid]);
-            const bool own = g.fi_i[fid] == i;
-            for (int v = 0; v < NV; ++v) Rr[v] = own ? -F[v] * S : F[v] * S;
-            const int o = own ? g.fi_j[fid] : g.fi_i[fid];
-            const double *qo = q + (size_t)o * NVM;
-            const R rf = R(0.5) * (qi[0] + R(qo[0])), Tf = R(0.5) * (qi[E] + R(qo[E]));
-            R un = R(0);
-            for (int a = 0; a < DIM; ++a) un += R(0.5) * (qi[1 + a] + R(qo[1 + a])) * R(g.fi_n[(size_t)fid * MGS + a]);
-            const R dn = R(g.fi_dn[fid]);
-            const R gb = fabs(un) + sound_speed(Tf) + R(2) * viscosity(Tf, m) / (rf * dn);
-            const R gR = R(2) * (R(1) / (R(3) * absorption(rf, m))) / dn;
-            gam[((size_t)i * MAXF + k) * 2] = gb;
-            gam[((size_t)i * MAXF + k) * 2 + 1] = gR;
-            gsum = gb * S;
-            gsumR = gR * S;
+            if (v < NV) {
+                const R x = Fx[(size_t)fid * NVM + v];
+                acc = g.own[i * MAXF + k] ? acc - x : acc + x;
+            }
+            const R gb = fgam[(size_t)fid * 2], gR = fgam[(size_t)fid * 2 + 1];
+            gs += gb;
+            gsR += gR;
+            if (v < 2 && valid) gam[((size_t)i * MAXF + k) * 2 + v] = v == 0 ? gb * hiv : (gb + gR) * hiv;
         } else {
             const int b = -1 - fid;
-            const R S = R(g.bf_S[b]);
-            for (int v = 0; v < NV; ++v) Rr[v] = -R(bflux[(size_t)b * NVM + v] + hot_b[(size_t)b * NVM + v]) * S;
+            const R *bg = c.bgeo + (size_t)b * 8;
+            const R S = bg[3], idn = bg[4];
+            if (v < NV) {
+                const double x = bflux[(size_t)b * NVM + v] + hot_b[(size_t)b * NVM + v];
+                acc = fma(-to_real<R>(x), S, acc);
+            }
             R un = R(0);
-            for (int a = 0; a < DIM; ++a) un += qi[1 + a] * R(g.bf_n[(size_t)b * MGS + a]);
-            const R db = R(g.bf_dn[b]);
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) un = fma(q[1 + a], bg[a], un);
             const bool mirror = g.patch_kind[g.bf_patch[b]] == 2;
             // a mirror face: the Rusanov part only, and nothing in the e_R row
-            const R gb = fabs(un) + sound_speed(qi[E]) + (mirror ? R(0) : R(2) * viscosity(qi[E], m) / (qi[0] * db));
-            const R gR = mirror ? -gb : R(2) * (R(1) / (R(3) * absorption(qi[0], m))) / db;
-            gsum = gb * S;
-            gsumR = gR * S;
+            R gb = fabs(un) + sound_speed(q[E]), gR = -gb;
+            if (!mirror) {
+                const R ir = rcp_r(q[0]);
+                gb += R(2) * viscosity(q[E], c) * ir * idn;
+                gR = R(2) * (c.dens ? c.kR0 * ir : c.kR0) * idn;
+            }
+            gs = fma(gb, S, gs);
+            gsR = fma(gR, S, gsR);
         }
     }
-    for (int o = 1; o < L; o <<= 1) {
-        for (int v = 0; v < NV; ++v) Rr[v] += __shfl_xor_sync(gmask, Rr[v], o);
-        gsum += __shfl_xor_sync(gmask, gsum, o);
-        gsumR += __shfl_xor_sync(gmask, gsumR, o);
-    }
-    double r2 = 0.0;
-    if (valid && k == 0) {
-        const R V = R(g.vol[i]);
-        R Q[NV];
-        source<R, DIM>(qi, m, Q);
-        for (int v = 0; v < NV; ++v) {
-            Rr[v] = Rr[v] / V + Q[v];
-            if (g.moff) Rr[v] += R(g.moff[(size_t)i * NVM + v]);
-            r2 += (double)Rr[v] * (double)Rr[v];
+    const R *so = src + (size_t)i * SRC;
+    const R iv = c.ivol[i];
+    R r = acc * iv;
+    if (v > E && v < NV) r += so[v - E - 1];
+    if (g.moff && v < NV) r += to_real<R>(g.moff[(size_t)i * NVM + v]);
+    const double r8 = v < NV && valid ? to_double(r) : 0.0;
+    double r2 = r8 * r8;
+    // relaxation form: the energy row holds the gas energy
+    const double rR = __shfl_sync(0xffffffffu, r8, l0 + ER);
+    const double rg = v == E ? r8 - rR : r8;
+    if (valid && v < NV) Rg[(size_t)i * NVM + v] = rg;
+    const R d0 = fma(gs, iv, so[3]), dR = fma(gs + gsR, iv, so[3]);
+    const EnergyD<R> D(d0, dR, so[4], so[5], so[6], so[7], so[8], so[9]);
+    double *Di = Dinv + (size_t)i * DSTR;
+    if (valid) {
+        if (v == 0) Di[0] = to_double(D.id0);
+        if (v < 4) {       // lane v: column v of the inverse
+            R x[4];
+            D.solve(R(v == 0), R(v == 1), R(v == 2), R(v == 3), x);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) Di[NVM + k * 4 + v] = to_double(x[k]);
         }
-        double *rg = Rg + (size_t)i * NVM;
-        for (int v = 0; v < NV; ++v) rg[v] = Rr[v];
-        rg[E] -= (double)Rr[ER];
-        // D = diag(1/dt + sum Gamma S / V) - dQ/dW (energy rows)
-        R um = R(0);
-        for (int a = 0; a < DIM; ++a) um += qi[1 + a] * qi[1 + a];
-        const R inv_dt = (sqrt(um) + sound_speed(qi[E])) / (R(cfl_macro) * R(g.dx[i]));
-        double *Di = Dinv + (size_t)i * DSTR;
-        const R d0 = inv_dt + gsum / V;
-        for (int v = 0; v < E; ++v) Di[v] = R(1) / d0;
-        R J[4][4], Dm[4][4], X[4][4];
-        source_jacobian<R, DIM>(qi, m, J);
-        for (int r = 0; r < 4; ++r)
-            for (int c = 0; c < 4; ++c)
-                Dm[r][c] = (r == c ? (r == 3 ? inv_dt + (gsum + gsumR) / V : d0) : R(0)) - J[r][c];
-        inverse4<R>(Dm, X);
-        for (int r = 0; r < 4; ++r)
-            for (int c = 0; c < 4; ++c) Di[NVM + r * 4 + c] = X[r][c];
     }
-    // deterministic per-CTA partial of |R|^2
+    // first sweep: dW = D^-1 R (in FP64), and its flux increments
+    double rr[NV], x4[4];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) rr[k] = __shfl_sync(0xffffffffu, rg, l0 + k);
+    if constexpr (sizeof(R) == 8) {
+        D.solve(rr[E], rr[E + 1], rr[E + 2], rr[E + 3], x4);
+    } else {
+        const EnergyD<double> D8(D);
+        D8.solve(rr[E], rr[E + 1], rr[E + 2], rr[E + 3], x4);
+    }
+    const double id0 = to_double(D.id0);
+    R u[DIM], dm[DIM];
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) {
+        u[a] = q[1 + a];
+        dm[a] = to_real<R>(id0 * rr[1 + a]);
+    }
+    const R drho = to_real<R>(id0 * rr[0]), dEg = to_real<R>(x4[0]), der = to_real<R>(x4[1]),
+            dev = to_real<R>(x4[2]), deR = to_real<R>(x4[3]);
+    const FluxIncrement<R, DIM> fi(q[0], u, drho, dm, dEg, der, dev);
+    if (valid && v < NV) {
+        Row<R> o;
+        o.x[1] = o.x[2] = R(0);
+        if (v <= DIM) {
+            R dmb = drho;
+#pragma unroll
+            for (int a = 0; a < DIM; ++a)
+                if (v == 1 + a) dmb = dm[a];
+            const R mb = v == 0 ? R(0) : q[0] * q[v];
+#pragma unroll
+            for (int a = 0; a < DIM; ++a)
+                o.x[a] = v == 0 ? dm[a] : fma(dmb, fi.u1[a], fma(mb, fi.du[a], v == 1 + a ? fi.dp : R(0)));
+            o.x[3] = dmb;
+        } else {
+            const R X = v == ER ? R(0) : so[10 + v - E], dX = v == E ? fi.dH : v == E + 1 ? der : v == E + 2 ? dev : R(0);
+            const R X1 = X + dX;
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) o.x[a] = fma(fi.du[a], X1, u[a] * dX);
+            o.x[3] = v == E ? dEg : v == E + 1 ? der : v == E + 2 ? dev : deR;
+        }
+        rows[(size_t)i * NVM + v] = o;
+    }
+    if (!st) return;
+    // deterministic per-CTA partial of |R|^2, then the last CTA
+    __shared__ double ws[4];
+    __shared__ bool last;
+#pragma unroll
     for (int o = 16; o > 0; o >>= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, o);
-    __shared__ double wsum[4];
-    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = r2;
+    if (lane == 0) ws[threadIdx.x >> 5] = r2;
     __syncthreads();
-    if (threadIdx.x == 0) rpart[blockIdx.x] = wsum[0] + wsum[1] + wsum[2] + wsum[3];
-}
-
-__global__ void k_macro_norm(int n_parts, const double *__restrict__ rpart, MacroState *__restrict__ st,
-                             double *__restrict__ history) {
-    __shared__ double buf[256];
-    if (st->done) return;
-    if (st->it >= st->max_inner) {
-        if (threadIdx.x == 0) st->done = 1;
-        return;
-    }
-    double s = 0.0;
-    for (int k = threadIdx.x; k < n_parts; k += blockDim.x) s += rpart[k];
-    buf[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) buf[threadIdx.x] += buf[threadIdx.x + w];
-        __syncthreads();
-    }
     if (threadIdx.x == 0) {
-        const double rn = sqrt(buf[0]);
-        if (st->it == 0) st->r0 = rn;
-        st->rn = rn;
-        if (history) history[st->it] = rn;
-        st->it += 1;
-        if (!isfinite(rn) || rn <= st->tol * st->r0) st->done = 1;
+        rpart[blockIdx.x] = (ws[0] + ws[1]) + (ws[2] + ws[3]);
+        __threadfence();
+        last = atomicAdd(&st->ticket, 1u) == gridDim.x - 1;
     }
-}
-
-// one point-relaxation sweep: every cell uses its neighbours' increments of the previous
-// sweep; increments are kept in the gas-energy form (row E holds d e_gas)
-// four lanes per cell (lane k = face k), summed with shuffles inside each group of four
-constexpr int LPC = 4;
-static_assert(LPC == MAXF, "one lane per cell face");
-
-// F_c(W + dW) . n - F_c(W) . n in FP32, from the primitive state q of W and the increment
-// dW (gas-energy form) without forming either flux: every term is a product of an increment
-// with a state value, so no two nearly equal fluxes are subtracted and the FP32 rounding
-// stays relative to the increment.
-//   rho1 = rho + drho, du = (dm - u drho) / rho1, d(rho |u|^2) = drho |u1|^2 + rho du.(u1 + u),
-//   dp = 2/3 (dEg - der - dev - d(rho |u|^2) / 2),
-//   d(m u_n) = dm u_n1 + rho u du_n, d(u_n X) = du_n X1 + u_n dX.
-template <int DIM>
-__device__ __forceinline__ void flux_increment(const double *q, const double *dW, const double *n,
-                                               const ModelDev &m, float *dF) {
-    constexpr int E = 1 + DIM;
-    const float rho = float(q[0]), T = float(q[E]);
-    const float er = 0.5f * float(m.d_r) * rho * float(q[E + 1]), ev = rho * vib_energy<float>(m, float(q[E + 2]));
-    float u[DIM], nf[DIM], dm[DIM], un = 0.0f, uu = 0.0f;
-    for (int a = 0; a < DIM; ++a) {
-        u[a] = float(q[1 + a]);
-        nf[a] = float(n[a]);
-        dm[a] = float(dW[1 + a]);
-        un += u[a] * nf[a];
-        uu += u[a] * u[a];
-    }
-    const float p = rho * T, Eg = 1.5f * p + 0.5f * rho * uu + er + ev;
-    const float drho = float(dW[0]), dEg = float(dW[E]), der = float(dW[E + 1]), dev = float(dW[E + 2]);
-    const float inv1 = 1.0f / (rho + drho);
-    float dun = 0.0f, dmn = 0.0f, uu1 = 0.0f, dq = 0.0f;
-    for (int a = 0; a < DIM; ++a) {
-        const float du = (dm[a] - u[a] * drho) * inv1, u1 = u[a] + du;
-        dun += du * nf[a];
-        dmn += dm[a] * nf[a];
-        uu1 += u1 * u1;
-        dq += du * (u1 + u[a]);
-    }
-    const float dK = drho * uu1 + rho * dq;
-    const float dp = (2.0f / 3.0f) * (dEg - der - dev - 0.5f * dK);
-    const float un1 = un + dun;
-    dF[0] = dmn;
-    for (int a = 0; a < DIM; ++a) dF[1 + a] = dm[a] * un1 + rho * u[a] * dun + dp * nf[a];
-    dF[E] = dun * (Eg + dEg + p + dp) + un * (dEg + dp);
-    dF[E + 1] = dun * (er + der) + un * der;
-    dF[E + 2] = dun * (ev + dev) + un * dev;
-    dF[E + 3] = 0.0f;
-}
-
-// R = double: the flux increment as the difference of the two fluxes in FP64; R = float:
-// flux_increment in FP32 (the residual side's FP32 mode)
-template <typename R, int DIM>
-__global__ void __launch_bounds__(128) k_macro_jacobi(MacroGeom g, ModelDev m, const MacroState *__restrict__ st,
-                                                      int first, int last, const double *__restrict__ W,
-                                                      const double *__restrict__ qW,
-                                                      const double *__restrict__ Rg, const double *__restrict__ Dinv,
-                                                      const double *__restrict__ gam,
-                                                      const double *__restrict__ dG_in, double *__restrict__ dG_out,
-                                                      double *__restrict__ W_next) {
-    constexpr int NV = DIM + 5, E = 1 + DIM, ER = 4 + DIM;
-    const int gt = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i = gt / LPC, k = gt % LPC;
-    const bool valid = i < g.n_cells;
-    const unsigned gmask = 0xFu << ((threadIdx.x & 31) & ~(LPC - 1));
-    if (st->done) {
-        if (last && valid && k == 0)
-            for (int v = 0; v < NV; ++v) W_next[(size_t)i * NVM + v] = W[(size_t)i * NVM + v];
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double s = 0.0;
+    for (unsigned k = threadIdx.x; k < gridDim.x; k += blockDim.x) s += __ldcg(rpart + k);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) ws[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    st->ticket = 0u;
+    if (st->it >= st->max_inner) {
+        st->done = 1;
         return;
     }
-    double off[NV];
-    for (int v = 0; v < NV; ++v) off[v] = 0.0;
-    if (valid && !first && k < g.info[i].x) {
-        const int fid = g.cface[i * MAXF + k];
-        if (fid >= 0) {
-            const bool own = g.fi_i[fid] == i;
-            const int o = own ? g.fi_j[fid] : g.fi_i[fid];
-            double n[3] = {0.0, 0.0, 0.0};
-            for (int a = 0; a < DIM; ++a) n[a] = own ? g.fi_n[(size_t)fid * MGS + a] : -g.fi_n[(size_t)fid * MGS + a];
-            const double *Wo = W + (size_t)o * NVM, *dGo = dG_in + (size_t)o * NVM;
-            const double S = g.fi_S[fid];
-            const double gb = gam[((size_t)i * MAXF + k) * 2], gR = gam[((size_t)i * MAXF + k) * 2 + 1];
-            if constexpr (std::is_same<R, double>::value) {
-                double Wp[NV], q0[NV], q1[NV], F0[NV], F1[NV];
-                for (int v = 0; v < NV; ++v) Wp[v] = Wo[v] + dGo[v];
-                Wp[E] += dGo[ER];
-                primitive<double, DIM>(Wo, m, q0);
-                primitive<double, DIM>(Wp, m, q1);
-                convective_flux<double, DIM>(q1, n, m, F1);
-                convective_flux<double, DIM>(q0, n, m, F0);
-                for (int v = 0; v < NV; ++v) {
-                    const double G = v == ER ? gb + gR : gb;
-                    off[v] = ((F1[v] - F0[v]) - G * dGo[v]) * S;
+    const double rn = sqrt((ws[0] + ws[1]) + (ws[2] + ws[3]));
+    if (st->it == 0) st->r0 = rn;
+    st->rn = rn;
+    if (history) history[st->it] = rn;
+    st->it += 1;
+    if (!isfinite(rn) || rn <= st->tol * st->r0) st->done = 1;
+}
+
+// One point-relaxation sweep from the neighbours' records of the previous sweep.  Four lanes
+// per cell: lane r holds row r (r < E) and row r of the energy block, so that its two rows'
+// neighbour terms, its row of the block's inverse and its two output rows are its own, and
+// only the increments are exchanged (by shuffles).  R = double: everything in FP64;
+// R = float: the neighbour terms in FP32 (as stored), their sum, the solve and the update in
+// FP64.  FIRST: no neighbour terms.  LAST: W += dW and the primitive variables of the new W.
+template <typename R, int DIM, bool FIRST, bool LAST>
+__global__ void __launch_bounds__(128) k_macro_jacobi(MacroGeom g, ModelDev m, const MacroState *__restrict__ st,
+                                                      const double *__restrict__ Rg, const double *__restrict__ Dinv,
+                                                      const R *__restrict__ gam, const R *__restrict__ src,
+                                                      const Row<R> *__restrict__ in, Row<R> *__restrict__ out,
+                                                      double *__restrict__ W, double *__restrict__ qd,
+                                                      float *__restrict__ qf) {
+    constexpr int E = 1 + DIM, ER = 4 + DIM, LPC = 4;
+    if (st->done) return;
+    const MacroReal<R> &c = real<R>(g);
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, r = t % LPC;
+    const bool valid = t / LPC < g.n_cells;
+    const int i = valid ? t / LPC : g.n_cells - 1;
+    const int l0 = (int)(threadIdx.x & 31 & ~(LPC - 1));
+    const bool two = r < E;        // row r of the first block exists (E = 2, 3, 4)
+    double x0 = two ? Rg[(size_t)i * NVM + r] : 0.0, x1 = Rg[(size_t)i * NVM + E + r];
+    if constexpr (!FIRST) {
+        const int4 nb = *reinterpret_cast<const int4 *>(g.nb + (size_t)i * MAXF);
+        const int nbk[MAXF] = {nb.x, nb.y, nb.z, nb.w};
+        Row<R> a0[MAXF], a1[MAXF];
+#pragma unroll
+        for (int k = 0; k < MAXF; ++k) {
+            const size_t o = (size_t)max(nbk[k], 0) * NVM;
+            if (nbk[k] >= 0) {
+                a0[k] = in[o + (two ? r : 0)];
+                a1[k] = in[o + E + r];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < MAXF; ++k) {
+            if (nbk[k] < 0) continue;
+            const R *nS = c.cnS + ((size_t)i * MAXF + k) * MGS;
+            const R gb = gam[((size_t)i * MAXF + k) * 2], gE = r == 3 ? gam[((size_t)i * MAXF + k) * 2 + 1] : gb;
+            if constexpr (sizeof(R) == 8) {
+                x0 = fma(gb, a0[k].x[3], x0);
+                x1 = fma(gE, a1[k].x[3], x1);
+#pragma unroll
+                for (int a = 0; a < DIM; ++a) {
+                    x0 = fma(-nS[a], a0[k].x[a], x0);
+                    x1 = fma(-nS[a], a1[k].x[a], x1);
                 }
             } else {
-                float dF[NV];
-                flux_increment<DIM>(qW + (size_t)o * NVM, dGo, n, m, dF);
-                for (int v = 0; v < NV; ++v) {
-                    const float G = float(v == ER ? gb + gR : gb);
-                    off[v] = double((dF[v] - G * float(dGo[v])) * float(S));
+                R t0 = -gb * a0[k].x[3], t1 = -gE * a1[k].x[3];
+#pragma unroll
+                for (int a = 0; a < DIM; ++a) {
+                    t0 = fma(nS[a], a0[k].x[a], t0);
+                    t1 = fma(nS[a], a1[k].x[a], t1);
                 }
+                x0 -= to_double(t0);
+                x1 -= to_double(t1);
             }
         }
     }
-    for (int v = 0; v < NV; ++v)
-        for (int o = 1; o < LPC; o <<= 1) off[v] += __shfl_xor_sync(gmask, off[v], o);
-    if (!valid || k != 0) return;
-    const double V = g.vol[i];
-    double x[NV];
-    const double *rg = Rg + (size_t)i * NVM;
-    for (int v = 0; v < NV; ++v) x[v] = rg[v] - off[v] / (2.0 * V);
     const double *Di = Dinv + (size_t)i * DSTR;
-    double dG[NV];
-    for (int v = 0; v < E; ++v) dG[v] = Di[v] * x[v];
-    for (int r = 0; r < 4; ++r) {
-        double s = 0.0;
-        for (int c = 0; c < 4; ++c) s += Di[NVM + r * 4 + c] * x[E + c];
-        dG[E + r] = s;
-    }
-    for (int v = 0; v < NV; ++v) dG_out[(size_t)i * NVM + v] = dG[v];
-    if (last) {
-        for (int v = 0; v < NV; ++v) W_next[(size_t)i * NVM + v] = W[(size_t)i * NVM + v] + dG[v];
-        W_next[(size_t)i * NVM + E] += dG[ER];
+    const double d0 = Di[0] * x0;
+    double d1 = 0.0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) d1 = fma(Di[NVM + r * 4 + k], __shfl_sync(0xffffffffu, x1, l0 + k), d1);
+    if constexpr (LAST) {
+        const double dE3 = __shfl_sync(0xffffffffu, d1, l0 + 3);
+        double w0 = 0.0, w1 = 0.0;
+        if (two) w0 = W[(size_t)i * NVM + r] + d0;
+        w1 = W[(size_t)i * NVM + E + r] + d1;
+        if (r == 0) w1 += dE3;
+        double w[DIM + 5], q[DIM + 5];
+#pragma unroll
+        for (int k = 0; k < E; ++k) w[k] = __shfl_sync(0xffffffffu, w0, l0 + k);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) w[E + k] = __shfl_sync(0xffffffffu, w1, l0 + k);
+        primitive<DIM>(w, m, g.d, q);
+        if (!valid) return;
+        double q0 = 0.0, q1 = q[E];
+#pragma unroll
+        for (int k = 0; k < E; ++k)
+            if (k == r) q0 = q[k];
+#pragma unroll
+        for (int k = 1; k < 4; ++k)
+            if (k == r) q1 = q[E + k];
+        if (two) {
+            W[(size_t)i * NVM + r] = w0;
+            qd[(size_t)i * NVM + r] = q0;
+            if (qf) qf[(size_t)i * NVM + r] = fp64::narrow(q0);
+        }
+        W[(size_t)i * NVM + E + r] = w1;
+        qd[(size_t)i * NVM + E + r] = q1;
+        if (qf) qf[(size_t)i * NVM + E + r] = fp64::narrow(q1);
+    } else {
+        const R s0 = to_real<R>(d0), s1 = to_real<R>(d1);
+        const R *q = c.q + (size_t)i * NVM;
+        R u[DIM], dm[DIM];
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+            u[a] = q[1 + a];
+            dm[a] = __shfl_sync(0xffffffffu, s0, l0 + 1 + a);
+        }
+        const R drho = __shfl_sync(0xffffffffu, s0, l0), dEg = __shfl_sync(0xffffffffu, s1, l0),
+                der = __shfl_sync(0xffffffffu, s1, l0 + 1), dev = __shfl_sync(0xffffffffu, s1, l0 + 2);
+        const R rho = q[0];
+        const FluxIncrement<R, DIM> fi(rho, u, drho, dm, dEg, der, dev);
+        if (!valid) return;
+        if (two) {
+            Row<R> o;
+            o.x[1] = o.x[2] = R(0);
+            const R mb = r == 0 ? R(0) : rho * q[r];
+#pragma unroll
+            for (int a = 0; a < DIM; ++a)
+                o.x[a] = r == 0 ? dm[a] : fma(s0, fi.u1[a], fma(mb, fi.du[a], r == 1 + a ? fi.dp : R(0)));
+            o.x[3] = s0;
+            out[(size_t)i * NVM + r] = o;
+        }
+        Row<R> o;
+        o.x[1] = o.x[2] = R(0);
+        const R X = r == 3 ? R(0) : src[(size_t)i * SRC + 10 + r], dX = r == 0 ? fi.dH : r == 3 ? R(0) : s1, X1 = X + dX;
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) o.x[a] = fma(fi.du[a], X1, u[a] * dX);
+        o.x[3] = s1;
+        out[(size_t)i * NVM + E + r] = o;
+        (void)ER;
     }
 }
 
-// closed domains: scale W so that its total mass equals that of the reference fields
-__global__ void k_macro_mass_rescale(int nv, int n_cells, const double *__restrict__ vol,
-                                     const double *__restrict__ F_ref, double *__restrict__ W) {
-    __shared__ double a[1024], b[1024];
+// closed domains: fac = (total mass of the reference fields) / (total mass of W), the factor
+// that k_macro_fields_from_W scales W by; CTA partials in a fixed order, added by the last CTA
+constexpr int MM_CTAS = 64;
+__global__ void __launch_bounds__(256) k_macro_mass(int n_cells, const double *__restrict__ vol,
+                                                    const double *__restrict__ F_ref, const double *__restrict__ W,
+                                                    double *__restrict__ part, MacroState *__restrict__ st,
+                                                    double *__restrict__ fac) {
+    __shared__ double a[8], b[8];
+    __shared__ bool last;
     double sa = 0.0, sb = 0.0;
-    for (int i = threadIdx.x; i < n_cells; i += blockDim.x) {
-        sa += F_ref[(size_t)i * NF] * vol[i];
-        sb += W[(size_t)i * NVM] * vol[i];
-    }
-    a[threadIdx.x] = sa;
-    b[threadIdx.x] = sb;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) {
-            a[threadIdx.x] += a[threadIdx.x + w];
-            b[threadIdx.x] += b[threadIdx.x + w];
+    auto reduce = [&] {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            sa += __shfl_xor_sync(0xffffffffu, sa, o);
+            sb += __shfl_xor_sync(0xffffffffu, sb, o);
         }
         __syncthreads();
+        if ((threadIdx.x & 31) == 0) {
+            a[threadIdx.x >> 5] = sa;
+            b[threadIdx.x >> 5] = sb;
+        }
+        __syncthreads();
+        sa = sb = 0.0;
+        for (int w = 0; w < 8; ++w) {
+            sa += a[w];
+            sb += b[w];
+        }
+    };
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < n_cells; i += gridDim.x * 256) {
+        sa = fma(F_ref[(size_t)i * NF], vol[i], sa);
+        sb = fma(W[(size_t)i * NVM], vol[i], sb);
     }
-    const double fac = a[0] / b[0];
-    for (int i = threadIdx.x; i < n_cells; i += blockDim.x)
-        for (int v = 0; v < nv; ++v) W[(size_t)i * NVM + v] *= fac;
+    reduce();
+    if (threadIdx.x == 0) {
+        part[blockIdx.x * 2] = sa;
+        part[blockIdx.x * 2 + 1] = sb;
+        __threadfence();
+        last = atomicAdd(&st->ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    sa = sb = 0.0;
+    if (threadIdx.x < gridDim.x) {
+        sa = __ldcg(part + threadIdx.x * 2);
+        sb = __ldcg(part + threadIdx.x * 2 + 1);
+    }
+    reduce();
+    if (threadIdx.x == 0) {
+        *fac = sa / sb;
+        st->ticket = 0u;
+    }
 }
 
 // ------------------------------------------------------------------ launchers
+// 1-D and 2-D (3-D meshes take macro3d.cu)
 #define MACRO_DISPATCH(dim, ...)          \
     do {                                  \
         if ((dim) == 1) {                 \
             constexpr int DIM = 1;        \
             __VA_ARGS__;                  \
-        } else if ((dim) == 2) {          \
-            constexpr int DIM = 2;        \
-            __VA_ARGS__;                  \
         } else {                          \
-            constexpr int DIM = 3;        \
+            constexpr int DIM = 2;        \
             __VA_ARGS__;                  \
         }                                 \
     } while (0)
-
-int macro_rpart_count(int n_cells) { return (n_cells * 4 + 127) / 128; }
-
-cudaError_t launch_macro_from_fields(cudaStream_t s, int dim, int n_cells, const ModelDev &m, const double *F,
-                                     double *W) {
-    const int nb = (n_cells + 127) / 128;
-    MACRO_DISPATCH(dim, (k_macro_from_fields<DIM><<<nb, 128, 0, s>>>(n_cells, m, F, W)));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_macro_fields_from_W(cudaStream_t s, int dim, int n_cells, const ModelDev &m, const double *W,
-                                       double *F) {
-    const int nb = (n_cells + 127) / 128;
-    MACRO_DISPATCH(dim, (k_macro_fields_from_W<DIM><<<nb, 128, 0, s>>>(n_cells, m, W, F)));
-    return cudaGetLastError();
-}
 
 #define MACRO_DISPATCH_R(fp32, ...)      \
     do {                                  \
@@ -982,48 +1149,98 @@ cudaError_t launch_macro_fields_from_W(cudaStream_t s, int dim, int n_cells, con
         }                                 \
     } while (0)
 
-cudaError_t launch_macro_grad(cudaStream_t s, const MacroGeom &g, int order, int fp32, const ModelDev &m,
-                              const MacroState *st, const double *W, double *q, double *grad, double *phi) {
-    const int nb = (g.n_cells + MR_NT - 1) / MR_NT;
+static int ctas(long long threads, int nt) { return (int)((threads + nt - 1) / nt); }
+
+int macro_rpart_count(int n_cells) { return std::max(ctas((long long)n_cells * NVM, 128), 2 * MM_CTAS); }
+
+cudaError_t launch_macro_from_fields(cudaStream_t s, int dim, int n_cells, const ModelDev &m, const double *F,
+                                     const MacroWork &w) {
+    MACRO_DISPATCH(dim, (k_macro_from_fields<DIM><<<ctas(n_cells, 64), 64, 0, s>>>(n_cells, m, F, w.W, w.qd, w.qf)));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_macro_fields_from_W(cudaStream_t s, const MacroGeom &g, const ModelDev &m, const MacroWork &w,
+                                       const double *F_ref, double *F) {
+    if (F_ref) {
+        k_macro_mass<<<MM_CTAS, 256, 0, s>>>(g.n_cells, g.vol, F_ref, w.W, w.rpart, w.state, w.fac);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    MACRO_DISPATCH(g.dim, (k_macro_fields_from_W<DIM><<<ctas(g.n_cells, 64), 64, 0, s>>>(
+                              g.n_cells, m, g.d, w.W, F_ref ? w.fac : nullptr, F)));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_macro_grad(cudaStream_t s, const MacroGeom &g, int order, int fp32, const MacroState *st,
+                              const MacroWork &w) {
+    const int nb = ctas((long long)g.n_cells * NVM, 128);
     MACRO_DISPATCH_R(fp32, MACRO_DISPATCH(g.dim, {
-        if (order == 2) k_macro_grad<R, DIM, 2><<<nb, MR_NT, 0, s>>>(g, m, st, W, q, grad, phi);
-        else k_macro_grad<R, DIM, 1><<<nb, MR_NT, 0, s>>>(g, m, st, W, q, grad, phi);
+        if (order == 2) k_macro_grad<R, DIM, 2><<<nb, 128, 0, s>>>(g, st, (R *)w.grad, (R *)w.rec);
+        else k_macro_grad<R, DIM, 1><<<nb, 128, 0, s>>>(g, st, (R *)w.grad, (R *)w.rec);
     }));
     return cudaGetLastError();
 }
 
-cudaError_t launch_macro_bflux(cudaStream_t s, const MacroGeom &g, int fp32, const ModelDev &m, const QuadD &vq,
-                               const QuadD &oq, const MacroState *st, const double *q, double *bflux) {
+cudaError_t launch_macro_flux(cudaStream_t s, const MacroGeom &g, int order, int fp32, const ModelDev &m,
+                              const QuadD &vq, const MacroState *st, const MacroWork &w, bool boundary_only) {
+    const int nf = boundary_only ? 0 : ctas(g.n_fi, MF_FACES), nc = boundary_only ? 0 : ctas(g.n_cells, MF_NT);
+    const int n = nf + g.n_bf + nc;
+    if (n == 0) return cudaSuccess;
+    MACRO_DISPATCH_R(fp32, MACRO_DISPATCH(g.dim, {
+        if (order == 2)
+            k_macro_flux<R, DIM, 2><<<n, MF_NT, 0, s>>>(g, m, vq, nf, g.n_bf, st, (const R *)w.grad, (const R *)w.rec,
+                                                        (R *)w.Fx, (R *)w.fgam, (R *)w.src, w.mbf);
+        else
+            k_macro_flux<R, DIM, 1><<<n, MF_NT, 0, s>>>(g, m, vq, nf, g.n_bf, st, (const R *)w.grad, (const R *)w.rec,
+                                                        (R *)w.Fx, (R *)w.fgam, (R *)w.src, w.mbf);
+    }));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_macro_binc(cudaStream_t s, const MacroGeom &g, const ModelDev &m, const QuadD &vq, const QuadD &oq,
+                              double *binc) {
     if (g.n_bf == 0) return cudaSuccess;
-    MACRO_DISPATCH_R(fp32, MACRO_DISPATCH(g.dim, (k_macro_bflux<R, DIM><<<g.n_bf, 128, 0, s>>>(g, m, vq, oq, st, q,
-                                                                                                bflux))));
+    MACRO_DISPATCH(g.dim, (k_macro_binc<DIM><<<g.n_bf, MF_NT, 0, s>>>(g, m, vq, oq, binc)));
     return cudaGetLastError();
 }
 
 cudaError_t launch_macro_hot(cudaStream_t s, const MacroGeom &g, int fp32, const ModelDev &m, const double *F_kin,
-                             const double *q, const double *grad, const double *kin_bflux, const double *mac_bflux,
-                             double *hot, double *hot_b) {
-    const int n = g.n_fi + g.n_bf, nb = (n + MR_NT - 1) / MR_NT;
+                             const MacroWork &w, const double *kin_bflux, double *hot_b) {
+    const int n = g.n_fi + g.n_bf;
     if (n == 0) return cudaSuccess;
-    MACRO_DISPATCH_R(fp32, MACRO_DISPATCH(g.dim, (k_macro_hot<R, DIM><<<nb, MR_NT, 0, s>>>(g, m, F_kin, q, grad,
-                                                                                          kin_bflux, mac_bflux, hot,
-                                                                                          hot_b))));
+    MACRO_DISPATCH_R(fp32, MACRO_DISPATCH(g.dim, (k_macro_hot<R, DIM><<<ctas(n, 32), 32, 0, s>>>(
+                                                     g, m, F_kin, (const R *)w.grad, kin_bflux, w.mbf, w.hot, w.hotf,
+                                                     hot_b))));
     return cudaGetLastError();
 }
 
-cudaError_t launch_macro_residual(cudaStream_t s, const MacroGeom &g, int order, int fp32, const ModelDev &m,
-                                  double cfl_macro, const MacroState *st, const double *W, const double *q,
-                                  const double *grad, const double *phi, const double *hot, const double *bflux,
-                                  const double *hot_b, double *Rg, double *Dinv, double *gam, double *rpart) {
-    (void)W;
-    const int nb = macro_rpart_count(g.n_cells);
+cudaError_t launch_macro_residual(cudaStream_t s, const MacroGeom &g, int fp32, MacroState *st, const MacroWork &w,
+                                  const double *hot_b, double *history) {
+    const int nb = ctas((long long)g.n_cells * NVM, 128);
+    MACRO_DISPATCH_R(fp32, MACRO_DISPATCH(g.dim, (k_macro_residual<R, DIM><<<nb, 128, 0, s>>>(
+                                                     g, st, (const R *)w.Fx, (const R *)w.fgam, (const R *)w.src, w.mbf,
+                                                     hot_b, w.Rg, w.Dinv, (R *)w.gam, (Row<R> *)w.rows[0], w.rpart,
+                                                     history))));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_macro_jacobi(cudaStream_t s, const MacroGeom &g, int fp32, const ModelDev &m, const MacroState *st,
+                                int sweep, bool last, const MacroWork &w) {
+    const int nb = ctas((long long)g.n_cells * 4, 128);
     MACRO_DISPATCH_R(fp32, MACRO_DISPATCH(g.dim, {
-        if (order == 2)
-            k_macro_residual<R, DIM, 2><<<nb, 128, 0, s>>>(g, m, cfl_macro, st, q, grad, phi, hot, bflux, hot_b, Rg,
-                                                              Dinv, gam, rpart);
+        const R *gam = (const R *)w.gam;
+        const R *src = (const R *)w.src;
+        const Row<R> *in = (const Row<R> *)w.rows[(sweep + 1) & 1];
+        Row<R> *out = (Row<R> *)w.rows[sweep & 1];
+        if (sweep == 0)
+            k_macro_jacobi<R, DIM, true, true><<<nb, 128, 0, s>>>(g, m, st, w.Rg, w.Dinv, gam, src, in, out, w.W, w.qd,
+                                                                  w.qf);
+        else if (last)
+            k_macro_jacobi<R, DIM, false, true><<<nb, 128, 0, s>>>(g, m, st, w.Rg, w.Dinv, gam, src, in, out, w.W,
+                                                                   w.qd, w.qf);
         else
-            k_macro_residual<R, DIM, 1><<<nb, 128, 0, s>>>(g, m, cfl_macro, st, q, grad, phi, hot, bflux, hot_b, Rg,
-                                                              Dinv, gam, rpart);
+            k_macro_jacobi<R, DIM, false, false><<<nb, 128, 0, s>>>(g, m, st, w.Rg, w.Dinv, gam, src, in, out, w.W,
+                                                                    w.qd, w.qf);
     }));
     return cudaGetLastError();
 }
@@ -1045,28 +1262,6 @@ __global__ void k_macro_offset(int n_cells, int nv, const double *__restrict__ R
 cudaError_t launch_macro_offset(cudaStream_t s, int dim, int n_cells, const double *Rg, const double *rows,
                                 double *moff) {
     k_macro_offset<<<(n_cells + 127) / 128, 128, 0, s>>>(n_cells, dim + 5, Rg, rows, moff);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_macro_norm(cudaStream_t s, int n_parts, const double *rpart, MacroState *st, double *history) {
-    k_macro_norm<<<1, 256, 0, s>>>(n_parts, rpart, st, history);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_macro_jacobi(cudaStream_t s, const MacroGeom &g, int fp32, const ModelDev &m,
-                                const MacroState *st, int first, int last, const double *W, const double *q,
-                                const double *Rg, const double *Dinv, const double *gam, const double *dG_in,
-                                double *dG_out, double *W_next) {
-    const int nb = (g.n_cells * LPC + 127) / 128;
-    MACRO_DISPATCH(g.dim, MACRO_DISPATCH_R(fp32, (k_macro_jacobi<R, DIM><<<nb, 128, 0, s>>>(
-                                                     g, m, st, first, last, W, q, Rg, Dinv, gam, dG_in, dG_out,
-                                                     W_next))));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_macro_mass_rescale(cudaStream_t s, int dim, int n_cells, const double *vol, const double *F_ref,
-                                      double *W) {
-    k_macro_mass_rescale<<<1, 1024, 0, s>>>(dim + 5, n_cells, vol, F_ref, W);
     return cudaGetLastError();
 }
 

@@ -218,28 +218,32 @@ __global__ void k_cell_features(MacroGeom g, ModelDev m, const double *__restric
     for (int d = 0; d < DIM; ++d) y[10 + d] = (float)((r[17 + d] + kR * gr(d, ER)) / sq);
 }
 
-// face high-order terms from predicted cell values (de-normalised, averaged over the two
-// cells); the boundary terms are zero
+// face high-order terms on the face normal from predicted cell values (de-normalised,
+// averaged over the two cells), laid out as k_macro_hot's; the boundary terms are zero
 template <int DIM>
-__global__ void k_hot_from_cells(MacroGeom g, const double *__restrict__ q, const float *__restrict__ Yc,
-                                 double *__restrict__ hot, double *__restrict__ hot_b) {
+__global__ void k_hot_from_cells(MacroGeom g, const float *__restrict__ Yc, double *__restrict__ hot,
+                                 float *__restrict__ hotf, double *__restrict__ hot_b) {
     constexpr int E = 1 + DIM;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < g.n_fi) {
-        double h[NHOT];
-        for (int k = 0; k < NHOT; ++k) h[k] = 0.0;
-        const int cells[2] = {g.fi_i[t], g.fi_j[t]};
+        double h[DIM + 4];
+        for (int k = 0; k < DIM + 4; ++k) h[k] = 0.0;
+        const double *n = g.d.fgeo + (size_t)t * FGEO;
+        const int cells[2] = {g.fi4[t].x, g.fi4[t].y};
         for (int c : cells) {
-            const double rho = q[(size_t)c * NVM], Tt = q[(size_t)c * NVM + E];
+            const double rho = g.d.q[(size_t)c * NVM], Tt = g.d.q[(size_t)c * NVM + E];
             const double srT = 0.5 * rho * Tt, sq = 0.5 * rho * Tt * sqrt(Tt);
             const float *y = Yc + (size_t)c * MLP_OUT;
             const int sidx[2][2] = {{0, 1}, {1, 2}};
             for (int a = 0; a < DIM; ++a)
-                for (int b = 0; b < DIM; ++b) h[a * DIM + b] += srT * y[sidx[a][b]];
+                for (int b = 0; b < DIM; ++b) h[a] += srT * y[sidx[a][b]] * n[b];
             for (int md = 0; md < 4; ++md)
-                for (int d = 0; d < DIM; ++d) h[DIM * DIM + md * DIM + d] += sq * y[4 + 2 * md + d];
+                for (int d = 0; d < DIM; ++d) h[DIM + md] += sq * y[4 + 2 * md + d] * n[d];
         }
-        for (int k = 0; k < NHOT; ++k) hot[(size_t)t * NHOT + k] = h[k];
+        for (int k = 0; k < DIM + 4; ++k) {
+            hot[(size_t)t * NVM + k] = h[k];
+            if (hotf) hotf[(size_t)t * NVM + k] = (float)h[k];
+        }
         return;
     }
     const int b = t - g.n_fi;
@@ -365,12 +369,12 @@ cudaError_t launch_cell_features(cudaStream_t s, const MacroGeom &g, const Model
     return cudaGetLastError();
 }
 
-cudaError_t launch_hot_from_cells(cudaStream_t s, const MacroGeom &g, const double *q, const float *Yc,
-                                  double *hot, double *hot_b) {
+cudaError_t launch_hot_from_cells(cudaStream_t s, const MacroGeom &g, const float *Yc, const MacroWork &w,
+                                  double *hot_b) {
     const int n = g.n_fi + g.n_bf, nb = (n + 127) / 128;
     if (n == 0) return cudaSuccess;
-    if (g.dim == 1) k_hot_from_cells<1><<<nb, 128, 0, s>>>(g, q, Yc, hot, hot_b);
-    else k_hot_from_cells<2><<<nb, 128, 0, s>>>(g, q, Yc, hot, hot_b);
+    if (g.dim == 1) k_hot_from_cells<1><<<nb, 128, 0, s>>>(g, Yc, w.hot, w.hotf, hot_b);
+    else k_hot_from_cells<2><<<nb, 128, 0, s>>>(g, Yc, w.hot, w.hotf, hot_b);
     return cudaGetLastError();
 }
 
