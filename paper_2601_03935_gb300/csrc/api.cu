@@ -934,6 +934,13 @@ int gsis_create(const gsis_mesh *m, const gsis_velocity_quad *vq, const gsis_pho
     md.sigma_R = mp->sigma_R;
     md.k_eff_density_scaled = mp->k_eff_density_scaled;
     md.cfl_meso = sp->cfl_meso;
+    md.i_Zr = 1.0 / mp->Z_r;
+    md.i_Zv = 1.0 / mp->Z_v;
+    md.i_Knp = 1.0 / mp->Kn_p;
+    md.i_half_dr = 2.0 / mp->d_r;
+    md.i_half_dv = 2.0 / mp->d_v;
+    md.i_heat = 1.0 / (3.0 + mp->d_r + mp->d_v);
+    md.i_4sigma = 1.0 / (4.0 * mp->sigma_R);
     md.dv_T = mp->dv_temperature_dependent ? 1 : 0;
     md.Tv_ref = mp->Tv_ref;
     md.userA = mp->A ? 1 : 0;

@@ -28,13 +28,14 @@ constexpr int ERR_TIMEOUT_BIT = 2;
 // ---- per-cell coefficient record (Real), built from the FP64 fields each iteration,
 // laid out for 16-byte vector loads:
 // u[3], pad | per Maxwellian a in {t, tr, tv} (16 each): A, B, T, K1 | Q[3], K2 |
-// R1[3], pad | R2[3], pad | rate (1/tau), inv_dt, sink, photon source g_R |
+// R1[3], S | R2[3], A2 | rate (1/tau), inv_dt, sink, photon source g_R |
 // photon rate k_eff, pad[3]
 namespace cf {
 constexpr int U = 0;
 constexpr int COMP = 4;        // first component block
 constexpr int CSZ = 16;        // size of one component block
 constexpr int A = 0, B = 1, T = 2, K1 = 3, Q = 4, K2 = 7, R1 = 8, R2 = 12;
+constexpr int S = 11, A2 = 15;   // FP64: -B in the units of fp64::exp2n, A m T (m hidden components)
 constexpr int RATE = COMP + 3 * CSZ;   // 52
 constexpr int INV_DT = RATE + 1;
 constexpr int SINK = RATE + 2;
@@ -114,6 +115,8 @@ struct ModelDev {
     double A[9];
     double Mix[9];             // (q0, q1, q2) = Mix (q_t, q_r, q_v)
     double cfl_meso;
+    double i_Zr, i_Zv, i_Knp;  // 1 / Z_r, 1 / Z_v, 1 / Kn_p
+    double i_half_dr, i_half_dv, i_heat, i_4sigma;   // 2/d_r, 2/d_v, 1/(3 + d_r + d_v), 1/(4 sigma_R)
     int dv_T;                  // d_v(T_v) = 2 x / (e^x - 1), x = Tv_ref / T_v; else d_v constant
     int userA;                 // A given by the caller (kept constant); else Mason-Monchick at d_v
     double Tv_ref;
