@@ -2155,10 +2155,12 @@ int mlp_malloc(gsis_ctx *c, void **p, size_t bytes) {
     return GSIS_OK;
 }
 
-void mlp_free(gsis_ctx *c, void *p) {
+template <typename T>
+void mlp_free(gsis_ctx *c, T *&p) {
     if (!p) return;
     cudaFree(p);
-    c->mlp_alloc.erase(std::remove(c->mlp_alloc.begin(), c->mlp_alloc.end(), p), c->mlp_alloc.end());
+    c->mlp_alloc.erase(std::remove(c->mlp_alloc.begin(), c->mlp_alloc.end(), (void *)p), c->mlp_alloc.end());
+    p = nullptr;
 }
 
 // parameters, moments and per-cell buffers once; work buffers for at least n rows
@@ -2170,6 +2172,8 @@ int mlp_ensure(gsis_ctx *c, int64_t n) {
         TRY(mlp_malloc(c, (void **)&d.m1, MLP_NW * sizeof(float)));
         TRY(mlp_malloc(c, (void **)&d.m2, MLP_NW * sizeof(float)));
         TRY(mlp_malloc(c, &d.pb, MLP_NW * 2));
+        TRY(mlp_malloc(c, (void **)&d.gpart, (size_t)MLP_SPLITS * MLP_NW * sizeof(float)));
+        TRY(mlp_malloc(c, (void **)&d.lpart, (MLP_CTAS + 1) * sizeof(double)));
         TRY(mlp_malloc(c, (void **)&c->mlp_X, (size_t)c->nc * MLP_IN * sizeof(float)));
         TRY(mlp_malloc(c, (void **)&c->mlp_Y, (size_t)c->nc * MLP_OUT * sizeof(float)));
         CUDA_TRY(c, cudaMemsetAsync(d.p, 0, MLP_NPARAM * sizeof(float), c->stream));
@@ -2179,18 +2183,13 @@ int mlp_ensure(gsis_ctx *c, int64_t n) {
     if (n > d.cap) {
         const int widths[MLP_LAYERS + 1] = {MLP_IN, MLP_H, MLP_H, MLP_H, MLP_OUT};
         for (int l = 0; l <= MLP_LAYERS; ++l) mlp_free(c, d.act[l]);
-        for (int l = 0; l < MLP_LAYERS; ++l) mlp_free(c, d.pre[l]);
-        mlp_free(c, d.dA[0]);
-        mlp_free(c, d.dA[1]);
+        for (int l = 0; l < MLP_LAYERS; ++l) mlp_free(c, d.dZ[l]);
         mlp_free(c, d.T);
-        mlp_free(c, d.lpart);
         mlp_free(c, c->mlp_idx);
+        d.cap = 0;
         for (int l = 0; l <= MLP_LAYERS; ++l) TRY(mlp_malloc(c, (void **)&d.act[l], n * widths[l] * sizeof(float)));
-        for (int l = 0; l < MLP_LAYERS; ++l) TRY(mlp_malloc(c, (void **)&d.pre[l], n * widths[l + 1] * sizeof(float)));
-        TRY(mlp_malloc(c, (void **)&d.dA[0], n * MLP_H * sizeof(float)));
-        TRY(mlp_malloc(c, (void **)&d.dA[1], n * MLP_H * sizeof(float)));
+        for (int l = 0; l < MLP_LAYERS; ++l) TRY(mlp_malloc(c, (void **)&d.dZ[l], n * widths[l + 1] * sizeof(float)));
         TRY(mlp_malloc(c, (void **)&d.T, n * MLP_OUT * sizeof(float)));
-        TRY(mlp_malloc(c, (void **)&d.lpart, (size_t)mlp_loss_parts((int)n) * sizeof(double)));
         TRY(mlp_malloc(c, (void **)&c->mlp_idx, n * sizeof(int)));
         d.cap = (int)n;
     }
@@ -2202,21 +2201,15 @@ const float *x_std(const gsis_ctx *c) { return c->mlp.p + MLP_NW + MLP_IN; }
 const float *y_mean(const gsis_ctx *c) { return c->mlp.p + MLP_NW + 2 * MLP_IN; }
 const float *y_std(const gsis_ctx *c) { return c->mlp.p + MLP_NW + 2 * MLP_IN + MLP_OUT; }
 
-// forward pass of n rows already standardised in act[0]; loss over standardised targets in T
-int mlp_loss(gsis_ctx *c, int n, double *loss) {
+// loss and gradients of n rows already standardised in act[0], targets in T; the host
+// copies are asynchronous (null: none)
+int mlp_loss(gsis_ctx *c, int n, double *loss, float *grad) {
     MlpDev &d = c->mlp;
-    CUDA_TRY(c, launch_mlp_forward(c->stream, d, n));
     CUDA_TRY(c, launch_mlp_loss_backward(c->stream, d, n));
-    c->launches += 4 + 1 + 3 + 4 + 3;
-    if (loss) {
-        const int np = mlp_loss_parts(n);
-        std::vector<double> part(np);
-        CUDA_TRY(c, cudaMemcpyAsync(part.data(), d.lpart, np * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-        CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-        double sum = 0.0;
-        for (double x : part) sum += x;
-        *loss = sum / ((double)n * MLP_OUT);
-    }
+    c->launches += 3;
+    if (loss)
+        CUDA_TRY(c, cudaMemcpyAsync(loss, d.lpart + d.loss_at, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    if (grad) CUDA_TRY(c, cudaMemcpyAsync(grad, d.g, MLP_NW * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
     return GSIS_OK;
 }
 
@@ -2272,11 +2265,8 @@ int gsis_mlp_loss_grad(gsis_ctx *c, const float *X, const float *Y, int64_t n, d
     CUDA_TRY(c, cudaMemcpyAsync(d.T, Y, n * MLP_OUT * sizeof(float), cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(c, launch_mlp_standardise(c->stream, (int)n, MLP_IN, d.act[0], x_mean(c), x_std(c), 0));
     CUDA_TRY(c, launch_mlp_standardise(c->stream, (int)n, MLP_OUT, d.T, y_mean(c), y_std(c), 0));
-    TRY(mlp_loss(c, (int)n, loss));
-    if (grad) {
-        CUDA_TRY(c, cudaMemcpyAsync(grad, d.g, MLP_NW * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
-        CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-    }
+    TRY(mlp_loss(c, (int)n, loss, grad));
+    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     return GSIS_OK;
 }
 
@@ -2292,7 +2282,7 @@ int gsis_mlp_predict(gsis_ctx *c, const float *X, int64_t n, float *Y) {
     CUDA_TRY(c, cudaMemcpyAsync(Y, d.act[MLP_LAYERS], n * MLP_OUT * sizeof(float), cudaMemcpyDeviceToHost,
                                 c->stream));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-    c->launches += 6;
+    c->launches += 3;
     return GSIS_OK;
 }
 
@@ -2351,7 +2341,7 @@ int gsis_mlp_train(gsis_ctx *c, const float *X, const float *Y, int64_t n, int32
             CUDA_TRY(c, launch_mlp_gather(c->stream, (int)b, MLP_IN, c->mlp_idx, Xd, d.act[0]));
             CUDA_TRY(c, launch_mlp_gather(c->stream, (int)b, MLP_OUT, c->mlp_idx, Yd, d.T));
             const bool report = ep == epochs - 1 && s0 + 2 * b > n;
-            TRY(mlp_loss(c, (int)b, report ? &last : nullptr));
+            TRY(mlp_loss(c, (int)b, report ? &last : nullptr, nullptr));
             CUDA_TRY(c, launch_mlp_adam(c->stream, d, (float)lr));
             c->launches += 3;
         }
@@ -2403,7 +2393,7 @@ int warm_start(gsis_ctx *c, int n_presolve, bool use_mlp) {
             CUDA_TRY(c, launch_mlp_forward(c->stream, d, (int)c->nc));
             CUDA_TRY(c, launch_mlp_standardise(c->stream, (int)c->nc, MLP_OUT, d.act[MLP_LAYERS], y_mean(c), y_std(c),
                                                1));
-            c->launches += 6;
+            c->launches += 3;
             TRY(launch(c, K_MLP, [&] {
                 return launch_hot_from_cells(c->stream, g, d.act[MLP_LAYERS], c->mw, c->hot_b);
             }));

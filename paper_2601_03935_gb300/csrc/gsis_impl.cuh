@@ -393,6 +393,7 @@ constexpr int MLP_IN = 16, MLP_H = 128, MLP_OUT = 12, MLP_LAYERS = 4;
 constexpr int MLP_NW = MLP_H * MLP_IN + MLP_H + 2 * (MLP_H * MLP_H + MLP_H) + MLP_OUT * MLP_H + MLP_OUT;
 constexpr int MLP_NSTAT = 2 * MLP_IN + 2 * MLP_OUT;
 constexpr int MLP_NPARAM = MLP_NW + MLP_NSTAT;
+constexpr int MLP_CTAS = 152, MLP_SPLITS = 32;   // CTAs of a pass over the rows; row ranges of the weight gradient
 
 struct MlpDev {
     int cap = 0;                       // rows the work buffers hold
@@ -400,21 +401,21 @@ struct MlpDev {
     float *g = nullptr, *m1 = nullptr, *m2 = nullptr;   // gradients and Adam moments [MLP_NW]
     void *pb = nullptr;                // BF16 copy of the weights and biases [MLP_NW]
     float *act[MLP_LAYERS + 1] = {};   // layer inputs/outputs [cap][width]
-    float *pre[MLP_LAYERS] = {};       // pre-activations [cap][width]
-    float *dA[2] = {nullptr, nullptr}; // back-propagated gradients [cap][MLP_H]
+    float *dZ[MLP_LAYERS] = {};        // gradients of the layers' pre-activations [cap][width]
     float *T = nullptr;                // targets [cap][MLP_OUT]
-    double *lpart = nullptr;           // loss partials
+    float *gpart = nullptr;            // weight-gradient partials [MLP_SPLITS][MLP_NW]
+    double *lpart = nullptr;           // loss partials [MLP_CTAS], then the loss
+    int loss_at = 0;                   // where in lpart the last loss is
     int64_t step = 0;                  // Adam step count
     bool trained = false;
 };
 
 cudaError_t launch_mlp_forward(cudaStream_t s, MlpDev &d, int n);       // act[0] (standardised) -> act[4]
-cudaError_t launch_mlp_loss_backward(cudaStream_t s, MlpDev &d, int n); // needs act/pre of a forward and T
+cudaError_t launch_mlp_loss_backward(cudaStream_t s, MlpDev &d, int n); // act[0], T -> g, loss
 cudaError_t launch_mlp_adam(cudaStream_t s, MlpDev &d, float lr);
 cudaError_t launch_mlp_to_bf16(cudaStream_t s, MlpDev &d);
 cudaError_t launch_mlp_standardise(cudaStream_t s, int n, int m, float *X, const float *mean, const float *sd,
                                    int inv);
-int mlp_loss_parts(int n);
 cudaError_t launch_mlp_gather(cudaStream_t s, int n, int width, const int *idx, const float *src, float *dst);
 cudaError_t launch_cell_features(cudaStream_t s, const MacroGeom &g, const ModelDev &m, const double *F,
                                  const double *q, const double *grad, float *X, float *Y);

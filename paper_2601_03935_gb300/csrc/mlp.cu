@@ -4,24 +4,22 @@
 //
 //  cell_features   per-cell inputs (state, gradient magnitudes, Kn, 1/Kn_p) and the
 //                  normalised high-order-term targets of Eq. (getHoTs) at the cell
-//  dense_fwd       Z = A W^T + b, A' = GELU(Z) (hidden) or Z (output); W staged in shared
-//                  memory transposed, one thread per output neuron, a tile of rows per CTA
-//  dense_bwd       dA = dZ W
-//  gelu_bwd        dZ = dA GELU'(Z)
-//  weight_grad     dW = dZ^T A, db = sum dZ; one thread per weight, fixed summation order
-//  mse             loss and dY = 2 (Y - T) / (n 12), per-CTA partial losses
+//  mlp_pass        all layers for a tile of rows in one kernel: forward, and in training the
+//                  loss and the back-propagated dZ of every layer
+//  weight_grad     dW = dZ^T A, db = sum dZ: 64 x 64 tiles over ranges of rows
+//  grad_reduce     sums of the ranges' tiles and of the loss partials, in a fixed order
 //  adam            FP32 master update and its BF16 copy
 //  hot_from_cells  face high-order terms from predicted cell values (face average)
+#include <algorithm>
 #include <cmath>
 #include <cuda_bf16.h>
 
+#include "fp64.cuh"
 #include "gsis_impl.cuh"
 
 namespace gsis {
 
 namespace {
-
-constexpr int TROWS = 32;          // rows (samples) per CTA of the dense kernels
 
 __device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_grad(float z) {
@@ -30,93 +28,291 @@ __device__ __forceinline__ float gelu_grad(float z) {
 
 }  // namespace
 
-// Y[r][o] = act(b[o] + sum_i X[r][i] W[o][i]); Z keeps the pre-activation when not null
-template <bool ACT>
-__global__ void __launch_bounds__(128) k_dense_fwd(int n, int in, int out, const float *__restrict__ X,
-                                                   const __nv_bfloat16 *__restrict__ W, const float *__restrict__ b,
-                                                   float *__restrict__ Z, float *__restrict__ Y) {
-    extern __shared__ float sm[];
-    float *Wt = sm;                    // [in][out]
-    float *Xs = sm + in * out;         // [TROWS][in]
-    const int r0 = blockIdx.x * TROWS;
-    for (int k = threadIdx.x; k < in * out; k += blockDim.x) {
-        const int o = k / in, i = k % in;
-        Wt[i * out + o] = __bfloat162float(W[k]);
+namespace {
+
+constexpr int layer_in(int l) { return l == 0 ? MLP_IN : MLP_H; }
+constexpr int layer_out(int l) { return l == MLP_LAYERS - 1 ? MLP_OUT : MLP_H; }
+constexpr int w_off(int l) {
+    int o = 0;
+    for (int k = 0; k < l; ++k) o += layer_out(k) * layer_in(k) + layer_out(k);
+    return o;
+}
+// Shared memory of mlp_pass: the four BF16 weight matrices with rows padded by 8 bytes (a
+// row's next one starts two banks on: 8-byte reads of 32 rows meet every bank twice), then
+// per warp PR rows of activations, of dZ (value-major, the PR rows side by side) and of the
+// pre-activations of the three hidden layers.
+constexpr int PR = 4;                                    // rows of a warp (a float4 of dZ)
+constexpr int ws_stride(int l) { return layer_in(l) + 4; }
+constexpr int ws_off(int l) {
+    int o = 0;
+    for (int k = 0; k < l; ++k) o += layer_out(k) * ws_stride(k);
+    return o;
+}
+constexpr int WS_BYTES = (ws_off(MLP_LAYERS) * 2 + 15) / 16 * 16;
+constexpr int WARP_FLOATS = PR * MLP_H * 5;
+constexpr int N_BIAS = 3 * MLP_H + MLP_OUT;
+constexpr int pass_smem(int warps, bool train) {
+    return WS_BYTES + (N_BIAS + 3) / 4 * 16 + warps * (train ? WARP_FLOATS : PR * MLP_H) * 4;
+}
+
+__device__ __forceinline__ void copy8_async(void *smem, const void *global) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(global)
+                 : "memory");
+}
+__device__ __forceinline__ float lo_bf16(uint32_t u) { return __uint_as_float(u << 16); }
+__device__ __forceinline__ float hi_bf16(uint32_t u) { return __uint_as_float(u & 0xffff0000u); }
+
+}  // namespace
+
+// One tile of WARPS * PR rows at a time through every layer; a warp keeps its PR rows to
+// itself, so only the staged weights are shared.  Forward: lane = output (lane + 32 j), the
+// sum over inputs in two interleaved FP32 chains on the packed FP32x2 pipe; backward: lane =
+// four consecutive inputs.  Reads act0 [n][16] (standardised) and T; writes Y [n][12], and in
+// training act1..3 [n][128], dZ0..3 [n][128 | 12] and the CTA's loss.
+// Bound by the instructions that feed the FP32 pipe (an 8-byte weight read and two
+// conversions serve PR rows); one thread per output with both operands from shared memory
+// per FMA, a kernel per layer and a serial weight gradient before: 2 048 rows, loss and
+// gradient 1.56 -> 0.107 ms end to end, of which this kernel takes 25 us.
+template <int WARPS, bool TRAIN>
+__global__ void __launch_bounds__(32 * WARPS) k_mlp_pass(int n, const __nv_bfloat16 *__restrict__ W,
+                                                         const float *__restrict__ P, const float *__restrict__ act0,
+                                                         float *__restrict__ Y, float *__restrict__ A1,
+                                                         float *__restrict__ A2, float *__restrict__ A3,
+                                                         const float *__restrict__ T, float *__restrict__ D0,
+                                                         float *__restrict__ D1, float *__restrict__ D2,
+                                                         float *__restrict__ D3, double *__restrict__ lpart) {
+    extern __shared__ __align__(16) unsigned char mlp_smem[];
+    __nv_bfloat16 *Ws = reinterpret_cast<__nv_bfloat16 *>(mlp_smem);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float *Bs = reinterpret_cast<float *>(mlp_smem + WS_BYTES);     // biases
+    float *A = Bs + (N_BIAS + 3) / 4 * 4 + warp * (TRAIN ? WARP_FLOATS : PR * MLP_H);
+    float *D = A + PR * MLP_H;                 // [o][PR]
+    float *Z = D + PR * MLP_H;                 // [3][PR][MLP_H]
+    float *const Aout[3] = {A1, A2, A3};
+    float *const Dout[4] = {D0, D1, D2, D3};
+#pragma unroll
+    for (int l = 0; l < MLP_LAYERS; ++l) {     // weights, four at a time
+        const int in4 = layer_in(l) / 4;
+        const uint2 *src = reinterpret_cast<const uint2 *>(W + w_off(l));
+        for (int k = threadIdx.x; k < layer_out(l) * in4; k += 32 * WARPS)
+            copy8_async(Ws + ws_off(l) + k / in4 * ws_stride(l) + k % in4 * 4, src + k);
     }
-    const int rows = min(TROWS, n - r0);
-    for (int k = threadIdx.x; k < rows * in; k += blockDim.x) Xs[k] = X[(size_t)r0 * in + k];
+    for (int k = threadIdx.x; k < N_BIAS; k += 32 * WARPS) {
+        const int l = k / MLP_H;
+        Bs[k] = P[w_off(l) + layer_out(l) * layer_in(l) + k % MLP_H];
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    const int o = threadIdx.x;
-    if (o >= out) return;
-    const float bo = b[o];
-    for (int r = 0; r < rows; ++r) {
-        float acc = bo;
-        for (int i = 0; i < in; ++i) acc = fmaf(Xs[r * in + i], Wt[i * out + o], acc);
-        const size_t idx = (size_t)(r0 + r) * out + o;
-        if (Z) Z[idx] = acc;
-        Y[idx] = ACT ? gelu(acc) : acc;
+    double loss = 0.0;
+    const int tiles = (n + WARPS * PR - 1) / (WARPS * PR);
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int r0 = (tile * WARPS + warp) * PR;
+        if (r0 >= n) continue;                  // the warp's rows only: no barrier below
+        const int rows = min(PR, n - r0);
+        __syncwarp();
+        for (int k = lane; k < PR * MLP_IN; k += 32) {
+            const int r = k / MLP_IN;
+            A[r * MLP_H + k % MLP_IN] = r < rows ? act0[(size_t)r0 * MLP_IN + k] : 0.0f;
+        }
+        __syncwarp();
+        // ---- hidden layers
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+            float2 acc[PR][4];
+#pragma unroll
+            for (int r = 0; r < PR; ++r)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[r][j] = make_float2(0.0f, 0.0f);
+            const __nv_bfloat16 *w0 = Ws + ws_off(l) + lane * ws_stride(l);
+#pragma unroll 2
+            for (int k = 0; k < layer_in(l); k += 4) {
+                float4 a[PR];
+                uint2 w[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) w[j] = *reinterpret_cast<const uint2 *>(w0 + 32 * j * ws_stride(l) + k);
+#pragma unroll
+                for (int r = 0; r < PR; ++r) a[r] = *reinterpret_cast<const float4 *>(A + r * MLP_H + k);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 p = make_float2(lo_bf16(w[j].x), hi_bf16(w[j].x));
+                    const float2 q = make_float2(lo_bf16(w[j].y), hi_bf16(w[j].y));
+#pragma unroll
+                    for (int r = 0; r < PR; ++r) {
+                        acc[r][j] = __ffma2_rn(make_float2(a[r].x, a[r].y), p, acc[r][j]);
+                        acc[r][j] = __ffma2_rn(make_float2(a[r].z, a[r].w), q, acc[r][j]);
+                    }
+                }
+            }
+            __syncwarp();
+            const float *b = Bs + l * MLP_H;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int o = lane + 32 * j;
+                const float bo = b[o];
+#pragma unroll
+                for (int r = 0; r < PR; ++r) {
+                    const float z = bo + (acc[r][j].x + acc[r][j].y), g = gelu(z);
+                    A[r * MLP_H + o] = g;
+                    if constexpr (TRAIN) {
+                        Z[(l * PR + r) * MLP_H + o] = z;
+                        if (r < rows) Aout[l][(size_t)(r0 + r) * MLP_H + o] = g;
+                    }
+                }
+            }
+            __syncwarp();
+        }
+        // ---- output layer: 12 x PR values over the lanes
+        for (int k = lane; k < PR * MLP_OUT; k += 32) {
+            const int r = k / MLP_OUT, o = k % MLP_OUT;
+            const __nv_bfloat16 *w0 = Ws + ws_off(3) + o * ws_stride(3);
+            float2 acc = make_float2(0.0f, 0.0f);
+#pragma unroll 4
+            for (int i = 0; i < MLP_H; i += 4) {
+                const uint2 w = *reinterpret_cast<const uint2 *>(w0 + i);
+                const float4 a = *reinterpret_cast<const float4 *>(A + r * MLP_H + i);
+                acc = __ffma2_rn(make_float2(a.x, a.y), make_float2(lo_bf16(w.x), hi_bf16(w.x)), acc);
+                acc = __ffma2_rn(make_float2(a.z, a.w), make_float2(lo_bf16(w.y), hi_bf16(w.y)), acc);
+            }
+            const float y = Bs[3 * MLP_H + o] + (acc.x + acc.y);
+            if (!TRAIN && r < rows) Y[(size_t)(r0 + r) * MLP_OUT + o] = y;
+            if constexpr (TRAIN) {
+                // loss and dZ = 2 (Y - T) / (n 12); rows past the end carry nothing
+                float dz = 0.0f;
+                if (r < rows) {
+                    const float d = y - T[(size_t)(r0 + r) * MLP_OUT + o];
+                    dz = 2.0f * d / (float)((double)n * MLP_OUT);
+                    const double d8 = to_double(d);
+                    loss = fma(d8, d8, loss);
+                    D3[(size_t)(r0 + r) * MLP_OUT + o] = dz;
+                }
+                D[o * PR + r] = dz;
+            }
+        }
+        if constexpr (TRAIN) {
+            // ---- backward: dA_l = dZ_l W_l, dZ_{l-1} = dA_l GELU'(Z_{l-1})
+#pragma unroll
+            for (int l = 3; l > 0; --l) {
+                __syncwarp();
+                float2 acc[PR][2];
+#pragma unroll
+                for (int r = 0; r < PR; ++r) acc[r][0] = acc[r][1] = make_float2(0.0f, 0.0f);
+                const __nv_bfloat16 *w0 = Ws + ws_off(l) + 4 * lane;
+#pragma unroll 4
+                for (int o = 0; o < layer_out(l); ++o) {
+                    const uint2 w = *reinterpret_cast<const uint2 *>(w0 + o * ws_stride(l));
+                    const float4 d = *reinterpret_cast<const float4 *>(D + o * PR);
+                    const float2 p = make_float2(lo_bf16(w.x), hi_bf16(w.x)), q = make_float2(lo_bf16(w.y), hi_bf16(w.y));
+                    const float dd[PR] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+                    for (int r = 0; r < PR; ++r) {
+                        acc[r][0] = __ffma2_rn(make_float2(dd[r], dd[r]), p, acc[r][0]);
+                        acc[r][1] = __ffma2_rn(make_float2(dd[r], dd[r]), q, acc[r][1]);
+                    }
+                }
+                __syncwarp();
+                float4 dz[PR];
+#pragma unroll
+                for (int r = 0; r < PR; ++r) {
+                    const float4 z = *reinterpret_cast<const float4 *>(Z + ((l - 1) * PR + r) * MLP_H + 4 * lane);
+                    dz[r] = make_float4(acc[r][0].x * gelu_grad(z.x), acc[r][0].y * gelu_grad(z.y),
+                                        acc[r][1].x * gelu_grad(z.z), acc[r][1].y * gelu_grad(z.w));
+                    if (r < rows)
+                        *reinterpret_cast<float4 *>(Dout[l - 1] + (size_t)(r0 + r) * MLP_H + 4 * lane) = dz[r];
+                }
+                float4 *Dv = reinterpret_cast<float4 *>(D) + 4 * lane;
+                Dv[0] = make_float4(dz[0].x, dz[1].x, dz[2].x, dz[3].x);
+                Dv[1] = make_float4(dz[0].y, dz[1].y, dz[2].y, dz[3].y);
+                Dv[2] = make_float4(dz[0].z, dz[1].z, dz[2].z, dz[3].z);
+                Dv[3] = make_float4(dz[0].w, dz[1].w, dz[2].w, dz[3].w);
+            }
+        }
     }
-}
-
-// dA[r][i] = sum_o dZ[r][o] W[o][i]
-__global__ void __launch_bounds__(128) k_dense_bwd(int n, int in, int out, const float *__restrict__ dZ,
-                                                   const __nv_bfloat16 *__restrict__ W, float *__restrict__ dA) {
-    extern __shared__ float sm[];
-    float *Ws = sm;                    // [out][in]
-    float *Ds = sm + in * out;         // [TROWS][out]
-    const int r0 = blockIdx.x * TROWS;
-    for (int k = threadIdx.x; k < in * out; k += blockDim.x) Ws[k] = __bfloat162float(W[k]);
-    const int rows = min(TROWS, n - r0);
-    for (int k = threadIdx.x; k < rows * out; k += blockDim.x) Ds[k] = dZ[(size_t)r0 * out + k];
-    __syncthreads();
-    const int i = threadIdx.x;
-    if (i >= in) return;
-    for (int r = 0; r < rows; ++r) {
-        float acc = 0.0f;
-        for (int o = 0; o < out; ++o) acc = fmaf(Ds[r * out + o], Ws[o * in + i], acc);
-        dA[(size_t)(r0 + r) * in + i] = acc;
-    }
-}
-
-__global__ void k_gelu_bwd(size_t n, const float *__restrict__ Z, float *__restrict__ dA) {
-    const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n) dA[k] *= gelu_grad(Z[k]);
-}
-
-// gW[o][i] = sum_r dZ[r][o] A[r][i] (thread per weight), gb[o] = sum_r dZ[r][o] (i == in)
-__global__ void k_weight_grad(int n, int in, int out, const float *__restrict__ dZ, const float *__restrict__ A,
-                              float *__restrict__ gW, float *__restrict__ gb) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= out * (in + 1)) return;
-    const int o = k / (in + 1), i = k % (in + 1);
-    float acc = 0.0f;
-    if (i < in) {
-        for (int r = 0; r < n; ++r) acc = fmaf(dZ[(size_t)r * out + o], A[(size_t)r * in + i], acc);
-        gW[o * in + i] = acc;
-    } else {
-        for (int r = 0; r < n; ++r) acc += dZ[(size_t)r * out + o];
-        gb[o] = acc;
-    }
-}
-
-// loss partial per CTA and dY = 2 (Y - T) / (n * m)
-__global__ void __launch_bounds__(256) k_mse(int n, int m, const float *__restrict__ Y, const float *__restrict__ T,
-                                             float *__restrict__ dY, double *__restrict__ part) {
-    __shared__ double buf[256];
-    const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    double l = 0.0;
-    if (k < (size_t)n * m) {
-        const float d = Y[k] - T[k];
-        dY[k] = 2.0f * d / (float)((double)n * m);
-        l = (double)d * d;
-    }
-    buf[threadIdx.x] = l;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) buf[threadIdx.x] += buf[threadIdx.x + w];
+    if constexpr (TRAIN) {
+        __shared__ double part[WARPS];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+        if (lane == 0) part[warp] = loss;
         __syncthreads();
+        if (threadIdx.x == 0) {
+            double sum = 0.0;
+            for (int w = 0; w < WARPS; ++w) sum += part[w];
+            lpart[blockIdx.x] = sum;
+        }
     }
-    if (threadIdx.x == 0) part[blockIdx.x] = buf[0];
+}
+
+// dW = dZ^T A and db = sum dZ of the rows [split chunk, + chunk) of all layers:
+// block = (64 x 64 tile of one layer's weights, split); part [split][MLP_NW] laid out as the
+// parameters.  256 threads, 4 x 4 weights each, rows staged 16 at a time.
+constexpr int WG_TILES = 12;      // 128 x 16: 2, 128 x 128: 4 each, 12 x 128: 2
+struct GradArgs {
+    const float *A[MLP_LAYERS], *D[MLP_LAYERS];
+};
+__global__ void __launch_bounds__(256) k_weight_grad(int n, int chunk, GradArgs g, float *__restrict__ part) {
+    constexpr int KB = 16;
+    __shared__ __align__(16) float sA[KB][64], sD[KB][64];
+    const int t = blockIdx.x;
+    const int l = t < 2 ? 0 : t < 6 ? 1 : t < 10 ? 2 : 3, u = t < 2 ? t : t < 6 ? t - 2 : t < 10 ? t - 6 : t - 10;
+    const int o0 = l == 0 ? u * 64 : l == 3 ? 0 : (u >> 1) * 64, i0 = l == 0 ? 0 : l == 3 ? u * 64 : (u & 1) * 64;
+    const int in = layer_in(l), out = layer_out(l);
+    const float *__restrict__ A = g.A[l], *__restrict__ Dz = g.D[l];
+    const int r0 = blockIdx.y * chunk, r1 = min(n, r0 + chunk);
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;       // inputs 4 tx.., outputs 4 ty..
+    float2 acc[4][2];
+    float bias[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int a = 0; a < 4; ++a) acc[a][0] = acc[a][1] = make_float2(0.0f, 0.0f);
+    const int lr = threadIdx.x >> 4, lc = (threadIdx.x & 15) * 4;  // staging: row, first of four columns
+    for (int r = r0; r < r1; r += KB) {
+        float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), d = a;
+        if (r + lr < r1) {
+            if (i0 + lc < in) a = *reinterpret_cast<const float4 *>(A + (size_t)(r + lr) * in + i0 + lc);
+            if (o0 + lc < out) d = *reinterpret_cast<const float4 *>(Dz + (size_t)(r + lr) * out + o0 + lc);
+        }
+        __syncthreads();
+        *reinterpret_cast<float4 *>(&sA[lr][lc]) = a;
+        *reinterpret_cast<float4 *>(&sD[lr][lc]) = d;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < KB; ++k) {
+            const float4 x = *reinterpret_cast<const float4 *>(&sA[k][4 * tx]), y = *reinterpret_cast<const float4 *>(&sD[k][4 * ty]);
+            const float yy[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+            for (int o = 0; o < 4; ++o) {
+                const float2 dd = make_float2(yy[o], yy[o]);
+                acc[o][0] = __ffma2_rn(dd, make_float2(x.x, x.y), acc[o][0]);
+                acc[o][1] = __ffma2_rn(dd, make_float2(x.z, x.w), acc[o][1]);
+                bias[o] += yy[o];
+            }
+        }
+    }
+    float *p = part + (size_t)blockIdx.y * MLP_NW + (l == 0 ? w_off(0) : l == 1 ? w_off(1) : l == 2 ? w_off(2) : w_off(3));
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+        const int oo = o0 + 4 * ty + o;
+        if (oo >= out) continue;
+        if (i0 + 4 * tx < in)
+            *reinterpret_cast<float4 *>(p + (size_t)oo * in + i0 + 4 * tx) =
+                make_float4(acc[o][0].x, acc[o][0].y, acc[o][1].x, acc[o][1].y);
+        if (i0 == 0 && tx == 0) p[(size_t)out * in + oo] = bias[o];
+    }
+}
+
+// g = sum of the splits' tiles; block 0 also sums the loss partials into lpart[0]
+__global__ void __launch_bounds__(128) k_grad_reduce(int splits, const float *__restrict__ part, float *__restrict__ g,
+                                                     int n_loss, double *__restrict__ lpart, double scale) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < MLP_NW) {
+        float s = 0.0f;
+        for (int q = 0; q < splits; ++q) s += part[(size_t)q * MLP_NW + k];
+        g[k] = s;
+    }
+    if (blockIdx.x != 0 || threadIdx.x >= 32) return;
+    double x = 0.0;
+    for (int q = threadIdx.x; q < n_loss; q += 32) x += lpart[q];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if (threadIdx.x == 0) lpart[n_loss] = x * scale;
 }
 
 __global__ void k_adam(size_t n, float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m1,
@@ -257,72 +453,49 @@ __global__ void k_hot_from_cells(MacroGeom g, const float *__restrict__ Yc, doub
 namespace gsis {
 
 namespace {
-int layer_in(int l) { return l == 0 ? MLP_IN : MLP_H; }
-int layer_out(int l) { return l == MLP_LAYERS - 1 ? MLP_OUT : MLP_H; }
-size_t w_off(int l) {
-    size_t o = 0;
-    for (int k = 0; k < l; ++k) o += (size_t)layer_out(k) * layer_in(k) + layer_out(k);
-    return o;
+
+// One CTA per SM at most: 4 warps (16 rows a tile) while that keeps every SM busy, else 8.
+template <bool TRAIN>
+cudaError_t mlp_pass(cudaStream_t s, MlpDev &d, int n, int *ctas) {
+    const int rows4 = 4 * PR, n4 = (n + rows4 - 1) / rows4;
+    auto run = [&](auto kern, int warps) {
+        const int tiles = (n + warps * PR - 1) / (warps * PR), smem = pass_smem(warps, TRAIN);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        *ctas = std::min(tiles, MLP_CTAS);
+        kern<<<*ctas, 32 * warps, smem, s>>>(n, static_cast<const __nv_bfloat16 *>(d.pb), d.p, d.act[0],
+                                             d.act[MLP_LAYERS], d.act[1], d.act[2], d.act[3], d.T, d.dZ[0], d.dZ[1],
+                                             d.dZ[2], d.dZ[3], d.lpart);
+        return cudaGetLastError();
+    };
+    return n4 <= MLP_CTAS ? run(k_mlp_pass<4, TRAIN>, 4) : run(k_mlp_pass<8, TRAIN>, 8);
 }
+
 }  // namespace
 
+// act[0] (standardised) -> act[4]
 cudaError_t launch_mlp_forward(cudaStream_t s, MlpDev &d, int n) {
-    const __nv_bfloat16 *pb = static_cast<const __nv_bfloat16 *>(d.pb);
-    for (int l = 0; l < MLP_LAYERS; ++l) {
-        const int in = layer_in(l), out = layer_out(l);
-        const size_t smem = (size_t)(in * out + TROWS * in) * sizeof(float);
-        const int nb = (n + TROWS - 1) / TROWS;
-        const size_t wo = w_off(l);
-        cudaError_t e;
-        if (l < MLP_LAYERS - 1) {
-            if ((e = cudaFuncSetAttribute(k_dense_fwd<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
-                return e;
-            k_dense_fwd<true><<<nb, 128, smem, s>>>(n, in, out, d.act[l], pb + wo, d.p + wo + (size_t)out * in,
-                                                    d.pre[l], d.act[l + 1]);
-        } else {
-            if ((e = cudaFuncSetAttribute(k_dense_fwd<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
-                return e;
-            k_dense_fwd<false><<<nb, 128, smem, s>>>(n, in, out, d.act[l], pb + wo, d.p + wo + (size_t)out * in,
-                                                     d.pre[l], d.act[l + 1]);
-        }
-        if ((e = cudaGetLastError())) return e;
-    }
-    return cudaSuccess;
+    int ctas = 0;
+    return mlp_pass<false>(s, d, n, &ctas);
 }
 
-int mlp_loss_parts(int n) { return (int)(((size_t)n * MLP_OUT + 255) / 256); }
-
+// act[0] and T -> gradients g and the mean squared error in lpart[d.loss_at]
 cudaError_t launch_mlp_loss_backward(cudaStream_t s, MlpDev &d, int n) {
-    const __nv_bfloat16 *pb = static_cast<const __nv_bfloat16 *>(d.pb);
-    const int nparts = mlp_loss_parts(n);
-    // dY into dA[0] (width MLP_OUT)
-    k_mse<<<nparts, 256, 0, s>>>(n, MLP_OUT, d.act[MLP_LAYERS], d.T, d.dA[0], d.lpart);
-    cudaError_t e = cudaGetLastError();
+    int ctas = 0;
+    cudaError_t e = mlp_pass<true>(s, d, n, &ctas);
     if (e) return e;
-    int cur = 0;
-    for (int l = MLP_LAYERS - 1; l >= 0; --l) {
-        const int in = layer_in(l), out = layer_out(l);
-        const size_t wo = w_off(l);
-        // dZ = dA (output layer) or dA * GELU'(pre) (hidden layers), in place in dA[cur]
-        if (l < MLP_LAYERS - 1) {
-            const size_t cnt = (size_t)n * out;
-            k_gelu_bwd<<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(cnt, d.pre[l], d.dA[cur]);
-            if ((e = cudaGetLastError())) return e;
-        }
-        const int nw = out * (in + 1);
-        k_weight_grad<<<(nw + 127) / 128, 128, 0, s>>>(n, in, out, d.dA[cur], d.act[l], d.g + wo,
-                                                       d.g + wo + (size_t)out * in);
-        if ((e = cudaGetLastError())) return e;
-        if (l > 0) {
-            const size_t smem = (size_t)(in * out + TROWS * out) * sizeof(float);
-            if ((e = cudaFuncSetAttribute(k_dense_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
-                return e;
-            k_dense_bwd<<<(n + TROWS - 1) / TROWS, 128, smem, s>>>(n, in, out, d.dA[cur], pb + wo, d.dA[1 - cur]);
-            if ((e = cudaGetLastError())) return e;
-            cur = 1 - cur;
-        }
+    const int splits = std::min(MLP_SPLITS, (n + 127) / 128), chunk = (n + splits - 1) / splits;
+    GradArgs g;
+    for (int l = 0; l < MLP_LAYERS; ++l) {
+        g.A[l] = d.act[l];
+        g.D[l] = d.dZ[l];
     }
-    return cudaSuccess;
+    k_weight_grad<<<dim3(WG_TILES, splits), 256, 0, s>>>(n, chunk, g, d.gpart);
+    if ((e = cudaGetLastError())) return e;
+    k_grad_reduce<<<(MLP_NW + 127) / 128, 128, 0, s>>>(splits, d.gpart, d.g, ctas, d.lpart,
+                                                       1.0 / ((double)n * MLP_OUT));
+    d.loss_at = ctas;
+    return cudaGetLastError();
 }
 
 cudaError_t launch_mlp_adam(cudaStream_t s, MlpDev &d, float lr) {
