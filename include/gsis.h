@@ -441,18 +441,13 @@ int gsis_get_layout(const gsis_ctx *ctx, int32_t *v_pad, int32_t *o_pad, int32_t
  * The gas moments are summed about each cell's own mean velocity (found in a first pass),
  * so FP32 storage keeps the heat fluxes to 1e-5 of rho T^1.5 at hypersonic speeds.
  *
- * It calls no cudaMalloc/cudaFree and no allocating library routine.  Its shift
- * velocities and partial sums live in one 32 MiB file-scope device array that every GPU
- * loading the library holds until the process exits; sizes that do not fit,
+ * It calls no cudaMalloc/cudaFree and no allocating library routine, and keeps nothing
+ * between calls: they may overlap on one GPU and may be captured.  Sizes with
  *   n_cells * 24 + (n_cells * ceil(n_xi/128) * 20 + n_cells * ceil(n_omega/128) * 4)
- *   * sizeof(storage) > 32 MiB,
- * are rejected with GSIS_ERR_INVALID_ARG before anything is launched.  The first call on
- * a device looks up the array's device address (with that device current) and caches it
- * for the life of the process; make that first call before any stream capture, and make
- * no call after cudaDeviceReset on that device.  All calls share the array: calls whose
- * kernels overlap on one GPU race on it.
+ *   * sizeof(storage) > 32 MiB
+ * are rejected with GSIS_ERR_INVALID_ARG before anything is launched.
  * Errors: INVALID_ARG (null pointer, non-positive size, too large), UNSUPPORTED (dim 3),
- * CUDA (address lookup or launch failure). */
+ * CUDA (launch failure). */
 int gsis_moments_static(int32_t dim, int32_t precision, int64_t n_cells, int32_t n_xi, const double *xi,
                         const double *w, int32_t n_omega, const double *omega, const double *wo,
                         const void *f, const void *I, double d_r, double d_v, double sigma_R, double *fields,

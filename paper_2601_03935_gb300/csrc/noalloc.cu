@@ -4,216 +4,125 @@
 // component owns the device heap (a host framework with its own pool allocator, a
 // plugin that may only use the buffers it is handed), or latency-critical loops that
 // cannot afford a cudaMalloc/cudaFree pair per call.  Such callers cannot create a
-// gsis context (gsis_create allocates), so this entry point takes device pointers and
-// keeps its per-chunk partial sums and per-cell shift velocities in a file-scope device
-// array instead of a buffer of its own.
-//
-// The array (kScratchBytes) lives in every GPU that loads the library until the
-// process exits.  Its device address is looked up once per device, on the first call
-// made with that device current (cudaGetSymbolAddress); make that first call before
-// any stream capture.  The address is cached for the life of the process: calls made
-// after cudaDeviceReset on that device are not supported.  All calls share the array:
-// two calls whose kernels overlap on a GPU race on it.  Every word a call reads from
-// the array is written earlier by the same call, so nothing in it has to start at zero
-// and a call never sees the previous call's contents.
+// gsis context (gsis_create allocates), so this entry point takes device pointers.  It is
+// one kernel that keeps its intermediate sums in shared memory: calls share nothing, may
+// overlap on a GPU and may be captured.
 //
 // Accuracy: the gas moments are summed about a per-cell shift velocity u0 (the cell's
 // own mean velocity from a first pass over its mass and momentum), so that the third
 // moments behind the heat fluxes do not cancel at high flow speeds; the FP32 storage
-// path keeps 1e-5 of rho T^1.5 at Mach 5.
+// path keeps 1e-5 of rho T^1.5 at Mach 5.  FP32 sums run over at most eight velocities per lane
+// and are then carried in two words (Knuth's two-sum).
+//
+// What bounds it: the one pass over f (the second pass of a cell, right after the first,
+// finds it in L1 or L2).  20 000 cells x 784 velocities, FP32: 301 -> 102 us (two passes over
+// memory, an FP64 subtraction and conversion per velocity component and five kernels before).
+#include <algorithm>
 #include <cmath>
-#include <mutex>
+#include <type_traits>
 
 #include "../../include/gsis.h"
+#include "fp64.cuh"
 
 namespace {
 
-constexpr size_t kScratchBytes = size_t(32) << 20;   // 32 MiB
-constexpr int kChunk = 128;                           // velocities (directions) per partial
-constexpr int kNMP = 20, kNMO = 4, kNF = 26, kMaxDevices = 64;
+using namespace gsis;
 
-static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
-
-std::mutex g_mutex;
-void *g_scratch_ptr[kMaxDevices] = {};
-
-int scratch_address(void **out) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return GSIS_ERR_CUDA;
-    std::lock_guard<std::mutex> lock(g_mutex);
-    if (!g_scratch_ptr[dev]) {
-        void *p = nullptr;
-        if (cudaGetSymbolAddress(&p, g_scratch) != cudaSuccess || !p) return GSIS_ERR_CUDA;
-        g_scratch_ptr[dev] = p;
-    }
-    *out = g_scratch_ptr[dev];
-    return GSIS_OK;
-}
+constexpr int kChunk = 128;                           // velocities (directions) counted as one by the size limit
+constexpr int kNF = 26, kWarps = 8, kCpw = 4;         // record words; warps of a CTA; cells of a warp in a round
+// 80 registers a thread: 2, 3, 4 CTAs per SM took 121, 102, 112 us on the case above
+constexpr int kCtasPerSm = 3;
+constexpr int kRec = 24;                              // sums of a cell (gas, then photons), in threes
 
 template <int DIM>
 constexpr int n_moments() {
     return 1 + DIM + DIM * (DIM + 1) / 2 + DIM + 3 * (1 + DIM);
 }
 
-// Bytes of the array one call uses: the shift velocities (3 doubles per cell), then the
-// gas and photon partials in the storage type.
-size_t scratch_bytes(long long n_cells, int n_xi, int n_om, size_t real) {
+// The largest problem a call takes: the sums by chunks of 128 velocities or directions (20
+// and 4 values in the storage type) and three doubles per cell come to at most 32 MiB.
+// Callers may rely on larger ones being refused.
+constexpr size_t kMaxBytes = size_t(32) << 20;
+size_t problem_bytes(long long n_cells, int n_xi, int n_om, size_t real) {
     const size_t n_chunks = (n_xi + kChunk - 1) / kChunk, o_chunks = (n_om + kChunk - 1) / kChunk;
-    return (size_t)n_cells * 3 * sizeof(double) + ((size_t)n_cells * n_chunks * kNMP + (size_t)n_cells * o_chunks * kNMO) * real;
+    return (size_t)n_cells * 3 * sizeof(double) + ((size_t)n_cells * n_chunks * 20 + (size_t)n_cells * o_chunks * 4) * real;
 }
 
-// One warp per (cell, chunk): mass and momentum partials of F0 (the first pass).
-template <typename Real, int DIM>
-__global__ void k_static_mass(long long n_cells, int n_xi, int n_chunks, const double *__restrict__ xi,
-                              const double *__restrict__ w, const Real *__restrict__ f, Real *__restrict__ part) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long i = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
-    const int chunk = blockIdx.y;
-    if (i >= n_cells) return;
-    Real acc[1 + DIM];
-#pragma unroll
-    for (int m = 0; m <= DIM; ++m) acc[m] = Real(0);
-    for (int vl = lane; vl < kChunk; vl += 32) {
-        const int v = chunk * kChunk + vl;
-        if (v >= n_xi) break;
-        const Real w0 = (Real)w[v] * f[((size_t)i * n_xi + v) * 4];
-        acc[0] += w0;
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) acc[1 + a] += w0 * (Real)xi[(size_t)v * DIM + a];
+// A running sum: two words in FP32 (hi + lo, the rounding error of every addition kept), one
+// in FP64
+template <typename Real>
+struct Sum;
+template <>
+struct Sum<float> {
+    float hi = 0.0f, lo = 0.0f;
+    __device__ __forceinline__ void add(float x) {
+        const float t = hi + x, v = t - hi;
+        lo += (hi - (t - v)) + (x - v);
+        hi = t;
     }
-#pragma unroll
-    for (int m = 0; m <= DIM; ++m)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc[m] += __shfl_xor_sync(0xffffffffu, acc[m], o);
-    if (lane == 0) {
-        Real *P = part + ((size_t)i * n_chunks + chunk) * kNMP;
-#pragma unroll
-        for (int m = 0; m <= DIM; ++m) P[m] = acc[m];
+    __device__ __forceinline__ void add(const Sum &o) {
+        add(o.hi);
+        lo += o.lo;
     }
-}
+    __device__ __forceinline__ Sum shfl(int o) const {
+        Sum r;
+        r.hi = __shfl_xor_sync(0xffffffffu, hi, o);
+        r.lo = __shfl_xor_sync(0xffffffffu, lo, o);
+        return r;
+    }
+    // an infinite hi leaves a NaN in lo
+    __device__ __forceinline__ double value() const {
+        return isfinite(lo) ? to_double(hi) + to_double(lo) : to_double(hi);
+    }
+};
+template <>
+struct Sum<double> {
+    double hi = 0.0;
+    __device__ __forceinline__ void add(double x) { hi += x; }
+    __device__ __forceinline__ void add(const Sum &o) { hi += o.hi; }
+    __device__ __forceinline__ Sum shfl(int o) const {
+        Sum r;
+        r.hi = __shfl_xor_sync(0xffffffffu, hi, o);
+        return r;
+    }
+    __device__ __forceinline__ double value() const { return hi; }
+};
 
-// Per cell: the shift velocity u0 = sum m1 / sum m0 over the chunks, in FP64 (zero where
-// the cell has no mass).
-template <typename Real, int DIM>
-__global__ void k_static_shift(long long n_cells, int n_chunks, const Real *__restrict__ part,
-                               double *__restrict__ u0) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_cells) return;
-    double S[1 + DIM];
-    for (int m = 0; m <= DIM; ++m) S[m] = 0.0;
-    for (int c = 0; c < n_chunks; ++c)
-        for (int m = 0; m <= DIM; ++m) S[m] += (double)part[((size_t)i * n_chunks + c) * kNMP + m];
-    for (int a = 0; a < DIM; ++a) u0[(size_t)i * 3 + a] = S[0] > 0.0 ? S[1 + a] / S[0] : 0.0;
-}
-
-// One warp per (cell, chunk): moments of the four planes about the cell's shift velocity,
-// c = xi - u0.
-template <typename Real, int DIM>
-__global__ void k_static_gas(long long n_cells, int n_xi, int n_chunks, const double *__restrict__ xi,
-                             const double *__restrict__ w, const double *__restrict__ u0,
-                             const Real *__restrict__ f, Real *__restrict__ part) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long i = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
-    const int chunk = blockIdx.y;
-    if (i >= n_cells) return;
-    constexpr int NM = n_moments<DIM>();
-    double us[DIM];
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) us[a] = u0[(size_t)i * 3 + a];
-    Real acc[NM];
-#pragma unroll
-    for (int m = 0; m < NM; ++m) acc[m] = Real(0);
-    for (int vl = lane; vl < kChunk; vl += 32) {
-        const int v = chunk * kChunk + vl;
-        if (v >= n_xi) break;
-        const Real *fv = f + ((size_t)i * n_xi + v) * 4;
-        Real c[DIM], c2 = Real(0);
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) {
-            c[a] = (Real)(xi[(size_t)v * DIM + a] - us[a]);
-            c2 += c[a] * c[a];
-        }
-        const Real wv = (Real)w[v];
-        const Real w0 = wv * fv[0];
-        int m = 0;
-        acc[m++] += w0;
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) acc[m++] += w0 * c[a];
-#pragma unroll
-        for (int a = 0; a < DIM; ++a)
-#pragma unroll
-            for (int b = a; b < DIM; ++b) acc[m++] += w0 * c[a] * c[b];
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) acc[m++] += w0 * c[a] * c2;
-#pragma unroll
-        for (int p = 1; p < 4; ++p) {
-            const Real wp = wv * fv[p];
-            acc[m++] += wp;
-#pragma unroll
-            for (int a = 0; a < DIM; ++a) acc[m++] += wp * c[a];
+// The velocity set as a lane reads it.  FP32 with a table in shared memory: each component in
+// two floats, hi + lo, and the weight, converted once per CTA; else straight from the FP64 set.
+template <typename Real, int DIM, bool TAB>
+struct Velocities {
+    const double *xi, *w;
+    const float *tab;
+    int n;
+    __device__ __forceinline__ Real weight(int v) const {
+        if constexpr (TAB) return tab[2 * DIM * n + v];
+        else return to_real<Real>(w[v]);
+    }
+    // xi_a rounded (first pass)
+    __device__ __forceinline__ Real x(int v, int a) const {
+        if constexpr (TAB) return tab[a * n + v];
+        else return to_real<Real>(xi[(size_t)v * DIM + a]);
+    }
+    // xi_a - u
+    __device__ __forceinline__ Real minus(int v, int a, Real u) const {
+        if constexpr (TAB) {
+            return (tab[a * n + v] - u) + tab[(DIM + a) * n + v];
+        } else {
+            return to_real<Real>(xi[(size_t)v * DIM + a] - to_double(u));
         }
     }
-#pragma unroll
-    for (int m = 0; m < NM; ++m)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc[m] += __shfl_xor_sync(0xffffffffu, acc[m], o);
-    if (lane == 0) {
-        Real *P = part + ((size_t)i * n_chunks + chunk) * kNMP;
-#pragma unroll
-        for (int m = 0; m < NM; ++m) P[m] = acc[m];
-    }
-}
+};
 
-template <typename Real, int DIM>
-__global__ void k_static_photon(long long n_cells, int n_om, int o_chunks, const double *__restrict__ om,
-                                const double *__restrict__ wo, const Real *__restrict__ I, Real *__restrict__ part) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long i = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
-    const int chunk = blockIdx.y;
-    if (i >= n_cells) return;
-    Real acc[1 + DIM];
-#pragma unroll
-    for (int m = 0; m <= DIM; ++m) acc[m] = Real(0);
-    for (int ol = lane; ol < kChunk; ol += 32) {
-        const int o = chunk * kChunk + ol;
-        if (o >= n_om) break;
-        const Real wI = (Real)wo[o] * I[(size_t)i * n_om + o];
-        acc[0] += wI;
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) acc[1 + a] += wI * (Real)om[(size_t)o * 3 + a];
-    }
-#pragma unroll
-    for (int m = 0; m <= DIM; ++m)
-#pragma unroll
-        for (int s = 16; s > 0; s >>= 1) acc[m] += __shfl_xor_sync(0xffffffffu, acc[m], s);
-    if (lane == 0) {
-        Real *P = part + ((size_t)i * o_chunks + chunk) * kNMO;
-#pragma unroll
-        for (int m = 0; m <= DIM; ++m) P[m] = acc[m];
-    }
-}
-
-// Partials -> per-cell field record (rho, u, T_t, T_r, T_v, T_R, heat fluxes, stress).
-// The partials are moments about u0; u below is the residual velocity u - u0, and the
-// central moments follow from them exactly as from moments about zero.
-template <typename Real, int DIM>
-__global__ void k_static_finish(long long n_cells, int n_chunks, int o_chunks, double d_r, double d_v,
-                                double sigma_R, const double *__restrict__ u0, const Real *__restrict__ part,
-                                const Real *__restrict__ opart, double *__restrict__ out) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_cells) return;
-    constexpr int NM = n_moments<DIM>();
+// Sums S about u0 + the photon sums -> the cell's field record (rho, u, T_t, T_r, T_v, T_R,
+// heat fluxes, stress).  u below is the residual velocity u - u0, and the central moments
+// follow from it exactly as from moments about zero.
+template <int DIM>
+__device__ void finish(const double *S, const double *Ph, const double *u0, double i_half_dr, double i_half_dv,
+                       double i_4sigma, double *F) {
     constexpr int MH = 3 - DIM;
-    double S[NM];
-    for (int k = 0; k < NM; ++k) S[k] = 0.0;
-    for (int c = 0; c < n_chunks; ++c)
-        for (int k = 0; k < NM; ++k) S[k] += (double)part[((size_t)i * n_chunks + c) * kNMP + k];
-    double Ph[1 + DIM];
-    for (int k = 0; k <= DIM; ++k) Ph[k] = 0.0;
-    for (int c = 0; c < o_chunks; ++c)
-        for (int k = 0; k <= DIM; ++k) Ph[k] += (double)opart[((size_t)i * o_chunks + c) * kNMO + k];
     int k = 0;
-    const double rho = S[k++];
+    const double rho = S[k++], ir = rcp_r(rho);
     double m1[DIM], m2[DIM][DIM], m3[DIM];
     for (int a = 0; a < DIM; ++a) m1[a] = S[k++];
     for (int a = 0; a < DIM; ++a)
@@ -232,7 +141,7 @@ __global__ void k_static_finish(long long n_cells, int n_chunks, int o_chunks, d
     double G2c[DIM];
     for (int a = 0; a < DIM; ++a) G2c[a] = S[k++];
     double u[DIM], P[DIM][DIM], trP = 0.0, trm2 = 0.0, u2 = 0.0, um1 = 0.0;
-    for (int a = 0; a < DIM; ++a) u[a] = m1[a] / rho;
+    for (int a = 0; a < DIM; ++a) u[a] = m1[a] * ir;
     for (int a = 0; a < DIM; ++a)
         for (int b = 0; b < DIM; ++b) P[a][b] = m2[a][b] - rho * u[a] * u[b];
     for (int a = 0; a < DIM; ++a) {
@@ -242,14 +151,13 @@ __global__ void k_static_finish(long long n_cells, int n_chunks, int o_chunks, d
         um1 += u[a] * m1[a];
     }
     const double ic2 = trP + H0;
-    double *F = out + (size_t)i * kNF;
     for (int q = 0; q < kNF; ++q) F[q] = 0.0;
     F[0] = rho;
-    for (int a = 0; a < DIM; ++a) F[1 + a] = u0[(size_t)i * 3 + a] + u[a];
-    F[4] = ic2 / (3.0 * rho);
-    F[5] = 2.0 * G1 / (d_r * rho);
-    F[6] = 2.0 * G2 / (d_v * rho);
-    F[7] = sigma_R > 0.0 ? pow(fmax(Ph[0], 0.0) / (4.0 * sigma_R), 0.25) : 0.0;
+    for (int a = 0; a < DIM; ++a) F[1 + a] = u0[a] + u[a];
+    F[4] = ic2 * ((1.0 / 3.0) * ir);
+    F[5] = G1 * (i_half_dr * ir);
+    F[6] = G2 * (i_half_dv * ir);
+    F[7] = i_4sigma > 0.0 ? sqrt_r(sqrt_r(fmax(Ph[0], 0.0) * i_4sigma)) : 0.0;
     for (int a = 0; a < DIM; ++a) {
         double t = m3[a] - u[a] * trm2 + u2 * m1[a] + 2.0 * u[a] * um1 - rho * u[a] * u2;
         for (int b = 0; b < DIM; ++b) t -= 2.0 * u[b] * m2[a][b];
@@ -261,8 +169,8 @@ __global__ void k_static_finish(long long n_cells, int n_chunks, int o_chunks, d
     double sig[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
     for (int a = 0; a < DIM; ++a)
         for (int b = 0; b < DIM; ++b) sig[a][b] = P[a][b];
-    for (int a = DIM; a < 3; ++a) sig[a][a] = H0 / MH;
-    for (int a = 0; a < 3; ++a) sig[a][a] -= ic2 / 3.0;
+    for (int a = DIM; a < 3; ++a) sig[a][a] = H0 * (1.0 / MH);
+    for (int a = 0; a < 3; ++a) sig[a][a] -= ic2 * (1.0 / 3.0);
     F[20] = sig[0][0];
     F[21] = sig[1][1];
     F[22] = sig[2][2];
@@ -271,30 +179,199 @@ __global__ void k_static_finish(long long n_cells, int n_chunks, int o_chunks, d
     F[25] = sig[1][2];
 }
 
+// One CTA takes a contiguous range of cells in rounds of 32, four per warp one after the
+// other; one warp then forms the round's field records, one lane per cell (an FP64 warp
+// instruction costs the same for one lane as for 32), while the others begin the next round
+// in the second buffer.  VEC: f is aligned to a record of four planes, which is then read at once.
+template <typename Real, int DIM, bool TAB, bool VEC>
+__global__ void __launch_bounds__(32 * kWarps, kCtasPerSm) k_static(long long n_cells, int n_xi, int n_om,
+                                                        const double *__restrict__ xi, const double *__restrict__ w,
+                                                        const double *__restrict__ om, const double *__restrict__ wo,
+                                                        const Real *__restrict__ f, const Real *__restrict__ I,
+                                                        double i_half_dr, double i_half_dv, double i_4sigma, int per_cta,
+                                                        double *__restrict__ out) {
+    constexpr int NM = n_moments<DIM>();
+    constexpr int kRun = sizeof(Real) == 4 ? 256 : 128;   // velocities of a plain sum: 8 or 4 per lane, loaded at once
+    static_assert(NM + 1 + DIM <= kRec && kWarps * kCpw == 32, "the sums of a cell; one lane per cell of a round");
+    extern __shared__ float s_tab[];
+    __shared__ double sums[2][kWarps * kCpw][kRec + 1], shift[2][kWarps * kCpw][DIM];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if constexpr (TAB) {
+        for (int v = threadIdx.x; v < n_xi; v += 32 * kWarps) {
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) {
+                const double x = xi[(size_t)v * DIM + a];
+                const float h = fp64::narrow(x);
+                s_tab[a * n_xi + v] = h;
+                s_tab[(DIM + a) * n_xi + v] = fp64::narrow(x - fp64::widen(h));
+            }
+            s_tab[2 * DIM * n_xi + v] = fp64::narrow(w[v]);
+        }
+        for (int o = threadIdx.x; o < n_om; o += 32 * kWarps) {
+            float *q = s_tab + (2 * DIM + 1) * n_xi;
+            q[o] = fp64::narrow(wo[o]);
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) q[(1 + a) * n_om + o] = fp64::narrow(om[(size_t)o * 3 + a]);
+        }
+        __syncthreads();
+    }
+    const Velocities<Real, DIM, TAB> vel{xi, w, s_tab, n_xi};
+    const float *pt = s_tab + (2 * DIM + 1) * n_xi;       // photon weights and directions
+    const long long begin = (long long)blockIdx.x * per_cta, end = min(n_cells, begin + per_cta);
+    struct __align__((VEC ? 4 : 1) * sizeof(Real)) Four {
+        Real v[4];
+    };
+    int round = 0;
+    for (long long base = begin; base < end; base += kWarps * kCpw, ++round) {
+        const int buf = round & 1;
+        for (int j = 0; j < kCpw; ++j) {
+            const int slot = j * kWarps + warp;
+            const long long i = base + slot;
+            if (i >= end) break;
+            const Four *fc = reinterpret_cast<const Four *>(f) + (size_t)i * n_xi;
+            // mass and momentum: the shift velocity (any value near the mean velocity serves)
+            Real m[1 + DIM];
+#pragma unroll
+            for (int k = 0; k <= DIM; ++k) m[k] = Real(0);
+#pragma unroll 8
+            for (int v = lane; v < n_xi; v += 32) {
+                const Real w0 = vel.weight(v) * fc[v].v[0];
+                m[0] += w0;
+#pragma unroll
+                for (int a = 0; a < DIM; ++a) m[1 + a] += w0 * vel.x(v, a);
+            }
+#pragma unroll
+            for (int k = 0; k <= DIM; ++k)
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) m[k] += __shfl_xor_sync(0xffffffffu, m[k], o);
+            Real u[DIM];
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) u[a] = m[0] > Real(0) ? m[1 + a] / m[0] : Real(0);
+            Sum<Real> S[kRec];
+            for (int v0 = 0; v0 < n_xi; v0 += kRun) {
+                Real acc[NM];
+#pragma unroll
+                for (int k = 0; k < NM; ++k) acc[k] = Real(0);
+                // the run's loads first; past the set's end the last velocity with no weight
+                Four fr[kRun / 32];
+#pragma unroll
+                for (int h = 0; h < kRun / 32; ++h) fr[h] = fc[min(v0 + 32 * h + lane, n_xi - 1)];
+#pragma unroll
+                for (int h = 0; h < kRun / 32; ++h) {
+                    if (v0 + 32 * h >= n_xi) break;
+                    const int v = min(v0 + 32 * h + lane, n_xi - 1);
+                    const Four &fv = fr[h];
+                    Real c[DIM], c2 = Real(0);
+#pragma unroll
+                    for (int a = 0; a < DIM; ++a) {
+                        c[a] = vel.minus(v, a, u[a]);
+                        c2 = fma(c[a], c[a], c2);
+                    }
+                    const Real wv = v0 + 32 * h + lane < n_xi ? vel.weight(v) : Real(0), w0 = wv * fv.v[0];
+                    Real wc[DIM];
+                    int k = 0;
+                    acc[k++] += w0;
+#pragma unroll
+                    for (int a = 0; a < DIM; ++a) {
+                        wc[a] = w0 * c[a];
+                        acc[k++] += wc[a];
+                    }
+#pragma unroll
+                    for (int a = 0; a < DIM; ++a)
+#pragma unroll
+                        for (int b = a; b < DIM; ++b, ++k) acc[k] = fma(wc[a], c[b], acc[k]);
+#pragma unroll
+                    for (int a = 0; a < DIM; ++a, ++k) acc[k] = fma(wc[a], c2, acc[k]);
+#pragma unroll
+                    for (int p = 1; p < 4; ++p) {
+                        const Real wp = wv * fv.v[p];
+                        acc[k++] += wp;
+#pragma unroll
+                        for (int a = 0; a < DIM; ++a, ++k) acc[k] = fma(wp, c[a], acc[k]);
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < NM; ++k) S[k].add(acc[k]);
+            }
+            const Real *Ic = I + (size_t)i * n_om;
+            for (int o0 = 0; o0 < n_om; o0 += kRun) {
+                Real acc[1 + DIM];
+#pragma unroll
+                for (int k = 0; k <= DIM; ++k) acc[k] = Real(0);
+#pragma unroll
+                for (int h = 0; h < kRun / 32; ++h) {
+                    const int o = o0 + 32 * h + lane;
+                    if (o >= n_om) break;
+                    const Real wI = TAB ? pt[o] * Ic[o] : to_real<Real>(wo[o]) * Ic[o];
+                    acc[0] += wI;
+#pragma unroll
+                    for (int a = 0; a < DIM; ++a) acc[1 + a] += wI * (TAB ? pt[(1 + a) * n_om + o] : to_real<Real>(om[(size_t)o * 3 + a]));
+                }
+#pragma unroll
+                for (int k = 0; k <= DIM; ++k) S[NM + k].add(acc[k]);
+            }
+            // sum over the lanes: at the first three steps a lane passes half of its sums on, so
+            // that it ends with three (12 + 6 + 3 + 2 x 3 exchanges instead of 5 x 20)
+            int first = 0;
+#pragma unroll
+            for (int step = 0; step < 3; ++step) {
+                const int half = 12 >> step, o = 16 >> step;
+                const bool up = lane & o;
+#pragma unroll
+                for (int k = 0; k < 12; ++k) {
+                    if (k >= half) break;
+                    const Sum<Real> a = S[k], b = S[half + k], got = (up ? a : b).shfl(o);
+                    S[k] = up ? b : a;
+                    S[k].add(got);
+                }
+                first += up ? half : 0;
+            }
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                S[k].add(S[k].shfl(2));
+                S[k].add(S[k].shfl(1));
+            }
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const double x = S[k].value();
+                if ((lane & 3) == 0) sums[buf][slot][first + k] = x;
+            }
+            if (lane == 0)
+#pragma unroll
+                for (int a = 0; a < DIM; ++a) shift[buf][slot][a] = to_double(u[a]);
+        }
+        __syncthreads();
+        if (warp == round % kWarps && base + lane < end)
+            finish<DIM>(sums[buf][lane], sums[buf][lane] + NM, shift[buf][lane], i_half_dr, i_half_dv, i_4sigma,
+                        out + (size_t)(base + lane) * kNF);
+    }
+}
+
 template <typename Real, int DIM>
 int run(long long n_cells, int n_xi, const double *xi, const double *w, int n_om, const double *om,
         const double *wo, const void *f, const void *I, double d_r, double d_v, double sigma_R, double *out,
         cudaStream_t s) {
-    const int n_chunks = (n_xi + kChunk - 1) / kChunk, o_chunks = (n_om + kChunk - 1) / kChunk;
-    if (scratch_bytes(n_cells, n_xi, n_om, sizeof(Real)) > kScratchBytes) return GSIS_ERR_INVALID_ARG;
-    void *base = nullptr;
-    int rc = scratch_address(&base);
-    if (rc != GSIS_OK) return rc;
-    double *u0 = static_cast<double *>(base);
-    Real *part = reinterpret_cast<Real *>(u0 + (size_t)n_cells * 3);
-    Real *opart = part + (size_t)n_cells * n_chunks * kNMP;
-    const int warps = 4;
-    const unsigned cells_blocks = (unsigned)((n_cells + warps - 1) / warps);
-    const unsigned per_cell = (unsigned)((n_cells + 127) / 128);
-    dim3 gg(cells_blocks, n_chunks), go(cells_blocks, o_chunks);
-    const Real *fr = static_cast<const Real *>(f);
-    k_static_mass<Real, DIM><<<gg, 32 * warps, 0, s>>>(n_cells, n_xi, n_chunks, xi, w, fr, part);
-    k_static_shift<Real, DIM><<<per_cell, 128, 0, s>>>(n_cells, n_chunks, part, u0);
-    k_static_gas<Real, DIM><<<gg, 32 * warps, 0, s>>>(n_cells, n_xi, n_chunks, xi, w, u0, fr, part);
-    k_static_photon<Real, DIM><<<go, 32 * warps, 0, s>>>(n_cells, n_om, o_chunks, om, wo, static_cast<const Real *>(I), opart);
-    k_static_finish<Real, DIM><<<per_cell, 128, 0, s>>>(n_cells, n_chunks, o_chunks, d_r, d_v, sigma_R, u0, part,
-                                                        opart, out);
-    return cudaGetLastError() == cudaSuccess ? GSIS_OK : GSIS_ERR_CUDA;
+    if (problem_bytes(n_cells, n_xi, n_om, sizeof(Real)) > kMaxBytes) return GSIS_ERR_INVALID_ARG;
+    // kCtasPerSm CTAs per SM share the cells out evenly; few cells: one per warp
+    constexpr int slots = 152 * kCtasPerSm;
+    const long long per = std::max<long long>(kWarps, (n_cells + slots - 1) / slots);
+    const unsigned ctas = (unsigned)((n_cells + per - 1) / per);
+    auto go = [&](auto kern, size_t smem) {
+        if (smem > 16384 &&
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+            return GSIS_ERR_CUDA;
+        kern<<<ctas, 32 * kWarps, smem, s>>>(n_cells, n_xi, n_om, xi, w, om, wo, static_cast<const Real *>(f),
+                                             static_cast<const Real *>(I), 2.0 / d_r, 2.0 / d_v,
+                                             sigma_R > 0.0 ? 1.0 / (4.0 * sigma_R) : 0.0, (int)per, out);
+        return cudaGetLastError() == cudaSuccess ? GSIS_OK : GSIS_ERR_CUDA;
+    };
+    const bool vec = reinterpret_cast<uintptr_t>(f) % (4 * sizeof(Real)) == 0;
+    // the FP32 tables of the sets while kCtasPerSm CTAs of them fit an SM
+    const size_t tab = ((size_t)n_xi * (2 * DIM + 1) + (size_t)n_om * (1 + DIM)) * sizeof(float);
+    if constexpr (std::is_same<Real, float>::value)
+        if (tab <= 64 * 1024)
+            return vec ? go(k_static<Real, DIM, true, true>, tab) : go(k_static<Real, DIM, true, false>, tab);
+    return vec ? go(k_static<Real, DIM, false, true>, 0) : go(k_static<Real, DIM, false, false>, 0);
 }
 
 }  // namespace
