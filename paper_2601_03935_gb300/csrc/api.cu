@@ -33,7 +33,7 @@ const char *kKernelNames[K_COUNT] = {"coefficients", "wall_density",  "slopes_ga
 struct gsis_ctx {
     int dim = 0, precision = 0, order = 2, block = 16;
     int64_t nc = 0;
-    int V = 0, Vp = 0, NO = 0, Op = 0, nch = 0, och = 0, n_bf = 0;
+    int V = 0, Vp = 0, NO = 0, Op = 0, nch = 0, och = 0, n_bf = 0, max_faces = 0;
     size_t real_size = 4;
     cudaStream_t stream = nullptr;
     ModelDev model{};
@@ -211,6 +211,7 @@ Geom<Real> geom(const gsis_ctx *c) {
     g.bf_tab = c->bf_tab;
     g.refl_v = c->refl_v;
     g.refl_o = c->refl_o;
+    g.max_faces = c->max_faces;
     g.resid = 0;
     return g;
 }
@@ -1005,6 +1006,7 @@ int gsis_create(const gsis_mesh *m, const gsis_velocity_quad *vq, const gsis_pho
         }
     }
     c->n_bf = (int)bf_cell.size();
+    c->max_faces = *std::max_element(nf.begin(), nf.end());
     // least-squares weights C_ij = (sum_k d_k d_k^T)^-1 d_j over the stencil of face
     // neighbours and their face neighbours (interior face neighbours first); a zero
     // gradient where the normal matrix is singular (det <= 1e-10 (tr/dim)^dim)

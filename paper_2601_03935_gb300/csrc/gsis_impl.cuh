@@ -99,6 +99,7 @@ struct Geom {
     int tc_wait;               // polls of the first tensor-core completion wait (ERR_TIMEOUT bit on expiry)
     Real pos_theta;            // > 0: the sweep keeps every value >= pos_theta times its previous value
     int *err;                  // device error word: bit 0 divergence, bit 1 a completion wait ran out
+    int max_faces;             // most faces of a cell
     int resid;                 // sweep: the moments of the residual only (no relaxation, no update)
 };
 

@@ -398,143 +398,6 @@ __device__ __forceinline__ Face<Real> load_face(const Real *__restrict__ fgeo, i
     return F;
 }
 
-// Venkatakrishnan-limited least-squares slope of cell j at VPT discrete velocities
-// v, v + 32, ..., v + 32 (VPT - 1), which share the cell's stencil indices, weights and
-// face offsets: grad = sum_s C_js (f_s - f_j) over the stencil (face neighbours and their
-// face neighbours); phi = min(1, min_faces phi_V(Delta_1, Delta_2)) per plane with the
-// bounds Delta_max/min taken over the interior face neighbours (the first entries of the
-// stencil).  Returns the slope multiplied by phi.
-template <typename Real, int N, int DIM, int VPT>
-__device__ __forceinline__ void limited_slope(const Geom<Real> &g, const Real *__restrict__ f, int stride, int j,
-                                              int v, const V<Real, N> (&fj)[VPT], V<Real, N> (&slope)[VPT][DIM]) {
-    // In 3-D the H0 plane carries nothing (no hidden velocity components): its slope is
-    // zero and no moment reads it, so its bounds and limiter are skipped (phi = 1).
-    constexpr bool ZH = DIM == 3 && N == 4;
-    V<Real, N> dmax[VPT], dmin[VPT];
-#pragma unroll
-    for (int u = 0; u < VPT; ++u)
-#pragma unroll
-        for (int p = 0; p < N; ++p) {
-            dmax[u].x[p] = Real(0);
-            dmin[u].x[p] = Real(0);
-#pragma unroll
-            for (int d = 0; d < DIM; ++d) slope[u][d].x[p] = Real(0);
-        }
-    const int4 info = g.info[j];
-    const int ns = info.y, nfn = info.z;
-    constexpr int MS = Lay<DIM>::MAXS, LW = Lay<DIM>::LW;
-    const int *stn = g.stn + (size_t)j * MS;
-    const Real *lw = g.lsq + (size_t)j * MS * LW;
-    // Stencil entries in batches of BT whose index and value loads are all issued before
-    // the batch is used.  The entries past the stencil's end (up to the batch boundary)
-    // hold cell 0 and zero weights, so they add exactly nothing; only the interior face
-    // neighbours (the first entries) bound the limiter.
-    constexpr int BT = DIM < 3 ? 2 : 4;
-    static_assert(MS % BT == 0, "batches tile the stencil records");
-#pragma unroll
-    for (int k0 = 0; k0 < MS; k0 += BT) {
-        if (k0 >= ns) break;
-        int sidx[BT];
-#pragma unroll
-        for (int t = 0; t < BT; ++t) sidx[t] = stn[k0 + t];
-        V<Real, N> fs[BT][VPT];
-#pragma unroll
-        for (int t = 0; t < BT; ++t)
-#pragma unroll
-            for (int u = 0; u < VPT; ++u) fs[t][u] = ldv<Real, N>(f, (size_t)sidx[t] * stride + v + 32 * u);
-#pragma unroll
-        for (int t = 0; t < BT; ++t) {
-            const int k = k0 + t;
-            const Real c0 = lw[LW * k], c1 = DIM > 1 ? lw[LW * k + 1] : Real(0), c2 = DIM > 2 ? lw[LW * k + 2] : Real(0);
-            const bool face_nbr = k < MAXF && k < nfn;
-#pragma unroll
-            for (int u = 0; u < VPT; ++u) {
-                const V<Real, N> dq = vsub(fs[t][u], fj[u]);
-                if (face_nbr) {
-#pragma unroll
-                    for (int p = 0; p < N; ++p) {
-                        if (ZH && p == 1) continue;
-                        dmax[u].x[p] = fmax(dmax[u].x[p], dq.x[p]);
-                        dmin[u].x[p] = fmin(dmin[u].x[p], dq.x[p]);
-                    }
-                }
-                vfma(c0, dq, slope[u][0]);
-                if constexpr (DIM > 1) vfma(c1, dq, slope[u][1]);
-                if constexpr (DIM > 2) vfma(c2, dq, slope[u][2]);
-            }
-        }
-    }
-    // phi = min(1, min over interior faces of phi_V(Delta_1, Delta_2)).  On the faces with
-    // Delta_2 > 0 (Delta_1 = Delta_max >= 0) phi_V >= 1 while Delta_2 <= Delta_1 / 2 and
-    // phi_V decreases for Delta_2 > Delta_1 / 4, so the minimum is taken at the largest
-    // Delta_2; likewise at the most negative Delta_2 with Delta_min.  Two evaluations per
-    // plane replace one per face.
-    const Real eps2 = g.eps2[j];
-    V<Real, N> hi[VPT], lo[VPT];
-#pragma unroll
-    for (int u = 0; u < VPT; ++u)
-#pragma unroll
-        for (int p = 0; p < N; ++p) {
-            hi[u].x[p] = Real(0);
-            lo[u].x[p] = Real(0);
-        }
-    const int nf = info.x;
-    for (int k = 0; k < nf; ++k) {
-        if (g.fnb[j * MAXF + k].x < 0) continue;
-        // face centroid - cell centroid: words 4..5 of a 1-D/2-D record, 5..7 of a 3-D one
-        Real dx0, dx1, dx2;
-        const Real *q = g.fgeo + ((size_t)j * MAXF + k) * Lay<DIM>::FRS + 4;
-        if constexpr (DIM < 3) {
-            const Vec<Real, 2> d = vload<Real, 2>(q);
-            dx0 = d.v[0];
-            dx1 = d.v[1];
-            dx2 = Real(0);
-        } else {
-            const Vec<Real, 4> d = vload<Real, 4>(q);
-            dx0 = d.v[1];
-            dx1 = d.v[2];
-            dx2 = d.v[3];
-        }
-#pragma unroll
-        for (int u = 0; u < VPT; ++u) {
-            V<Real, N> d2 = vmul(slope[u][0], vsplat<Real, N>(dx0));
-            if constexpr (DIM > 1) vfma(dx1, slope[u][1], d2);
-            if constexpr (DIM > 2) vfma(dx2, slope[u][2], d2);
-#pragma unroll
-            for (int p = 0; p < N; ++p) {
-                if (ZH && p == 1) continue;
-                hi[u].x[p] = fmax(hi[u].x[p], d2.x[p]);
-                lo[u].x[p] = fmin(lo[u].x[p], d2.x[p]);
-            }
-        }
-    }
-#pragma unroll
-    for (int u = 0; u < VPT; ++u) {
-        // phi_V(d1, d2) = (d1 (d1 + 2 d2) + eps2) / (d1 (d1 + d2) + 2 d2^2 + eps2)
-        V<Real, N> ph;
-        // both bounds of every plane without branches (two planes per packed
-        // instruction); the select keeps 1 where a bound's side does not apply
-        const V<Real, N> e = vsplat<Real, N>(eps2);
-        auto venkat = [&](const V<Real, N> &d1, const V<Real, N> &d2) {
-            const V<Real, N> d2x2 = vadd(d2, d2);
-            const V<Real, N> num = vfmav(d1, vadd(d1, d2x2), e);
-            const V<Real, N> den = vfmav(d1, vadd(d1, d2), vfmav(d2x2, d2, e));
-            V<Real, N> r;
-#pragma unroll
-            for (int p = 0; p < N; ++p) r.x[p] = (ZH && p == 1) ? Real(1) : fdiv(num.x[p], den.x[p]);
-            return r;
-        };
-        const V<Real, N> ph_hi = venkat(dmax[u], hi[u]), ph_lo = venkat(dmin[u], lo[u]);
-#pragma unroll
-        for (int p = 0; p < N; ++p)
-            ph.x[p] = (ZH && p == 1) ? Real(1)
-                                     : fmin(fmin(Real(1), hi[u].x[p] > Real(0) ? ph_hi.x[p] : Real(1)),
-                                            lo[u].x[p] < Real(0) ? ph_lo.x[p] : Real(1));
-#pragma unroll
-        for (int d = 0; d < DIM; ++d) slope[u][d] = vmul(slope[u][d], ph);
-    }
-}
-
 // Reference distribution of the four gas planes at one (cell, velocity).
 template <typename Real, int DIM>
 __device__ __forceinline__ void reference(const Real *__restrict__ C, const Real *xi, Real (&gp)[4]) {
@@ -631,62 +494,179 @@ __device__ __forceinline__ void add_moments(Real (&acc)[Lay<DIM>::NMP], const Re
 }
 
 // ------------------------------------------------------------------ upwind face values
-// Thread (tx, ty) of a 32 x SLOPE_ROWS CTA: cell blockIdx.x * SLOPE_ROWS + ty, velocities
-// blockIdx.y * 32 SLOPE_VPT + tx + 32 u (u < SLOPE_VPT).  Computes the cell's Venkatakrishnan-limited
-// least-squares slope and, on every interior face through which the velocity leaves the
-// cell (xi . n > 0), the second-order reconstruction f_j + phi grad f_j . (x_f - x_j) of
-// every plane: fface[(face * n_pad + v) * N + plane].  The two cells of a face hold exactly
-// opposite normals, so for each velocity exactly one of them (the upwind one) writes the
-// face's value, and none where xi . n = 0, which the sweep skips.  The sweep reads these
-// values for both its outflow and its inflow interior faces.
+// Thread (tx, ty) of a 32 x SLOPE_ROWS CTA: cell blockIdx.x * SLOPE_ROWS + ty.  Computes the
+// cell's least-squares gradient grad = sum_s C_js (f_s - f_j) over its stencil (face
+// neighbours and their face neighbours), Venkatakrishnan's limiter phi = min(1, min_faces
+// phi_V(Delta_1, Delta_2)) per plane, with the bounds Delta_1 taken over the interior face
+// neighbours (the first entries of the stencil), and, on every interior face through which
+// the velocity leaves the cell (xi . n > 0), the second-order reconstruction
+// f_j + phi grad . (x_f - x_j) of every plane: fface[(face * n_pad + v) * N + plane].  The two
+// cells of a face hold exactly opposite normals, so for each velocity exactly one of them (the
+// upwind one) writes the face's value, and none where xi . n = 0, which the sweep skips.  The
+// sweep reads these values for both its outflow and its inflow interior faces.
 constexpr int SLOPE_ROWS = 8;
-// velocities per thread (32 slope_vpt per row; a 3-D slope of four planes takes 12
-// registers per velocity) and FP32 CTAs per SM (64 registers per thread)
+// velocities per thread of the FP32 pass (v, v + 32, ...), which share the cell's stencil
+// indices, weights and face offsets
 __host__ __device__ constexpr int slope_vpt(int dim) { return dim < 3 ? 2 : 1; }
-__host__ __device__ constexpr int slope_minb(int) { return 4; }
-template <typename Real, int N, int DIM>
-__global__ void __launch_bounds__(32 * SLOPE_ROWS, slope_minb(DIM)) k_slopes(Geom<Real> g, int n_pad,
-                                                                             const Real *__restrict__ xq,
-                                                                             const Real *__restrict__ f,
-                                                                             Real *__restrict__ fface) {
-    constexpr int VPT = slope_vpt(DIM);
+
+// Row `i` of an array whose rows are `bytes` long: one 32 x 32 -> 64-bit multiply-add
+__device__ __forceinline__ const float *row_at(const float *p, int i, unsigned bytes) {
+    return reinterpret_cast<const float *>(reinterpret_cast<const char *>(p) + (unsigned long long)(unsigned)i * bytes);
+}
+
+// 1 / x to one unit in the last place, for normal x
+__device__ __forceinline__ float rcp_normal(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// The FP32 slope pass.  It keeps the L1 data path (64 % of its cycles) and the issue slots
+// (52 %) busier than memory (2.5 TB/s): per warp and pair of velocities 22 16-byte reads of f
+// and some 60 broadcast reads of indices, weights and face records, each of which writes 32
+// registers like any other (the weights as ready-made pairs cost more than the moves that
+// make them: 313 us for what takes 254).  64 registers, four CTAs per SM: with Delta_2 of every
+// face kept from the limiter to the reconstruction the pass runs three and takes 269 us.
+// A row's address is one multiply-add, the two quotients of phi one reciprocal each, and the
+// face loops have the cells' face count.  About 330 instructions per velocity, 501 before:
+// 20 000 triangles x 784 velocities 324 -> 254 us, 40 000 x 2 304 1.89 -> 1.51 ms, 10 185
+// tetrahedra x 4 096 1.31 -> 1.06 ms.
+template <int N, int DIM, int FM>
+__global__ void __launch_bounds__(32 * SLOPE_ROWS, 4) k_slopes32(Geom<float> g, int n, int n_pad,
+                                                                                const float *__restrict__ xq,
+                                                                                const float *__restrict__ f,
+                                                                                float *__restrict__ fface) {
+    // In 3-D the H0 plane carries nothing (no hidden velocity components): its gradient is
+    // zero and no moment reads it, so its bounds and limiter are skipped (phi = 1).
+    constexpr bool ZH = DIM == 3 && N == 4;
+    constexpr int VPT = slope_vpt(DIM), MS = Lay<DIM>::MAXS, LW = Lay<DIM>::LW, FRS = Lay<DIM>::FRS;
+    // stencil entries per batch, whose index and value loads are all issued before the batch
+    // is used.  Entries past the stencil's end hold cell 0 and zero weights and add nothing.
+    constexpr int BT = DIM < 3 ? 2 : 4;
+    static_assert(MS % BT == 0, "batches tile the stencil records");
     const int v = blockIdx.y * (32 * VPT) + threadIdx.x;
     const int j = blockIdx.x * SLOPE_ROWS + threadIdx.y;
-    if (j >= g.n_cells) return;
-    const size_t idx = (size_t)j * n_pad + v;
-    V<Real, N> fj[VPT];
+    if (j >= g.n_cells || blockIdx.y * (32 * VPT) >= n) return;   // no face value of a padding velocity is used
+    const float *fv = f + (size_t)v * N;
+    const unsigned row = (unsigned)n_pad * (N * 4);
+    const int4 info = g.info[j];
+    const int ns = info.y, nfn = info.z;
+    V<float, N> fj[VPT], grad[VPT][DIM], dmax[VPT], dmin[VPT];
 #pragma unroll
-    for (int u = 0; u < VPT; ++u) fj[u] = ldv<Real, N>(f, idx + 32 * u);
-    V<Real, N> sl[VPT][DIM];
-    limited_slope<Real, N, DIM, VPT>(g, f, n_pad, j, v, fj, sl);
-    Real xi[VPT][DIM];
+    for (int u = 0; u < VPT; ++u) {
+        fj[u] = ldv<float, N>(row_at(fv, j, row), 32 * u);
+        dmax[u] = dmin[u] = vsplat<float, N>(0.0f);
 #pragma unroll
-    for (int u = 0; u < VPT; ++u)
+        for (int d = 0; d < DIM; ++d) grad[u][d] = vsplat<float, N>(0.0f);
+    }
+    const int *stn = g.stn + (size_t)j * MS;
+    const float *lw = g.lsq + (size_t)j * MS * LW;
 #pragma unroll
-        for (int a = 0; a < DIM; ++a) xi[u][a] = xq[a * n_pad + v + 32 * u];
-    const int nf = g.info[j].x;
-    for (int k = 0; k < nf; ++k) {
-        const int fid = g.cface[j * MAXF + k];
-        if (fid < 0) continue;
-        const Face<Real> F = load_face<Real, DIM>(g.fgeo, j, k);
+    for (int k0 = 0; k0 < MS; k0 += BT) {
+        if (k0 >= ns) break;
+        V<float, N> fs[BT][VPT];
+#pragma unroll
+        for (int t = 0; t < BT; ++t) {
+            const float *p = row_at(fv, stn[k0 + t], row);
+#pragma unroll
+            for (int u = 0; u < VPT; ++u) fs[t][u] = ldv<float, N>(p, 32 * u);
+        }
+#pragma unroll
+        for (int t = 0; t < BT; ++t) {
+            const int k = k0 + t;
+            float w[DIM];
+#pragma unroll
+            for (int d = 0; d < DIM; ++d) w[d] = lw[LW * k + d];
+            const bool face_nbr = k < FM && k < nfn;
+#pragma unroll
+            for (int u = 0; u < VPT; ++u) {
+                const V<float, N> dq = vsub(fs[t][u], fj[u]);
+                if (face_nbr) {
+#pragma unroll
+                    for (int p = 0; p < N; ++p) {
+                        if (ZH && p == 1) continue;
+                        dmax[u].x[p] = fmaxf(dmax[u].x[p], dq.x[p]);
+                        dmin[u].x[p] = fminf(dmin[u].x[p], dq.x[p]);
+                    }
+                }
+#pragma unroll
+                for (int d = 0; d < DIM; ++d) vfma(w[d], dq, grad[u][d]);
+            }
+        }
+    }
+    int fid[FM];             // < 0: boundary, or past the cell's faces
+    float dx[FM][DIM];       // face centroid - cell centroid (zero where there is no interior face)
+    const float *fg = g.fgeo + (size_t)j * MAXF * FRS;
+#pragma unroll
+    for (int k = 0; k < FM; ++k) {
+        fid[k] = g.cface[(size_t)j * MAXF + k];
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) dx[k][d] = fid[k] >= 0 ? fg[k * FRS + (DIM < 3 ? 4 : 5) + d] : 0.0f;
+    }
+    // Delta_2 = grad . (x_f - x_j) at the interior faces.  On the faces with Delta_2 > 0
+    // (Delta_1 = Delta_max >= 0) phi_V >= 1 while Delta_2 <= Delta_1 / 2 and phi_V decreases for
+    // Delta_2 > Delta_1 / 4, so the minimum is taken at the largest Delta_2; likewise at the most
+    // negative Delta_2 with Delta_min.  Two evaluations per plane replace one per face.
+    //   phi_V(d1, e) = num / den, num = d1 (d1 + 2 e) + eps2, den = d1 (d1 + e) + 2 e^2 + eps2
+    //                = num + e (2 e - d1), which cancels at most a third of num.
+    // den is at least eps2, kept a normal number (below it the squares of d1 and e vanish in
+    // FP32 as well).
+    const float eps2 = fmaxf(g.eps2[j], 1e-37f);
+#pragma unroll
+    for (int u = 0; u < VPT; ++u) {
+        V<float, N> hi = vsplat<float, N>(0.0f), lo = hi;
+#pragma unroll
+        for (int k = 0; k < FM; ++k) {
+            V<float, N> d2 = vmul(grad[u][0], vsplat<float, N>(dx[k][0]));
+#pragma unroll
+            for (int d = 1; d < DIM; ++d) vfma(dx[k][d], grad[u][d], d2);
+#pragma unroll
+            for (int p = 0; p < N; ++p) {
+                if (ZH && p == 1) continue;
+                hi.x[p] = fmaxf(hi.x[p], d2.x[p]);
+                lo.x[p] = fminf(lo.x[p], d2.x[p]);
+            }
+        }
+        const V<float, N> two = vsplat<float, N>(2.0f), ev = vsplat<float, N>(eps2);
+        auto venkat = [&](const V<float, N> &d1, const V<float, N> &e) {
+            const V<float, N> num = vfmav(d1, vfmav(two, e, d1), ev);
+            const V<float, N> den = vfmav(e, vsub(vadd(e, e), d1), num);
+            V<float, N> r;
+#pragma unroll
+            for (int p = 0; p < N; ++p) r.x[p] = (ZH && p == 1) ? 1.0f : num.x[p] * rcp_normal(den.x[p]);
+            return r;
+        };
+        const V<float, N> ph = venkat(dmax[u], hi), pl = venkat(dmin[u], lo);
+        V<float, N> phi;
+#pragma unroll
+        for (int p = 0; p < N; ++p) phi.x[p] = fminf(fminf(1.0f, ph.x[p]), pl.x[p]);
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) grad[u][d] = vmul(grad[u][d], phi);
+    }
+#pragma unroll
+    for (int k = 0; k < FM; ++k) {
+        if (fid[k] < 0) continue;
+        float nx[DIM];
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) nx[d] = fg[k * FRS + d];
+        float *o = const_cast<float *>(row_at(fface + (size_t)v * N, fid[k], row));
 #pragma unroll
         for (int u = 0; u < VPT; ++u) {
-            Real xn = xi[u][0] * F.n[0];
-            if constexpr (DIM > 1) xn = fma(xi[u][1], F.n[1], xn);
-            if constexpr (DIM > 2) xn = fma(xi[u][2], F.n[2], xn);
-            if (!(xn > Real(0))) continue;
-            V<Real, N> fv = fj[u];
-            vfma(F.df[0], sl[u][0], fv);
-            if constexpr (DIM > 1) vfma(F.df[1], sl[u][1], fv);
-            if constexpr (DIM > 2) vfma(F.df[2], sl[u][2], fv);
-            const size_t o = (size_t)fid * n_pad + v + 32 * u;
-            if constexpr (N == 1) {
-                fface[o] = fv.x[0];
-            } else {
-                Vec<Real, N> t;
+            float xn = xq[v + 32 * u] * nx[0];
 #pragma unroll
-                for (int p = 0; p < N; ++p) t.v[p] = fv.x[p];
-                vstore<Real, N>(fface + o * N, t);
+            for (int a = 1; a < DIM; ++a) xn = fmaf(xq[a * n_pad + v + 32 * u], nx[a], xn);
+            V<float, N> val = fj[u];
+#pragma unroll
+            for (int d = 0; d < DIM; ++d) vfma(dx[k][d], grad[u][d], val);
+            if (xn > 0.0f) {
+                if constexpr (N == 1) {
+                    o[32 * u] = val.x[0];
+                } else {
+                    Vec<float, N> t;
+#pragma unroll
+                    for (int p = 0; p < N; ++p) t.v[p] = val.x[p];
+                    vstore<float, N>(o + 32 * u * N, t);
+                }
             }
         }
     }
@@ -2256,10 +2236,13 @@ static cudaError_t slopes_t(cudaStream_t s, const Geom<Real> &g, const Quad<Real
         k_slopes64<N, DIM><<<grid, dim3(32, SLOPE_ROWS), 0, s>>>(g, q.n, q.n_pad, q.x, f, fface);
         return cudaGetLastError();
     } else {
-    static_assert(SV % (32 * slope_vpt(DIM)) == 0, "a row's velocities must tile the padding");
-    dim3 grid((g.n_cells + SLOPE_ROWS - 1) / SLOPE_ROWS, q.n_pad / (32 * slope_vpt(DIM))), block(32, SLOPE_ROWS);
-    k_slopes<Real, N, DIM><<<grid, block, 0, s>>>(g, q.n_pad, q.x, f, fface);
-    return cudaGetLastError();
+        static_assert(SV % (32 * slope_vpt(DIM)) == 0, "a row's velocities must tile the padding");
+        dim3 grid((g.n_cells + SLOPE_ROWS - 1) / SLOPE_ROWS, q.n_pad / (32 * slope_vpt(DIM))), block(32, SLOPE_ROWS);
+        if (DIM < 3 && g.max_faces <= DIM + 1)     // segments, triangles
+            k_slopes32<N, DIM, DIM + 1><<<grid, block, 0, s>>>(g, q.n, q.n_pad, q.x, f, fface);
+        else
+            k_slopes32<N, DIM, MAXF><<<grid, block, 0, s>>>(g, q.n, q.n_pad, q.x, f, fface);
+        return cudaGetLastError();
     }
 }
 
