@@ -35,7 +35,7 @@ constexpr int U = 0;
 constexpr int COMP = 4;        // first component block
 constexpr int CSZ = 16;        // size of one component block
 constexpr int A = 0, B = 1, T = 2, K1 = 3, Q = 4, K2 = 7, R1 = 8, R2 = 12;
-constexpr int S = 11, A2 = 15;   // FP64: -B in the units of fp64::exp2n, A m T (m hidden components)
+constexpr int S = 11, A2 = 15;   // -B in the units of fp64::exp2n (FP64) or times log2 e (FP32), A m T (m hidden components)
 constexpr int RATE = COMP + 3 * CSZ;   // 52
 constexpr int INV_DT = RATE + 1;
 constexpr int SINK = RATE + 2;

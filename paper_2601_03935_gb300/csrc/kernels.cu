@@ -135,6 +135,8 @@ __global__ void k_coefficients(Geom<Real> g, ModelDev m, const double *__restric
         } else {
             A = alpha[c] * rho * pow_neg_half_dim<DIM>(two_pi * T);
             B = CT(0.5) / T;
+            Cc[cf::S] = CT(-0.7213475204444817) / T;      // -B log2 e
+            Cc[cf::A2] = A * (CT(3 - DIM) * T);
             s = CT(2) / (CT(15) * T * rho * T);
             irT = CT(1) / (rho * T);
         }
@@ -863,9 +865,9 @@ __global__ void __launch_bounds__(SV * ROWS, sizeof(Real) == 4 ? (DIM < 3 ? 8 : 
     Real *sC = reinterpret_cast<Real *>(reinterpret_cast<unsigned char *>(Nf) +
                                         ((size_t)g.block * MAXF * NFS * sizeof(Real) + 31) / 32 * 32);   // [block][NC]
     // the tensor-core epilogue's basis covers the 1-D and 2-D moments
-    constexpr bool TCM = std::is_same<Real, float>::value && N == 4 && DIM < 3;
+    constexpr bool tc = std::is_same<Real, float>::value && N == 4;
+    static_assert(!tc || (DIM < 3 && !RESID), "FP32 gas without the tensor cores is k_sweep_gas32's");
     constexpr int NMPD = Lay<DIM>::NMP;
-    const bool tc = TCM && g.tc && !RESID;
     Real *sxi = reinterpret_cast<Real *>(smem_raw + sweep_main_bytes(g.block, N, DIM, sizeof(Real), tc));   // [DIM+1][SV]
     signed char *Lg = reinterpret_cast<signed char *>(sxi + (DIM + 1) * SV);   // [block][MAXF] in-block neighbour or -1
     tcm::Ctl *ctl = reinterpret_cast<tcm::Ctl *>(Lg + ((g.block * MAXF + 15) & ~15));
@@ -883,12 +885,7 @@ __global__ void __launch_bounds__(SV * ROWS, sizeof(Real) == 4 ? (DIM < 3 ? 8 : 
         for (int a = 0; a < DIM; ++a) sxi[a * SV + tx] = xi[a];
         sxi[DIM * SV + tx] = q.w[v];
     }
-    if constexpr (TCM) {
-        if (tc)
-            tcm::start(ctl, ty * SV + tx);   // the allocation completes during phase 1
-        else if (ty == 0 && tx < 32)
-            tcm::relinquish();               // CUDA-core epilogue: let further CTAs onto the SM
-    }
+    if constexpr (tc) tcm::start(ctl, ty * SV + tx);   // the allocation completes during phase 1
 
     // ---- 0. face records: source = interior face id (order 2) or neighbour cell (order 1),
     // -1 - boundary face, NO_FACE past the cell's faces
@@ -1081,63 +1078,61 @@ __global__ void __launch_bounds__(SV * ROWS, sizeof(Real) == 4 ? (DIM < 3 ? 8 : 
     __syncthreads();
 
     // ---- 3. f^{k+1/2} = f^k + delta
-    if constexpr (TCM) {
-        if (tc) {
-            // Tensor-core moments: the tile's operand stage overlays R, the dead diagonal
-            // and inflow areas and B; f^{k+1/2} waits in registers until every R read is done.
-            unsigned char *stage = smem_raw;
-            const int tile = c0 / MT * MT, lt0 = c0 - tile;
-            constexpr int PER = MT / ROWS;
-            Vec<float, 4> th[PER];
+    if constexpr (tc) {
+        // Tensor-core moments: the tile's operand stage overlays R, the dead diagonal
+        // and inflow areas and B; f^{k+1/2} waits in registers until every R read is done.
+        unsigned char *stage = smem_raw;
+        const int tile = c0 / MT * MT, lt0 = c0 - tile;
+        constexpr int PER = MT / ROWS;
+        Vec<float, 4> th[PER];
 #pragma unroll
-            for (int j = 0; j < PER; ++j) {
-                const int l = ty + j * ROWS;
-                if (l < nb) {
-                    const size_t idx = (size_t)(c0 + l) * stride + v;
-                    const Vec<float, 4> fo = vload<float, 4>(reinterpret_cast<const float *>(f_in) + idx * 4);
-                    Vec<float, 4> t = *reinterpret_cast<const Vec<float, 4> *>(&R[l * SV + tx]);
+        for (int j = 0; j < PER; ++j) {
+            const int l = ty + j * ROWS;
+            if (l < nb) {
+                const size_t idx = (size_t)(c0 + l) * stride + v;
+                const Vec<float, 4> fo = vload<float, 4>(reinterpret_cast<const float *>(f_in) + idx * 4);
+                Vec<float, 4> t = *reinterpret_cast<const Vec<float, 4> *>(&R[l * SV + tx]);
 #pragma unroll
-                    for (int p = 0; p < 4; ++p) t.v[p] += fo.v[p];
-                    if (g.pos_theta > 0.0f) {
+                for (int p = 0; p < 4; ++p) t.v[p] += fo.v[p];
+                if (g.pos_theta > 0.0f) {
 #pragma unroll
-                        for (int p = 0; p < 4; ++p) t.v[p] = fmaxf(t.v[p], g.pos_theta * fo.v[p]);
-                    }
-                    vstore<float, 4>(reinterpret_cast<float *>(f_out) + idx * 4, t);
-                    th[j] = t;
+                    for (int p = 0; p < 4; ++p) t.v[p] = fmaxf(t.v[p], g.pos_theta * fo.v[p]);
                 }
+                vstore<float, 4>(reinterpret_cast<float *>(f_out) + idx * 4, t);
+                th[j] = t;
             }
-            __syncthreads();
-#pragma unroll
-            for (int j = 0; j < PER; ++j) {
-                const int l = ty + j * ROWS;
-                if (l < nb) tcm::put_a4(stage, lt0 + l, tx, th[j].v);
-            }
-            if (ty == 0) {
-                const Vec<float, 4> u4 =
-                    vload<float, 4>(reinterpret_cast<const float *>(coef) + (size_t)tile * cf::NC + cf::U);
-                float c[DIM];
-#pragma unroll
-                for (int a = 0; a < DIM; ++a) c[a] = (float)sxi[a * SV + tx] - u4.v[a];
-                tcm::put_b<DIM>(stage, tx, c, (float)sxi[DIM * SV + tx]);
-            }
-            tcm::fence_smem_to_async();
-            __syncthreads();
-            // ---- 4. moments: one M = 128, N = 16, K = 64 contraction per CTA
-            const int tid = ty * SV + tx;
-            const uint32_t taddr = tcm::accumulator(ctl);
-            float m[tcm::NBASIS];
-            bool ok;
-            if (tcm::contract(ctl, taddr, stage, tid, m, ok, g.tc_wait)) {
-                const int l = (tid & 15) - lt0;
-                if (l >= 0 && l < nb)
-                    tcm::store_row<DIM>(reinterpret_cast<float *>(partial) +
-                                            ((size_t)(c0 + l) * gridDim.y + chunk) * NMPD,
-                                        tid >> 5, m);
-            }
-            if (!ok && tid == 0) atomicOr(g.err, ERR_TIMEOUT_BIT);
-            tcm::end(ctl, taddr, tid, ok, 0);
-            return;
         }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const int l = ty + j * ROWS;
+            if (l < nb) tcm::put_a4(stage, lt0 + l, tx, th[j].v);
+        }
+        if (ty == 0) {
+            const Vec<float, 4> u4 =
+                vload<float, 4>(reinterpret_cast<const float *>(coef) + (size_t)tile * cf::NC + cf::U);
+            float c[DIM];
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) c[a] = (float)sxi[a * SV + tx] - u4.v[a];
+            tcm::put_b<DIM>(stage, tx, c, (float)sxi[DIM * SV + tx]);
+        }
+        tcm::fence_smem_to_async();
+        __syncthreads();
+        // ---- 4. moments: one M = 128, N = 16, K = 64 contraction per CTA
+        const int tid = ty * SV + tx;
+        const uint32_t taddr = tcm::accumulator(ctl);
+        float m[tcm::NBASIS];
+        bool ok;
+        if (tcm::contract(ctl, taddr, stage, tid, m, ok, g.tc_wait)) {
+            const int l = (tid & 15) - lt0;
+            if (l >= 0 && l < nb)
+                tcm::store_row<DIM>(reinterpret_cast<float *>(partial) +
+                                        ((size_t)(c0 + l) * gridDim.y + chunk) * NMPD,
+                                    tid >> 5, m);
+        }
+        if (!ok && tid == 0) atomicOr(g.err, ERR_TIMEOUT_BIT);
+        tcm::end(ctl, taddr, tid, ok, 0);
+        return;
     }
     for (int l = ty; l < nb && !RESID; l += ROWS) {
         const size_t idx = (size_t)(c0 + l) * stride + v;
@@ -1220,12 +1215,12 @@ __global__ void __launch_bounds__(SV * ROWS, sizeof(Real) == 4 ? (DIM < 3 ? 8 : 
         }
         return;
     }
-    constexpr int TPC = 8;
-    const int tid = ty * SV + tx;
-    const int sub = tid % TPC;
-    const unsigned gmask = 0xFFu << ((tid & 31) & ~(TPC - 1));
-    for (int l = tid / TPC; l < nb; l += SV * ROWS / TPC) {
-        if constexpr (PHOTON) {
+    if constexpr (PHOTON) {
+        constexpr int TPC = 8;
+        const int tid = ty * SV + tx;
+        const int sub = tid % TPC;
+        const unsigned gmask = 0xFFu << ((tid & 31) & ~(TPC - 1));
+        for (int l = tid / TPC; l < nb; l += SV * ROWS / TPC) {
             Real acc[1 + DIM];
 #pragma unroll
             for (int m = 0; m <= DIM; ++m) acc[m] = Real(0);
@@ -1244,29 +1239,463 @@ __global__ void __launch_bounds__(SV * ROWS, sizeof(Real) == 4 ? (DIM < 3 ? 8 : 
 #pragma unroll
                 for (int m = 0; m <= DIM; ++m) P[m] = acc[m];
             }
+        }
+    }
+}
+
+// ------------------------------------------------------------------ the FP32 gas sweep
+__device__ __forceinline__ float2 dup2(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float ex2_ftz(float x) {   // 2^x, results below 2^-126 as 0
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// 1 / x, one Newton step beyond rcp_normal
+__device__ __forceinline__ float rcp_refined(float x) {
+    const float y = rcp_normal(x);
+    return fmaf(y, fmaf(-x, y, 1.0f), y);
+}
+
+// Shared memory of a k_sweep_gas32 CTA.
+template <int DIM>
+struct S32 {
+    static constexpr int ROWS = 4;                        // warps: a lane takes velocities tx and tx + 32
+    static constexpr int NK = (6 + 3 * DIM + 3) / 4;      // float4 of a Maxwellian: S B A A2 | K1 K2, then Q R1 R2 per axis
+    static constexpr int CF = 2 + 3 * NK;                 // float4 of a cell's coefficients: u, Maxwellians, rates
+    static constexpr int XS = DIM + 1;
+    __host__ __device__ static constexpr size_t bytes(int block) {
+        return (size_t)block * SV * 16                    // R: residuals, increments, f
+               + (size_t)block * MAXF * 16                // face records
+               + (size_t)block * MAXF * 16                // in-block neighbours
+               + (size_t)block * CF * 16                  // coefficients
+               + (size_t)block * SV * 4                   // 1 / diagonal
+               + (size_t)XS * SV * 4                      // velocities and weights
+               + ((size_t)block * 4 + 15) / 16 * 16;      // in-block neighbour counts
+    }
+};
+
+// The reference distribution of the four planes at a pair of velocities (reference() above,
+// with the second bracket as the first plus q.c).  A coefficient read from shared memory
+// costs a register write per lane: it is read once for the pair, its products are scalar
+// instructions, and what follows is packed.
+template <int DIM>
+__device__ __forceinline__ void reference32(const float4 *__restrict__ C, const float2 (&xi)[DIM], float2 (&gp)[4]) {
+    constexpr int MH = 3 - DIM;
+    const float4 u4 = C[0];
+    const float uu[3] = {u4.x, u4.y, u4.z};
+    float2 c[DIM], c2;
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) {
+        c[a] = make_float2(xi[a].x - uu[a], xi[a].y - uu[a]);
+        c2 = a == 0 ? __fmul2_rn(c[0], c[0]) : __ffma2_rn(c[a], c[a], c2);
+    }
+    auto mul = [](float s, float2 x) { return make_float2(s * x.x, s * x.y); };
+    auto fma_ = [](float s, float2 x, float2 y) { return make_float2(fmaf(s, x.x, y.x), fmaf(s, x.y, y.y)); };
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        float w[4 * S32<DIM>::NK];
+#pragma unroll
+        for (int t = 0; t < S32<DIM>::NK; ++t) {
+            const float4 x = C[1 + k * S32<DIM>::NK + t];
+            w[4 * t] = x.x;
+            w[4 * t + 1] = x.y;
+            w[4 * t + 2] = x.z;
+            w[4 * t + 3] = x.w;
+        }
+        const float2 e = make_float2(ex2_ftz(w[0] * c2.x), ex2_ftz(w[0] * c2.y));
+        float2 qc = mul(w[6], c[0]), r1 = mul(w[7], c[0]), r2 = mul(w[8], c[0]);
+#pragma unroll
+        for (int a = 1; a < DIM; ++a) {
+            qc = fma_(w[6 + 3 * a], c[a], qc);
+            r1 = fma_(w[7 + 3 * a], c[a], r1);
+            r2 = fma_(w[8 + 3 * a], c[a], r2);
+        }
+        const float2 tb = make_float2(fmaf(w[1], c2.x, 0.5f * MH - 2.5f), fmaf(w[1], c2.y, 0.5f * MH - 2.5f));
+        const float2 p0 = __ffma2_rn(qc, tb, dup2(1.0f)), E = mul(w[2], e);
+        const float2 t1 = fma_(w[4], p0, r1), t2 = fma_(w[5], p0, r2);
+        if (k == 0) {
+            gp[0] = __fmul2_rn(E, p0);
+            gp[1] = MH > 0 ? __fmul2_rn(mul(w[3], e), __fadd2_rn(p0, qc)) : dup2(0.0f);
+            gp[2] = __fmul2_rn(E, t1);
+            gp[3] = __fmul2_rn(E, t2);
         } else {
-            constexpr int NM = n_gas_moments<DIM>();
-            const Vec<Real, 4> u4 = vload<Real, 4>(coef + (size_t)((c0 + l) / MT * MT) * cf::NC + cf::U);
-            Real acc[NMPD];
+            gp[0] = __ffma2_rn(E, p0, gp[0]);
+            if constexpr (MH > 0) gp[1] = __ffma2_rn(mul(w[3], e), __fadd2_rn(p0, qc), gp[1]);
+            gp[2] = __ffma2_rn(E, t1, gp[2]);
+            gp[3] = __ffma2_rn(E, t2, gp[3]);
+        }
+    }
+}
+
+// k_sweep for the four FP32 gas planes with CUDA-core moments: the same phases, a warp taking a
+// cell's 64 velocities in pairs per lane, so that what is read for the cell is read once for
+// both, without branches on the direction of a velocity.  FM: the most faces of a cell.
+// It waits more than it works (43 % of the issue slots, L1 60 %, 3.3 TB/s): the relaxation,
+// a serial chain over the block's cells in one warp, takes a quarter of the time (two warps of
+// one velocity per lane, or reading ahead of it, took longer: more instructions).  Six CTAs of
+// 80 registers per SM where no cell has more faces than a triangle, else five of 96 (at six,
+// spills: 396 us; at four 358).  About 290 instructions per velocity, 497 before: 20 000
+// triangles x 784 velocities at order 2 354 -> 292 us, 40 000 x 2 304 1.91 -> 1.56 ms, 10 185
+// tetrahedra x 4 096 946 -> 814 us.
+template <int DIM, int ORDER, bool RESID, int FM>
+__global__ void __launch_bounds__(32 * S32<DIM>::ROWS, FM < MAXF ? 6 : 5)
+    k_sweep_gas32(Geom<float> g, Quad<float> q, const float *__restrict__ coef, const float *__restrict__ bcoef,
+                  const float *__restrict__ f_in, const float *__restrict__ fface, float *__restrict__ f_out,
+                  float *__restrict__ partial) {
+    using S = S32<DIM>;
+    constexpr int ROWS = S::ROWS, NT = 32 * ROWS;
+    extern __shared__ float4 smem32[];
+    float4 *R = smem32;                                   // [block][SV]
+    float4 *Fa = R + g.block * SV;                        // [block][MAXF]: n, S/V (3-D: S/V n), source
+    float4 *Gr = Fa + g.block * MAXF;                     // [block][MAXF]: S/V n, index; lower in-block neighbours from
+                                                          // the front, upper ones from the back
+    float4 *Cs = Gr + g.block * MAXF;                     // [block][CF]
+    float *Dg = reinterpret_cast<float *>(Cs + g.block * S::CF);   // [block][SV]
+    float *sxi = Dg + g.block * SV;                       // [DIM + 1][SV]
+    int *Ln = reinterpret_cast<int *>(sxi + S::XS * SV);  // [block] lower + 8 upper in-block neighbours
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int c0 = blockIdx.x * g.block;
+    const int nb = min(g.block, g.n_cells - c0);
+    const int chunk = blockIdx.y;
+    const int v = chunk * SV + tx;
+    const int stride = q.n_pad;
+    const unsigned row = (unsigned)stride * 16;
+    const float *f_v = f_in + (size_t)v * 4;
+    float2 xi[DIM];
 #pragma unroll
-            for (int m = 0; m < NMPD; ++m) acc[m] = Real(0);
-            for (int vl = sub; vl < SV; vl += TPC) {
-                const Vec<Real, N> fv4 = R[l * SV + vl];
-                Real fv[4] = {fv4.v[0], fv4.v[1], fv4.v[2], fv4.v[3]};
-                Real c[DIM];
+    for (int a = 0; a < DIM; ++a) xi[a] = make_float2(q.x[a * stride + v], q.x[a * stride + v + 32]);
+
+    // ---- 0. face records, in-block neighbours, coefficients
+    for (int t = threadIdx.x; t < nb * MAXF; t += NT) {
+        const int l = t / MAXF, k = t - l * MAXF, i = c0 + l, nf = g.info[i].x;
+        float4 fa = make_float4(0.0f, 0.0f, 0.0f, __int_as_float(NO_FACE));
+        int lj = -1, lower = 0, upper = 0, before = 0;
+        float sn[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
-                for (int a = 0; a < DIM; ++a) c[a] = sxi[a * SV + vl] - u4.v[a];
-                add_moments<Real, DIM>(acc, c, sxi[DIM * SV + vl], fv);
+        for (int m = 0; m < MAXF; ++m) {
+            int o = m < nf ? g.fnb[i * MAXF + m].y : -1;
+            if (o == l) o = -1;                           // a cell that is its own periodic neighbour
+            lower += o >= 0 && o < l;
+            upper += o > l;
+            if (m == k) lj = o;
+        }
+#pragma unroll
+        for (int m = 0; m < MAXF; ++m) {
+            const int o = m < nf ? g.fnb[i * MAXF + m].y : -1;
+            before += m < k && o >= 0 && o != l && (o < l) == (lj < l);
+        }
+        if (k < nf) {
+            const Face<float> F = load_face<float, DIM>(g.fgeo, i, k);
+            const int src = ORDER == 2 ? g.cface[i * MAXF + k] : g.fnb[i * MAXF + k].x;
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) sn[a] = F.sv * F.n[a];
+            if constexpr (DIM < 3) fa = make_float4(F.n[0], DIM > 1 ? F.n[1] : 0.0f, F.sv, __int_as_float(src));
+            else fa = make_float4(sn[0], sn[1], sn[2], __int_as_float(src));
+        }
+        Fa[t] = fa;
+        if (lj >= 0)
+            Gr[l * MAXF + (lj < l ? before : MAXF - 1 - before)] = make_float4(sn[0], sn[1], sn[2], __int_as_float(lj));
+        if (k == 0) Ln[l] = lower + 8 * upper;
+    }
+    for (int t = threadIdx.x; t < nb * 4; t += NT) {
+        const int l = t >> 2, k = t & 3;
+        const float *C = coef + (size_t)(c0 + l) * cf::NC;
+        float4 *o = Cs + l * S::CF;
+        if (k == 3) {
+            o[0] = *reinterpret_cast<const float4 *>(C + cf::U);
+            o[S::CF - 1] = *reinterpret_cast<const float4 *>(C + cf::RATE);
+        } else {
+            const float4 *P = reinterpret_cast<const float4 *>(C + cf::COMP + k * cf::CSZ);
+            const float4 x0 = P[0], x1 = P[1], x2 = P[2], x3 = P[3];   // A B T K1 | Q K2 | R1 S | R2 A2
+            const float Q[3] = {x1.x, x1.y, x1.z}, R1[3] = {x2.x, x2.y, x2.z}, R2[3] = {x3.x, x3.y, x3.z};
+            float w[4 * S::NK];
+            w[0] = x2.w;
+            w[1] = x0.y;
+            w[2] = x0.x;
+            w[3] = x3.w;
+            w[4] = x0.w;
+            w[5] = x1.w;
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) {
+                w[6 + 3 * a] = Q[a];
+                w[7 + 3 * a] = R1[a];
+                w[8 + 3 * a] = R2[a];
             }
 #pragma unroll
-            for (int m = 0; m < NM; ++m)
+            for (int a = 6 + 3 * DIM; a < 4 * S::NK; ++a) w[a] = 0.0f;
 #pragma unroll
-                for (int o = 1; o < TPC; o <<= 1) acc[m] += __shfl_xor_sync(gmask, acc[m], o);
-            if (sub == 0) {
-                Real *P = partial + ((size_t)(c0 + l) * gridDim.y + chunk) * NMPD;
+            for (int a = 0; a < S::NK; ++a)
+                o[1 + k * S::NK + a] = make_float4(w[4 * a], w[4 * a + 1], w[4 * a + 2], w[4 * a + 3]);
+        }
+    }
+    if (threadIdx.x < SV) {
 #pragma unroll
-                for (int m = 0; m < NM; ++m) P[m] = acc[m];
+        for (int a = 0; a < DIM; ++a) sxi[a * SV + threadIdx.x] = q.x[a * stride + chunk * SV + threadIdx.x];
+        sxi[DIM * SV + threadIdx.x] = q.w[chunk * SV + threadIdx.x];
+    }
+    __syncthreads();
+
+    // ---- 1. residuals and diagonals; a cell's loads are issued before its reference
+    for (int l = ty; l < nb; l += ROWS) {
+        const float *nbr = (ORDER == 2 ? fface : f_in) + (size_t)v * 4;
+        V<float, 4> fi[2], fk[FM][2], r[2];
+        const float *own = row_at(f_v, c0 + l, row);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) fi[u] = ldv<float, 4>(own, 32 * u);
+#pragma unroll
+        for (int k = 0; k < FM; ++k) {
+            const int src = __float_as_int(Fa[l * MAXF + k].w);
+            if (src < 0) continue;
+            const float *p = row_at(nbr, src, row);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) fk[k][u] = ldv<float, 4>(p, 32 * u);
+        }
+        float2 gp[4];
+        reference32<DIM>(Cs + l * S::CF, xi, gp);
+        const float4 cc = Cs[l * S::CF + S::CF - 1];      // rate, 1 / dt, sink
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            r[0].x[p] = (gp[p].x - fi[0].x[p]) * cc.x;
+            r[1].x[p] = (gp[p].y - fi[1].x[p]) * cc.x;
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) r[u].x[3] = fmaf(cc.z, fi[u].x[0], r[u].x[3]);
+        float d[2] = {cc.y + cc.x, cc.y + cc.x};
+#pragma unroll
+        for (int k = 0; k < FM; ++k) {
+            const float4 fa = Fa[l * MAXF + k];
+            const int src = __float_as_int(fa.w);
+            if (src == NO_FACE) continue;
+            float a[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                a[u] = (u ? xi[0].y : xi[0].x) * fa.x;
+                if constexpr (DIM > 1) a[u] = fmaf(u ? xi[1].y : xi[1].x, fa.y, a[u]);
+                if constexpr (DIM > 2) a[u] = fmaf(u ? xi[2].y : xi[2].x, fa.z, a[u]);
+                if constexpr (DIM < 3) {
+                    d[u] = fmaf(fa.z, fmaxf(a[u], 0.0f), d[u]);
+                    a[u] *= fa.z;
+                } else {
+                    d[u] += fmaxf(a[u], 0.0f);
+                }
             }
+            if (src >= 0) {
+                // order 2: the face's upwind value serves both directions (a = 0: zero, never
+                // written); order 1: the neighbour's value where it enters, the cell's where it
+                // leaves
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    vfma(ORDER == 2 ? -a[u] : -fminf(a[u], 0.0f), fk[k][u], r[u]);
+                    if (ORDER == 1) vfma(-fmaxf(a[u], 0.0f), fi[u], r[u]);
+                }
+                continue;
+            }
+            const int bf = -1 - src, tab = g.bf_tab[bf];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                V<float, 4> fv;
+                if (tab >= 0) {
+                    // mirror plane: what enters at this velocity leaves at its mirror image
+                    fv = ldv<float, 4>(row_at(f_in, c0 + l, row), g.refl_v[(size_t)tab * stride + v + 32 * u]);
+                } else {
+                    const float *B = bcoef + (size_t)bf * bc::NB;
+                    float c2 = 0.0f;
+#pragma unroll
+                    for (int m = 0; m < DIM; ++m) {
+                        const float c = (u ? xi[m].y : xi[m].x) - B[bc::U + m];
+                        c2 = fmaf(c, c, c2);
+                    }
+                    const float E = B[bc::A] * fexp(-B[bc::B] * c2);
+                    fv.x[0] = E * B[bc::M0];
+                    fv.x[1] = E * B[bc::MH];
+                    fv.x[2] = E * B[bc::M1];
+                    fv.x[3] = E * B[bc::M2];
+                }
+                vfma(-fminf(a[u], 0.0f), fv, r[u]);
+                vfma(-fmaxf(a[u], 0.0f), fi[u], r[u]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            R[l * SV + tx + 32 * u] = make_float4(r[u].x[0], r[u].x[1], r[u].x[2], r[u].x[3]);
+            Dg[l * SV + tx + 32 * u] = rcp_refined(d[u]);
+        }
+    }
+    __syncthreads();
+
+    // ---- 2. Gauss-Seidel inside the block, one warp; the neighbour just relaxed stays in
+    // registers.  The other warps meanwhile load f for phase 3.
+    const float *R1 = reinterpret_cast<const float *>(R);
+    constexpr int PRE = 2;                                // cells of phase 3 loaded ahead
+    V<float, 4> fo[PRE][2];
+    auto load_f = [&](int l, V<float, 4> (&x)[2]) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) x[u] = ldv<float, 4>(row_at(f_v, c0 + l, row), 32 * u);
+    };
+    auto load_ahead = [&] {
+#pragma unroll
+        for (int j = 0; j < PRE; ++j)
+            if (ty + j * ROWS < nb) load_f(ty + j * ROWS, fo[j]);
+    };
+    if (!RESID && ty != 0) load_ahead();
+    if (!RESID && ty == 0) {
+        auto entering = [&](const float4 &gr, float (&a)[2]) {        // min(S/V xi . n, 0)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                a[u] = (u ? xi[0].y : xi[0].x) * gr.x;
+                if constexpr (DIM > 1) a[u] = fmaf(u ? xi[1].y : xi[1].x, gr.y, a[u]);
+                if constexpr (DIM > 2) a[u] = fmaf(u ? xi[2].y : xi[2].x, gr.z, a[u]);
+                a[u] = fminf(a[u], 0.0f);
+            }
+        };
+        V<float, 4> prev[2];
+        auto pass = [&](bool up) {
+            const int step = up ? -1 : 1;
+            int l = up ? nb - 1 : 0;
+            for (int t = 0; t < nb; ++t, l += step) {
+                const int n = up ? Ln[l] >> 3 : Ln[l] & 7;
+                float inv[2];
+                V<float, 4> own[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    inv[u] = Dg[l * SV + tx + 32 * u];
+                    own[u] = ldv<float, 4>(R1, l * SV + tx + 32 * u);
+                }
+                if (n > 0) {
+                    const float4 g0 = Gr[l * MAXF + (up ? MAXF - 1 : 0)];
+                    const int lj = __float_as_int(g0.w);
+                    if (lj != l - step) {
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) prev[u] = ldv<float, 4>(R1, lj * SV + tx + 32 * u);
+                    }
+                    // up: the sum of a dq over the neighbours; else r minus it
+                    V<float, 4> s[2] = {up ? vsplat<float, 4>(0.0f) : own[0], up ? vsplat<float, 4>(0.0f) : own[1]};
+                    float a[2];
+                    entering(g0, a);
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) vfma(up ? a[u] : -a[u], prev[u], s[u]);
+                    for (int e = 1; e < n; ++e) {
+                        const float4 gr = Gr[l * MAXF + (up ? MAXF - 1 - e : e)];
+                        entering(gr, a);
+#pragma unroll
+                        for (int u = 0; u < 2; ++u)
+                            vfma(up ? a[u] : -a[u], ldv<float, 4>(R1, __float_as_int(gr.w) * SV + tx + 32 * u), s[u]);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        if (up) {
+                            prev[u] = own[u];
+                            vfma(-inv[u], s[u], prev[u]);
+                        } else {
+                            prev[u] = vmul(s[u], vsplat<float, 4>(inv[u]));
+                        }
+                    }
+                } else {
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) prev[u] = up ? own[u] : vmul(own[u], vsplat<float, 4>(inv[u]));
+                }
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+                    R[l * SV + tx + 32 * u] = make_float4(prev[u].x[0], prev[u].x[1], prev[u].x[2], prev[u].x[3]);
+            }
+        };
+        pass(false);
+        pass(true);
+        load_ahead();
+    }
+    __syncthreads();
+
+    // ---- 3. f^{k+1/2} = f^k + delta
+    if constexpr (!RESID) {
+        auto update = [&](int l, const V<float, 4> (&x)[2]) {
+            float *to = const_cast<float *>(row_at(f_out + (size_t)v * 4, c0 + l, row));
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                V<float, 4> t = vadd(ldv<float, 4>(R1, l * SV + tx + 32 * u), x[u]);
+                if (g.pos_theta > 0.0f) {   // the positivity bound of the implicit update
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) t.x[p] = fmaxf(t.x[p], g.pos_theta * x[u].x[p]);
+                }
+                const float4 o = make_float4(t.x[0], t.x[1], t.x[2], t.x[3]);
+                R[l * SV + tx + 32 * u] = o;
+                *reinterpret_cast<float4 *>(to + 128 * u) = o;
+            }
+        };
+        V<float, 4> more[PRE][2];
+        for (int l0 = ty; l0 < nb; l0 += PRE * ROWS) {
+            const int l1 = l0 + PRE * ROWS;
+#pragma unroll
+            for (int j = 0; j < PRE; ++j)
+                if (l1 + j * ROWS < nb) load_f(l1 + j * ROWS, more[j]);
+#pragma unroll
+            for (int j = 0; j < PRE; ++j)
+                if (l0 + j * ROWS < nb) update(l0 + j * ROWS, fo[j]);
+#pragma unroll
+            for (int j = 0; j < PRE; ++j)
+#pragma unroll
+                for (int u = 0; u < 2; ++u) fo[j][u] = more[j][u];
+        }
+        __syncthreads();
+    }
+
+    // ---- 4. velocity moments per (cell, chunk), eight lanes per cell
+    constexpr int NM = n_gas_moments<DIM>(), NB0 = 1 + DIM + DIM * (DIM + 1) / 2 + DIM, NMPD = Lay<DIM>::NMP;
+    const int sub = threadIdx.x & 7;
+    for (int l = threadIdx.x >> 3; l < nb; l += NT / 8) {
+        const float4 u4 = *reinterpret_cast<const float4 *>(coef + (size_t)((c0 + l) / MT * MT) * cf::NC + cf::U);
+        const float uu[3] = {u4.x, u4.y, u4.z};
+        // lin: planes (F0, H0) and (f1, f2) times 1, c; hi: F0 times cc, c |c|^2
+        float2 lin[DIM + 1][2];
+        float hi[NB0 - 1 - DIM];
+#pragma unroll
+        for (int b = 0; b <= DIM; ++b) lin[b][0] = lin[b][1] = dup2(0.0f);
+#pragma unroll
+        for (int b = 0; b < NB0 - 1 - DIM; ++b) hi[b] = 0.0f;
+#pragma unroll 2
+        for (int vl = sub; vl < SV; vl += 8) {
+            const float4 x = R[l * SV + vl];
+            const float w = sxi[DIM * SV + vl];
+            float c[DIM], c2 = 0.0f, wc[DIM];
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) {
+                c[a] = sxi[a * SV + vl] - uu[a];
+                c2 = fmaf(c[a], c[a], c2);
+            }
+            const float2 p0 = __fmul2_rn(dup2(w), make_float2(x.x, x.y)), p1 = __fmul2_rn(dup2(w), make_float2(x.z, x.w));
+            lin[0][0] = __fadd2_rn(lin[0][0], p0);
+            lin[0][1] = __fadd2_rn(lin[0][1], p1);
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) {
+                lin[1 + a][0] = __ffma2_rn(dup2(c[a]), p0, lin[1 + a][0]);
+                lin[1 + a][1] = __ffma2_rn(dup2(c[a]), p1, lin[1 + a][1]);
+                wc[a] = p0.x * c[a];
+            }
+            int m = 0;
+#pragma unroll
+            for (int a = 0; a < DIM; ++a)
+#pragma unroll
+                for (int b = a; b < DIM; ++b, ++m) hi[m] = fmaf(wc[a], c[b], hi[m]);
+#pragma unroll
+            for (int a = 0; a < DIM; ++a, ++m) hi[m] = fmaf(wc[a], c2, hi[m]);
+        }
+        float acc[24];
+        int m = 0;
+#pragma unroll
+        for (int b = 0; b <= DIM; ++b) acc[m++] = lin[b][0].x;
+#pragma unroll
+        for (int b = 0; b < NB0 - 1 - DIM; ++b) acc[m++] = hi[b];
+#pragma unroll
+        for (int p = (DIM < 3 ? 1 : 2); p < 4; ++p)
+#pragma unroll
+            for (int b = 0; b <= DIM; ++b) acc[m++] = p & 1 ? lin[b][p >> 1].y : lin[b][p >> 1].x;
+#pragma unroll
+        for (int b = NM; b < 24; ++b) acc[b] = 0.0f;
+        fold8(acc, sub);
+        float *P = partial + ((size_t)(c0 + l) * gridDim.y + chunk) * NMPD;
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {
+            const int b = fold8_index(sub, t);
+            if (b < NM) P[b] = acc[t];
         }
     }
 }
@@ -2267,20 +2696,31 @@ static cudaError_t sweep_t(cudaStream_t s, const Geom<Real> &g, const Quad<Real>
                            const Real *bcoef, const Real *f_in, const Real *fface, Real *f_out, Real *partial) {
     const bool tc = N == 4 && sizeof(Real) == 4 && DIM < 3 && g.tc && !RESID;
     if (g.tc && (DIM == 3 || MT % g.block != 0)) return cudaErrorInvalidValue;
-    const size_t smem = sweep_smem_bytes(g.block, N, DIM, sizeof(Real), tc);
     dim3 grid((g.n_cells + g.block - 1) / g.block, q.n_pad / SV);
-    auto run = [&](auto kern, int rows) {
+    auto run = [&](auto kern, dim3 block, size_t smem) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        kern<<<grid, dim3(SV, rows), smem, s>>>(g, q, coef, bcoef, f_in, fface, f_out, partial);
+        kern<<<grid, block, smem, s>>>(g, q, coef, bcoef, f_in, fface, f_out, partial);
         return cudaGetLastError();
     };
-    // FP64 on fewer CTAs than SMs (1-D meshes of a few hundred cells): a CTA's time is its
-    // longest chain of FP64 instructions, so its cells are dealt to 8 rows instead of 2
-    // (64 cells x 32 velocities: 72 -> 53 us; 800 x 64: 71 -> 55 us)
-    if constexpr (std::is_same<Real, double>::value)
-        if ((long long)grid.x * grid.y < 152) return run(k_sweep<Real, N, DIM, ORDER, RESID, 8>, 8);
-    return run(k_sweep<Real, N, DIM, ORDER, RESID>, SROWS);
+    const size_t smem = sweep_smem_bytes(g.block, N, DIM, sizeof(Real), tc);
+    if constexpr (N == 4 && std::is_same<Real, float>::value) {
+        if constexpr (DIM < 3 && !RESID)
+            if (tc) return run(k_sweep<Real, N, DIM, ORDER>, dim3(SV, SROWS), smem);
+        // segments and triangles, whose faces' values leave room for one more CTA per SM, or
+        // any cells (the 20 000-triangle cavity as "any cells": 326 us, as triangles 306 us)
+        const size_t bytes = S32<DIM>::bytes(g.block);
+        if (DIM < 3 && g.max_faces <= DIM + 1) return run(k_sweep_gas32<DIM, ORDER, RESID, DIM + 1>, dim3(128), bytes);
+        return run(k_sweep_gas32<DIM, ORDER, RESID, MAXF>, dim3(128), bytes);
+    } else {
+        // FP64 on fewer CTAs than SMs (1-D meshes of a few hundred cells): a CTA's time is its
+        // longest chain of FP64 instructions, so its cells are dealt to 8 rows instead of 2
+        // (64 cells x 32 velocities: 72 -> 53 us; 800 x 64: 71 -> 55 us)
+        if constexpr (std::is_same<Real, double>::value)
+            if ((long long)grid.x * grid.y < 152)
+                return run(k_sweep<Real, N, DIM, ORDER, RESID, 8>, dim3(SV, 8), smem);
+        return run(k_sweep<Real, N, DIM, ORDER, RESID>, dim3(SV, SROWS), smem);
+    }
 }
 
 template <typename Real>
