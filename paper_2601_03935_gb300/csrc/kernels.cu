@@ -2531,6 +2531,114 @@ __global__ void k_equilibrium(int n_cells, Quad<Real> vq, Quad<Real> oq, ModelDe
     for (int o = threadIdx.x; o < oq.n_pad; o += blockDim.x) I[(size_t)i * oq.n_pad + o] = (Real)B;
 }
 
+// ---- two-word FP32: a value as x + y with |y| at most about a unit of x's last place.  FP32
+// storage needs its equilibria to FP32 rounding, which exp in FP32 alone does not give (its
+// argument reaches 100); an FP64 instruction takes the time of some 70 of these.
+__device__ __forceinline__ float2 two_sum(float a, float b) {
+    const float s = __fadd_rn(a, b), t = __fadd_rn(s, -a);
+    return make_float2(s, __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -t)), __fadd_rn(b, -t)));
+}
+__device__ __forceinline__ float2 two_sum_ordered(float a, float b) {   // |a| >= |b|
+    const float s = __fadd_rn(a, b);
+    return make_float2(s, __fadd_rn(b, -__fadd_rn(s, -a)));
+}
+__device__ __forceinline__ float2 two_diff(float x, float uh, float ul) {   // x - (uh + ul)
+    const float2 d = two_sum(x, -uh);
+    return make_float2(d.x, __fadd_rn(d.y, -ul));
+}
+__device__ __forceinline__ float2 square2(float2 d) {
+    const float p = __fmul_rn(d.x, d.x);
+    return make_float2(p, fmaf(__fadd_rn(d.x, d.x), d.y, fmaf(d.x, d.x, -p)));
+}
+__device__ __forceinline__ float2 add2w(float2 a, float2 b) {
+    const float2 s = two_sum(a.x, b.x);
+    return make_float2(s.x, __fadd_rn(s.y, __fadd_rn(a.y, b.y)));
+}
+// 2^(j / 8)
+__constant__ float2 EXP2_8TH[8] = {
+    {1.000000000e+00f, 0.000000000e+00f},   {1.090507746e+00f, -1.307753994e-08f},
+    {1.189207077e+00f, 3.797635273e-08f},   {1.296839595e+00f, -4.018999533e-08f},
+    {1.414213538e+00f, 2.420323497e-08f},   {1.542210817e+00f, 8.070904833e-09f},
+    {1.681792855e+00f, -2.475532668e-08f},  {1.834008098e+00f, -1.123927795e-08f}};
+// 2^(s c2) = v 2^k: 2^(j/8) from a table times e^r, |r| <= ln 2 / 16, by its Taylor sum
+struct Exp2 {
+    float2 v;
+    float scale;       // v carries the other half of the exponent, so that both are normal numbers
+};
+__device__ __forceinline__ Exp2 exp2_two(const float2 *__restrict__ table, float2 s, float2 c2) {
+    float y = __fmul_rn(s.x, c2.x), yl = fmaf(s.y, c2.x, fmaf(s.x, c2.y, fmaf(s.x, c2.x, -y)));
+    if (fabsf(y) > 250.0f) {         // 0 or infinite in FP32
+        y = copysignf(250.0f, y);
+        yl = 0.0f;
+    }
+    const float k = rintf(8.0f * y), f = fmaf(-0.125f, k, y);
+    const float2 g = two_sum_ordered(f, yl);
+    const float L = 0.693147182f, Ll = -1.90465421e-9f;      // ln 2
+    const float r = __fmul_rn(g.x, L), rl = fmaf(g.y, L, fmaf(g.x, Ll, fmaf(g.x, L, -r)));
+    const float p = fmaf(r, fmaf(r, fmaf(r, 1.0f / 120.0f, 1.0f / 24.0f), 1.0f / 6.0f), 0.5f);
+    const float2 q = two_sum_ordered(r, fmaf(__fmul_rn(r, r), p, rl));      // e^r - 1
+    const int ki = (int)k, n = ki >> 3, n1 = n >> 1;
+    const float2 T = table[ki & 7];
+    const float t = __fmul_rn(T.x, q.x);
+    const float2 e = two_sum_ordered(T.x, t);
+    const float el = __fadd_rn(e.y, fmaf(T.x, q.y, fmaf(T.y, q.x, __fadd_rn(T.y, fmaf(T.x, q.x, -t)))));
+    const float s1 = __int_as_float((n1 + 127) << 23);
+    Exp2 o;
+    o.v = make_float2(__fmul_rn(e.x, s1), __fmul_rn(el, s1));
+    o.scale = __int_as_float((n - n1 + 127) << 23);
+    return o;
+}
+__device__ __forceinline__ float scaled(float2 N, const Exp2 &e) {   // (N 2^..) to FP32
+    const float r = __fmul_rn(N.x, e.v.x);
+    return __fmul_rn(__fadd_rn(r, fmaf(N.x, e.v.y, fmaf(N.y, e.v.x, fmaf(N.x, e.v.x, -r)))), e.scale);
+}
+
+// The equilibrium in FP32 storage: the start of a run writes f once, and in FP64 arithmetic
+// (the kernel above) its time is that of 17 FP64 instructions per velocity.  Here each cell's
+// constants are formed in FP64 by one thread and kept as two FP32 words, and a velocity takes
+// about 100 FP32 instructions; a value is within 0.502 units in the last place (0.500 before).
+template <int DIM>
+__global__ void __launch_bounds__(256) k_equilibrium32(int n_cells, int cells, Quad<float> vq, Quad<float> oq,
+                                                       ModelDev m, const double *__restrict__ F,
+                                                       float *__restrict__ f, float *__restrict__ I) {
+    constexpr int MAXC = 16;                                   // cells of a CTA at most
+    __shared__ float2 tab[8], K[MAXC][DIM + 5];                // u, -log2 e / (2 T), the four planes' factors
+    __shared__ float B[MAXC];
+    const int c0 = blockIdx.x * cells, nc = min(cells, n_cells - c0);
+    if (threadIdx.x >= 32 && threadIdx.x < 40) tab[threadIdx.x - 32] = EXP2_8TH[threadIdx.x - 32];
+    if (threadIdx.x < nc) {
+        const double *M = F + (size_t)(c0 + threadIdx.x) * NF;
+        auto put = [&](int k, double x) {
+            const float h = (float)x;
+            K[threadIdx.x][k] = make_float2(h, (float)(x - (double)h));
+        };
+        const double Tt = M[4];
+        const double norm = M[0] * pow_neg_half_dim<DIM>(6.283185307179586 * Tt);
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) put(a, M[1 + a]);
+        put(DIM, -1.4426950408889634 / (2.0 * Tt));
+        put(DIM + 1, norm);
+        put(DIM + 2, (3 - DIM) * Tt * norm);
+        put(DIM + 3, 0.5 * m.d_r * M[5] * norm);
+        put(DIM + 4, vib_energy<double>(m, M[6]) * norm);
+        B[threadIdx.x] = (float)(m.sigma_R * M[7] * M[7] * M[7] * M[7] / 3.141592653589793);
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31, nw = vq.n_pad / 32;
+    for (int t = threadIdx.x >> 5; t < nc * nw; t += 8) {
+        const int c = t / nw, v = (t - c * nw) * 32 + lane;
+        float2 c2 = square2(two_diff(vq.x[v], K[c][0].x, K[c][0].y));
+#pragma unroll
+        for (int a = 1; a < DIM; ++a)
+            c2 = add2w(c2, square2(two_diff(vq.x[a * vq.n_pad + v], K[c][a].x, K[c][a].y)));
+        const Exp2 e = exp2_two(tab, K[c][DIM], c2);
+        *reinterpret_cast<float4 *>(f + ((size_t)(c0 + c) * vq.n_pad + v) * 4) =
+            make_float4(scaled(K[c][DIM + 1], e), DIM < 3 ? scaled(K[c][DIM + 2], e) : 0.0f, scaled(K[c][DIM + 3], e),
+                        scaled(K[c][DIM + 4], e));
+    }
+    for (int t = threadIdx.x; t < nc * oq.n_pad; t += 256) I[(size_t)c0 * oq.n_pad + t] = B[t / oq.n_pad];
+}
+
 // ------------------------------------------------------------------ launchers
 #define GSIS_DISPATCH_DIM(dim, ...)                    \
     switch (dim) {                                     \
@@ -2775,7 +2883,14 @@ cudaError_t launch_finish(cudaStream_t s, int dim, int n_cells, int n_chunks, in
 template <typename Real>
 cudaError_t launch_equilibrium(cudaStream_t s, int dim, int n_cells, const Quad<Real> &vq, const Quad<Real> &oq,
                                const ModelDev &m, const double *fields, Real *f, Real *I) {
-    GSIS_DISPATCH_DIM3(dim, (k_equilibrium<Real, DIM><<<n_cells, 256, 0, s>>>(n_cells, vq, oq, m, fields, f, I)));
+    if constexpr (std::is_same<Real, float>::value) {
+        // a cell's constants cost one thread about as much as 70 velocities cost a warp: 16 cells
+        // to a CTA, fewer where that leaves SMs without one
+        const int cells = std::max(1, std::min(16, n_cells / 304)), grid = (n_cells + cells - 1) / cells;
+        GSIS_DISPATCH_DIM3(dim, (k_equilibrium32<DIM><<<grid, 256, 0, s>>>(n_cells, cells, vq, oq, m, fields, f, I)));
+    } else {
+        GSIS_DISPATCH_DIM3(dim, (k_equilibrium<Real, DIM><<<n_cells, 256, 0, s>>>(n_cells, vq, oq, m, fields, f, I)));
+    }
     return cudaGetLastError();
 }
 
