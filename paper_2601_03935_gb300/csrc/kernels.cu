@@ -2266,9 +2266,64 @@ __global__ void k_kbflux_combine(MacroGeom g, const double *__restrict__ raw, do
 // tile's first cell, the shift every gas moment pass uses):
 // with delta = S_c / rho the flow velocity is u0 + delta and every central moment
 // follows from the binomial shift by delta.
+// Sums of a cell's gas moment partials over the chunks first, first + step, ...: in FP32 two
+// words per sum (Knuth's two-sum, the rounding error of every addition carried in the second
+// word, itself summed plainly), off the slow FP64 pipe.  The fields stay within 1e-5 of the
+// FP64 oracle from 13 chunks (784 velocities) up to 216 (13 824 velocities of the 3-D capsule)
+// in the parity tests.
+template <typename Real, int NM>
+struct MomentSum {
+    double s[NM];
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int k = 0; k < NM; ++k) s[k] = 0.0;
+    }
+    __device__ __forceinline__ void add(int k, double x) { s[k] += x; }
+    __device__ __forceinline__ double word(int k) const { return s[k]; }
+    __device__ __forceinline__ void add_word(int k, double x) { s[k] += x; }
+    __device__ __forceinline__ double value(int k) const { return s[k]; }
+};
+template <int NM>
+struct MomentSum<float, NM> {
+    float hi[NM], lo[NM];
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int k = 0; k < NM; ++k) hi[k] = lo[k] = 0.0f;
+    }
+    __device__ __forceinline__ void add(int k, float b) {
+        const float a = hi[k], t = a + b, bv = t - a;
+        lo[k] += (a - (t - bv)) + (b - bv);
+        hi[k] = t;
+    }
+    __device__ __forceinline__ float2 word(int k) const { return make_float2(hi[k], lo[k]); }
+    __device__ __forceinline__ void add_word(int k, float2 x) {
+        add(k, x.x);
+        lo[k] += x.y;
+    }
+    __device__ __forceinline__ double value(int k) const { return to_double(hi[k]) + to_double(lo[k]); }
+};
 template <typename Real, int DIM>
-__device__ __forceinline__ void finish_cell(int i, int n_chunks, int o_chunks, const ModelDev &m,
-                                            const Real *__restrict__ coef, const Real *__restrict__ partial,
+__device__ __forceinline__ void sum_chunks(int i, int first, int step, int n_chunks, const Real *__restrict__ partial,
+                                           MomentSum<Real, n_gas_moments<DIM>()> &S) {
+    constexpr int NM = n_gas_moments<DIM>(), NMPD = Lay<DIM>::NMP;   // partial stride
+    static_assert(NMPD % 4 == 0 && NM <= NMPD && NMO == 4 && DIM + 1 <= NMO, "partial records are read as 4-vectors");
+    S.zero();
+#pragma unroll 2
+    for (int c = first; c < n_chunks; c += step) {
+        const Real *P = partial + ((size_t)i * n_chunks + c) * NMPD;
+#pragma unroll
+        for (int q = 0; q < NMPD / 4; ++q) {
+            const Vec<Real, 4> p4 = vload<Real, 4>(P + 4 * q);
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (4 * q + e < NM) S.add(4 * q + e, p4.v[e]);
+        }
+    }
+}
+
+template <typename Real, int DIM>
+__device__ __forceinline__ void finish_cell(int i, int o_chunks, const ModelDev &m, const Real *__restrict__ coef,
+                                            const MomentSum<Real, n_gas_moments<DIM>()> &sums,
                                             const Real *__restrict__ opartial, const double *__restrict__ vol,
                                             const double *__restrict__ F_old, double *__restrict__ F_new,
                                             double *__restrict__ eps_terms, int *__restrict__ err, int have_old,
@@ -2277,8 +2332,6 @@ __device__ __forceinline__ void finish_cell(int i, int n_chunks, int o_chunks, c
     constexpr int MH = 3 - DIM;
     double S[NM];
     double Ph[1 + DIM];
-    constexpr int NMPD = Lay<DIM>::NMP;   // partial stride
-    static_assert(NMPD % 4 == 0 && NM <= NMPD && NMO == 4 && DIM + 1 <= NMO, "partial records are read as 4-vectors");
     if (X) {
         // per-cell sums of a velocity-sharded context, already summed over the ranks
         // (velocity shards are built for 1-D and 2-D)
@@ -2289,46 +2342,9 @@ __device__ __forceinline__ void finish_cell(int i, int n_chunks, int o_chunks, c
 #pragma unroll
             for (int k = 0; k <= DIM; ++k) Ph[k] = X[(size_t)i * NXC + NMP + k];
         }
-    } else if constexpr (std::is_same<Real, float>::value) {
-        // FP32 partials: a compensated FP32 sum (Knuth's two-sum, the rounding error of
-        // every addition carried in lo, lo itself summed plainly), off the slow FP64 pipe.
-        // The fields stay within 1e-5 of the FP64 oracle from 13 chunks (784 velocities)
-        // up to 216 (13 824 velocities of the 3-D capsule) in the parity tests.
-        float hi[NM], lo[NM];
-#pragma unroll
-        for (int k = 0; k < NM; ++k) hi[k] = lo[k] = 0.0f;
-#pragma unroll 2
-        for (int c = 0; c < n_chunks; ++c) {
-            const Real *P = partial + ((size_t)i * n_chunks + c) * NMPD;
-#pragma unroll
-            for (int q = 0; q < NMPD / 4; ++q) {
-                const Vec<Real, 4> p4 = vload<Real, 4>(P + 4 * q);
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    if (4 * q + e < NM) {
-                        const int k = 4 * q + e;
-                        const float a = hi[k], b = p4.v[e], t = a + b, bv = t - a;
-                        lo[k] += (a - (t - bv)) + (b - bv);
-                        hi[k] = t;
-                    }
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < NM; ++k) S[k] = to_double(hi[k]) + to_double(lo[k]);
     } else {
 #pragma unroll
-        for (int k = 0; k < NM; ++k) S[k] = 0.0;
-#pragma unroll 2
-        for (int c = 0; c < n_chunks; ++c) {
-            const Real *P = partial + ((size_t)i * n_chunks + c) * NMPD;
-#pragma unroll
-            for (int q = 0; q < NMPD / 4; ++q) {
-                const Vec<Real, 4> p4 = vload<Real, 4>(P + 4 * q);
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    if (4 * q + e < NM) S[4 * q + e] += (double)p4.v[e];
-            }
-        }
+        for (int k = 0; k < NM; ++k) S[k] = sums.value(k);
     }
     if (!X) {
 #pragma unroll
@@ -2459,44 +2475,63 @@ __device__ __forceinline__ void finish_cell(int i, int n_chunks, int o_chunks, c
 // each CTA adds its 32 cells in a fixed shuffle order, and the last CTA to finish (counted
 // with an atomic ticket after a fence, no waiting) adds the CTA partials in a fixed order,
 // so the result does not depend on scheduling.
-template <typename Real, int DIM>
-__global__ void __launch_bounds__(32) k_finish(int n_cells, int n_chunks, int o_chunks, ModelDev m,
-                                               const Real *__restrict__ coef, const Real *__restrict__ partial,
-                                               const Real *__restrict__ opartial, const double *__restrict__ vol,
-                                               const double *__restrict__ F_old, double *__restrict__ F_new,
-                                               double *__restrict__ eps_terms, int *__restrict__ err, int have_old,
-                                               int reduce, double *__restrict__ eps_part,
-                                               unsigned int *__restrict__ ticket, double *__restrict__ eps_sums,
-                                               const double *__restrict__ X) {
-    const int i = blockIdx.x * 32 + threadIdx.x;
+template <typename Real, int DIM, int FW>
+__global__ void __launch_bounds__(32 * FW) k_finish(int n_cells, int n_chunks, int o_chunks, ModelDev m,
+                                                    const Real *__restrict__ coef, const Real *__restrict__ partial,
+                                                    const Real *__restrict__ opartial, const double *__restrict__ vol,
+                                                    const double *__restrict__ F_old, double *__restrict__ F_new,
+                                                    double *__restrict__ eps_terms, int *__restrict__ err, int have_old,
+                                                    int reduce, double *__restrict__ eps_part,
+                                                    unsigned int *__restrict__ ticket, double *__restrict__ eps_sums,
+                                                    const double *__restrict__ X) {
+    constexpr int NM = n_gas_moments<DIM>();
+    using Sum = MomentSum<Real, NM>;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane;
+    Sum S;
+    if (i < n_cells && !X) sum_chunks<Real, DIM>(i, w, FW, n_chunks, partial, S);
+    if constexpr (FW > 1) {
+        __shared__ double words[FW - 1][NM][32];     // a double, or the two FP32 words of a sum
+        using Word = decltype(S.word(0));
+        if (w > 0) {
+#pragma unroll
+            for (int k = 0; k < NM; ++k) *reinterpret_cast<Word *>(&words[w - 1][k][lane]) = S.word(k);
+        }
+        __syncthreads();
+        if (w > 0) return;
+#pragma unroll
+        for (int v = 0; v < FW - 1; ++v)
+#pragma unroll
+            for (int k = 0; k < NM; ++k) S.add_word(k, *reinterpret_cast<const Word *>(&words[v][k][lane]));
+    }
     double E[NEPS];
     for (int q = 0; q < NEPS; ++q) E[q] = 0.0;
     if (i < n_cells)
-        finish_cell<Real, DIM>(i, n_chunks, o_chunks, m, coef, partial, opartial, vol, F_old, F_new, eps_terms, err,
-                               have_old, X, E);
+        finish_cell<Real, DIM>(i, o_chunks, m, coef, S, opartial, vol, F_old, F_new, eps_terms, err, have_old, X, E);
     if (!reduce) return;
 #pragma unroll
     for (int q = 0; q < NEPS; ++q)
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) E[q] += __shfl_xor_sync(0xffffffffu, E[q], o);
-    __shared__ bool last;
-    if (threadIdx.x == 0) {
+    bool last = false;
+    if (lane == 0) {
         for (int q = 0; q < NEPS; ++q) eps_part[(size_t)blockIdx.x * NEPS + q] = E[q];
         __threadfence();
         last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     }
-    __syncthreads();
-    if (!last) return;
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
     __threadfence();
     double acc[NEPS];
     for (int q = 0; q < NEPS; ++q) acc[q] = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += 32)
+#pragma unroll 4
+    for (int b = lane; b < (int)gridDim.x; b += 32)
+#pragma unroll
         for (int q = 0; q < NEPS; ++q) acc[q] += __ldcg(eps_part + (size_t)b * NEPS + q);   // L2: other CTAs' writes
 #pragma unroll
     for (int q = 0; q < NEPS; ++q)
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
-    if (threadIdx.x == 0) {
+    if (lane == 0) {
         for (int q = 0; q < NEPS; ++q) eps_sums[q] = acc[q];
         *ticket = 0u;
     }
@@ -2870,12 +2905,14 @@ cudaError_t launch_finish(cudaStream_t s, int dim, int n_cells, int n_chunks, in
                           const double *fields_old, double *fields_new, double *eps_terms, int *err_flag,
                           int have_old, double *eps_part, unsigned int *ticket, double *eps_sums,
                           const double *X) {
-    const int nt = 32, nbk = (n_cells + nt - 1) / nt;
-    const int reduce = eps_sums != nullptr;
-    GSIS_DISPATCH_DIM3(dim, (k_finish<Real, DIM><<<nbk, nt, 0, s>>>(n_cells, n_chunks, o_chunks, m, coef, partial,
-                                                                    opartial, vol, fields_old, fields_new, eps_terms,
-                                                                    err_flag, have_old, reduce, eps_part, ticket,
-                                                                    eps_sums, X)));
+    const int nbk = (n_cells + 31) / 32, reduce = eps_sums != nullptr;
+    auto go = [&](auto kern, int warps) {
+        kern<<<nbk, 32 * warps, 0, s>>>(n_cells, n_chunks, o_chunks, m, coef, partial, opartial, vol, fields_old,
+                                        fields_new, eps_terms, err_flag, have_old, reduce, eps_part, ticket, eps_sums,
+                                        X);
+    };
+    if (n_chunks >= 4 && !X) GSIS_DISPATCH_DIM3(dim, go(k_finish<Real, DIM, 4>, 4))
+    else GSIS_DISPATCH_DIM3(dim, go(k_finish<Real, DIM, 1>, 1))
     return cudaGetLastError();
 }
 
