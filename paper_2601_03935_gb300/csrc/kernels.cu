@@ -24,6 +24,7 @@
 // epilogue when a relaxation block lies inside one tile.
 #include <algorithm>
 #include <cmath>
+#include <cooperative_groups.h>
 #include <cstdio>
 #include <type_traits>
 
@@ -690,7 +691,7 @@ __global__ void __launch_bounds__(32 * SLOPE_ROWS) k_slopes64(Geom<double> g, in
     constexpr bool ZH = DIM == 3 && N == 4;      // the H0 plane of 3-D: slope not limited (phi = 1)
     constexpr int MS = Lay<DIM>::MAXS, LW = Lay<DIM>::LW;
     const int v = blockIdx.y * 32 + threadIdx.x;
-    const int j = blockIdx.x * SLOPE_ROWS + threadIdx.y;
+    const int j = blockIdx.x * blockDim.y + threadIdx.y;
     if (j >= g.n_cells || blockIdx.y * 32 >= n) return;     // no face value of a padding velocity is used
     const V<double, N> fj = ldv<double, N>(f, (size_t)j * n_pad + v);
     const int4 info = g.info[j];
@@ -849,7 +850,10 @@ __host__ __device__ constexpr size_t sweep_main_bytes(int block, int planes, int
 //     operator, one thread per velocity (row 0);
 //  3. f^{k+1/2} = f^k + delta, staged in shared memory;
 //  4. velocity moments per (cell, chunk), eight lanes per cell.
-template <typename Real, int N, int DIM, int ORDER, bool RESID = false, int ROWS = SROWS>
+// CL > 1: a cluster of CL CTAs takes the block.  Its cells are dealt to the rows of all of
+// them; the residuals go to the first CTA's shared memory, which relaxes, and every CTA
+// updates and sums its own cells.
+template <typename Real, int N, int DIM, int ORDER, bool RESID = false, int ROWS = SROWS, int CL = 1>
 __global__ void __launch_bounds__(SV * ROWS, sizeof(Real) == 4 ? (DIM < 3 ? 8 : 6) : 1) k_sweep(Geom<Real> g, Quad<Real> q, const Real *__restrict__ coef,
                                                       const Real *__restrict__ bcoef, const Real *__restrict__ f_in,
                                                       const Real *__restrict__ fface, Real *__restrict__ f_out,
@@ -872,11 +876,25 @@ __global__ void __launch_bounds__(SV * ROWS, sizeof(Real) == 4 ? (DIM < 3 ? 8 : 
     signed char *Lg = reinterpret_cast<signed char *>(sxi + (DIM + 1) * SV);   // [block][MAXF] in-block neighbour or -1
     tcm::Ctl *ctl = reinterpret_cast<tcm::Ctl *>(Lg + ((g.block * MAXF + 15) & ~15));
     const int tx = threadIdx.x, ty = threadIdx.y;
-    const int c0 = blockIdx.x * g.block;
+    const int rank = CL > 1 ? blockIdx.x % CL : 0, row0 = rank * ROWS + ty;
+    const int c0 = blockIdx.x / CL * g.block;
+    auto barrier = [] {
+        if constexpr (CL > 1) cooperative_groups::this_cluster().sync();
+        else __syncthreads();
+    };
+    // where the residuals and diagonals are relaxed
+    Vec<Real, N> *Rr = R;
+    Real *Dr = Dg;
+    if constexpr (CL > 1 && !RESID) {
+        Rr = cooperative_groups::this_cluster().map_shared_rank(R, 0);
+        Dr = cooperative_groups::this_cluster().map_shared_rank(Dg, 0);
+    }
     const int nb = min(g.block, g.n_cells - c0);
     const int chunk = blockIdx.y;
     const int v = chunk * SV + tx;
     const int stride = q.n_pad;
+    // FP64: a warp of padding velocities alone leaves f as it is
+    const bool idle = std::is_same<Real, double>::value && chunk * SV + (tx & 32) >= q.n;
     Real xi[DIM];
 #pragma unroll
     for (int a = 0; a < DIM; ++a) xi[a] = q.x[a * stride + v];
@@ -924,7 +942,7 @@ __global__ void __launch_bounds__(SV * ROWS, sizeof(Real) == 4 ? (DIM < 3 ? 8 : 
     if constexpr (!PHOTON)
         for (int t = ty * SV + tx; t < nb * (cf::NC / 4); t += SV * ROWS)
             reinterpret_cast<Vec<Real, 4> *>(sC)[t] = vload<Real, 4>(coef + (size_t)c0 * cf::NC + 4 * t);
-    __syncthreads();
+    barrier();      // a cluster's CTAs have all started before one writes to another's shared memory
 
     // ---- 1. residuals and diagonals.  A cell's loads (its own value and the interior faces'
     // values: order 2 the face's upwind value, whichever side wrote it; order 1 the
@@ -943,15 +961,20 @@ __global__ void __launch_bounds__(SV * ROWS, sizeof(Real) == 4 ? (DIM < 3 ? 8 : 
     };
     constexpr bool AHEAD = PHOTON;
     V<Real, N> fi_next, fk_next[MAXF];
-    if (AHEAD && ty < nb) issue(ty, fi_next, fk_next);
-    for (int l = ty; l < nb; l += ROWS) {
+    if (AHEAD && row0 < nb) issue(row0, fi_next, fk_next);
+    for (int l = row0; l < nb; l += CL * ROWS) {
+        if (idle) {
+            Rr[l * SV + tx] = Vec<Real, N>{};
+            Dr[l * SV + tx] = Real(1);
+            continue;
+        }
         const Real *C = PHOTON ? coef + (size_t)(c0 + l) * cf::NC : sC + l * cf::NC;
         V<Real, N> fi, fk[MAXF];
         if constexpr (AHEAD) {
             fi = fi_next;
 #pragma unroll
             for (int k = 0; k < MAXF; ++k) fk[k] = fk_next[k];
-            if (l + ROWS < nb) issue(l + ROWS, fi_next, fk_next);
+            if (l + CL * ROWS < nb) issue(l + CL * ROWS, fi_next, fk_next);
         } else {
             issue(l, fi, fk);
         }
@@ -1021,10 +1044,10 @@ __global__ void __launch_bounds__(SV * ROWS, sizeof(Real) == 4 ? (DIM < 3 ? 8 : 
         Vec<Real, N> t;
 #pragma unroll
         for (int p = 0; p < N; ++p) t.v[p] = r.x[p];
-        R[l * SV + tx] = t;
-        Dg[l * SV + tx] = rcp_r(d);          // the relaxation multiplies by 1/d
+        Rr[l * SV + tx] = t;
+        Dr[l * SV + tx] = rcp_r(d);          // the relaxation multiplies by 1/d
     }
-    __syncthreads();
+    barrier();
 
     // ---- 2. Gauss-Seidel inside the block with the first-order operator; a = S/V xi_n from
     // the in-block face records of phase 0, used where a < 0 (in-block inflow):
@@ -1032,7 +1055,7 @@ __global__ void __launch_bounds__(SV * ROWS, sizeof(Real) == 4 ? (DIM < 3 ? 8 : 
     //   backward delta_l  = delta*_l - (sum_{j>l} a delta_j) / d_l
     // (RESID: the residuals themselves are the result; phases 2 and 3 are skipped and
     // phase 4 takes their moments)
-    if (ty == 0 && !RESID) {
+    if (ty == 0 && rank == 0 && !RESID && !idle) {
         for (int l = 0; l < nb; ++l) {
             Vec<Real, N> acc = R[l * SV + tx];
 #pragma unroll
@@ -1075,7 +1098,7 @@ __global__ void __launch_bounds__(SV * ROWS, sizeof(Real) == 4 ? (DIM < 3 ? 8 : 
             R[l * SV + tx] = acc;
         }
     }
-    __syncthreads();
+    barrier();
 
     // ---- 3. f^{k+1/2} = f^k + delta
     if constexpr (tc) {
@@ -1134,10 +1157,10 @@ __global__ void __launch_bounds__(SV * ROWS, sizeof(Real) == 4 ? (DIM < 3 ? 8 : 
         tcm::end(ctl, taddr, tid, ok, 0);
         return;
     }
-    for (int l = ty; l < nb && !RESID; l += ROWS) {
+    for (int l = row0; l < nb && !RESID; l += CL * ROWS) {
         const size_t idx = (size_t)(c0 + l) * stride + v;
         V<Real, N> fo = ldv<Real, N>(f_in, idx);
-        Vec<Real, N> t = R[l * SV + tx];
+        Vec<Real, N> t = Rr[l * SV + tx];
 #pragma unroll
         for (int p = 0; p < N; ++p) t.v[p] += fo.x[p];
         if (g.pos_theta > Real(0)) {   // the positivity bound of the implicit update
@@ -1151,7 +1174,7 @@ __global__ void __launch_bounds__(SV * ROWS, sizeof(Real) == 4 ? (DIM < 3 ? 8 : 
             vstore<Real, N>(f_out + idx * N, t);
         }
     }
-    __syncthreads();
+    barrier();      // and the first CTA's residuals have been read
 
     // ---- 4. moments of the new distribution on CUDA cores, eight lanes per cell
     if constexpr (sizeof(Real) == 8 && !PHOTON) {
@@ -1188,6 +1211,7 @@ __global__ void __launch_bounds__(SV * ROWS, sizeof(Real) == 4 ? (DIM < 3 ? 8 : 
             __syncthreads();
             const int l0 = max(t0 - c0, 0), l1 = min(t0 + MT - c0, nb);
             for (int l = l0 + tid / 8; l < l1; l += SV * ROWS / 8) {
+                if (CL > 1 && l / ROWS % CL != rank) continue;
                 Real acc[24];
 #pragma unroll
                 for (int m = 0; m < 24; ++m) acc[m] = Real(0);
@@ -2804,8 +2828,10 @@ template <typename Real, int N, int DIM>
 static cudaError_t slopes_t(cudaStream_t s, const Geom<Real> &g, const Quad<Real> &q, const Real *f,
                             Real *fface) {
     if constexpr (std::is_same<Real, double>::value) {
-        dim3 grid((g.n_cells + SLOPE_ROWS - 1) / SLOPE_ROWS, q.n_pad / 32);
-        k_slopes64<N, DIM><<<grid, dim3(32, SLOPE_ROWS), 0, s>>>(g, q.n, q.n_pad, q.x, f, fface);
+        // few cells: one warp per CTA, so that the FP64 work reaches every SM
+        const int cols = (q.n + 31) / 32, rows = (long long)g.n_cells * cols < 152 * SLOPE_ROWS ? 1 : SLOPE_ROWS;
+        k_slopes64<N, DIM><<<dim3((g.n_cells + rows - 1) / rows, cols), dim3(32, rows), 0, s>>>(g, q.n, q.n_pad, q.x, f,
+                                                                                             fface);
         return cudaGetLastError();
     } else {
         static_assert(SV % (32 * slope_vpt(DIM)) == 0, "a row's velocities must tile the padding");
@@ -2859,9 +2885,29 @@ static cudaError_t sweep_t(cudaStream_t s, const Geom<Real> &g, const Quad<Real>
         // FP64 on fewer CTAs than SMs (1-D meshes of a few hundred cells): a CTA's time is its
         // longest chain of FP64 instructions, so its cells are dealt to 8 rows instead of 2
         // (64 cells x 32 velocities: 72 -> 53 us; 800 x 64: 71 -> 55 us)
-        if constexpr (std::is_same<Real, double>::value)
+        if constexpr (N == 4) {
+            if ((long long)grid.x * grid.y < 152) {
+                auto kern = k_sweep<Real, N, DIM, ORDER, RESID, SROWS, 8>;
+                cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                if (e != cudaSuccess) return e;
+                cudaLaunchConfig_t cfg = {};
+                cfg.gridDim = dim3(grid.x * 8, grid.y);
+                cfg.blockDim = dim3(SV, SROWS);
+                cfg.dynamicSmemBytes = smem;
+                cfg.stream = s;
+                cudaLaunchAttribute at = {};
+                at.id = cudaLaunchAttributeClusterDimension;
+                at.val.clusterDim.x = 8;
+                at.val.clusterDim.y = at.val.clusterDim.z = 1;
+                cfg.attrs = &at;
+                cfg.numAttrs = 1;
+                e = cudaLaunchKernelEx(&cfg, kern, g, q, coef, bcoef, f_in, fface, f_out, partial);
+                return e != cudaSuccess ? e : cudaGetLastError();
+            }
+        } else if constexpr (std::is_same<Real, double>::value) {
             if ((long long)grid.x * grid.y < 152)
                 return run(k_sweep<Real, N, DIM, ORDER, RESID, 8>, dim3(SV, 8), smem);
+        }
         return run(k_sweep<Real, N, DIM, ORDER, RESID>, dim3(SV, SROWS), smem);
     }
 }
