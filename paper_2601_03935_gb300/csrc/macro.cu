@@ -49,6 +49,31 @@ namespace {
 
 constexpr double PI = 3.14159265358979323846;
 
+// The kernels of the inner loop start while their predecessor in the stream still runs
+// (launch_after): a kernel lets its successor's blocks in as soon as all of its own have
+// started, and reads and writes nothing before every block of its predecessor has ended and
+// its writes are visible.  Every thread waits, so that the end of a kernel implies the end of
+// all before it.  The kernels take plain pointers and hand them to a body that holds the
+// __restrict__: a load through a __restrict__ argument of the kernel itself may be moved
+// above the wait.
+__device__ __forceinline__ void wait_for_previous() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_after(cudaStream_t s, void (*kernel)(P...), int grid, int block, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Device functions are templates on the compute type R (double for the plain FP64 path,
 // float for the FP32 path's residual evaluation).
 template <typename R>
@@ -222,8 +247,7 @@ __global__ void k_macro_fields_from_W(int n_cells, ModelDev m, MacroReal<double>
 // most negative Delta_2 (phi_V falls beyond Delta_1 / 4 and exceeds 1 below Delta_1 / 2), and
 // in FP64 the smaller of the two quotients is found without dividing (their terms are positive).
 template <typename R, int DIM, int ORDER>
-__global__ void __launch_bounds__(128) k_macro_grad(MacroGeom g, const MacroState *__restrict__ st,
-                                                    R *__restrict__ grad, R *__restrict__ rec) {
+__device__ __forceinline__ void k_macro_grad_body(MacroGeom g, const MacroState *__restrict__ st, R *__restrict__ grad, R *__restrict__ rec) {
     constexpr int NV = DIM + 5, MS = Lay<DIM>::MAXS, LW = Lay<DIM>::LW;
     if (st && st->done) return;
     const MacroReal<R> &c = real<R>(g);
@@ -285,6 +309,11 @@ __global__ void __launch_bounds__(128) k_macro_grad(MacroGeom g, const MacroStat
         for (int k = 0; k < MAXF; ++k)
             if (g.nb[i * MAXF + k] >= 0) rec[((size_t)i * MAXF + k) * NVM + v] = fma(phi, d2[k], qi);
     }
+}
+template <typename R, int DIM, int ORDER>
+__global__ void __launch_bounds__(128) k_macro_grad(MacroGeom g, const MacroState *st, R *grad, R *rec) {
+    wait_for_previous();
+    k_macro_grad_body<R, DIM, ORDER>(g, st, grad, rec);
 }
 
 // ------------------------------------------------------------------ face fluxes
@@ -556,11 +585,7 @@ __global__ void __launch_bounds__(MF_NT) k_macro_binc(MacroGeom g, ModelDev m, Q
 // Blocks [n_face_cta, n_face_cta + n_bf): one boundary face each.  The rest: the sources of
 // MF_NT cells each, src [nc][SRC].
 template <typename R, int DIM, int ORDER>
-__global__ void __launch_bounds__(MF_NT) k_macro_flux(MacroGeom g, ModelDev m, QuadD vq, int n_face_cta, int n_bf_cta,
-                                                      const MacroState *__restrict__ st,
-                                                      const R *__restrict__ grad, const R *__restrict__ rec,
-                                                      R *__restrict__ Fx, R *__restrict__ fgam, R *__restrict__ src,
-                                                      double *__restrict__ bflux) {
+__device__ __forceinline__ void k_macro_flux_body(MacroGeom g, ModelDev m, QuadD vq, int n_face_cta, int n_bf_cta, const MacroState *__restrict__ st, const R *__restrict__ grad, const R *__restrict__ rec, R *__restrict__ Fx, R *__restrict__ fgam, R *__restrict__ src, double *__restrict__ bflux) {
     constexpr int NV = DIM + 5, E = 1 + DIM;
     if (st && st->done) return;
     const MacroReal<R> &c = real<R>(g);
@@ -661,6 +686,11 @@ __global__ void __launch_bounds__(MF_NT) k_macro_flux(MacroGeom g, ModelDev m, Q
     o[10] = fma(R(2.5), p, fma(R(0.5), ke, er + ev));
     o[11] = er;
     o[12] = ev;
+}
+template <typename R, int DIM, int ORDER>
+__global__ void __launch_bounds__(MF_NT) k_macro_flux(MacroGeom g, ModelDev m, QuadD vq, int n_face_cta, int n_bf_cta, const MacroState *st, const R *grad, const R *rec, R *Fx, R *fgam, R *src, double *bflux) {
+    wait_for_previous();
+    k_macro_flux_body<R, DIM, ORDER>(g, m, vq, n_face_cta, n_bf_cta, st, grad, rec, Fx, fgam, src, bflux);
 }
 
 // ------------------------------------------------------------------ high-order terms
@@ -788,13 +818,7 @@ struct __align__(4 * sizeof(R)) Row {
 // a fence, no waiting) adds the CTA partials of |R|^2 in a fixed order and sets the norm,
 // the iteration count and the stop flag.
 template <typename R, int DIM>
-__global__ void __launch_bounds__(128) k_macro_residual(MacroGeom g, MacroState *__restrict__ st,
-                                                        const R *__restrict__ Fx, const R *__restrict__ fgam,
-                                                        const R *__restrict__ src, const double *__restrict__ bflux,
-                                                        const double *__restrict__ hot_b, double *__restrict__ Rg,
-                                                        double *__restrict__ Dinv, R *__restrict__ gam,
-                                                        Row<R> *__restrict__ rows, double *__restrict__ rpart,
-                                                        double *__restrict__ history) {
+__device__ __forceinline__ void k_macro_residual_body(MacroGeom g, MacroState *__restrict__ st, const R *__restrict__ Fx, const R *__restrict__ fgam, const R *__restrict__ src, const double *__restrict__ bflux, const double *__restrict__ hot_b, double *__restrict__ Rg, double *__restrict__ Dinv, R *__restrict__ gam, Row<R> *__restrict__ rows, double *__restrict__ rpart, double *__restrict__ history) {
     constexpr int NV = DIM + 5, E = 1 + DIM, ER = 4 + DIM;
     if (st && st->done) return;
     const MacroReal<R> &c = real<R>(g);
@@ -943,6 +967,11 @@ __global__ void __launch_bounds__(128) k_macro_residual(MacroGeom g, MacroState 
     st->it += 1;
     if (!isfinite(rn) || rn <= st->tol * st->r0) st->done = 1;
 }
+template <typename R, int DIM>
+__global__ void __launch_bounds__(128) k_macro_residual(MacroGeom g, MacroState *st, const R *Fx, const R *fgam, const R *src, const double *bflux, const double *hot_b, double *Rg, double *Dinv, R *gam, Row<R> *rows, double *rpart, double *history) {
+    wait_for_previous();
+    k_macro_residual_body<R, DIM>(g, st, Fx, fgam, src, bflux, hot_b, Rg, Dinv, gam, rows, rpart, history);
+}
 
 // One point-relaxation sweep from the neighbours' records of the previous sweep.  Four lanes
 // per cell: lane r holds row r (r < E) and row r of the energy block, so that its two rows'
@@ -951,12 +980,7 @@ __global__ void __launch_bounds__(128) k_macro_residual(MacroGeom g, MacroState 
 // R = float: the neighbour terms in FP32 (as stored), their sum, the solve and the update in
 // FP64.  FIRST: no neighbour terms.  LAST: W += dW and the primitive variables of the new W.
 template <typename R, int DIM, bool FIRST, bool LAST>
-__global__ void __launch_bounds__(128) k_macro_jacobi(MacroGeom g, ModelDev m, const MacroState *__restrict__ st,
-                                                      const double *__restrict__ Rg, const double *__restrict__ Dinv,
-                                                      const R *__restrict__ gam, const R *__restrict__ src,
-                                                      const Row<R> *__restrict__ in, Row<R> *__restrict__ out,
-                                                      double *__restrict__ W, double *__restrict__ qd,
-                                                      float *__restrict__ qf) {
+__device__ __forceinline__ void k_macro_jacobi_body(MacroGeom g, ModelDev m, const MacroState *__restrict__ st, const double *__restrict__ Rg, const double *__restrict__ Dinv, const R *__restrict__ gam, const R *__restrict__ src, const Row<R> *__restrict__ in, Row<R> *__restrict__ out, double *__restrict__ W, double *__restrict__ qd, float *__restrict__ qf) {
     constexpr int E = 1 + DIM, ER = 4 + DIM, LPC = 4;
     if (st->done) return;
     const MacroReal<R> &c = real<R>(g);
@@ -1070,6 +1094,11 @@ __global__ void __launch_bounds__(128) k_macro_jacobi(MacroGeom g, ModelDev m, c
         (void)ER;
     }
 }
+template <typename R, int DIM, bool FIRST, bool LAST>
+__global__ void __launch_bounds__(128) k_macro_jacobi(MacroGeom g, ModelDev m, const MacroState *st, const double *Rg, const double *Dinv, const R *gam, const R *src, const Row<R> *in, Row<R> *out, double *W, double *qd, float *qf) {
+    wait_for_previous();
+    k_macro_jacobi_body<R, DIM, FIRST, LAST>(g, m, st, Rg, Dinv, gam, src, in, out, W, qd, qf);
+}
 
 // closed domains: fac = (total mass of the reference fields) / (total mass of W), the factor
 // that k_macro_fields_from_W scales W by; CTA partials in a fixed order, added by the last CTA
@@ -1175,8 +1204,8 @@ cudaError_t launch_macro_grad(cudaStream_t s, const MacroGeom &g, int order, int
                               const MacroWork &w) {
     const int nb = ctas((long long)g.n_cells * NVM, 128);
     MACRO_DISPATCH_R(fp32, MACRO_DISPATCH(g.dim, {
-        if (order == 2) k_macro_grad<R, DIM, 2><<<nb, 128, 0, s>>>(g, st, (R *)w.grad, (R *)w.rec);
-        else k_macro_grad<R, DIM, 1><<<nb, 128, 0, s>>>(g, st, (R *)w.grad, (R *)w.rec);
+        if (order == 2) launch_after(s, k_macro_grad<R, DIM, 2>, nb, 128, g, st, (R *)w.grad, (R *)w.rec);
+        else launch_after(s, k_macro_grad<R, DIM, 1>, nb, 128, g, st, (R *)w.grad, (R *)w.rec);
     }));
     return cudaGetLastError();
 }
@@ -1188,10 +1217,10 @@ cudaError_t launch_macro_flux(cudaStream_t s, const MacroGeom &g, int order, int
     if (n == 0) return cudaSuccess;
     MACRO_DISPATCH_R(fp32, MACRO_DISPATCH(g.dim, {
         if (order == 2)
-            k_macro_flux<R, DIM, 2><<<n, MF_NT, 0, s>>>(g, m, vq, nf, g.n_bf, st, (const R *)w.grad, (const R *)w.rec,
+            launch_after(s, k_macro_flux<R, DIM, 2>, n, MF_NT, g, m, vq, nf, g.n_bf, st, (const R *)w.grad, (const R *)w.rec,
                                                         (R *)w.Fx, (R *)w.fgam, (R *)w.src, w.mbf);
         else
-            k_macro_flux<R, DIM, 1><<<n, MF_NT, 0, s>>>(g, m, vq, nf, g.n_bf, st, (const R *)w.grad, (const R *)w.rec,
+            launch_after(s, k_macro_flux<R, DIM, 1>, n, MF_NT, g, m, vq, nf, g.n_bf, st, (const R *)w.grad, (const R *)w.rec,
                                                         (R *)w.Fx, (R *)w.fgam, (R *)w.src, w.mbf);
     }));
     return cudaGetLastError();
@@ -1217,7 +1246,7 @@ cudaError_t launch_macro_hot(cudaStream_t s, const MacroGeom &g, int fp32, const
 cudaError_t launch_macro_residual(cudaStream_t s, const MacroGeom &g, int fp32, MacroState *st, const MacroWork &w,
                                   const double *hot_b, double *history) {
     const int nb = ctas((long long)g.n_cells * NVM, 128);
-    MACRO_DISPATCH_R(fp32, MACRO_DISPATCH(g.dim, (k_macro_residual<R, DIM><<<nb, 128, 0, s>>>(
+    MACRO_DISPATCH_R(fp32, MACRO_DISPATCH(g.dim, (launch_after(s, k_macro_residual<R, DIM>, nb, 128, 
                                                      g, st, (const R *)w.Fx, (const R *)w.fgam, (const R *)w.src, w.mbf,
                                                      hot_b, w.Rg, w.Dinv, (R *)w.gam, (Row<R> *)w.rows[0], w.rpart,
                                                      history))));
@@ -1233,13 +1262,13 @@ cudaError_t launch_macro_jacobi(cudaStream_t s, const MacroGeom &g, int fp32, co
         const Row<R> *in = (const Row<R> *)w.rows[(sweep + 1) & 1];
         Row<R> *out = (Row<R> *)w.rows[sweep & 1];
         if (sweep == 0)
-            k_macro_jacobi<R, DIM, true, true><<<nb, 128, 0, s>>>(g, m, st, w.Rg, w.Dinv, gam, src, in, out, w.W, w.qd,
+            launch_after(s, k_macro_jacobi<R, DIM, true, true>, nb, 128, g, m, st, w.Rg, w.Dinv, gam, src, in, out, w.W, w.qd,
                                                                   w.qf);
         else if (last)
-            k_macro_jacobi<R, DIM, false, true><<<nb, 128, 0, s>>>(g, m, st, w.Rg, w.Dinv, gam, src, in, out, w.W,
+            launch_after(s, k_macro_jacobi<R, DIM, false, true>, nb, 128, g, m, st, w.Rg, w.Dinv, gam, src, in, out, w.W,
                                                                    w.qd, w.qf);
         else
-            k_macro_jacobi<R, DIM, false, false><<<nb, 128, 0, s>>>(g, m, st, w.Rg, w.Dinv, gam, src, in, out, w.W,
+            launch_after(s, k_macro_jacobi<R, DIM, false, false>, nb, 128, g, m, st, w.Rg, w.Dinv, gam, src, in, out, w.W,
                                                                     w.qd, w.qf);
     }));
     return cudaGetLastError();
