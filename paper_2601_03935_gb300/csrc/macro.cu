@@ -49,13 +49,16 @@ namespace {
 
 constexpr double PI = 3.14159265358979323846;
 
-// The kernels of the inner loop start while their predecessor in the stream still runs
-// (launch_after): a kernel lets its successor's blocks in as soon as all of its own have
-// started, and reads and writes nothing before every block of its predecessor has ended and
-// its writes are visible.  Every thread waits, so that the end of a kernel implies the end of
-// all before it.  The kernels take plain pointers and hand them to a body that holds the
-// __restrict__: a load through a __restrict__ argument of the kernel itself may be moved
-// above the wait.
+// The kernels of the inner loop are launched before their predecessor in the stream has ended
+// (launch_after), so that only the wait for its last block remains of the time between two
+// kernels; a kernel reads and writes nothing before every block of its predecessor has ended
+// and its writes are visible.  Every thread waits, so that the end of a kernel implies the end
+// of all before it.  300 inner iterations: 800 cells FP64 14.4 -> 13.7 ms, 2 048 cells FP64
+// 22.5 -> 22.1, 20 000 cells mixed 17.2 -> 16.9.  With the next kernel's blocks let in when
+// those of the current one have started (griddepcontrol.launch_dependents) these took 14.8,
+// 28.6 and 19.4 ms, and halfway through the kernels 13.8, 22.0 and 18.2.
+// The kernels take plain pointers and hand them to a body that holds the __restrict__: a load
+// through a __restrict__ argument of the kernel itself may be moved above the wait.
 __device__ __forceinline__ void wait_for_previous() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
