@@ -50,10 +50,11 @@ struct gsis_ctx {
     cudaStream_t copy_stream = nullptr;
     cudaEvent_t stage_ready = nullptr, stage_free = nullptr;
     // the photon slope pass and sweep run on side_stream, between fork_ev (recorded on the
-    // context stream after the wall densities) and join_ev (waited on before the moments
-    // are finished), concurrently with the gas kernels; created on first use
+    // context stream) and join_ev (waited on before the moments are finished), concurrently
+    // with the gas kernels; at order 2 the wall densities too, up to wall_ev (waited on
+    // before the gas sweep); created on first use
     cudaStream_t side_stream = nullptr;
-    cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
+    cudaEvent_t fork_ev = nullptr, join_ev = nullptr, wall_ev = nullptr;
     bool staged = false;
     void *coef = nullptr, *bcoef = nullptr, *partial = nullptr, *opartial = nullptr;
     // defect correction (solver.defect_correction): coefficients of M^{k+1/2}, the moment
@@ -317,13 +318,18 @@ int refresh(gsis_ctx *c) { return c->precision == GSIS_FP64 ? refresh_fields<dou
 template <typename Real>
 int kinetic_step(gsis_ctx *c, int nxt) {
     const Geom<Real> g = geom<Real>(c);
-    TRY(launch(c, K_WALL, [&] {
-        return launch_wall_density<Real>(c->stream, c->dim, g, vquad<Real>(c), c->patch_T, c->bf_inc, c->patch_kind,
-                                         (const Real *)c->f[c->cur], c->sharded ? c->wout_g : nullptr,
-                                         (Real *)c->bcoef);
-    }));
+    auto wall = [&](cudaStream_t st) {
+        return launch(c, K_WALL, [&] {
+            return launch_wall_density<Real>(st, c->dim, g, vquad<Real>(c), c->patch_T, c->bf_inc, c->patch_kind,
+                                             (const Real *)c->f[c->cur], c->sharded ? c->wout_g : nullptr,
+                                             (Real *)c->bcoef);
+        }, st);
+    };
+    // the gas slope pass needs no wall densities: at order 2 they are found beside it
+    const bool wall_aside = c->order == 2;
+    if (!wall_aside) TRY(wall(c->stream));
     // photon transport is independent of the gas planes: it runs on the side stream
-    if (!c->side_stream) {   // the events first: a side stream implies both events exist
+    if (!c->side_stream) {   // the events first: a side stream implies that they exist
         cudaEvent_t e = nullptr;
         if (!c->fork_ev) {
             CUDA_TRY(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -333,6 +339,10 @@ int kinetic_step(gsis_ctx *c, int nxt) {
             CUDA_TRY(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
             c->join_ev = e;
         }
+        if (!c->wall_ev) {
+            CUDA_TRY(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+            c->wall_ev = e;
+        }
         cudaStream_t st = nullptr;
         CUDA_TRY(c, cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
         c->side_stream = st;
@@ -340,6 +350,10 @@ int kinetic_step(gsis_ctx *c, int nxt) {
     CUDA_TRY(c, cudaEventRecord(c->fork_ev, c->stream));
     CUDA_TRY(c, cudaStreamWaitEvent(c->side_stream, c->fork_ev, 0));
     const cudaStream_t ps = c->side_stream;
+    if (wall_aside) {
+        TRY(wall(ps));
+        CUDA_TRY(c, cudaEventRecord(c->wall_ev, ps));
+    }
     if (c->order == 2) {
         TRY(launch(c, K_SLOPE_PHOTON, [&] {
             return launch_slopes<Real>(ps, c->dim, 1, g, oquad<Real>(c), (const Real *)c->I[c->cur],
@@ -358,6 +372,7 @@ int kinetic_step(gsis_ctx *c, int nxt) {
                                        (Real *)c->fface);
         }));
     }
+    if (wall_aside) CUDA_TRY(c, cudaStreamWaitEvent(c->stream, c->wall_ev, 0));
     TRY(launch(c, K_SWEEP_GAS, [&] {
         return launch_sweep_gas<Real>(c->stream, c->dim, c->order, g, vquad<Real>(c), (const Real *)c->coef,
                                       (const Real *)c->bcoef, (const Real *)c->f[c->cur], (const Real *)c->fface,
@@ -892,6 +907,7 @@ void gsis_destroy(gsis_ctx *ctx) {
     for (cudaEvent_t ev : ctx->poll_ev)
         if (ev) cudaEventDestroy(ev);
     if (ctx->join_ev) cudaEventDestroy(ctx->join_ev);
+    if (ctx->wall_ev) cudaEventDestroy(ctx->wall_ev);
     if (ctx->stage_ready) cudaEventDestroy(ctx->stage_ready);
     if (ctx->stage_free) cudaEventDestroy(ctx->stage_free);
     if (ctx->macro_exec) cudaGraphExecDestroy(ctx->macro_exec);
