@@ -2495,10 +2495,11 @@ __device__ __forceinline__ void finish_cell(int i, int o_chunks, const ModelDev 
     for (int q = 0; q < NEPS; ++q) eps_terms[(size_t)i * NEPS + q] = E[q];
 }
 
-// One cell per lane, 32-lane CTAs.  With `reduce`, the convergence terms are summed too:
-// each CTA adds its 32 cells in a fixed shuffle order, and the last CTA to finish (counted
-// with an atomic ticket after a fence, no waiting) adds the CTA partials in a fixed order,
-// so the result does not depend on scheduling.
+// One cell per lane of the first warp; FW warps share the sums over the chunks (from four
+// chunks on: 10 000 cells x 36 chunks 39 -> 30 us, 20 000 x 13 34 -> 33).  With `reduce`, the
+// convergence terms are summed too: each CTA adds its 32 cells in a fixed shuffle order, and
+// the last CTA to finish (counted with an atomic ticket after a fence, no waiting) adds the
+// CTA partials in a fixed order, so the result does not depend on scheduling.
 template <typename Real, int DIM, int FW>
 __global__ void __launch_bounds__(32 * FW) k_finish(int n_cells, int n_chunks, int o_chunks, ModelDev m,
                                                     const Real *__restrict__ coef, const Real *__restrict__ partial,
@@ -2882,9 +2883,10 @@ static cudaError_t sweep_t(cudaStream_t s, const Geom<Real> &g, const Quad<Real>
         if (DIM < 3 && g.max_faces <= DIM + 1) return run(k_sweep_gas32<DIM, ORDER, RESID, DIM + 1>, dim3(128), bytes);
         return run(k_sweep_gas32<DIM, ORDER, RESID, MAXF>, dim3(128), bytes);
     } else {
-        // FP64 on fewer CTAs than SMs (1-D meshes of a few hundred cells): a CTA's time is its
-        // longest chain of FP64 instructions, so its cells are dealt to 8 rows instead of 2
-        // (64 cells x 32 velocities: 72 -> 53 us; 800 x 64: 71 -> 55 us)
+        // FP64 on fewer blocks than SMs (1-D meshes of a few hundred cells): a block's time is
+        // the FP64 pipe of the SM it runs on.  Gas: a cluster of eight CTAs per block (64 cells
+        // x 32 velocities: 72 us by one CTA of two rows, 53 of eight rows, 32 by the cluster;
+        // 800 x 64: 71, 55, 45).  Photons, with few instructions per value: eight rows.
         if constexpr (N == 4) {
             if ((long long)grid.x * grid.y < 152) {
                 auto kern = k_sweep<Real, N, DIM, ORDER, RESID, SROWS, 8>;

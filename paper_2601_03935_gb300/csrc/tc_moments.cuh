@@ -115,16 +115,12 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
 }
 
 // ---- tensor memory, barriers and fences
+// A CTA of a kernel that contains tcgen05.alloc holds the SM's allocation permit until it
+// relinquishes it, and while it holds it no further CTA of the kernel is scheduled on that SM.
 __device__ __forceinline__ void tmem_alloc(uint32_t slot_addr) {   // one full warp
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot_addr),
                  "r"(TMEM_COLS)
                  : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-// A CTA of a kernel that contains tcgen05.alloc holds the SM's allocation permit until it
-// relinquishes it, and while it holds it no further CTA of the kernel is scheduled on that
-// SM.  CTAs that take a path without tensor memory therefore give it up at once (one warp).
-__device__ __forceinline__ void relinquish() {
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr) {     // the allocating warp
