@@ -99,7 +99,7 @@ struct gsis_ctx {
         double *W[2], *q, *grad, *phi, *Rg, *Dinv, *gam, *dG[2], *rpart, *hot, *mbf;
     } w3{};
     double *hot_b = nullptr, *kbf = nullptr, *fields_h = nullptr, *fields_n = nullptr, *mhist = nullptr;
-    MacroState *h_mstate = nullptr;   // pinned: initial state, then two states as polled
+    MacroState *h_mstate = nullptr;   // pinned: the host's state, then two states as polled
     cudaEvent_t poll_ev[2] = {};      // after the copy of each
     int last_inner = 0;
     cudaGraphExec_t macro_exec = nullptr;   // POLL inner iterations, captured once
@@ -545,7 +545,10 @@ int macro_solve(gsis_ctx *c) {
     c->h_mstate->r0 = 0.0;
     c->h_mstate->rn = 0.0;
     c->h_mstate->tol = sp.tol_inner;
-    CUDA_TRY(c, cudaMemcpyAsync(mstate, c->h_mstate, sizeof(MacroState), cudaMemcpyHostToDevice, c->stream));
+    // the state goes to the device as a kernel's argument, which is taken when the launch
+    // returns: a copy from h_mstate might still be waiting when the next solve rewrites it
+    auto start = [&] { return launch(c, K_MCONV, [&] { return launch_macro_start(c->stream, *c->h_mstate, mstate); }); };
+    TRY(start());
     const bool graph = !c->prof && c->stream != nullptr;
     if (graph && !c->macro_exec) TRY(capture_inner(c, fp_main, &c->macro_exec, &c->macro_nodes));
     if (graph && mixed && !c->macro_exec64) TRY(capture_inner(c, 0, &c->macro_exec64, &c->macro_nodes64));
@@ -590,7 +593,7 @@ int macro_solve(gsis_ctx *c) {
         // the FP64 residual side for up to `tail` more iterations, from where the FP32 ones stopped
         c->h_mstate->done = 0;
         c->h_mstate->max_inner = c->h_mstate->it + tail;
-        CUDA_TRY(c, cudaMemcpyAsync(mstate, c->h_mstate, sizeof(MacroState), cudaMemcpyHostToDevice, c->stream));
+        TRY(start());
         TRY(phase(true, tail, false));
     }
     return GSIS_OK;

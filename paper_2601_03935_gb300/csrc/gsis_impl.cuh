@@ -296,6 +296,8 @@ struct MacroWork {
 
 cudaError_t launch_macro_from_fields(cudaStream_t s, int dim, int n_cells, const ModelDev &m, const double *F,
                                      const MacroWork &w);
+// the state that a solve, or its FP64 tail, starts from
+cudaError_t launch_macro_start(cudaStream_t s, const MacroState &value, MacroState *st);
 // F_ref: null, or the fields whose total mass W is scaled to
 cudaError_t launch_macro_fields_from_W(cudaStream_t s, const MacroGeom &g, const ModelDev &m, const MacroWork &w,
                                        const double *F_ref, double *F);

@@ -1103,6 +1103,8 @@ __global__ void __launch_bounds__(128) k_macro_jacobi(MacroGeom g, ModelDev m, c
     k_macro_jacobi_body<R, DIM, FIRST, LAST>(g, m, st, Rg, Dinv, gam, src, in, out, W, qd, qf);
 }
 
+__global__ void k_macro_start(MacroState value, MacroState *st) { *st = value; }
+
 // closed domains: fac = (total mass of the reference fields) / (total mass of W), the factor
 // that k_macro_fields_from_W scales W by; CTA partials in a fixed order, added by the last CTA
 constexpr int MM_CTAS = 64;
@@ -1184,6 +1186,11 @@ __global__ void __launch_bounds__(256) k_macro_mass(int n_cells, const double *_
 static int ctas(long long threads, int nt) { return (int)((threads + nt - 1) / nt); }
 
 int macro_rpart_count(int n_cells) { return std::max(ctas((long long)n_cells * NVM, 128), 2 * MM_CTAS); }
+
+cudaError_t launch_macro_start(cudaStream_t s, const MacroState &value, MacroState *st) {
+    k_macro_start<<<1, 1, 0, s>>>(value, st);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_macro_from_fields(cudaStream_t s, int dim, int n_cells, const ModelDev &m, const double *F,
                                      const MacroWork &w) {

@@ -1,0 +1,39 @@
+"""The order in which the host gives work to the device, on the CPU: libgsis is linked with a
+runtime that records instead of running (fake_cudart.cpp)."""
+import numpy as np
+import pytest
+
+import gsis_inputs as gi
+
+import _fake
+
+STREAM = 0x1000          # a stream of the caller's own
+
+
+@pytest.fixture(scope="module")
+def G(tmp_path_factory):
+    return _fake.load(str(tmp_path_factory.mktemp("fake")))
+
+
+def _create(G, wl, stream=STREAM):
+    m = wl.mesh
+    return G.gsis_create(m.dim, m.face_owner, m.face_nbr, m.face_normal, m.face_area, m.face_centroid,
+                         m.cell_volume, m.cell_centroid, m.patches, wl.xi[:, :m.dim], wl.w, wl.omega, wl.wo,
+                         wl.model, wl.solver, stream, period=getattr(m, "period", 0.0))
+
+
+@pytest.mark.parametrize("max_inner", [3, 8, 9, 16, 17, 40])
+@pytest.mark.parametrize("macro_fp32", [0, 1, 2])
+def test_solver_state_is_not_rewritten_under_a_copy(G, macro_fp32, max_inner):
+    # steps in a row without a read between them, and two pre-solves
+    wl = gi.workloads.with_solver(gi.workloads.slab(n_cells=12, n_xi=16, n_mu=8), precision="fp32",
+                                  macro_fp32=macro_fp32, max_inner=max_inner)
+    ctx = _create(G, wl)
+    G.fake.fake_reset()
+    try:
+        for _ in range(3):
+            assert G.load().gsis_step_async(ctx, G.GSIS_MODE_GSIS) == G.GSIS_OK
+        G.load().gsis_warm_start(ctx, 2, 0)
+    finally:
+        G.gsis_destroy(ctx)
+    assert _fake.report(G, "rewritten") == []
