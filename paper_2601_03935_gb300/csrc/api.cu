@@ -172,20 +172,24 @@ int dalloc_real(gsis_ctx *c, void **p, size_t n) {
     return GSIS_OK;
 }
 
+// Uploads (and the clearing of new buffers) are work of the context's stream, which is not
+// ordered after the default stream: cudaMemcpy from pageable memory and cudaMemset return
+// before the device memory holds the values.  The sources may go out of scope: the call
+// returns once they are staged.
 // upload a host double array as Real
 int upload_real(gsis_ctx *c, void *dst, const std::vector<double> &src) {
     if (c->precision == GSIS_FP64) {
-        CUDA_TRY(c, cudaMemcpy(dst, src.data(), src.size() * sizeof(double), cudaMemcpyHostToDevice));
+        CUDA_TRY(c, cudaMemcpyAsync(dst, src.data(), src.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream));
     } else {
         std::vector<float> t(src.begin(), src.end());
-        CUDA_TRY(c, cudaMemcpy(dst, t.data(), t.size() * sizeof(float), cudaMemcpyHostToDevice));
+        CUDA_TRY(c, cudaMemcpyAsync(dst, t.data(), t.size() * sizeof(float), cudaMemcpyHostToDevice, c->stream));
     }
     return GSIS_OK;
 }
 
 template <typename T>
 int upload(gsis_ctx *c, T *dst, const std::vector<T> &src) {
-    CUDA_TRY(c, cudaMemcpy(dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice));
+    CUDA_TRY(c, cudaMemcpyAsync(dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice, c->stream));
     return GSIS_OK;
 }
 
@@ -428,9 +432,11 @@ int macro_velocity_set(gsis_ctx *c) {
     if (c->mfp32) {
         const size_t n = 4 * (size_t)c->Vdp;
         std::vector<double> h(n);
-        CUDA_TRY(c, cudaMemcpy(h.data(), c->vqd_x, 3 * (size_t)c->Vdp * sizeof(double), cudaMemcpyDeviceToHost));
-        CUDA_TRY(c, cudaMemcpy(h.data() + 3 * (size_t)c->Vdp, c->vqd_w, (size_t)c->Vdp * sizeof(double),
-                               cudaMemcpyDeviceToHost));
+        CUDA_TRY(c, cudaMemcpyAsync(h.data(), c->vqd_x, 3 * (size_t)c->Vdp * sizeof(double), cudaMemcpyDeviceToHost,
+                                    c->stream));
+        CUDA_TRY(c, cudaMemcpyAsync(h.data() + 3 * (size_t)c->Vdp, c->vqd_w, (size_t)c->Vdp * sizeof(double),
+                                    cudaMemcpyDeviceToHost, c->stream));
+        CUDA_TRY(c, cudaStreamSynchronize(c->stream));
         const std::vector<float> hf(h.begin(), h.end());
         float *p = nullptr;
         TRY(dalloc(c, &p, n));
@@ -860,7 +866,7 @@ int init_uniform(gsis_ctx *c) {
         M[i * NF + 0] = 1.0;
         for (int k = 4; k < 8; ++k) M[i * NF + k] = 1.0;
     }
-    CUDA_TRY(c, cudaMemcpy(c->fields, M.data(), M.size() * sizeof(double), cudaMemcpyHostToDevice));
+    TRY(upload(c, c->fields, M));
     TRY(launch(c, K_EQUIL, [&] {
         return launch_equilibrium<Real>(c->stream, c->dim, (int)c->nc, vquad<Real>(c), oquad<Real>(c), c->model,
                                         c->fields, (Real *)c->f[c->cur], (Real *)c->I[c->cur]);
@@ -1290,7 +1296,7 @@ int gsis_create(const gsis_mesh *m, const gsis_velocity_quad *vq, const gsis_pho
         A_(dalloc_real(c, &c->fface, nfi1 * c->Vp * 4));
         A_(dalloc_real(c, &c->oface, nfi1 * c->Op));
         // values that no cell writes (xi . n = 0) are read with the factor xi . n
-        if (cudaMemset(c->fface, 0, nfi1 * c->Vp * 4 * c->real_size) != cudaSuccess) return bail(GSIS_ERR_CUDA);
+        if (cudaMemsetAsync(c->fface, 0, nfi1 * c->Vp * 4 * c->real_size, c->stream) != cudaSuccess) return bail(GSIS_ERR_CUDA);
     }
     A_(dalloc(c, &c->fields, (size_t)nc * NF));
     A_(dalloc(c, &c->fields_old, (size_t)nc * NF));
@@ -1337,7 +1343,7 @@ int gsis_create(const gsis_mesh *m, const gsis_velocity_quad *vq, const gsis_pho
             A_(work(&w.gam, (size_t)nc * MAXF * 2));
             for (int k = 0; k < 2; ++k) {
                 A_(work(&w.rows[k], (size_t)nc * NVM * 4));
-                if (cudaMemset(w.rows[k], 0, (size_t)nc * NVM * 4 * R8) != cudaSuccess) return bail(GSIS_ERR_CUDA);
+                if (cudaMemsetAsync(w.rows[k], 0, (size_t)nc * NVM * 4 * R8, c->stream) != cudaSuccess) return bail(GSIS_ERR_CUDA);
             }
             A_(dalloc(c, &w.Rg, (size_t)nc * NVM));
             A_(dalloc(c, &w.Dinv, (size_t)nc * 24));
@@ -1347,12 +1353,12 @@ int gsis_create(const gsis_mesh *m, const gsis_velocity_quad *vq, const gsis_pho
             A_(dalloc(c, &w.mbf, nbf1 * NVM));
         }
         A_(dalloc(c, &w.state, 1));
-        if (cudaMemset(w.state, 0, sizeof(MacroState)) != cudaSuccess) return bail(GSIS_ERR_CUDA);
+        if (cudaMemsetAsync(w.state, 0, sizeof(MacroState), c->stream) != cudaSuccess) return bail(GSIS_ERR_CUDA);
         if (sp->defect_correction) {
             A_(dalloc_real(c, &c->coef_h, (size_t)nc * cf::NC));
             A_(dalloc(c, &c->rrow, (size_t)nc * NVM));
             A_(dalloc(c, &c->moff, (size_t)nc * NVM));
-            if (cudaMemset(c->moff, 0, (size_t)nc * NVM * sizeof(double)) != cudaSuccess) return bail(GSIS_ERR_CUDA);
+            if (cudaMemsetAsync(c->moff, 0, (size_t)nc * NVM * sizeof(double), c->stream) != cudaSuccess) return bail(GSIS_ERR_CUDA);
         }
         A_(dalloc(c, &c->hot_b, nbf1 * NVM));
         A_(dalloc(c, &c->kbf, nbf1 * NVM));
@@ -1540,8 +1546,8 @@ int gsis_create(const gsis_mesh *m, const gsis_velocity_quad *vq, const gsis_pho
     if (bf_cell.empty()) { bf_cell.push_back(0); bf_patch.push_back(0); }
     A_(upload(c, c->vol, vol));
     A_(upload(c, c->cell_dx, cdx));
-    CUDA_TRY(c, cudaMemcpy(c->g_info, info.data(), info.size() * sizeof(int), cudaMemcpyHostToDevice));
-    CUDA_TRY(c, cudaMemcpy(c->g_fnb, fnb.data(), fnb.size() * sizeof(int), cudaMemcpyHostToDevice));
+    A_(upload(c, reinterpret_cast<int *>(c->g_info), info));
+    A_(upload(c, reinterpret_cast<int *>(c->g_fnb), fnb));
     A_(upload(c, c->g_stn, stn));
     A_(upload(c, c->bf_cell, bf_cell));
     A_(upload(c, c->bf_patch, bf_patch));
@@ -1644,10 +1650,10 @@ int gsis_create(const gsis_mesh *m, const gsis_velocity_quad *vq, const gsis_pho
         A_(upload(c, c->bf_inc, inc));
     }
     A_(macro_velocity_set(c));
-    if (cudaMemset(c->eps_ticket, 0, sizeof(unsigned int)) != cudaSuccess) return bail(GSIS_ERR_CUDA);
+    if (cudaMemsetAsync(c->eps_ticket, 0, sizeof(unsigned int), c->stream) != cudaSuccess) return bail(GSIS_ERR_CUDA);
     A_(upload(c, c->patch_kind, pk));
-    if (cudaMemset(c->err, 0, sizeof(int)) != cudaSuccess) return bail(GSIS_ERR_CUDA);
-    if (cudaMemset(c->coef, 0, (size_t)nc * cf::NC * c->real_size) != cudaSuccess) return bail(GSIS_ERR_CUDA);
+    if (cudaMemsetAsync(c->err, 0, sizeof(int), c->stream) != cudaSuccess) return bail(GSIS_ERR_CUDA);
+    if (cudaMemsetAsync(c->coef, 0, (size_t)nc * cf::NC * c->real_size, c->stream) != cudaSuccess) return bail(GSIS_ERR_CUDA);
     A_(c->precision == GSIS_FP64 ? init_uniform<double>(c) : init_uniform<float>(c));
     A_(refresh(c));
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return bail(GSIS_ERR_CUDA);
@@ -1807,16 +1813,15 @@ int gsis_import_state(gsis_ctx *c, const void *buf, int64_t len) {
     if (h.n_hist) std::memcpy(hist.data(), p, (size_t)h.n_hist * 8);
     p += (size_t)h.n_hist * 8;
     const size_t rs = c->real_size;
-    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-    CUDA_TRY(c, cudaMemcpy(c->fields, p, (size_t)c->nc * NF * 8, cudaMemcpyHostToDevice));
+    CUDA_TRY(c, cudaMemcpyAsync(c->fields, p, (size_t)c->nc * NF * 8, cudaMemcpyHostToDevice, c->stream));
     p += (size_t)c->nc * NF * 8;
-    CUDA_TRY(c, cudaMemset(c->f[c->cur], 0, (size_t)c->nc * c->Vp * 4 * rs));
-    CUDA_TRY(c, cudaMemset(c->I[c->cur], 0, (size_t)c->nc * c->Op * rs));
-    CUDA_TRY(c, cudaMemcpy2D(c->f[c->cur], (size_t)c->Vp * 4 * rs, p, (size_t)c->V * 4 * rs, (size_t)c->V * 4 * rs,
-                             (size_t)c->nc, cudaMemcpyHostToDevice));
+    CUDA_TRY(c, cudaMemsetAsync(c->f[c->cur], 0, (size_t)c->nc * c->Vp * 4 * rs, c->stream));
+    CUDA_TRY(c, cudaMemsetAsync(c->I[c->cur], 0, (size_t)c->nc * c->Op * rs, c->stream));
+    CUDA_TRY(c, cudaMemcpy2DAsync(c->f[c->cur], (size_t)c->Vp * 4 * rs, p, (size_t)c->V * 4 * rs, (size_t)c->V * 4 * rs,
+                                  (size_t)c->nc, cudaMemcpyHostToDevice, c->stream));
     p += (size_t)c->nc * c->V * 4 * rs;
-    CUDA_TRY(c, cudaMemcpy2D(c->I[c->cur], (size_t)c->Op * rs, p, (size_t)c->NO * rs, (size_t)c->NO * rs,
-                             (size_t)c->nc, cudaMemcpyHostToDevice));
+    CUDA_TRY(c, cudaMemcpy2DAsync(c->I[c->cur], (size_t)c->Op * rs, p, (size_t)c->NO * rs, (size_t)c->NO * rs,
+                                  (size_t)c->nc, cudaMemcpyHostToDevice, c->stream));
     // the next iteration reads the coefficient record built from the fields, exactly as
     // after the iteration that produced them
     int rc = c->precision == GSIS_FP64 ? launch(c, K_COEF, [&] {
@@ -2046,8 +2051,9 @@ int gsis_shard_setup(gsis_ctx *c, int32_t n_xi_all, const double *xi_all, const 
     c->xcount = (int64_t)((size_t)c->nc * NXC + nbf1 * (1 + KBR));
     TRY(dalloc(c, &c->xbuf, (size_t)c->xcount));
     TRY(dalloc(c, &c->wout_g, nbf1));
-    CUDA_TRY(c, cudaMemset(c->xbuf, 0, (size_t)c->xcount * sizeof(double)));
-    CUDA_TRY(c, cudaMemset(c->wout_g, 0, nbf1 * sizeof(double)));
+    CUDA_TRY(c, cudaMemsetAsync(c->xbuf, 0, (size_t)c->xcount * sizeof(double), c->stream));
+    CUDA_TRY(c, cudaMemsetAsync(c->wout_g, 0, nbf1 * sizeof(double), c->stream));
+    CUDA_TRY(c, cudaStreamSynchronize(c->stream));      // the buffer may be used on another stream from here on
     c->sharded = true;
     c->shard_state = 0;
     return GSIS_OK;

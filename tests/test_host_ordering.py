@@ -37,3 +37,31 @@ def test_solver_state_is_not_rewritten_under_a_copy(G, macro_fp32, max_inner):
     finally:
         G.gsis_destroy(ctx)
     assert _fake.report(G, "rewritten") == []
+
+
+@pytest.mark.parametrize("precision,macro_fp32", [("fp64", 0), ("fp32", 0), ("fp32", 2)])
+@pytest.mark.parametrize("name,order,defect", [("slab", 1, 0), ("cavity", 2, 1), ("capsule", 2, 0)])
+def test_the_context_stream_orders_all_work(G, name, order, defect, precision, macro_fp32):
+    # nothing that a kernel reads or overwrites is left to the default stream
+    base = {"slab": lambda: gi.workloads.slab(n_cells=12, n_xi=16, n_mu=8),
+            "cavity": lambda: gi.workloads.cavity(n_side=4, n_v=8),
+            "capsule": lambda: gi.workloads.capsule(n=4, n_v=6, n_polar=4, n_azim=4)}[name]()
+    wl = gi.workloads.with_solver(base, precision=precision, order=order, macro_fp32=macro_fp32, max_inner=10,
+                                  defect_correction=defect)
+    lib = G.load()
+    G.fake.fake_reset()
+    ctx = _create(G, wl)
+    try:
+        n = wl.mesh.n_cells
+        for mode in (G.GSIS_MODE_CIS, G.GSIS_MODE_GSIS):
+            assert lib.gsis_step_async(ctx, mode) == G.GSIS_OK
+        G.gsis_set_distributions(ctx, np.ones((n, wl.w.size, 4)), np.ones((n, wl.wo.size)))
+        image = G.gsis_export_state(ctx)
+        G.gsis_import_state(ctx, image)
+        assert lib.gsis_step_async(ctx, G.GSIS_MODE_CIS) == G.GSIS_OK
+        if wl.dim < 3 and not defect:
+            G.gsis_shard_setup(ctx, wl.xi[:, :wl.dim], wl.w, wl.omega, wl.wo)
+            assert lib.gsis_shard_begin(ctx, G.GSIS_MODE_GSIS) == G.GSIS_OK
+    finally:
+        G.gsis_destroy(ctx)
+    assert _fake.report(G, "unordered") == []
