@@ -2861,6 +2861,14 @@ size_t sweep_smem_bytes(int block, int planes, int dim, size_t real_size, bool t
            (size_t)((block * MAXF + 15) & ~15) + (tc ? sizeof(tcm::Ctl) : 0);
 }
 
+// The dynamic shared memory a sweep may take: always the most a CTA can have, never this
+// context's need.  The limit belongs to the kernel, and another thread's context, with another
+// relaxation block, may set it between here and the launch.
+template <typename K>
+static cudaError_t allow_smem(K kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+}
+
 template <typename Real, int N, int DIM, int ORDER, bool RESID>
 static cudaError_t sweep_t(cudaStream_t s, const Geom<Real> &g, const Quad<Real> &q, const Real *coef,
                            const Real *bcoef, const Real *f_in, const Real *fface, Real *f_out, Real *partial) {
@@ -2868,7 +2876,7 @@ static cudaError_t sweep_t(cudaStream_t s, const Geom<Real> &g, const Quad<Real>
     if (g.tc && (DIM == 3 || MT % g.block != 0)) return cudaErrorInvalidValue;
     dim3 grid((g.n_cells + g.block - 1) / g.block, q.n_pad / SV);
     auto run = [&](auto kern, dim3 block, size_t smem) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(kern);
         if (e != cudaSuccess) return e;
         kern<<<grid, block, smem, s>>>(g, q, coef, bcoef, f_in, fface, f_out, partial);
         return cudaGetLastError();
@@ -2890,7 +2898,7 @@ static cudaError_t sweep_t(cudaStream_t s, const Geom<Real> &g, const Quad<Real>
         if constexpr (N == 4) {
             if ((long long)grid.x * grid.y < 152) {
                 auto kern = k_sweep<Real, N, DIM, ORDER, RESID, SROWS, 8>;
-                cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                cudaError_t e = allow_smem(kern);
                 if (e != cudaSuccess) return e;
                 cudaLaunchConfig_t cfg = {};
                 cfg.gridDim = dim3(grid.x * 8, grid.y);

@@ -32,6 +32,7 @@ constexpr int kChunk = 128;                           // velocities (directions)
 constexpr int kNF = 26, kWarps = 8, kCpw = 4;         // record words; warps of a CTA; cells of a warp in a round
 // 80 registers a thread: 2, 3, 4 CTAs per SM took 121, 102, 112 us on the case above
 constexpr int kCtasPerSm = 3;
+constexpr int kMaxTable = 64 * 1024;                  // bytes of the velocity sets in shared memory at most
 constexpr int kRec = 24;                              // sums of a cell (gas, then photons), in threes
 
 template <int DIM>
@@ -357,8 +358,10 @@ int run(long long n_cells, int n_xi, const double *xi, const double *w, int n_om
     const long long per = std::max<long long>(kWarps, (n_cells + slots - 1) / slots);
     const unsigned ctas = (unsigned)((n_cells + per - 1) / per);
     auto go = [&](auto kern, size_t smem) {
+        // always the bound, never this call's size: the limit belongs to the kernel, and another
+        // thread's call may set it between here and the launch
         if (smem > 16384 &&
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxTable) != cudaSuccess)
             return GSIS_ERR_CUDA;
         kern<<<ctas, 32 * kWarps, smem, s>>>(n_cells, n_xi, n_om, xi, w, om, wo, static_cast<const Real *>(f),
                                              static_cast<const Real *>(I), 2.0 / d_r, 2.0 / d_v,
@@ -369,7 +372,7 @@ int run(long long n_cells, int n_xi, const double *xi, const double *w, int n_om
     // the FP32 tables of the sets while kCtasPerSm CTAs of them fit an SM
     const size_t tab = ((size_t)n_xi * (2 * DIM + 1) + (size_t)n_om * (1 + DIM)) * sizeof(float);
     if constexpr (std::is_same<Real, float>::value)
-        if (tab <= 64 * 1024)
+        if (tab <= kMaxTable)
             return vec ? go(k_static<Real, DIM, true, true>, tab) : go(k_static<Real, DIM, true, false>, tab);
     return vec ? go(k_static<Real, DIM, false, true>, 0) : go(k_static<Real, DIM, false, false>, 0);
 }

@@ -65,3 +65,34 @@ def test_the_context_stream_orders_all_work(G, name, order, defect, precision, m
     finally:
         G.gsis_destroy(ctx)
     assert _fake.report(G, "unordered") == []
+
+
+def test_kernel_attributes_are_the_same_for_every_caller(G):
+    # a kernel's shared-memory limit belongs to the process: calls of other threads, with other
+    # velocity sets or relaxation blocks, may come between one call's setting and its launch
+    G.fake.fake_reset()
+    a = np.zeros(64)
+    p = a.ctypes.data
+    for dim, precision in ((1, "fp32"), (2, "fp32"), (1, "fp64"), (2, "fp64")):
+        for n_xi in (100, 900, 2000, 3000, 5000):
+            for f in (p, p + 8):
+                assert G.gsis_moments_static(dim, precision, 40, n_xi, p, p, 64, p, p, f, p, 2.0, 2.0, 0.01, p,
+                                             STREAM) == G.GSIS_OK
+    cases = [(gi.workloads.slab(n_cells=70, n_xi=16, n_mu=8), "fp64"), (gi.workloads.cavity(n_side=9, n_v=8), "fp32"),
+             (gi.workloads.cavity(n_side=9, n_v=40), "fp64"), (gi.workloads.capsule(n=4, n_v=6, n_polar=4, n_azim=4), "fp32")]
+    for base, precision in cases:
+        for order in (1, 2):
+            for block in (1, 16, 48):
+                ctx = _create(G, gi.workloads.with_solver(base, precision=precision, order=order, relax_block=block))
+                try:
+                    assert G.load().gsis_step_async(ctx, G.GSIS_MODE_CIS) == G.GSIS_OK
+                finally:
+                    G.gsis_destroy(ctx)
+    G.gsis_mlp_init(ctx := _create(G, gi.workloads.slab(n_cells=8, n_xi=16, n_mu=8)), 1)
+    try:
+        for n in (1, 2000, 5000):
+            G.gsis_mlp_predict(ctx, np.zeros((n, 16), np.float32))
+            G.gsis_mlp_loss_grad(ctx, np.zeros((n, 16), np.float32), np.zeros((n, 12), np.float32))
+    finally:
+        G.gsis_destroy(ctx)
+    assert _fake.report(G, "attribute") == []
