@@ -2211,15 +2211,18 @@ void mlp_free(gsis_ctx *c, T *&p) {
 int mlp_ensure(gsis_ctx *c, int64_t n) {
     MlpDev &d = c->mlp;
     if (!d.p) {
-        TRY(mlp_malloc(c, (void **)&d.p, MLP_NPARAM * sizeof(float)));
-        TRY(mlp_malloc(c, (void **)&d.g, MLP_NW * sizeof(float)));
-        TRY(mlp_malloc(c, (void **)&d.m1, MLP_NW * sizeof(float)));
-        TRY(mlp_malloc(c, (void **)&d.m2, MLP_NW * sizeof(float)));
-        TRY(mlp_malloc(c, &d.pb, MLP_NW * 2));
-        TRY(mlp_malloc(c, (void **)&d.gpart, (size_t)MLP_SPLITS * MLP_NW * sizeof(float)));
-        TRY(mlp_malloc(c, (void **)&d.lpart, (MLP_CTAS + 1) * sizeof(double)));
-        TRY(mlp_malloc(c, (void **)&c->mlp_X, (size_t)c->nc * MLP_IN * sizeof(float)));
-        TRY(mlp_malloc(c, (void **)&c->mlp_Y, (size_t)c->nc * MLP_OUT * sizeof(float)));
+        // what an earlier call got before one of its allocations failed is kept; the parameters,
+        // by which the other entry points know that there is a network, come last
+        auto get = [&](auto **p, size_t bytes) { return *p ? GSIS_OK : mlp_malloc(c, (void **)p, bytes); };
+        TRY(get(&d.g, MLP_NW * sizeof(float)));
+        TRY(get(&d.m1, MLP_NW * sizeof(float)));
+        TRY(get(&d.m2, MLP_NW * sizeof(float)));
+        TRY(get(&d.pb, MLP_NW * 2));
+        TRY(get(&d.gpart, (size_t)MLP_SPLITS * MLP_NW * sizeof(float)));
+        TRY(get(&d.lpart, (MLP_CTAS + 1) * sizeof(double)));
+        TRY(get(&c->mlp_X, (size_t)c->nc * MLP_IN * sizeof(float)));
+        TRY(get(&c->mlp_Y, (size_t)c->nc * MLP_OUT * sizeof(float)));
+        TRY(get(&d.p, MLP_NPARAM * sizeof(float)));
         CUDA_TRY(c, cudaMemsetAsync(d.p, 0, MLP_NPARAM * sizeof(float), c->stream));
         CUDA_TRY(c, cudaMemsetAsync(d.m1, 0, MLP_NW * sizeof(float), c->stream));
         CUDA_TRY(c, cudaMemsetAsync(d.m2, 0, MLP_NW * sizeof(float), c->stream));
@@ -2365,6 +2368,7 @@ int gsis_mlp_train(gsis_ctx *c, const float *X, const float *Y, int64_t n, int32
     const int64_t need = n * (MLP_IN + MLP_OUT);
     if (need > c->mlp_data_cap) {
         mlp_free(c, c->mlp_data);
+        c->mlp_data_cap = 0;
         TRY(mlp_malloc(c, (void **)&c->mlp_data, need * sizeof(float)));
         c->mlp_data_cap = need;
     }

@@ -29,6 +29,7 @@ def load(folder):
     G.fake.fake_report.restype = C.c_char_p
     G.fake.fake_launch.restype = C.c_char_p
     G.fake.fake_cleared.argtypes = [C.c_size_t]
+    G.fake.fake_device_bytes.restype = C.c_size_t
     G.fake.fake_fail_malloc_after.argtypes = [C.c_longlong]
     return G
 

@@ -14,6 +14,7 @@
 // Reported (fake_report, one line each):
 //  unordered <name>   work on another stream while default-stream work is incomplete
 //  rewritten          a pinned source that changed between a copy's enqueueing and its completion
+//  null               a copy or clear of a null pointer
 //  attribute <kernel> a kernel's attribute set to another value than before (the attribute
 //                     belongs to the kernel, for every thread of the process)
 #include <cuda_runtime_api.h>
@@ -92,6 +93,12 @@ void record(const void *fun, dim3 g, dim3 b, size_t smem, cudaStream_t st) {
     enqueue(st, S().names[fun]);
 }
 
+// a null pointer among the buffers of a copy or clear
+cudaError_t null_buffer() {
+    say("null");
+    return cudaErrorInvalidValue;
+}
+
 void note_clear(void *p, size_t n) {
     auto it = S().device.find((const char *)p);
     if (it != S().device.end() && n >= it->second) S().cleared.push_back(it->second);
@@ -112,6 +119,11 @@ void fake_reset() {
     s.mallocs_left = -1;
 }
 void fake_fail_malloc_after(long long n) { S().mallocs_left = n; }
+size_t fake_device_bytes() {
+    size_t n = 0;
+    for (auto &p : S().device) n += p.second;
+    return n;
+}
 int fake_launch_count() { return (int)S().launches.size(); }
 const char *fake_launch(int k, int *grid, int *block) {
     const Launch &l = S().launches[k];
@@ -209,35 +221,41 @@ cudaError_t cudaFreeHost(void *p) {
 }
 
 cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind k) {
+    if (!d || !s) return null_buffer();
     complete(nullptr, S().seq);
     std::memcpy(d, s, n);
     if (k == cudaMemcpyHostToDevice) enqueue(nullptr, "copy");
     return cudaSuccess;
 }
 cudaError_t cudaMemcpy2D(void *d, size_t dp, const void *s, size_t sp, size_t w, size_t h, cudaMemcpyKind k) {
+    if (!d || !s) return null_buffer();
     complete(nullptr, S().seq);
     for (size_t r = 0; r < h; ++r) std::memcpy((char *)d + r * dp, (const char *)s + r * sp, w);
     if (k == cudaMemcpyHostToDevice) enqueue(nullptr, "copy");
     return cudaSuccess;
 }
 cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind k, cudaStream_t st) {
+    if (!d || !s) return null_buffer();
     enqueue(st, "copy", k == cudaMemcpyHostToDevice ? s : nullptr, n);
     std::memcpy(d, s, n);
     return cudaSuccess;
 }
 cudaError_t cudaMemcpy2DAsync(void *d, size_t dp, const void *s, size_t sp, size_t w, size_t h, cudaMemcpyKind,
                               cudaStream_t st) {
+    if (!d || !s) return null_buffer();
     enqueue(st, "copy");
     for (size_t r = 0; r < h; ++r) std::memcpy((char *)d + r * dp, (const char *)s + r * sp, w);
     return cudaSuccess;
 }
 cudaError_t cudaMemset(void *p, int v, size_t n) {
+    if (!p) return null_buffer();
     std::memset(p, v, n);
     note_clear(p, n);
     enqueue(nullptr, "clear");
     return cudaSuccess;
 }
 cudaError_t cudaMemsetAsync(void *p, int v, size_t n, cudaStream_t st) {
+    if (!p) return null_buffer();
     std::memset(p, v, n);
     note_clear(p, n);
     enqueue(st, "clear");

@@ -96,3 +96,41 @@ def test_kernel_attributes_are_the_same_for_every_caller(G):
     finally:
         G.gsis_destroy(ctx)
     assert _fake.report(G, "attribute") == []
+
+
+def _network_calls(G, ctx):
+    X, Y = np.ones((40, 16), np.float32), np.ones((40, 12), np.float32)
+    G.gsis_mlp_init(ctx, 1)
+    G.gsis_mlp_loss_grad(ctx, X, Y)
+    G.gsis_mlp_train(ctx, X, Y, epochs=1, batch=20)
+    G.gsis_mlp_train(ctx, X[:20], Y[:20], epochs=1, batch=20)
+
+
+def test_closure_buffers_after_a_failed_allocation(G):
+    # whichever allocation fails, the call is refused and a later one finds every buffer there
+    wl = gi.workloads.slab(n_cells=8, n_xi=16, n_mu=8)
+    G.fake.fake_reset()
+    ctx = _create(G, wl)
+    _network_calls(G, ctx)
+    whole = G.fake.fake_device_bytes()
+    G.gsis_destroy(ctx)
+    for k in range(100):
+        ctx = _create(G, wl)
+        try:
+            G.fake.fake_fail_malloc_after(k)
+            failed = False
+            for _ in range(2):
+                try:
+                    _network_calls(G, ctx)
+                except G.GsisError as e:
+                    assert e.code == G.GSIS_ERR_OUT_OF_MEMORY
+                    failed = True
+                    G.fake.fake_fail_malloc_after(-1)
+            G.fake.fake_fail_malloc_after(-1)
+            assert G.fake.fake_device_bytes() == whole, k
+            if not failed:
+                break
+        finally:
+            G.fake.fake_fail_malloc_after(-1)
+            G.gsis_destroy(ctx)
+    assert k > 20 and _fake.report(G, "freed") == []
