@@ -1295,8 +1295,11 @@ int gsis_create(const gsis_mesh *m, const gsis_velocity_quad *vq, const gsis_pho
     if (c->order == 2) {
         A_(dalloc_real(c, &c->fface, nfi1 * c->Vp * 4));
         A_(dalloc_real(c, &c->oface, nfi1 * c->Op));
-        // values that no cell writes (xi . n = 0) are read with the factor xi . n
-        if (cudaMemsetAsync(c->fface, 0, nfi1 * c->Vp * 4 * c->real_size, c->stream) != cudaSuccess) return bail(GSIS_ERR_CUDA);
+        // values that no cell writes (xi . n = 0) are read with the factor xi . n, which in 3-D the
+        // sweep forms as (S/V n) . xi: not always zero where the slope pass's is
+        if (cudaMemsetAsync(c->fface, 0, nfi1 * c->Vp * 4 * c->real_size, c->stream) != cudaSuccess ||
+            cudaMemsetAsync(c->oface, 0, nfi1 * c->Op * c->real_size, c->stream) != cudaSuccess)
+            return bail(GSIS_ERR_CUDA);
     }
     A_(dalloc(c, &c->fields, (size_t)nc * NF));
     A_(dalloc(c, &c->fields_old, (size_t)nc * NF));

@@ -134,3 +134,16 @@ def test_closure_buffers_after_a_failed_allocation(G):
             G.fake.fake_fail_malloc_after(-1)
             G.gsis_destroy(ctx)
     assert k > 20 and _fake.report(G, "freed") == []
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_face_values_are_defined_before_the_first_sweep(G, precision):
+    # an upwind value is written where xi . n > 0 on one side; in 3-D the sweep's S/V xi . n may
+    # round to something else than zero where xi . n is zero, and then reads what nobody wrote
+    wl = gi.workloads.with_solver(gi.workloads.capsule(n=4, n_v=6, n_polar=4, n_azim=4), precision=precision, order=2)
+    faces, real = int((wl.mesh.face_nbr >= 0).sum()), 4 if precision == "fp32" else 8
+    pad = lambda n: (n + 63) // 64 * 64  # noqa: E731
+    G.fake.fake_reset()
+    G.gsis_destroy(_create(G, wl))
+    assert G.fake.fake_cleared(faces * pad(wl.w.size) * 4 * real) == 1       # gas
+    assert G.fake.fake_cleared(faces * pad(wl.wo.size) * real) == 1          # photons
