@@ -1506,11 +1506,16 @@ __global__ void __launch_bounds__(32 * S32<DIM>::ROWS, FM < MAXF ? 6 : 5)
             if (src >= 0) {
                 // order 2: the face's upwind value serves both directions (a = 0: zero, never
                 // written); order 1: the neighbour's value where it enters, the cell's where it
-                // leaves
+                // leaves (chosen, not multiplied by zero: a value that is not finite moves with
+                // the flow only)
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
-                    vfma(ORDER == 2 ? -a[u] : -fminf(a[u], 0.0f), fk[k][u], r[u]);
-                    if (ORDER == 1) vfma(-fmaxf(a[u], 0.0f), fi[u], r[u]);
+                    V<float, 4> up = fk[k][u];
+                    if (ORDER == 1) {
+#pragma unroll
+                        for (int p = 0; p < 4; ++p) up.x[p] = a[u] < 0.0f ? up.x[p] : fi[u].x[p];
+                    }
+                    vfma(-a[u], up, r[u]);
                 }
                 continue;
             }
