@@ -1269,9 +1269,9 @@ __global__ void __launch_bounds__(SV * ROWS, sizeof(Real) == 4 ? (DIM < 3 ? 8 : 
 
 // ------------------------------------------------------------------ the FP32 gas sweep
 __device__ __forceinline__ float2 dup2(float x) { return make_float2(x, x); }
-__device__ __forceinline__ float ex2_ftz(float x) {   // 2^x, results below 2^-126 as 0
+__device__ __forceinline__ float ex2(float x) {       // 2^x, subnormal results included
     float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    asm("ex2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 // 1 / x, one Newton step beyond rcp_normal
@@ -1326,7 +1326,7 @@ __device__ __forceinline__ void reference32(const float4 *__restrict__ C, const 
             w[4 * t + 2] = x.z;
             w[4 * t + 3] = x.w;
         }
-        const float2 e = make_float2(ex2_ftz(w[0] * c2.x), ex2_ftz(w[0] * c2.y));
+        const float2 e = make_float2(ex2(w[0] * c2.x), ex2(w[0] * c2.y));
         float2 qc = mul(w[6], c[0]), r1 = mul(w[7], c[0]), r2 = mul(w[8], c[0]);
 #pragma unroll
         for (int a = 1; a < DIM; ++a) {
