@@ -5,8 +5,8 @@
 // plugin that may only use the buffers it is handed), or latency-critical loops that
 // cannot afford a cudaMalloc/cudaFree pair per call.  Such callers cannot create a
 // gsis context (gsis_create allocates), so this entry point takes device pointers.  It is
-// one kernel that keeps its intermediate sums in shared memory: calls share nothing, may
-// overlap on a GPU and may be captured.
+// one kernel (one of two) that keeps its intermediate sums in shared memory: calls share
+// nothing, may overlap on a GPU and may be captured.
 //
 // Accuracy: the gas moments are summed about a per-cell shift velocity u0 (the cell's
 // own mean velocity from a first pass over its mass and momentum), so that the third
@@ -15,10 +15,14 @@
 // and are then carried in two words (Knuth's two-sum).
 //
 // What bounds it: the one pass over f (the second pass of a cell, right after the first,
-// finds it in L1 or L2).  20 000 cells x 784 velocities, FP32: 301 -> 102 us (two passes over
+// finds it in L1 or L2).  20 000 cells x 784 velocities, FP32: 301 -> 108 us (two passes over
 // memory, an FP64 subtraction and conversion per velocity component and five kernels before).
+// Few cells of large sets would leave most of the chip idle with a warp per cell: there a
+// cluster of CTAs takes a cell (FP32, one cell of 9 216 velocities: 308 us by one warp, 19 by
+// eight CTAs, 126 by the five kernels; FP64 389, 35 and 96).
 #include <algorithm>
 #include <cmath>
+#include <cooperative_groups.h>
 #include <type_traits>
 
 #include "../../include/gsis.h"
@@ -32,7 +36,16 @@ constexpr int kChunk = 128;                           // velocities (directions)
 constexpr int kNF = 26, kWarps = 8, kCpw = 4;         // record words; warps of a CTA; cells of a warp in a round
 // 80 registers a thread: 2, 3, 4 CTAs per SM took 121, 102, 112 us on the case above
 constexpr int kCtasPerSm = 3;
-constexpr int kMaxTable = 64 * 1024;                  // bytes of the velocity sets in shared memory at most
+// bytes of the velocity sets in shared memory at most (three CTAs per SM hold 61 KB of them
+// each, beside 14 KB of sums; between that and the limit two run)
+constexpr int kMaxTable = 64 * 1024;
+constexpr int kWideRun = 128;                         // velocities of a plain sum where a cell is split
+// FP64: a cell is split among CTAs (k_static_wide) up to kWideCells cells, from kWideSet
+// velocities or directions on.  us, split and whole: 64 x 784 22 and 74, 456 x 784 48 and 75,
+// 700 x 784 74 and 75, 1 000 x 784 101 and 76, 700 x 9 216 484 and 738, 1 000 x 9 216 674 and
+// 739; one cell of 9 216 35 and 389.
+constexpr long long kWideCells = 700;
+constexpr int kWideSet = 256;
 constexpr int kRec = 24;                              // sums of a cell (gas, then photons), in threes
 
 template <int DIM>
@@ -89,7 +102,7 @@ struct Sum<double> {
     __device__ __forceinline__ double value() const { return hi; }
 };
 
-// The velocity set as a lane reads it.  FP32 with a table in shared memory: each component in
+// The velocity set as a lane reads it.  With a table in shared memory (FP32): each component in
 // two floats, hi + lo, and the weight, converted once per CTA; else straight from the FP64 set.
 template <typename Real, int DIM, bool TAB>
 struct Velocities {
@@ -114,6 +127,145 @@ struct Velocities {
         }
     }
 };
+
+// The photon directions likewise: weights and components in floats where TAB.
+template <typename Real, int DIM, bool TAB>
+struct Directions {
+    const double *om, *wo;
+    const float *tab;
+    int n;
+    __device__ __forceinline__ Real weight(int o) const {
+        if constexpr (TAB) return tab[o];
+        else return to_real<Real>(wo[o]);
+    }
+    __device__ __forceinline__ Real x(int o, int a) const {
+        if constexpr (TAB) return tab[(1 + a) * n + o];
+        else return to_real<Real>(om[(size_t)o * 3 + a]);
+    }
+};
+
+// The four planes of a velocity; VEC: f is aligned to such a record, which is read at once
+template <typename Real, bool VEC>
+struct __align__((VEC ? 4 : 1) * sizeof(Real)) Planes {
+    Real v[4];
+};
+
+// Mass and momentum of the velocities first, first + step, ... (a lane's), summed over the warp
+template <int DIM, typename Real, typename Vel, typename Four>
+__device__ __forceinline__ void mass_momentum(const Vel &vel, const Four *fc, int first, int step, int n_xi,
+                                              Real (&m)[1 + DIM]) {
+#pragma unroll
+    for (int k = 0; k <= DIM; ++k) m[k] = Real(0);
+#pragma unroll 8
+    for (int v = first; v < n_xi; v += step) {
+        const Real w0 = vel.weight(v) * fc[v].v[0];
+        m[0] += w0;
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) m[1 + a] += w0 * vel.x(v, a);
+    }
+#pragma unroll
+    for (int k = 0; k <= DIM; ++k)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m[k] += __shfl_xor_sync(0xffffffffu, m[k], o);
+}
+
+// Adds a lane's share of the gas moments of the RUN velocities from v0 on, about u, to S
+template <int DIM, int RUN, typename Real, typename Vel, typename Four>
+__device__ __forceinline__ void add_gas_run(const Vel &vel, const Four *fc, int v0, int n_xi, int lane,
+                                            const Real (&u)[DIM], Sum<Real> (&S)[kRec]) {
+    constexpr int NM = n_moments<DIM>();
+    Real acc[NM];
+#pragma unroll
+    for (int k = 0; k < NM; ++k) acc[k] = Real(0);
+    // the run's loads first; past the set's end the last velocity with no weight
+    Four fr[RUN / 32];
+#pragma unroll
+    for (int h = 0; h < RUN / 32; ++h) fr[h] = fc[min(v0 + 32 * h + lane, n_xi - 1)];
+#pragma unroll
+    for (int h = 0; h < RUN / 32; ++h) {
+        if (v0 + 32 * h >= n_xi) break;
+        const int v = min(v0 + 32 * h + lane, n_xi - 1);
+        const Four &fv = fr[h];
+        Real c[DIM], c2 = Real(0);
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+            c[a] = vel.minus(v, a, u[a]);
+            c2 = fma(c[a], c[a], c2);
+        }
+        const Real wv = v0 + 32 * h + lane < n_xi ? vel.weight(v) : Real(0), w0 = wv * fv.v[0];
+        Real wc[DIM];
+        int k = 0;
+        acc[k++] += w0;
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+            wc[a] = w0 * c[a];
+            acc[k++] += wc[a];
+        }
+#pragma unroll
+        for (int a = 0; a < DIM; ++a)
+#pragma unroll
+            for (int b = a; b < DIM; ++b, ++k) acc[k] = fma(wc[a], c[b], acc[k]);
+#pragma unroll
+        for (int a = 0; a < DIM; ++a, ++k) acc[k] = fma(wc[a], c2, acc[k]);
+#pragma unroll
+        for (int p = 1; p < 4; ++p) {
+            const Real wp = wv * fv.v[p];
+            acc[k++] += wp;
+#pragma unroll
+            for (int a = 0; a < DIM; ++a, ++k) acc[k] = fma(wp, c[a], acc[k]);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < NM; ++k) S[k].add(acc[k]);
+}
+
+// the photon moments of the RUN directions from o0 on likewise
+template <int DIM, int RUN, typename Real, typename Dir>
+__device__ __forceinline__ void add_photon_run(const Dir &dir, const Real *Ic, int o0, int n_om, int lane,
+                                               Sum<Real> (&S)[kRec]) {
+    constexpr int NM = n_moments<DIM>();
+    Real acc[1 + DIM];
+#pragma unroll
+    for (int k = 0; k <= DIM; ++k) acc[k] = Real(0);
+#pragma unroll
+    for (int h = 0; h < RUN / 32; ++h) {
+        const int o = o0 + 32 * h + lane;
+        if (o >= n_om) break;
+        const Real wI = dir.weight(o) * Ic[o];
+        acc[0] += wI;
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) acc[1 + a] += wI * dir.x(o, a);
+    }
+#pragma unroll
+    for (int k = 0; k <= DIM; ++k) S[NM + k].add(acc[k]);
+}
+
+// Sums S over the lanes: at the first three steps a lane passes half of its sums on, so that
+// it ends with three, S[0..2], numbers first, first + 1, first + 2 (returned; the same in four
+// consecutive lanes): 12 + 6 + 3 + 2 x 3 exchanges instead of 5 x 20
+template <typename Real>
+__device__ __forceinline__ int fold_lanes(int lane, Sum<Real> (&S)[kRec]) {
+    int first = 0;
+#pragma unroll
+    for (int step = 0; step < 3; ++step) {
+        const int half = 12 >> step, o = 16 >> step;
+        const bool up = lane & o;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            if (k >= half) break;
+            const Sum<Real> a = S[k], b = S[half + k], got = (up ? a : b).shfl(o);
+            S[k] = up ? b : a;
+            S[k].add(got);
+        }
+        first += up ? half : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        S[k].add(S[k].shfl(2));
+        S[k].add(S[k].shfl(1));
+    }
+    return first;
+}
 
 // Sums S about u0 + the photon sums -> the cell's field record (rho, u, T_t, T_r, T_v, T_R,
 // heat fluxes, stress).  u below is the residual velocity u - u0, and the central moments
@@ -219,9 +371,8 @@ __global__ void __launch_bounds__(32 * kWarps, kCtasPerSm) k_static(long long n_
     const Velocities<Real, DIM, TAB> vel{xi, w, s_tab, n_xi};
     const float *pt = s_tab + (2 * DIM + 1) * n_xi;       // photon weights and directions
     const long long begin = (long long)blockIdx.x * per_cta, end = min(n_cells, begin + per_cta);
-    struct __align__((VEC ? 4 : 1) * sizeof(Real)) Four {
-        Real v[4];
-    };
+    const Directions<Real, DIM, TAB> dir{om, wo, pt, n_om};
+    using Four = Planes<Real, VEC>;
     int round = 0;
     for (long long base = begin; base < end; base += kWarps * kCpw, ++round) {
         const int buf = round & 1;
@@ -231,107 +382,16 @@ __global__ void __launch_bounds__(32 * kWarps, kCtasPerSm) k_static(long long n_
             if (i >= end) break;
             const Four *fc = reinterpret_cast<const Four *>(f) + (size_t)i * n_xi;
             // mass and momentum: the shift velocity (any value near the mean velocity serves)
-            Real m[1 + DIM];
-#pragma unroll
-            for (int k = 0; k <= DIM; ++k) m[k] = Real(0);
-#pragma unroll 8
-            for (int v = lane; v < n_xi; v += 32) {
-                const Real w0 = vel.weight(v) * fc[v].v[0];
-                m[0] += w0;
-#pragma unroll
-                for (int a = 0; a < DIM; ++a) m[1 + a] += w0 * vel.x(v, a);
-            }
-#pragma unroll
-            for (int k = 0; k <= DIM; ++k)
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) m[k] += __shfl_xor_sync(0xffffffffu, m[k], o);
-            Real u[DIM];
+            Real m[1 + DIM], u[DIM];
+            mass_momentum<DIM>(vel, fc, lane, 32, n_xi, m);
 #pragma unroll
             for (int a = 0; a < DIM; ++a) u[a] = m[0] > Real(0) ? m[1 + a] / m[0] : Real(0);
             Sum<Real> S[kRec];
-            for (int v0 = 0; v0 < n_xi; v0 += kRun) {
-                Real acc[NM];
-#pragma unroll
-                for (int k = 0; k < NM; ++k) acc[k] = Real(0);
-                // the run's loads first; past the set's end the last velocity with no weight
-                Four fr[kRun / 32];
-#pragma unroll
-                for (int h = 0; h < kRun / 32; ++h) fr[h] = fc[min(v0 + 32 * h + lane, n_xi - 1)];
-#pragma unroll
-                for (int h = 0; h < kRun / 32; ++h) {
-                    if (v0 + 32 * h >= n_xi) break;
-                    const int v = min(v0 + 32 * h + lane, n_xi - 1);
-                    const Four &fv = fr[h];
-                    Real c[DIM], c2 = Real(0);
-#pragma unroll
-                    for (int a = 0; a < DIM; ++a) {
-                        c[a] = vel.minus(v, a, u[a]);
-                        c2 = fma(c[a], c[a], c2);
-                    }
-                    const Real wv = v0 + 32 * h + lane < n_xi ? vel.weight(v) : Real(0), w0 = wv * fv.v[0];
-                    Real wc[DIM];
-                    int k = 0;
-                    acc[k++] += w0;
-#pragma unroll
-                    for (int a = 0; a < DIM; ++a) {
-                        wc[a] = w0 * c[a];
-                        acc[k++] += wc[a];
-                    }
-#pragma unroll
-                    for (int a = 0; a < DIM; ++a)
-#pragma unroll
-                        for (int b = a; b < DIM; ++b, ++k) acc[k] = fma(wc[a], c[b], acc[k]);
-#pragma unroll
-                    for (int a = 0; a < DIM; ++a, ++k) acc[k] = fma(wc[a], c2, acc[k]);
-#pragma unroll
-                    for (int p = 1; p < 4; ++p) {
-                        const Real wp = wv * fv.v[p];
-                        acc[k++] += wp;
-#pragma unroll
-                        for (int a = 0; a < DIM; ++a, ++k) acc[k] = fma(wp, c[a], acc[k]);
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < NM; ++k) S[k].add(acc[k]);
-            }
+            for (int v0 = 0; v0 < n_xi; v0 += kRun) add_gas_run<DIM, kRun>(vel, fc, v0, n_xi, lane, u, S);
             const Real *Ic = I + (size_t)i * n_om;
-            for (int o0 = 0; o0 < n_om; o0 += kRun) {
-                Real acc[1 + DIM];
-#pragma unroll
-                for (int k = 0; k <= DIM; ++k) acc[k] = Real(0);
-#pragma unroll
-                for (int h = 0; h < kRun / 32; ++h) {
-                    const int o = o0 + 32 * h + lane;
-                    if (o >= n_om) break;
-                    const Real wI = TAB ? pt[o] * Ic[o] : to_real<Real>(wo[o]) * Ic[o];
-                    acc[0] += wI;
-#pragma unroll
-                    for (int a = 0; a < DIM; ++a) acc[1 + a] += wI * (TAB ? pt[(1 + a) * n_om + o] : to_real<Real>(om[(size_t)o * 3 + a]));
-                }
-#pragma unroll
-                for (int k = 0; k <= DIM; ++k) S[NM + k].add(acc[k]);
-            }
-            // sum over the lanes: at the first three steps a lane passes half of its sums on, so
-            // that it ends with three (12 + 6 + 3 + 2 x 3 exchanges instead of 5 x 20)
-            int first = 0;
-#pragma unroll
-            for (int step = 0; step < 3; ++step) {
-                const int half = 12 >> step, o = 16 >> step;
-                const bool up = lane & o;
-#pragma unroll
-                for (int k = 0; k < 12; ++k) {
-                    if (k >= half) break;
-                    const Sum<Real> a = S[k], b = S[half + k], got = (up ? a : b).shfl(o);
-                    S[k] = up ? b : a;
-                    S[k].add(got);
-                }
-                first += up ? half : 0;
-            }
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                S[k].add(S[k].shfl(2));
-                S[k].add(S[k].shfl(1));
-            }
+            for (int o0 = 0; o0 < n_om; o0 += kRun)
+                add_photon_run<DIM, kRun>(dir, Ic, o0, n_om, lane, S);
+            const int first = fold_lanes(lane, S);
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 const double x = S[k].value();
@@ -345,6 +405,82 @@ __global__ void __launch_bounds__(32 * kWarps, kCtasPerSm) k_static(long long n_
         if (warp == round % kWarps && base + lane < end)
             finish<DIM>(sums[buf][lane], sums[buf][lane] + NM, shift[buf][lane], i_half_dr, i_half_dv, i_4sigma,
                         out + (size_t)(base + lane) * kNF);
+    }
+}
+
+// One cell by a cluster of CTAs, whose warps take the cell's velocities in runs: for few cells,
+// which k_static would leave to as many warps, and for FP32 sets too large for its tables (each
+// component is then taken from the FP64 set).  The sums are added per warp, per CTA and over
+// the cluster, each in a fixed order.
+template <typename Real, int DIM, bool VEC>
+__global__ void __launch_bounds__(32 * kWarps, kCtasPerSm) k_static_wide(int n_xi, int n_om, const double *__restrict__ xi,
+                                                             const double *__restrict__ w,
+                                                             const double *__restrict__ om,
+                                                             const double *__restrict__ wo,
+                                                             const Real *__restrict__ f, const Real *__restrict__ I,
+                                                             double i_half_dr, double i_half_dv, double i_4sigma,
+                                                             double *__restrict__ out) {
+    constexpr int NM = n_moments<DIM>();
+    __shared__ Real m_warp[kWarps][1 + DIM], m_cta[1 + DIM];
+    __shared__ double sums[kRec], words[(kWarps + 1) * kRec];       // a Sum of either type is 8 bytes
+    static_assert(sizeof(Sum<Real>) == sizeof(double), "sums in shared memory");
+    Sum<Real> *s_warp = reinterpret_cast<Sum<Real> *>(words), *s_cta = s_warp + kWarps * kRec;
+    const auto cluster = cooperative_groups::this_cluster();
+    const int cs = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wi = rank * kWarps + warp, nw = cs * kWarps;
+    const size_t i = blockIdx.x / (unsigned)cs;
+    using Four = Planes<Real, VEC>;
+    const Four *fc = reinterpret_cast<const Four *>(f) + i * n_xi;
+    const Velocities<Real, DIM, false> vel{xi, w, nullptr, n_xi};
+    const Directions<Real, DIM, false> dir{om, wo, nullptr, n_om};
+    Real m[1 + DIM], u[DIM];
+    mass_momentum<DIM>(vel, fc, wi * 32 + lane, nw * 32, n_xi, m);
+    if (lane == 0)
+#pragma unroll
+        for (int k = 0; k <= DIM; ++k) m_warp[warp][k] = m[k];
+    __syncthreads();
+    if (threadIdx.x <= DIM) {
+        Real t = m_warp[0][threadIdx.x];
+        for (int q = 1; q < kWarps; ++q) t += m_warp[q][threadIdx.x];
+        m_cta[threadIdx.x] = t;
+    }
+    cluster.sync();
+#pragma unroll
+    for (int k = 0; k <= DIM; ++k) m[k] = Real(0);
+    for (int r = 0; r < cs; ++r) {
+        const Real *t = cluster.map_shared_rank(m_cta, r);
+#pragma unroll
+        for (int k = 0; k <= DIM; ++k) m[k] += t[k];
+    }
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) u[a] = m[0] > Real(0) ? m[1 + a] / m[0] : Real(0);
+    Sum<Real> S[kRec];
+    for (int v0 = wi * kWideRun; v0 < n_xi; v0 += nw * kWideRun)
+        add_gas_run<DIM, kWideRun>(vel, fc, v0, n_xi, lane, u, S);
+    for (int o0 = wi * kWideRun; o0 < n_om; o0 += nw * kWideRun)
+        add_photon_run<DIM, kWideRun>(dir, I + i * n_om, o0, n_om, lane, S);
+    const int first = fold_lanes(lane, S);
+    if ((lane & 3) == 0)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s_warp[warp * kRec + first + k] = S[k];
+    __syncthreads();
+    if (threadIdx.x < kRec) {
+        Sum<Real> t = s_warp[threadIdx.x];
+        for (int q = 1; q < kWarps; ++q) t.add(s_warp[q * kRec + threadIdx.x]);
+        s_cta[threadIdx.x] = t;
+    }
+    cluster.sync();
+    if (rank == 0 && threadIdx.x < kRec) {
+        Sum<Real> t = s_cta[threadIdx.x];
+        for (int r = 1; r < cs; ++r) t.add(cluster.map_shared_rank(s_cta, r)[threadIdx.x]);
+        sums[threadIdx.x] = t.value();
+    }
+    cluster.sync();      // the other CTAs' shared memory has been read
+    if (rank == 0 && threadIdx.x == 0) {
+        double u0[DIM];
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) u0[a] = to_double(u[a]);
+        finish<DIM>(sums, sums + NM, u0, i_half_dr, i_half_dv, i_4sigma, out + i * kNF);
     }
 }
 
@@ -369,12 +505,33 @@ int run(long long n_cells, int n_xi, const double *xi, const double *w, int n_om
         return cudaGetLastError() == cudaSuccess ? GSIS_OK : GSIS_ERR_CUDA;
     };
     const bool vec = reinterpret_cast<uintptr_t>(f) % (4 * sizeof(Real)) == 0;
-    // the FP32 tables of the sets while kCtasPerSm CTAs of them fit an SM
+    auto go_wide = [&](auto kern) {
+        // as many CTAs per cell as give every warp a run and leave no SM without work
+        int cs = 1;
+        while (cs < 8 && n_cells * cs * 2 <= 2 * 152 && std::max(n_xi, n_om) > cs * kWarps * kWideRun) cs *= 2;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(n_cells * cs));
+        cfg.blockDim = dim3(32 * kWarps);
+        cfg.stream = s;
+        cudaLaunchAttribute at = {};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = cs;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, n_xi, n_om, xi, w, om, wo, static_cast<const Real *>(f),
+                                                 static_cast<const Real *>(I), 2.0 / d_r, 2.0 / d_v,
+                                                 sigma_R > 0.0 ? 1.0 / (4.0 * sigma_R) : 0.0, out);
+        return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? GSIS_OK : GSIS_ERR_CUDA;
+    };
+    // FP32: the tables of the sets while they fit (4 000 cells x 2 304 velocities with them 99 us,
+    // one cell 23); beyond, split, with or without few cells (4 096 velocities, one cell 15 us and
+    // 131 unsplit, 1 000 cells 86 and 156, 4 000 cells 294 and 441)
     const size_t tab = ((size_t)n_xi * (2 * DIM + 1) + (size_t)n_om * (1 + DIM)) * sizeof(float);
-    if constexpr (std::is_same<Real, float>::value)
-        if (tab <= kMaxTable)
-            return vec ? go(k_static<Real, DIM, true, true>, tab) : go(k_static<Real, DIM, true, false>, tab);
-    return vec ? go(k_static<Real, DIM, false, true>, 0) : go(k_static<Real, DIM, false, false>, 0);
+    constexpr bool fp32 = std::is_same<Real, float>::value;
+    if (fp32 ? tab > kMaxTable : n_cells <= kWideCells && std::max(n_xi, n_om) >= kWideSet)
+        return vec ? go_wide(k_static_wide<Real, DIM, true>) : go_wide(k_static_wide<Real, DIM, false>);
+    return vec ? go(k_static<Real, DIM, fp32, true>, fp32 ? tab : 0) : go(k_static<Real, DIM, fp32, false>, fp32 ? tab : 0);
 }
 
 }  // namespace

@@ -1,5 +1,7 @@
-"""The order in which the host gives work to the device, on the CPU: libgsis is linked with a
+"""What the host gives to the device and in which order, on the CPU: libgsis is linked with a
 runtime that records instead of running (fake_cudart.cpp)."""
+import ctypes as C
+
 import numpy as np
 import pytest
 
@@ -147,3 +149,19 @@ def test_face_values_are_defined_before_the_first_sweep(G, precision):
     G.gsis_destroy(_create(G, wl))
     assert G.fake.fake_cleared(faces * pad(wl.w.size) * 4 * real) == 1       # gas
     assert G.fake.fake_cleared(faces * pad(wl.wo.size) * real) == 1          # photons
+
+
+@pytest.mark.parametrize("dim,precision,n_cells,n_xi,ctas", [
+    (2, "fp32", 1, 9216, 8), (2, "fp32", 16, 16384, 128), (2, "fp32", 152, 4096, 152), (2, "fp32", 4000, 4096, 4000),
+    (1, "fp32", 1, 9216, 8), (2, "fp64", 1, 9216, 8), (2, "fp64", 64, 4096, 128), (2, "fp64", 300, 784, 300),
+    (1, "fp64", 64, 784, 64)])
+def test_few_cells_of_large_sets_fill_the_chip(G, dim, precision, n_cells, n_xi, ctas):
+    # one CTA of eight warps per eight cells, whatever the set, left all but a few SMs idle
+    G.fake.fake_reset()
+    a = np.zeros(64)
+    p = a.ctypes.data
+    assert G.gsis_moments_static(dim, precision, n_cells, n_xi, p, p, 64, p, p, p, p, 2.0, 2.0, 0.01, p, STREAM) == G.GSIS_OK
+    grid, block = C.c_int(), C.c_int()
+    assert G.fake.fake_launch_count() == 1
+    G.fake.fake_launch(0, C.byref(grid), C.byref(block))
+    assert grid.value >= ctas and block.value == 256
