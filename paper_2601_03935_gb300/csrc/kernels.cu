@@ -2619,13 +2619,25 @@ __device__ __forceinline__ float2 add2w(float2 a, float2 b) {
     const float2 s = two_sum(a.x, b.x);
     return make_float2(s.x, __fadd_rn(s.y, __fadd_rn(a.y, b.y)));
 }
-// 2^(j / 8)
-__constant__ float2 EXP2_8TH[8] = {
-    {1.000000000e+00f, 0.000000000e+00f},   {1.090507746e+00f, -1.307753994e-08f},
-    {1.189207077e+00f, 3.797635273e-08f},   {1.296839595e+00f, -4.018999533e-08f},
-    {1.414213538e+00f, 2.420323497e-08f},   {1.542210817e+00f, 8.070904833e-09f},
-    {1.681792855e+00f, -2.475532668e-08f},  {1.834008098e+00f, -1.123927795e-08f}};
-// 2^(s c2) = v 2^k: 2^(j/8) from a table times e^r, |r| <= ln 2 / 16, by its Taylor sum
+// 2^(j / EXP2_N) in two words, built by the compiler from the table of fp64.cuh
+constexpr int EXP2_N = 64;
+struct Exp2Table {
+    float hi[EXP2_N], lo[EXP2_N];
+};
+constexpr Exp2Table make_exp2_table() {
+    constexpr fp64::ExpTable E = fp64::make_exp_table();
+    Exp2Table T{};
+    for (int j = 0; j < EXP2_N; ++j) {
+        const double x = E.t[j * (fp64::EXP_N / EXP2_N)];
+        T.hi[j] = (float)x;
+        T.lo[j] = (float)(x - (double)T.hi[j]);
+    }
+    return T;
+}
+__constant__ const Exp2Table g_exp2_table = make_exp2_table();
+// 2^(s c2) = v 2^k: 2^(j/EXP2_N) from the table times e^r, |r| <= ln 2 / (2 EXP2_N), by its
+// Taylor sum.  The rounding of the sum's r^2/2 term is what the result is off by beyond its own
+// rounding: 4e-5 units in the last place (2e-3 with EXP2_N = 8).
 struct Exp2 {
     float2 v;
     float scale;       // v carries the other half of the exponent, so that both are normal numbers
@@ -2636,14 +2648,15 @@ __device__ __forceinline__ Exp2 exp2_two(const float2 *__restrict__ table, float
         y = copysignf(250.0f, y);
         yl = 0.0f;
     }
-    const float k = rintf(8.0f * y), f = fmaf(-0.125f, k, y);
+    const float k = rintf((float)EXP2_N * y), f = fmaf(-1.0f / EXP2_N, k, y);
     const float2 g = two_sum_ordered(f, yl);
     const float L = 0.693147182f, Ll = -1.90465421e-9f;      // ln 2
     const float r = __fmul_rn(g.x, L), rl = fmaf(g.y, L, fmaf(g.x, Ll, fmaf(g.x, L, -r)));
-    const float p = fmaf(r, fmaf(r, fmaf(r, 1.0f / 120.0f, 1.0f / 24.0f), 1.0f / 6.0f), 0.5f);
+    const float p = fmaf(r, fmaf(r, 1.0f / 24.0f, 1.0f / 6.0f), 0.5f);
     const float2 q = two_sum_ordered(r, fmaf(__fmul_rn(r, r), p, rl));      // e^r - 1
-    const int ki = (int)k, n = ki >> 3, n1 = n >> 1;
-    const float2 T = table[ki & 7];
+    const int ki = (int)k, n = ki >> 6, n1 = n >> 1;
+    static_assert(EXP2_N == 64, "the integer part is a shift by 6");
+    const float2 T = table[ki & (EXP2_N - 1)];
     const float t = __fmul_rn(T.x, q.x);
     const float2 e = two_sum_ordered(T.x, t);
     const float el = __fadd_rn(e.y, fmaf(T.x, q.y, fmaf(T.y, q.x, __fadd_rn(T.y, fmaf(T.x, q.x, -t)))));
@@ -2661,16 +2674,18 @@ __device__ __forceinline__ float scaled(float2 N, const Exp2 &e) {   // (N 2^..)
 // The equilibrium in FP32 storage: the start of a run writes f once, and in FP64 arithmetic
 // (the kernel above) its time is that of 17 FP64 instructions per velocity.  Here each cell's
 // constants are formed in FP64 by one thread and kept as two FP32 words, and a velocity takes
-// about 100 FP32 instructions; a value is within 0.502 units in the last place (0.500 before).
+// about 100 FP32 instructions; a value is within 0.5001 units in the last place (0.5000 in FP64
+// arithmetic).
 template <int DIM>
 __global__ void __launch_bounds__(256) k_equilibrium32(int n_cells, int cells, Quad<float> vq, Quad<float> oq,
                                                        ModelDev m, const double *__restrict__ F,
                                                        float *__restrict__ f, float *__restrict__ I) {
     constexpr int MAXC = 16;                                   // cells of a CTA at most
-    __shared__ float2 tab[8], K[MAXC][DIM + 5];                // u, -log2 e / (2 T), the four planes' factors
+    __shared__ float2 tab[EXP2_N], K[MAXC][DIM + 5];                // u, -log2 e / (2 T), the four planes' factors
     __shared__ float B[MAXC];
     const int c0 = blockIdx.x * cells, nc = min(cells, n_cells - c0);
-    if (threadIdx.x >= 32 && threadIdx.x < 40) tab[threadIdx.x - 32] = EXP2_8TH[threadIdx.x - 32];
+    if (threadIdx.x >= 32 && threadIdx.x < 32 + EXP2_N)
+        tab[threadIdx.x - 32] = make_float2(g_exp2_table.hi[threadIdx.x - 32], g_exp2_table.lo[threadIdx.x - 32]);
     if (threadIdx.x < nc) {
         const double *M = F + (size_t)(c0 + threadIdx.x) * NF;
         auto put = [&](int k, double x) {
