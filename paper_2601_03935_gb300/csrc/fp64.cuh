@@ -115,14 +115,15 @@ __device__ __forceinline__ double rcp_d(double x) {
     const double e = fma(-x, r, 1.0);
     return fma(r, fma(e, e, e), r);
 }
-// a / b to within an ulp
+// a / b to within an ulp; where b or the quotient is not moderate (a zero, infinity or NaN
+// among them) as CUDA's division has it
 __device__ __forceinline__ double div_d(double a, double b) {
-    if (!moderate(b)) return a / b;
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
     const double e = fma(-b, r, 1.0);
     r = fma(r, fma(e, e, e), r);
     const double q = a * r;
+    if (!moderate(b) || !moderate(q)) return a / b;
     return fma(fma(-b, q, a), r, q);
 }
 __device__ __forceinline__ double sqrt_d(double x) {
