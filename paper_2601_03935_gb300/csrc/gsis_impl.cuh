@@ -9,6 +9,7 @@ namespace gsis {
 constexpr int MAXF = 4;        // faces per cell (segments, triangles, quads, tetrahedra)
 constexpr int MAXS = 12;       // least-squares stencil: face neighbours and their face neighbours
 constexpr int NF = 26;         // per-cell field record, see gsis.h
+constexpr int SMS = 152;       // SMs of a GB300, for rules on how far a launch fills it
 constexpr int SV = 64;         // discrete velocities (or photon directions) per sweep CTA
 constexpr int SROWS = 2;       // thread rows of a sweep CTA (the block's cells are dealt to them)
 constexpr int VCH = SV;        // velocity chunk of the gas moment partials
@@ -396,7 +397,7 @@ constexpr int MLP_IN = 16, MLP_H = 128, MLP_OUT = 12, MLP_LAYERS = 4;
 constexpr int MLP_NW = MLP_H * MLP_IN + MLP_H + 2 * (MLP_H * MLP_H + MLP_H) + MLP_OUT * MLP_H + MLP_OUT;
 constexpr int MLP_NSTAT = 2 * MLP_IN + 2 * MLP_OUT;
 constexpr int MLP_NPARAM = MLP_NW + MLP_NSTAT;
-constexpr int MLP_CTAS = 152, MLP_SPLITS = 32;   // CTAs of a pass over the rows; row ranges of the weight gradient
+constexpr int MLP_CTAS = SMS, MLP_SPLITS = 32;   // CTAs of a pass over the rows; row ranges of the weight gradient
 
 struct MlpDev {
     int cap = 0;                       // rows the work buffers hold

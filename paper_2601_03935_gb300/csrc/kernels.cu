@@ -61,8 +61,6 @@ __device__ __forceinline__ T pow_neg_half_dim(T x) {
     else if constexpr (DIM == 1) return T(1) / sqrt(x);
     else return T(1) / (x * sqrt(x));
 }
-__device__ __forceinline__ float fdiv(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double fdiv(double a, double b) { return a / b; }
 
 // ------------------------------------------------------------------ coefficients
 template <typename Real, int DIM>
@@ -2850,7 +2848,7 @@ static cudaError_t slopes_t(cudaStream_t s, const Geom<Real> &g, const Quad<Real
                             Real *fface) {
     if constexpr (std::is_same<Real, double>::value) {
         // few cells: one warp per CTA, so that the FP64 work reaches every SM
-        const int cols = (q.n + 31) / 32, rows = (long long)g.n_cells * cols < 152 * SLOPE_ROWS ? 1 : SLOPE_ROWS;
+        const int cols = (q.n + 31) / 32, rows = (long long)g.n_cells * cols < SMS * SLOPE_ROWS ? 1 : SLOPE_ROWS;
         k_slopes64<N, DIM><<<dim3((g.n_cells + rows - 1) / rows, cols), dim3(32, rows), 0, s>>>(g, q.n, q.n_pad, q.x, f,
                                                                                              fface);
         return cudaGetLastError();
@@ -2916,7 +2914,7 @@ static cudaError_t sweep_t(cudaStream_t s, const Geom<Real> &g, const Quad<Real>
         // x 32 velocities: 72 us by one CTA of two rows, 53 of eight rows, 32 by the cluster;
         // 800 x 64: 71, 55, 45).  Photons, with few instructions per value: eight rows.
         if constexpr (N == 4) {
-            if ((long long)grid.x * grid.y < 152) {
+            if ((long long)grid.x * grid.y < SMS) {
                 auto kern = k_sweep<Real, N, DIM, ORDER, RESID, SROWS, 8>;
                 cudaError_t e = allow_smem(kern);
                 if (e != cudaSuccess) return e;
@@ -2935,7 +2933,7 @@ static cudaError_t sweep_t(cudaStream_t s, const Geom<Real> &g, const Quad<Real>
                 return e != cudaSuccess ? e : cudaGetLastError();
             }
         } else if constexpr (std::is_same<Real, double>::value) {
-            if ((long long)grid.x * grid.y < 152)
+            if ((long long)grid.x * grid.y < SMS)
                 return run(k_sweep<Real, N, DIM, ORDER, RESID, 8>, dim3(SV, 8), smem);
         }
         return run(k_sweep<Real, N, DIM, ORDER, RESID>, dim3(SV, SROWS), smem);
@@ -2999,7 +2997,7 @@ cudaError_t launch_equilibrium(cudaStream_t s, int dim, int n_cells, const Quad<
     if constexpr (std::is_same<Real, float>::value) {
         // a cell's constants cost one thread about as much as 70 velocities cost a warp: 16 cells
         // to a CTA, fewer where that leaves SMs without one
-        const int cells = std::max(1, std::min(16, n_cells / 304)), grid = (n_cells + cells - 1) / cells;
+        const int cells = std::max(1, std::min(16, n_cells / (2 * SMS))), grid = (n_cells + cells - 1) / cells;
         GSIS_DISPATCH_DIM3(dim, (k_equilibrium32<DIM><<<grid, 256, 0, s>>>(n_cells, cells, vq, oq, m, fields, f, I)));
     } else {
         GSIS_DISPATCH_DIM3(dim, (k_equilibrium<Real, DIM><<<n_cells, 256, 0, s>>>(n_cells, vq, oq, m, fields, f, I)));

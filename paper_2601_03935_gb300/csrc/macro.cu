@@ -20,9 +20,8 @@
 //  macro_jacobi        one further point-relaxation sweep of
 //                      D dW_i + (1/(2V)) sum_j (dF_j - Gamma dW_j) S = R_i
 //                      in the gas-energy form; the last one adds dW to W
-//  kinetic_bflux       moments of the kinetic boundary fluxes of the current distribution
-//  sync                f <- f + w [f_eq(M^{k+1}) - f_eq(M^{k+1/2})] (Section 3) fused with
-//                      the velocity moments of the result
+// (kinetic_bflux, the kinetic boundary fluxes, and sync, the update of f by the synthetic
+// solution, are in kernels.cu.)
 //
 // Every kernel of the inner loop returns at once when the solve's stop flag is set,
 // so a fixed launch sequence can run past convergence without changing W.
@@ -35,8 +34,8 @@
 // face fluxes once per face, and the relaxation reads its neighbours' flux increments as
 // vectors F_a that the neighbour formed once, not once per adjacent face.
 // Per inner iteration (six sweeps, a GSIS iteration less its kinetic part over 100): 20 000
-// cells, mixed schedule 307 -> 74 us; 2 048 cells, FP64 209 -> 61 us, mixed 112 -> 43 us;
-// 800 cells in 1-D, FP64, order 2, 174 -> 45 us.
+// cells, mixed schedule 307 -> 72 us; 2 048 cells, FP64 209 -> 61 us, mixed 112 -> 40 us;
+// 800 cells in 1-D, FP64, order 2, 174 -> 43 us.
 #include <algorithm>
 #include <cmath>
 
@@ -518,7 +517,7 @@ __device__ void boundary_face(const MacroGeom &g, const ModelDev &m, const QuadD
     const double *in = g.binc + (size_t)b * BINC;
     // F0 = rho (2 pi T)^(-DIM/2) exp(-c^2 / 2T)
     const R i2piT = rcp_r(R(2.0 * PI) * Tt);
-    const R Ac = qc[0] * (DIM == 2 ? i2piT : DIM == 1 ? sqrt_r(i2piT) : i2piT * sqrt_r(i2piT));
+    const R Ac = qc[0] * (DIM == 2 ? i2piT : sqrt_r(i2piT));
     const R hr = c.half_dr * qc[E + 1], hv = vib_e(qc[E + 2], m, c);
     R r[NS];
     r[0] = Ac * acc[0];
@@ -984,7 +983,7 @@ __global__ void __launch_bounds__(128) k_macro_residual(MacroGeom g, MacroState 
 // FP64.  FIRST: no neighbour terms.  LAST: W += dW and the primitive variables of the new W.
 template <typename R, int DIM, bool FIRST, bool LAST>
 __device__ __forceinline__ void k_macro_jacobi_body(MacroGeom g, ModelDev m, const MacroState *__restrict__ st, const double *__restrict__ Rg, const double *__restrict__ Dinv, const R *__restrict__ gam, const R *__restrict__ src, const Row<R> *__restrict__ in, Row<R> *__restrict__ out, double *__restrict__ W, double *__restrict__ qd, float *__restrict__ qf) {
-    constexpr int E = 1 + DIM, ER = 4 + DIM, LPC = 4;
+    constexpr int E = 1 + DIM, LPC = 4;
     if (st->done) return;
     const MacroReal<R> &c = real<R>(g);
     const int t = blockIdx.x * blockDim.x + threadIdx.x, r = t % LPC;
@@ -1094,7 +1093,6 @@ __device__ __forceinline__ void k_macro_jacobi_body(MacroGeom g, ModelDev m, con
         for (int a = 0; a < DIM; ++a) o.x[a] = fma(fi.du[a], X1, u[a] * dX);
         o.x[3] = s1;
         out[(size_t)i * NVM + E + r] = o;
-        (void)ER;
     }
 }
 template <typename R, int DIM, bool FIRST, bool LAST>

@@ -27,6 +27,7 @@
 
 #include "../../include/gsis.h"
 #include "fp64.cuh"
+#include "gsis_impl.cuh"
 
 namespace {
 
@@ -336,7 +337,7 @@ __device__ void finish(const double *S, const double *Ph, const double *u0, doub
 // other; one warp then forms the round's field records, one lane per cell (an FP64 warp
 // instruction costs the same for one lane as for 32), while the others begin the next round
 // in the second buffer.  VEC: f is aligned to a record of four planes, which is then read at once.
-template <typename Real, int DIM, bool TAB, bool VEC>
+template <typename Real, int DIM, bool VEC>
 __global__ void __launch_bounds__(32 * kWarps, kCtasPerSm) k_static(long long n_cells, int n_xi, int n_om,
                                                         const double *__restrict__ xi, const double *__restrict__ w,
                                                         const double *__restrict__ om, const double *__restrict__ wo,
@@ -344,6 +345,7 @@ __global__ void __launch_bounds__(32 * kWarps, kCtasPerSm) k_static(long long n_
                                                         double i_half_dr, double i_half_dv, double i_4sigma, int per_cta,
                                                         double *__restrict__ out) {
     constexpr int NM = n_moments<DIM>();
+    constexpr bool TAB = std::is_same<Real, float>::value;      // the FP32 sets are in shared memory
     constexpr int kRun = sizeof(Real) == 4 ? 256 : 128;   // velocities of a plain sum: 8 or 4 per lane, loaded at once
     static_assert(NM + 1 + DIM <= kRec && kWarps * kCpw == 32, "the sums of a cell; one lane per cell of a round");
     extern __shared__ float s_tab[];
@@ -490,7 +492,7 @@ int run(long long n_cells, int n_xi, const double *xi, const double *w, int n_om
         cudaStream_t s) {
     if (problem_bytes(n_cells, n_xi, n_om, sizeof(Real)) > kMaxBytes) return GSIS_ERR_INVALID_ARG;
     // kCtasPerSm CTAs per SM share the cells out evenly; few cells: one per warp
-    constexpr int slots = 152 * kCtasPerSm;
+    constexpr int slots = SMS * kCtasPerSm;
     const long long per = std::max<long long>(kWarps, (n_cells + slots - 1) / slots);
     const unsigned ctas = (unsigned)((n_cells + per - 1) / per);
     auto go = [&](auto kern, size_t smem) {
@@ -508,7 +510,7 @@ int run(long long n_cells, int n_xi, const double *xi, const double *w, int n_om
     auto go_wide = [&](auto kern) {
         // as many CTAs per cell as give every warp a run and leave no SM without work
         int cs = 1;
-        while (cs < 8 && n_cells * cs * 2 <= 2 * 152 && std::max(n_xi, n_om) > cs * kWarps * kWideRun) cs *= 2;
+        while (cs < 8 && n_cells * cs <= SMS && std::max(n_xi, n_om) > cs * kWarps * kWideRun) cs *= 2;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(n_cells * cs));
         cfg.blockDim = dim3(32 * kWarps);
@@ -531,7 +533,7 @@ int run(long long n_cells, int n_xi, const double *xi, const double *w, int n_om
     constexpr bool fp32 = std::is_same<Real, float>::value;
     if (fp32 ? tab > kMaxTable : n_cells <= kWideCells && std::max(n_xi, n_om) >= kWideSet)
         return vec ? go_wide(k_static_wide<Real, DIM, true>) : go_wide(k_static_wide<Real, DIM, false>);
-    return vec ? go(k_static<Real, DIM, fp32, true>, fp32 ? tab : 0) : go(k_static<Real, DIM, fp32, false>, fp32 ? tab : 0);
+    return vec ? go(k_static<Real, DIM, true>, fp32 ? tab : 0) : go(k_static<Real, DIM, false>, fp32 ? tab : 0);
 }
 
 }  // namespace
