@@ -2909,12 +2909,20 @@ static cudaError_t sweep_t(cudaStream_t s, const Geom<Real> &g, const Quad<Real>
         if (DIM < 3 && g.max_faces <= DIM + 1) return run(k_sweep_gas32<DIM, ORDER, RESID, DIM + 1>, dim3(128), bytes);
         return run(k_sweep_gas32<DIM, ORDER, RESID, MAXF>, dim3(128), bytes);
     } else {
-        // FP64 on fewer blocks than SMs (1-D meshes of a few hundred cells): a block's time is
-        // the FP64 pipe of the SM it runs on.  Gas: a cluster of eight CTAs per block (64 cells
-        // x 32 velocities: 72 us by one CTA of two rows, 53 of eight rows, 32 by the cluster;
-        // 800 x 64: 71, 55, 45).  Photons, with few instructions per value: eight rows.
+        // FP64 on fewer (block, chunk) pairs than SMs: a pair's time is the FP64 pipe of the SM it
+        // runs on.
+        const long long pairs = (long long)grid.x * grid.y;
         if constexpr (N == 4) {
-            if ((long long)grid.x * grid.y < SMS) {
+            // Gas: a cluster of eight CTAs per pair, while the chip holds all clusters at once (51,
+            // 36 or 15 of them at three, two or one CTA per SM; a second wave costs as much as the
+            // first) and the blocks have cells for the CTAs.  us of the 1-D sweep, cluster and one
+            // CTA of eight rows: blocks of 16 cells 32 and 55 at 10 pairs, 45 and 55 at 50, 72 and
+            // 55 at 57; of 32, 65 and 102 at 24, 118 and 102 at 38; of 64, 99 and 198 at 10, 193 and
+            // 198 at 19, 383 and 198 at 50; of 8, 33 and 33 at 50; of 4, 21 and 22 at 10, 28 and 22
+            // at 38; of 1, 18 and 16 at 10.
+            const int per_sm = std::min<int>(3, 228 * 1024 / (smem + 1024));
+            const int fit = per_sm == 3 ? 51 : per_sm == 2 ? 36 : 15;
+            if (g.block >= 4 && pairs <= std::min(fit, 4 * g.block)) {
                 auto kern = k_sweep<Real, N, DIM, ORDER, RESID, SROWS, 8>;
                 cudaError_t e = allow_smem(kern);
                 if (e != cudaSuccess) return e;
@@ -2932,9 +2940,11 @@ static cudaError_t sweep_t(cudaStream_t s, const Geom<Real> &g, const Quad<Real>
                 e = cudaLaunchKernelEx(&cfg, kern, g, q, coef, bcoef, f_in, fface, f_out, partial);
                 return e != cudaSuccess ? e : cudaGetLastError();
             }
-        } else if constexpr (std::is_same<Real, double>::value) {
-            if ((long long)grid.x * grid.y < SMS)
-                return run(k_sweep<Real, N, DIM, ORDER, RESID, 8>, dim3(SV, 8), smem);
+        }
+        // one CTA of eight rows (blocks of 16 cells at 100 pairs: 55 us, of two rows 59); photons,
+        // with few instructions per value, always
+        if constexpr (std::is_same<Real, double>::value) {
+            if (pairs < SMS) return run(k_sweep<Real, N, DIM, ORDER, RESID, 8>, dim3(SV, 8), smem);
         }
         return run(k_sweep<Real, N, DIM, ORDER, RESID>, dim3(SV, SROWS), smem);
     }

@@ -165,3 +165,24 @@ def test_few_cells_of_large_sets_fill_the_chip(G, dim, precision, n_cells, n_xi,
     assert G.fake.fake_launch_count() == 1
     G.fake.fake_launch(0, C.byref(grid), C.byref(block))
     assert grid.value >= ctas and block.value == 256
+
+
+@pytest.mark.parametrize("block,pairs,clusters", [
+    (1, 4, False), (3, 10, False), (2, 100, False), (4, 16, True), (4, 17, False), (16, 51, True), (16, 52, False),
+    (16, 151, False), (16, 152, False), (32, 36, True), (32, 37, False), (64, 15, True), (64, 16, False), (64, 52, False)])
+def test_fp64_sweep_takes_clusters_while_the_chip_holds_them(G, block, pairs, clusters):
+    # one chunk of velocities: as many pairs as relaxation blocks.  More clusters than fit at once
+    # (or with more CTAs than cells) took up to 4.6 times as long as one CTA per pair
+    wl = gi.workloads.with_solver(gi.workloads.slab(n_cells=block * pairs, n_xi=16, n_mu=8), precision="fp64",
+                                  order=1, relax_block=block)
+    ctx = _create(G, wl)
+    G.fake.fake_reset()
+    try:
+        assert G.load().gsis_step_async(ctx, G.GSIS_MODE_CIS) == G.GSIS_OK
+    finally:
+        G.gsis_destroy(ctx)
+    grid, threads, grids = C.c_int(), C.c_int(), []
+    for k in range(G.fake.fake_launch_count()):
+        if b"7k_sweepIdLi4" in G.fake.fake_launch(k, C.byref(grid), C.byref(threads)):
+            grids.append(grid.value)
+    assert grids == [8 * pairs if clusters else pairs]
