@@ -1281,7 +1281,6 @@ __device__ __forceinline__ float rcp_refined(float x) {
 // Shared memory of a k_sweep_gas32 CTA.
 template <int DIM>
 struct S32 {
-    static constexpr int ROWS = 4;                        // warps: a lane takes velocities tx and tx + 32
     static constexpr int NK = (6 + 3 * DIM + 3) / 4;      // float4 of a Maxwellian: S B A A2 | K1 K2, then Q R1 R2 per axis
     static constexpr int CF = 2 + 3 * NK;                 // float4 of a cell's coefficients: u, Maxwellians, rates
     static constexpr int XS = DIM + 1;
@@ -1359,13 +1358,16 @@ __device__ __forceinline__ void reference32(const float4 *__restrict__ C, const 
 // spills: 396 us; at four 358).  About 290 instructions per velocity, 497 before: 20 000
 // triangles x 784 velocities at order 2 354 -> 292 us, 40 000 x 2 304 1.91 -> 1.56 ms, 10 185
 // tetrahedra x 4 096 946 -> 814 us.
-template <int DIM, int ORDER, bool RESID, int FM>
-__global__ void __launch_bounds__(32 * S32<DIM>::ROWS, FM < MAXF ? 6 : 5)
+// ROWS: its warps; one where a block has no more than two cells, which leave the others without
+// work and the SM without warps (10 000 tetrahedra x 1 728, blocks of one cell, order 1: 690 us
+// with four, 241 with one; of two cells 403 and 172).
+template <int DIM, int ORDER, bool RESID, int FM, int ROWS>
+__global__ void __launch_bounds__(32 * ROWS, (FM < MAXF ? 24 : 20) / ROWS)
     k_sweep_gas32(Geom<float> g, Quad<float> q, const float *__restrict__ coef, const float *__restrict__ bcoef,
                   const float *__restrict__ f_in, const float *__restrict__ fface, float *__restrict__ f_out,
                   float *__restrict__ partial) {
     using S = S32<DIM>;
-    constexpr int ROWS = S::ROWS, NT = 32 * ROWS;
+    constexpr int NT = 32 * ROWS;
     extern __shared__ float4 smem32[];
     float4 *R = smem32;                                   // [block][SV]
     float4 *Fa = R + g.block * SV;                        // [block][MAXF]: n, S/V (3-D: S/V n), source
@@ -1450,10 +1452,10 @@ __global__ void __launch_bounds__(32 * S32<DIM>::ROWS, FM < MAXF ? 6 : 5)
                 o[1 + k * S::NK + a] = make_float4(w[4 * a], w[4 * a + 1], w[4 * a + 2], w[4 * a + 3]);
         }
     }
-    if (threadIdx.x < SV) {
+    for (int t = threadIdx.x; t < SV; t += NT) {
 #pragma unroll
-        for (int a = 0; a < DIM; ++a) sxi[a * SV + threadIdx.x] = q.x[a * stride + chunk * SV + threadIdx.x];
-        sxi[DIM * SV + threadIdx.x] = q.w[chunk * SV + threadIdx.x];
+        for (int a = 0; a < DIM; ++a) sxi[a * SV + t] = q.x[a * stride + chunk * SV + t];
+        sxi[DIM * SV + t] = q.w[chunk * SV + t];
     }
     __syncthreads();
 
@@ -2906,8 +2908,9 @@ static cudaError_t sweep_t(cudaStream_t s, const Geom<Real> &g, const Quad<Real>
         // segments and triangles, whose faces' values leave room for one more CTA per SM, or
         // any cells (the 20 000-triangle cavity as "any cells": 326 us, as triangles 306 us)
         const size_t bytes = S32<DIM>::bytes(g.block);
-        if (DIM < 3 && g.max_faces <= DIM + 1) return run(k_sweep_gas32<DIM, ORDER, RESID, DIM + 1>, dim3(128), bytes);
-        return run(k_sweep_gas32<DIM, ORDER, RESID, MAXF>, dim3(128), bytes);
+        if (g.block <= 2) return run(k_sweep_gas32<DIM, ORDER, RESID, MAXF, 1>, dim3(32), bytes);
+        if (DIM < 3 && g.max_faces <= DIM + 1) return run(k_sweep_gas32<DIM, ORDER, RESID, DIM + 1, 4>, dim3(128), bytes);
+        return run(k_sweep_gas32<DIM, ORDER, RESID, MAXF, 4>, dim3(128), bytes);
     } else {
         // FP64 on fewer (block, chunk) pairs than SMs: a pair's time is the FP64 pipe of the SM it
         // runs on.

@@ -186,3 +186,23 @@ def test_fp64_sweep_takes_clusters_while_the_chip_holds_them(G, block, pairs, cl
         if b"7k_sweepIdLi4" in G.fake.fake_launch(k, C.byref(grid), C.byref(threads)):
             grids.append(grid.value)
     assert grids == [8 * pairs if clusters else pairs]
+
+
+@pytest.mark.parametrize("name", ["slab", "cavity", "capsule"])
+@pytest.mark.parametrize("block,threads", [(1, 32), (2, 32), (3, 128), (16, 128)])
+def test_fp32_sweep_has_no_idle_warps_on_small_blocks(G, name, block, threads):
+    # four warps on a block of one cell left three of them idle, and the SM short of warps
+    base = {"slab": lambda: gi.workloads.slab(n_cells=12, n_xi=16, n_mu=8),
+            "cavity": lambda: gi.workloads.cavity(n_side=4, n_v=8),
+            "capsule": lambda: gi.workloads.capsule(n=4, n_v=6, n_polar=4, n_azim=4)}[name]()
+    ctx = _create(G, gi.workloads.with_solver(base, precision="fp32", order=2, relax_block=block))
+    G.fake.fake_reset()
+    try:
+        assert G.load().gsis_step_async(ctx, G.GSIS_MODE_CIS) == G.GSIS_OK
+    finally:
+        G.gsis_destroy(ctx)
+    grid, n, found = C.c_int(), C.c_int(), []
+    for k in range(G.fake.fake_launch_count()):
+        if b"k_sweep_gas32" in G.fake.fake_launch(k, C.byref(grid), C.byref(n)):
+            found.append(n.value)
+    assert found == [threads]
