@@ -51,7 +51,7 @@ METRIC = "DVM cell-velocity updates/s (% HBM roofline); time-to-steady vs plain 
 # SHA-256 of the kernel sources the capture ran; the figure is reported only while those
 # sources are unchanged, and as null once a kernel has changed since the counters were taken.
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "sweep_gas_cavity20k_order2.md")
-KERNEL_SOURCES = ("kernels.cu", "gsis_impl.cuh", "tc_moments.cuh")
+KERNEL_SOURCES = ("kernels.cu", "gsis_impl.cuh", "tc_moments.cuh", "fp64.cuh")
 
 
 def kernel_sources_sha256(csrc=None):

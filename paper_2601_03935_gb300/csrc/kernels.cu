@@ -678,9 +678,8 @@ __global__ void __launch_bounds__(32 * SLOPE_ROWS, 4) k_slopes32(Geom<float> g, 
 // patterns, every face's Delta_2 = grad . (x_f - x_j) is formed once and serves the limiter
 // and the reconstruction f_j + phi Delta_2, and each plane takes one reciprocal: the smaller
 // of the two quotients num / den of phi is found by cross-multiplication (all four terms
-// are positive).  About 220 instructions per update in 2-D; k_slopes compiled for double
-// took 370 (divisions 9 each, comparisons 1 to 2).  20 000 triangles x 784 velocities,
-// order 2: 11.1 -> 5.9 ms.
+// are positive).  About 220 instructions per update in 2-D, 370 before (divisions 9 each,
+// comparisons 1 to 2).  20 000 triangles x 784 velocities, order 2: 11.1 -> 5.9 ms.
 template <int N, int DIM>
 __global__ void __launch_bounds__(32 * SLOPE_ROWS) k_slopes64(Geom<double> g, int n, int n_pad,
                                                               const double *__restrict__ xq,
@@ -1355,7 +1354,7 @@ __device__ __forceinline__ void reference32(const float4 *__restrict__ C, const 
 // a serial chain over the block's cells in one warp, takes a quarter of the time (two warps of
 // one velocity per lane, or reading ahead of it, took longer: more instructions).  Six CTAs of
 // 80 registers per SM where no cell has more faces than a triangle, else five of 96 (at six,
-// spills: 396 us; at four 358).  About 290 instructions per velocity, 497 before: 20 000
+// spills: 396 us; at four 358).  About 300 instructions per velocity, 497 before: 20 000
 // triangles x 784 velocities at order 2 354 -> 292 us, 40 000 x 2 304 1.91 -> 1.56 ms, 10 185
 // tetrahedra x 4 096 946 -> 814 us.
 // ROWS: its warps; one where a block has no more than two cells, which leave the others without
