@@ -178,14 +178,14 @@ __device__ __forceinline__ void add_gas_run(const Vel &vel, const Four *fc, int 
     Real acc[NM];
 #pragma unroll
     for (int k = 0; k < NM; ++k) acc[k] = Real(0);
-    // the run's loads first; past the set's end the last velocity with no weight
+    // the run's loads first; past the set's end the last velocity again, which is not used
     Four fr[RUN / 32];
 #pragma unroll
     for (int h = 0; h < RUN / 32; ++h) fr[h] = fc[min(v0 + 32 * h + lane, n_xi - 1)];
 #pragma unroll
     for (int h = 0; h < RUN / 32; ++h) {
-        if (v0 + 32 * h >= n_xi) break;
-        const int v = min(v0 + 32 * h + lane, n_xi - 1);
+        const int v = v0 + 32 * h + lane;
+        if (v >= n_xi) break;
         const Four &fv = fr[h];
         Real c[DIM], c2 = Real(0);
 #pragma unroll
@@ -193,7 +193,7 @@ __device__ __forceinline__ void add_gas_run(const Vel &vel, const Four *fc, int 
             c[a] = vel.minus(v, a, u[a]);
             c2 = fma(c[a], c[a], c2);
         }
-        const Real wv = v0 + 32 * h + lane < n_xi ? vel.weight(v) : Real(0), w0 = wv * fv.v[0];
+        const Real wv = vel.weight(v), w0 = wv * fv.v[0];
         Real wc[DIM];
         int k = 0;
         acc[k++] += w0;
